@@ -202,7 +202,7 @@ int pd_bind_arena(pd_ctx *ctx, void *device_arena, size_t bytes);
  * the context stream; the step sequence runs as captured CUDA graphs.  The
  * contact neighbourhoods S^nbr (Algorithm 1, nodes within R_c) are taken from
  * per-node candidate lists of radius R_c + skin (skin = 0.1 R_c), rebuilt by
- * a hash-grid counting sort in a conditional graph node only in steps where
+ * a grid counting sort in a conditional graph node only in steps where
  * some node has moved more than 0.45 skin since the last rebuild; every pair
  * is still tested against R_c exactly, so the forces are those of a full
  * search.  status[PD_STATUS_REBUILDS] counts the rebuilds.
@@ -278,7 +278,7 @@ int pd_set_wait_test(pd_ctx *ctx, int withhold_block, long long max_spins);
 /* Scalar facts of the context (out has 15 slots): out[0] N, out[1] directed
  * bonds, out[2] grains, out[3] h_min, out[4] R_c, out[5] K_n (aggregate 0),
  * out[6] dt, out[7] completed steps, out[8] max bonds per node, out[9] contact
- * hash buckets, out[10] step path (0 graph of kernels, 1 persistent kernel),
+ * grid cells, out[10] step path (0 graph of kernels, 1 persistent kernel),
  * out[11] threads per node, out[12] threads per block of the persistent
  * kernel, out[13] aggregates, out[14] bond-network templates (grains of one
  * shape meshed at the same h/R share one lattice and one bond network). */
@@ -350,7 +350,7 @@ int pd_set_path(pd_ctx *ctx, int mode, int lanes, int block);
 
 /* ---- kernel timing (instrumentation) ----------------------------------------- */
 #define PD_TIMER_PREDICT 0      /* memset + displacement update / positions / bucket counts */
-#define PD_TIMER_BIN 1          /* scan + scatter of the contact hash grid               */
+#define PD_TIMER_BIN 1          /* scan + scatter of the contact grid                    */
 #define PD_TIMER_FORCE 2        /* force + acceleration + velocity kernel                */
 #define PD_TIMER_COUNT 4
 

@@ -1,6 +1,6 @@
 // pd_common.cu -- precision-independent kernels of the multi-kernel step path:
-// displacement update and positions (Algorithm 1), contact binning (hash-grid
-// counting sort: bucket counts, device-wide exclusive scan, scatter),
+// displacement update and positions (Algorithm 1), contact binning (grid
+// counting sort: cell counts, device-wide exclusive scan, scatter),
 // positions for readout and the diagnostics reductions; plus the launch
 // dispatchers.  Compiled without FMA contraction.
 #include <algorithm>
@@ -52,22 +52,21 @@ __global__ void __launch_bounds__(kBlock) k_predict(DevPtrs d, KParams k, int vi
     }
 }
 
-// Rebuild of the contact candidate lists: bucket counts, a device-wide
+// Rebuild of the contact candidate lists: cell counts, a device-wide
 // exclusive scan of the counts (reduce, top, apply), the counting-sort
 // scatter and the lists (the list kernel clears the counts for the next
 // rebuild).  Every
 // kernel returns at once when the rebuild flag is clear.
 __global__ void __launch_bounds__(kBlock) k_bin(DevPtrs d, KParams k) {
     if (!*(volatile int *)d.rebuild) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < k.N) bin_node<false>(d, k, i);
+    bin_nodes<false>(d, k, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
 __global__ void __launch_bounds__(kBlock) k_build_list(DevPtrs d, KParams k) {
     if (!*(volatile int *)d.rebuild) return;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) atomicAdd(&d.status[PD_STATUS_REBUILDS], 1);
-    // the bucket counts were consumed by the scan: zero them for the next
+    // the cell counts were consumed by the scan: zero them for the next
     // rebuild (the grid covers max(N, T / 4) threads: one int4 per thread)
     if ((unsigned)i < k.T / 4) reinterpret_cast<int4 *>(d.count)[i] = make_int4(0, 0, 0, 0);
     if (i < k.N) build_list_node<false>(d, k, i);
@@ -147,11 +146,11 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_top(int *blocksums, int n
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_apply(int *count, const int *__restrict__ blocksums,
-                                                             int *start, int *cursor, unsigned T, int N,
+                                                             int *start, unsigned T, int N,
                                                              const int *flag) {
     if (!*(volatile const int *)flag) return;
     __shared__ int sm[33];
-    // T is a power of two >= 1024 and bases are multiples of 4: whole int4 per thread
+    // T and the bases are multiples of 4: whole int4 per thread
     const size_t base = (size_t)blockIdx.x * kScanTile + (size_t)threadIdx.x * kScanItems;
     int4 c4 = make_int4(0, 0, 0, 0);
     if (base < T) {
@@ -163,16 +162,13 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(int *count, const i
     if (base < T) {
         const int4 st = make_int4(v[0] + off, v[1] + off, v[2] + off, v[3] + off);
         *reinterpret_cast<int4 *>(start + base) = st;
-        *reinterpret_cast<int4 *>(cursor + base) = st;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) start[T] = N;
 }
 
 __global__ void __launch_bounds__(kBlock) k_scatter(DevPtrs d, KParams k) {
     if (!*(volatile int *)d.rebuild) return;
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= k.N) return;
-    scatter_node<false>(d, k, i);
+    scatter_nodes<false>(d, k, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
 __global__ void __launch_bounds__(kBlock) k_positions(DevPtrs d, KParams k) {
@@ -360,11 +356,11 @@ cudaError_t launch_narrow(const double2 *src, float2 *dst, size_t n, cudaStream_
 }
 
 cudaError_t launch_rebuild(const DevPtrs &d, const KParams &k, cudaStream_t s) {
-    const int nb = nblk(k.T, kScanTile), nn = nblk(k.N, kBlock);
+    const int nb = nblk(k.T, kScanTile), nn = nblk(k.N, kBlock * kBinBatch);
     k_bin<<<nn, kBlock, 0, s>>>(d, k);
     k_scan_reduce<<<nb, kScanThreads, 0, s>>>(d.count, d.blocksums, k.T, d.rebuild);
     k_scan_top<<<1, kScanThreads, 0, s>>>(d.blocksums, nb, d.rebuild);
-    k_scan_apply<<<nb, kScanThreads, 0, s>>>(d.count, d.blocksums, d.start, d.cursor, k.T, k.N, d.rebuild);
+    k_scan_apply<<<nb, kScanThreads, 0, s>>>(d.count, d.blocksums, d.start, k.T, k.N, d.rebuild);
     k_scatter<<<nn, kBlock, 0, s>>>(d, k);
     k_build_list<<<nblk(std::max<long long>(k.N, k.T / 4), kBlock), kBlock, 0, s>>>(d, k);
     return cudaGetLastError();

@@ -3,6 +3,8 @@
 // contact / wall / precision helpers they use.
 #pragma once
 
+#include <type_traits>
+
 #include "pd_internal.h"
 #include "peridem.h"
 
@@ -23,11 +25,15 @@ __device__ __forceinline__ T ldm(const T *p) {
 // ---------------------------------------------------------------------------
 // contact search grid
 
-// Square cells of side >= R_c hashed (with the aggregate id) into T buckets
-// (T a power of two >= 2N): every pair closer than R_c lies in the 3x3 cell
-// block around either node; aliasing cells only add candidates, which the
-// distance test rejects.
-// Hash-grid cell index of a coordinate (inv_cell = 1 / cell side).  Only the
+// Square cells of side >= R_c + skin.  Each aggregate has a grid of gw x gh
+// cells in row order behind its base; a cell coordinate outside the grid wraps
+// around (the grid covers the wall box unless that has more than four cells per
+// node).  Every pair closer than R_c + skin lies in the 3 x 3 cell block around
+// either node; wrapped cells only add candidates, which the distance test
+// rejects.  The three cells of a row of the block are neighbours in memory, and
+// so are those of nearby nodes (a hash of the cell instead scattered every
+// node's nine buckets over the whole table).
+// Grid cell of a coordinate (inv_cell = 1 / cell side).  Only the
 // binning kernel calls this; the force kernels read the stored cells.
 __device__ __forceinline__ int cell_coord_f(float x, float inv_cell) {
     float f = floorf(x * inv_cell);
@@ -43,10 +49,13 @@ __device__ __forceinline__ int cell_coord(double x, double origin, double inv_ce
     return (int)f;
 }
 
-constexpr unsigned kHashX = 73856093u, kHashY = 19349663u, kHashA = 83492791u;
-
-__device__ __forceinline__ unsigned cell_bucket(int cx, int cy, int agg, unsigned T) {
-    return ((unsigned)cx * kHashX ^ (unsigned)cy * kHashY ^ (unsigned)agg * kHashA) & (T - 1u);
+__device__ __forceinline__ int wrap_cell(int c, int n) {
+    if ((unsigned)c < (unsigned)n) return c;
+    const int r = c % n;
+    return r < 0 ? r + n : r;
+}
+__device__ __forceinline__ int grid_cell(const AggParams &A, int cx, int cy) {
+    return A.gbase + wrap_cell(cy, A.gh) * A.gw + wrap_cell(cx, A.gw);
 }
 
 // ---------------------------------------------------------------------------
@@ -191,55 +200,65 @@ __device__ __forceinline__ void corner_region_stable(double di, double dj, doubl
 // the S_li cap S_lj term (inclusion-exclusion); friction and damping follow by
 // substituting e -> e^l, V_y -> |S_l|, p(y) -> c_l.  A node past a wall is
 // treated as touching it and counted in status[PD_STATUS_PENETRATION].
+//
+// Distance of the node from wall l, not below 0 (the node past the wall: past).
+__device__ __forceinline__ double wall_distance(const AggParams &A, int l, double t, double px, double py, bool &past) {
+    const double w = A.w0[l] + A.wv[l] * t;
+    const double x = l < 2 ? px : py;
+    const double d = (l & 1) ? w - x : x - w;
+    past = d < 0.0;
+    return past ? 0.0 : d;
+}
+// The own-segment term of wall l at distance d.
+__device__ __forceinline__ void wall_single64(const KParams &k, const AggParams &A, double Kn, double rho, int l, double d,
+                                              double vx, double vy, double Vx, double &gx, double &gy) {
+    gx = gy = 0.0;
+    const double Rc = A.Rc;
+    if (!(d < Rc)) return;
+    double Ar, gap;
+    wall_segment_stable(d, Rc, Ar, gap);
+    if (!(Ar > 0.0) || !(gap > 0.0)) return;
+    const double Fr = Kn * gap * Vx * Ar;
+    const double ex = l == 0 ? -1.0 : (l == 1 ? 1.0 : 0.0), ey = l == 2 ? -1.0 : (l == 3 ? 1.0 : 0.0);
+    const double wvx = (l < 2) ? A.wv[l] : 0.0, wvy = (l < 2) ? 0.0 : A.wv[l];
+    gx = -Fr * ex, gy = -Fr * ey;
+    damping_friction64(k, Kn, rho, rho, ex, ey, vx - wvx, vy - wvy, Fr, Vx, Ar, gx, gy);
+}
+// The term of corner c, (x_lo|x_hi) x (y_lo|y_hi), at distances di, dj from its walls.
+__device__ __forceinline__ void wall_corner64(const KParams &k, const AggParams &A, double Kn, double rho, int c, double di,
+                                              double dj, double vx, double vy, double Vx, double &gx, double &gy) {
+    gx = gy = 0.0;
+    const double Rc = A.Rc;
+    const int i = c >> 1, j = 2 + (c & 1);
+    if (!(di < Rc) || !(dj < Rc) || !(sqrt(di * di + dj * dj) < Rc)) return;
+    double Ar, lx, ly;
+    corner_region_stable(di, dj, Rc, Ar, lx, ly);
+    if (!(Ar > 0.0)) return;
+    const double cx = (i == 0 ? -1.0 : 1.0) * lx, cy = (j == 2 ? -1.0 : 1.0) * ly;
+    const double cd = sqrt(cx * cx + cy * cy);
+    if (!(cd < Rc) || !(cd > 0.0)) return;
+    const double ux = cx / cd, uy = cy / cd;
+    const double Fr = Kn * (Rc - cd) * Vx * Ar;
+    gx = -Fr * ux, gy = -Fr * uy;
+    damping_friction64(k, Kn, rho, rho, ux, uy, vx - A.wv[i], vy - A.wv[j], Fr, Vx, Ar, gx, gy);
+}
 __device__ __forceinline__ void wall_terms64(const KParams &k, const AggParams &A, double Kn, double rho, double t,
                                              double px, double py, double vx, double vy, double Vx,
                                              double (&single)[4][2], double (&corner)[4][2], int *status) {
-    const double Rc = A.Rc;
-    double d[4], ex[4], ey[4];
-    d[0] = px - (A.w0[0] + A.wv[0] * t); ex[0] = -1.0; ey[0] = 0.0;
-    d[1] = (A.w0[1] + A.wv[1] * t) - px; ex[1] = 1.0;  ey[1] = 0.0;
-    d[2] = py - (A.w0[2] + A.wv[2] * t); ex[2] = 0.0;  ey[2] = -1.0;
-    d[3] = (A.w0[3] + A.wv[3] * t) - py; ex[3] = 0.0;  ey[3] = 1.0;
+    double d[4];
     bool near = false;
 #pragma unroll
     for (int l = 0; l < 4; ++l) {
         single[l][0] = single[l][1] = corner[l][0] = corner[l][1] = 0.0;
-        if (d[l] < 0.0) {
-            if (status) atomicAdd(&status[PD_STATUS_PENETRATION], 1);
-            d[l] = 0.0;
-        }
-        near |= d[l] < Rc;
+        bool past;
+        d[l] = wall_distance(A, l, t, px, py, past);
+        if (past && status) atomicAdd(&status[PD_STATUS_PENETRATION], 1);
+        near |= d[l] < A.Rc;
     }
     if (!near) return;
-    for (int l = 0; l < 4; ++l) {
-        if (!(d[l] < Rc)) continue;
-        double Ar, gap;
-        wall_segment_stable(d[l], Rc, Ar, gap);
-        if (!(Ar > 0.0) || !(gap > 0.0)) continue;
-        double Fr = Kn * gap * Vx * Ar;
-        double wvx = (l < 2) ? A.wv[l] : 0.0, wvy = (l < 2) ? 0.0 : A.wv[l];
-        double gx = -Fr * ex[l], gy = -Fr * ey[l];
-        damping_friction64(k, Kn, rho, rho, ex[l], ey[l], vx - wvx, vy - wvy, Fr, Vx, Ar, gx, gy);
-        single[l][0] = gx;
-        single[l][1] = gy;
-    }
-    for (int c = 0; c < 4; ++c) {
-        const int i = c >> 1, j = 2 + (c & 1);  // (x_lo|x_hi) x (y_lo|y_hi)
-        double di = d[i], dj = d[j];
-        if (!(sqrt(di * di + dj * dj) < Rc)) continue;
-        double Ar, lx, ly;
-        corner_region_stable(di, dj, Rc, Ar, lx, ly);
-        if (!(Ar > 0.0)) continue;
-        double cx = lx * ex[i] + ly * ex[j], cy = lx * ey[i] + ly * ey[j];
-        double cd = sqrt(cx * cx + cy * cy);
-        if (!(cd < Rc) || !(cd > 0.0)) continue;
-        double ux = cx / cd, uy = cy / cd;
-        double Fr = Kn * (Rc - cd) * Vx * Ar;
-        double gx = -Fr * ux, gy = -Fr * uy;
-        damping_friction64(k, Kn, rho, rho, ux, uy, vx - A.wv[i], vy - A.wv[j], Fr, Vx, Ar, gx, gy);
-        corner[c][0] = gx;
-        corner[c][1] = gy;
-    }
+    for (int l = 0; l < 4; ++l) wall_single64(k, A, Kn, rho, l, d[l], vx, vy, Vx, single[l][0], single[l][1]);
+    for (int c = 0; c < 4; ++c)
+        wall_corner64(k, A, Kn, rho, c, d[c >> 1], d[2 + (c & 1)], vx, vy, Vx, corner[c][0], corner[c][1]);
 }
 
 // Wall force on a node at (px, py) with velocity (vx, vy) and volume Vx:
@@ -298,15 +317,21 @@ __device__ __forceinline__ float ff_diff(float ah, float al, float bh, float bl)
     return __fsub_rn(ah, bh) + (al - bl);
 }
 
-// Square root and quotient of the bond loop by the approximate special-function
+// Square root and reciprocal of the bond loop by the approximate special-function
 // instructions (relative error about 2^-22) instead of the correctly rounded
 // sequences: the FP32-split bond force carries a 1e-5 tolerance, and stretches
 // within 1e-4 of the critical one are re-decided in FP64 after the loop, so
-// the break decisions do not change.  (The operands here are far from the
-// ranges where __fdividef returns 0.)
+// the break decisions do not change.  The flush-to-zero forms are one
+// instruction each; the others scale subnormal operands, which take lattices
+// finer than 1e-12 m to occur.
 __device__ __forceinline__ float sqrt_approx(float x) {
     float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
 
@@ -572,19 +597,26 @@ __device__ __forceinline__ float4 *cur_pq(const DevPtrs &d) {
     else return d.pq;
 }
 
+// What a node's velocity and displacement update reads besides its forces.
+struct Update32 {
+    double2 v, u, xs;       // velocity, displacement, reference position + shift
+    float4 sref;            // position at the last rebuild
+    float2 a;               // previous acceleration
+    int2 cell;
+};
+
 // Shifted position xs + u of node i as a float-float pair into q_out[i], and
 // the rebuild test: the displacement since the last rebuild from the float-float
-// positions (error ~1e-7 of the displacement, far below the trigger's margin).
-template <bool PERSIST>
-__device__ __forceinline__ bool position32(const DevPtrs &d, const KParams &k, int i, double2 u, float4 *q_out) {
-    const double2 xs = __ldg(&d.xs[i]);
+// positions (error ~1e-7 of the displacement, far below the trigger's margin);
+// xs, r: the node's reference position + shift and its position at the last rebuild.
+__device__ __forceinline__ bool position32(const DevPtrs &d, const KParams &k, int i, double2 u, double2 xs, float4 r,
+                                           float4 *q_out) {
     const double qx = xs.x + u.x, qy = xs.y + u.y;
     // float-float split by bit operations (no FP64-pipe conversions)
     float4 q;
     dbl_to_ff(qx, q.x, q.z);
     dbl_to_ff(qy, q.y, q.w);
     q_out[i] = q;
-    const float4 r = ldm<PERSIST>(&d.sref[i]);
     const float ex = __fsub_rn(q.x, r.x) + (q.z - r.z), ey = __fsub_rn(q.y, r.y) + (q.w - r.w);
     return !(ex * ex + ey * ey <= k.dmax2);
 }
@@ -595,13 +627,13 @@ __device__ __forceinline__ bool position32(const DevPtrs &d, const KParams &k, i
 // kSkinTrigger * skin since the last rebuild.  The persistent kernel's velocity
 // update calls it for the next step with the same operands that the update
 // phase would load, so both give the same bits.
-template <bool PERSIST>
 __device__ __forceinline__ bool advance_node32(const DevPtrs &d, const KParams &k, int i, double2 u, double2 v,
-                                               float ax, float ay, double2 *u_out, float4 *q_out) {
+                                               float ax, float ay, double2 xs, float4 r, double2 *u_out,
+                                               float4 *q_out) {
     u.x = fma(k.dt, v.x, fma(k.half_dt2, f2d_bits(ax), u.x));
     u.y = fma(k.dt, v.y, fma(k.half_dt2, f2d_bits(ay), u.y));
     u_out[i] = u;
-    return position32<PERSIST>(d, k, i, u, q_out);
+    return position32(d, k, i, u, xs, r, q_out);
 }
 
 // Algorithm 1: u <- u + dt v + dt^2/2 a (when advancing) and the positions.
@@ -621,12 +653,14 @@ __device__ __forceinline__ bool predict_node(const DevPtrs &d, const KParams &k,
     double2 u = advance ? ldm<PERSIST>(&d.ub[vin][i]) : ldm<PERSIST>(&uc[i]);
     const float dmax2 = k.dmax2;
     if (d.pq) {
+        const double2 xs = __ldg(&d.xs[i]);
+        const float4 r = ldm<PERSIST>(&d.sref[i]);
         if (advance) {
             const double2 v = ldm<PERSIST>(&d.v[vin][i]);
             const float2 a = ldm<PERSIST>(&d.af[i]);       // FP32 acceleration, widened exactly
-            return advance_node32<PERSIST>(d, k, i, u, v, a.x, a.y, uc, cur_pq<PERSIST>(d));
+            return advance_node32(d, k, i, u, v, a.x, a.y, xs, r, uc, cur_pq<PERSIST>(d));
         }
-        return position32<PERSIST>(d, k, i, u, cur_pq<PERSIST>(d));
+        return position32(d, k, i, u, xs, r, cur_pq<PERSIST>(d));
     }
     if (advance) {
         // explicit round-to-nearest operations: never contracted into FMAs
@@ -651,28 +685,47 @@ __device__ __forceinline__ double2 position64(const DevPtrs &d, int i) {
     return make_double2(__dadd_rn(X.x, u.x), __dadd_rn(X.y, u.y));
 }
 
-// Rebuild, step 1: hash-grid cell and bucket of node i at its current
-// position, counted into its bucket.
+// Grid cell of node i at its current position.
 template <bool PERSIST>
-__device__ __forceinline__ void bin_node(const DevPtrs &d, const KParams &k, int i) {
-    const int ag = __ldg(&d.g_agg[__ldg(&d.grain[i])]);
-    const AggParams &A = d.agg[ag];
-    int cx, cy;
+__device__ __forceinline__ int2 node_cell(const DevPtrs &d, const AggParams &A, int i) {
     if (d.pq) {
         // FP32-split: the cell from the shifted float position (error below 1e-3
         // cell; the cells of this path are 0.4 % wider to absorb it)
         const float4 q = ldm<PERSIST>(&cur_pq<PERSIST>(d)[i]);
-        cx = cell_coord_f((q.x - A.oxs) + q.z, A.inv_cell_f);
-        cy = cell_coord_f((q.y - A.oys) + q.w, A.inv_cell_f);
-    } else {
-        const double2 p = ldm<PERSIST>(&d.p[i]);
-        cx = cell_coord(p.x, A.ox, A.inv_cell);
-        cy = cell_coord(p.y, A.oy, A.inv_cell);
+        return make_int2(cell_coord_f((q.x - A.oxs) + q.z, A.inv_cell_f), cell_coord_f((q.y - A.oys) + q.w, A.inv_cell_f));
     }
-    d.cell[i] = make_int2(cx, cy);
-    unsigned b = cell_bucket(cx, cy, ag, k.T);
-    d.key[i] = (int)b;
-    atomicAdd(&d.count[b], 1);
+    const double2 p = ldm<PERSIST>(&d.p[i]);
+    return make_int2(cell_coord(p.x, A.ox, A.inv_cell), cell_coord(p.y, A.oy, A.inv_cell));
+}
+
+// Rebuild, step 1: cells of the nodes i, i + stride, ... (kBinBatch of them,
+// those below N), each counted into its cell; its rank there is its place in
+// the counting sort.  The batch's atomics are in flight together.
+constexpr int kBinBatch = 4;
+template <bool PERSIST>
+__device__ __forceinline__ void bin_nodes(const DevPtrs &d, const KParams &k, int i, int stride) {
+    int2 c[kBinBatch];
+    int key[kBinBatch], rank[kBinBatch];
+#pragma unroll
+    for (int m = 0; m < kBinBatch; ++m) {
+        const long long at = i + (long long)m * stride;
+        key[m] = -1;
+        if (at >= k.N) continue;
+        const AggParams &A = d.agg[__ldg(&d.g_agg[__ldg(&d.grain[at])])];
+        c[m] = node_cell<PERSIST>(d, A, (int)at);
+        key[m] = grid_cell(A, c[m].x, c[m].y);
+    }
+#pragma unroll
+    for (int m = 0; m < kBinBatch; ++m)
+        if (key[m] >= 0) rank[m] = atomicAdd(&d.count[key[m]], 1);
+#pragma unroll
+    for (int m = 0; m < kBinBatch; ++m) {
+        if (key[m] < 0) continue;
+        const size_t at = i + (size_t)m * stride;
+        d.cell[at] = c[m];
+        d.key[at] = key[m];
+        d.rank[at] = rank[m];
+    }
 }
 
 // L2 prefetch of a byte range, one 128-byte line per index of a grid stride g
@@ -728,7 +781,7 @@ __device__ __forceinline__ void prefetch_force_inputs(const DevPtrs &d, const KP
     }
 }
 
-// Hash-grid cells of the four walls of every aggregate at time t (written once
+// Grid cells of the four walls of every aggregate at time t (written once
 // per force evaluation by the threads of one block, one aggregate each): a node
 // two or more cells away from all of them is farther than R_c from every wall
 // and feels no wall force.
@@ -757,102 +810,73 @@ __device__ __forceinline__ bool cells_far_from_walls(int2 c, int4 w) {
     return c.x - w.x >= 2 && w.y - c.x >= 2 && c.y - w.z >= 2 && w.w - c.y >= 2;
 }
 
-// Counting-sort scatter of node i into its bucket, with its position record.
+// Counting-sort scatter of the nodes i, i + stride, ... (kBinBatch of them) into
+// their cells, with their position records.
 template <bool PERSIST>
-__device__ __forceinline__ void scatter_node(const DevPtrs &d, const KParams &k, int i) {
-    const int pos = atomicAdd(&d.cursor[ldm<PERSIST>(&d.key[i])], 1);
-    d.sorted[pos] = i;
-    uint4 rec;
-    if (k.fp32) {
-        const float4 q = ldm<PERSIST>(&cur_pq<PERSIST>(d)[i]);
-        rec = make_uint4(__float_as_uint(q.x), __float_as_uint(q.y), __float_as_uint(q.z), __float_as_uint(q.w));
-    } else {
-        const double2 p = ldm<PERSIST>(&d.p[i]);
-        rec = make_uint4((unsigned)__double2loint(p.x), (unsigned)__double2hiint(p.x), (unsigned)__double2loint(p.y),
-                         (unsigned)__double2hiint(p.y));
+__device__ __forceinline__ void scatter_nodes(const DevPtrs &d, const KParams &k, int i, int stride) {
+    int pos[kBinBatch];
+    uint4 rec[kBinBatch];
+#pragma unroll
+    for (int m = 0; m < kBinBatch; ++m) {
+        const long long at = i + (long long)m * stride;
+        pos[m] = -1;
+        if (at >= k.N) continue;
+        pos[m] = ldm<PERSIST>(&d.start[ldm<PERSIST>(&d.key[at])]) + ldm<PERSIST>(&d.rank[at]);
+        if (k.fp32) {
+            const float4 q = ldm<PERSIST>(&cur_pq<PERSIST>(d)[at]);
+            rec[m] = make_uint4(__float_as_uint(q.x), __float_as_uint(q.y), __float_as_uint(q.z), __float_as_uint(q.w));
+        } else {
+            const double2 p = ldm<PERSIST>(&d.p[at]);
+            rec[m] = make_uint4((unsigned)__double2loint(p.x), (unsigned)__double2hiint(p.x),
+                                (unsigned)__double2loint(p.y), (unsigned)__double2hiint(p.y));
+        }
     }
-    d.srec[pos] = rec;
+#pragma unroll
+    for (int m = 0; m < kBinBatch; ++m) {
+        if (pos[m] < 0) continue;
+        d.sorted[pos[m]] = (int)(i + (long long)m * stride);
+        d.srec[pos[m]] = rec[m];
+    }
 }
 
-// Rebuild, last step: the candidate list of node i -- every node y != i of
-// its aggregate with |p(y) - p(i)| < R_c + skin, gathered from the 3x3 block
-// of hash-grid cells around its cell (cells are wider than R_c + skin) and
-// kept in ascending node index -- and the position it was built at.  The
-// bucket records hold the positions in bucket order, so only nodes inside
-// the radius are looked up.  The three buckets of a row of the block are
-// walked as one range of records, so that the threads of a warp step through
-// rows rather than through nine buckets of different lengths.
-template <bool PERSIST>
-__device__ __forceinline__ void build_list_node(const DevPtrs &d, const KParams &k, int i) {
-    const int ag = __ldg(&d.g_agg[__ldg(&d.grain[i])]);
-    const AggParams &A = d.agg[ag];
-    const int2 cc = ldm<PERSIST>(&d.cell[i]);
-    const unsigned ha = (unsigned)ag * kHashA, mask = k.T - 1u;
-    unsigned hx[3], bk[9];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) hx[c] = (unsigned)(cc.x + c - 1) * kHashX;
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        const unsigned hy = (unsigned)(cc.y + r - 1) * kHashY ^ ha;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) bk[3 * r + c] = (hx[c] ^ hy) & mask;
+// sqrt(di^2 + dj^2) of the stencil offsets (compile-time for a fixed offset)
+__host__ __device__ constexpr float stn_sqrt_n(int n) {
+    return n == 1 ? 1.0f : (n == 2 ? 1.41421356f : (n == 4 ? 2.0f : (n == 5 ? 2.23606798f : 2.82842712f)));
+}
+
+// Offset o (0..23) of the bond stencil: the 5 x 5 lattice block without its
+// centre, in (dj, di) order.
+__host__ __device__ constexpr int stn_di(int o) { return (o + (o >= 12 ? 1 : 0)) % 5 - 2; }
+__host__ __device__ constexpr int stn_dj(int o) { return (o + (o >= 12 ? 1 : 0)) / 5 - 2; }
+
+// Offset of the neighbour row dj from a stencil record.
+__device__ __forceinline__ int stn_row(const uint4 &st, int dj) {
+    return dj == -2 ? (int)(short)(st.y & 0xFFFFu) : (dj == -1 ? (int)(short)(st.y >> 16)
+           : (dj == 0 ? 0 : (dj == 1 ? (int)(short)(st.z & 0xFFFFu) : (int)(short)(st.z >> 16))));
+}
+// Bits of the stencil's intact bonds: the broken-bond bits w follow the order
+// of the node's bonds (the rank of the offset among the stencil bits), so each
+// set bit clears the stencil bit of that rank (a node seldom has a broken
+// bond: the loop is skipped).
+__device__ __forceinline__ uint32_t stn_alive(uint32_t mask, uint32_t w) {
+    uint32_t alive = mask;
+    for (; w; w &= w - 1u) {
+        uint32_t m = mask;
+        for (int t = __ffs(w) - 1; t > 0; --t) m &= m - 1u;
+        alive &= ~(m & (0u - m));
     }
-    float4 qi = make_float4(0.f, 0.f, 0.f, 0.f);
-    double2 pi = make_double2(0.0, 0.0);
-    if (d.pq) qi = ldm<PERSIST>(&cur_pq<PERSIST>(d)[i]);
-    else pi = ldm<PERSIST>(&d.p[i]);
-    int lst[kMaxList];
-    int n = 0, over = 0;
+    return alive;
+}
+// Is the node whose number differs by `delta` the partner of one of the intact
+// stencil bonds?
+__device__ __forceinline__ bool stn_bonded(const uint4 &st, uint32_t alive, int delta) {
+    bool hit = false;
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        int t0[3], m[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const int cell = 3 * r + c;
-            bool dup = false;      // two cells of the block hashed to one bucket: visit it once
-#pragma unroll
-            for (int q = 0; q < cell; ++q) dup |= bk[q] == bk[cell];
-            t0[c] = dup ? 0 : ldm<PERSIST>(&d.start[bk[cell]]);
-            m[c] = dup ? 0 : ldm<PERSIST>(&d.start[bk[cell] + 1]) - t0[c];
-        }
-        const int tot = m[0] + m[1] + m[2];
-        for (int e = 0; e < tot; ++e) {
-            const int t = e < m[0] ? t0[0] + e : (e < m[0] + m[1] ? t0[1] + (e - m[0]) : t0[2] + (e - m[0] - m[1]));
-            const uint4 rec = ldm<PERSIST>(&d.srec[t]);
-            float dx, dy;
-            if (d.pq) {
-                dx = (__uint_as_float(rec.x) - qi.x) + (__uint_as_float(rec.z) - qi.z);
-                dy = (__uint_as_float(rec.y) - qi.y) + (__uint_as_float(rec.w) - qi.w);
-            } else {
-                dx = (float)(__hiloint2double((int)rec.y, (int)rec.x) - pi.x);
-                dy = (float)(__hiloint2double((int)rec.w, (int)rec.z) - pi.y);
-            }
-            if (!(dx * dx + dy * dy < A.rs2)) continue;
-            const int j = ldm<PERSIST>(&d.sorted[t]);
-            // hash aliasing can bring nodes of another aggregate: never in contact
-            if (j == i || __ldg(&d.g_agg[__ldg(&d.grain[j])]) != ag) continue;
-            if (n < kMaxList) {
-                int w = n++;
-                while (w > 0 && lst[w - 1] > j) {
-                    lst[w] = lst[w - 1];
-                    --w;
-                }
-                lst[w] = j;
-            } else {
-                over = 1;
-            }
-        }
+    for (int dj = -2; dj <= 2; ++dj) {
+        const int di = delta - stn_row(st, dj), oo = (dj + 2) * 5 + di + 2, o = oo < 12 ? oo : oo - 1;
+        if (di >= -2 && di <= 2 && oo != 12) hit |= (alive >> o) & 1u;
     }
-    const size_t N = (size_t)k.N;
-    for (int q = 0; q < n; ++q) d.nbr[q * N + i] = lst[q];
-    d.nbr_cnt[i] = n;
-    if (d.pq) {
-        d.sref[i] = qi;
-    } else {
-        const double2 u = ldm<PERSIST>(&cur_u<PERSIST>(d)[i]);
-        d.sref[i] = make_float4((float)u.x, (float)u.y, 0.f, 0.f);
-    }
-    if (over) atomicAdd(&d.status[PD_STATUS_OVERFLOW], 1);
+    return hit;
 }
 
 // Is the bond x -> j intact?  (row columns ascending: binary search; broken
@@ -868,6 +892,124 @@ __device__ __forceinline__ bool bonded_intact(const DevPtrs &d, const KParams &k
         return !((__ldcg(&d.bits[(size_t)i * k.wpn + (kk >> 5)]) >> (kk & 31)) & 1u);
     }
     return false;
+}
+
+// The node's bonds broken since the last rebuild, whose partners its candidate
+// list leaves out: their number (any: it may have broken bonds; words read past
+// L1, since its lanes may have just set them), and the partner of the m-th.
+__device__ __forceinline__ uint32_t fresh_word(const DevPtrs &d, const KParams &k, int i, int w) {
+    const size_t at = (size_t)i * k.wpn + w;
+    return __ldcg(&d.bits[at]) & ~__ldcg(&d.bref[at]);
+}
+__device__ __forceinline__ int fresh_bonds(const DevPtrs &d, const KParams &k, int i, bool any) {
+    int n = 0;
+    if (any)
+        for (int w = 0; w < k.wpn; ++w) n += __popc(fresh_word(d, k, i, w));
+    return n;
+}
+__device__ __forceinline__ int fresh_partner(const DevPtrs &d, const KParams &k, int i, int r0, int m) {
+    for (int w = 0;; ++w) {
+        uint32_t b = fresh_word(d, k, i, w);
+        const int n = __popc(b);
+        if (m < n || w + 1 == k.wpn) {
+            for (; m > 0; --m) b &= b - 1u;
+            return __ldg(&d.col[r0 + 32 * w + __ffs(b) - 1]);
+        }
+        m -= n;
+    }
+}
+
+// Rebuild, last step: the candidate list of node i -- every node y != i of
+// its aggregate with |p(y) - p(i)| < R_c + skin that it has no intact bond with
+// (an intact bond excludes self-contact: without this rule the nodes of every
+// grain whose spacing is within 4.5 % of the smallest list their four lattice
+// neighbours; bonds that break later come from their bits, see fresh_bonds) --
+// gathered from the 3 x 3 block of grid cells around its cell (cells are wider
+// than R_c + skin) and kept in ascending node index, and the position and the
+// broken bits it was built at.  The records hold the positions in cell order,
+// so only nodes inside the radius are looked up, and the bonds of a stencil
+// node are told from the difference of the node numbers.
+template <bool PERSIST>
+__device__ __forceinline__ void build_list_node(const DevPtrs &d, const KParams &k, int i) {
+    const int gi = __ldg(&d.grain[i]);
+    const AggParams &A = d.agg[__ldg(&d.g_agg[gi])];
+    const int2 cc = ldm<PERSIST>(&d.cell[i]);
+    const int wx = wrap_cell(cc.x, A.gw);
+    // the block's rows, each one range of records unless it wraps around
+    const bool whole = wx > 0 && wx < A.gw - 1;
+    int row[3], t0[3] = {0, 0, 0}, t1[3] = {0, 0, 0};
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        row[r] = A.gbase + wrap_cell(cc.y + r - 1, A.gh) * A.gw;
+        if (whole) {
+            t0[r] = ldm<PERSIST>(&d.start[row[r] + wx - 1]);
+            t1[r] = ldm<PERSIST>(&d.start[row[r] + wx + 2]);
+        }
+    }
+    const int s0 = __ldg(&d.g_start[gi]), s1 = __ldg(&d.g_start[gi + 1]);
+    const uint4 st = k.stencil ? __ldg(&d.stn[i]) : make_uint4(kStnIrregular, 0u, 0u, 0u);
+    const uint32_t w0 = __ldcg(&d.bits[(size_t)i * k.wpn]);
+    d.bref[(size_t)i * k.wpn] = w0;
+    for (int w = 1; w < k.wpn; ++w) d.bref[(size_t)i * k.wpn + w] = __ldcg(&d.bits[(size_t)i * k.wpn + w]);
+    float4 qi = make_float4(0.f, 0.f, 0.f, 0.f);
+    double2 pi = make_double2(0.0, 0.0);
+    if (d.pq) qi = ldm<PERSIST>(&cur_pq<PERSIST>(d)[i]);
+    else pi = ldm<PERSIST>(&d.p[i]);
+    int lst[kMaxList];
+    int n = 0, over = 0;
+    auto visit = [&](int t) {
+        const uint4 rec = ldm<PERSIST>(&d.srec[t]);
+        float dx, dy;
+        if (d.pq) {
+            dx = (__uint_as_float(rec.x) - qi.x) + (__uint_as_float(rec.z) - qi.z);
+            dy = (__uint_as_float(rec.y) - qi.y) + (__uint_as_float(rec.w) - qi.w);
+        } else {
+            dx = (float)(__hiloint2double((int)rec.y, (int)rec.x) - pi.x);
+            dy = (float)(__hiloint2double((int)rec.w, (int)rec.z) - pi.y);
+        }
+        if (!(dx * dx + dy * dy < A.rs2)) return;
+        const int j = ldm<PERSIST>(&d.sorted[t]);
+        if (j == i) return;
+        if (j >= s0 && j < s1) {
+            if (st.x & kStnIrregular) {
+                if (bonded_intact(d, k, i, __ldg(&d.row_ptr[i]), __ldg(&d.row_ptr[i + 1]), j)) return;
+            } else if (stn_bonded(st, stn_alive(st.x, w0), j - i)) {
+                return;
+            }
+        }
+        if (n < kMaxList) {
+            int w = n++;
+            while (w > 0 && lst[w - 1] > j) {
+                lst[w] = lst[w - 1];
+                --w;
+            }
+            lst[w] = j;
+        } else {
+            over = 1;
+        }
+    };
+    if (whole) {
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+            for (int t = t0[r]; t < t1[r]; ++t) visit(t);
+    } else {
+        // (a grid has at least three cells each way: the nine are different)
+        for (int r = 0; r < 3; ++r)
+            for (int c = -1; c <= 1; ++c) {
+                const int cell = row[r] + wrap_cell(cc.x + c, A.gw);
+                for (int t = ldm<PERSIST>(&d.start[cell]), e = ldm<PERSIST>(&d.start[cell + 1]); t < e; ++t) visit(t);
+            }
+    }
+    const size_t N = (size_t)k.N;
+    for (int q = 0; q < n; ++q) d.nbr[q * N + i] = lst[q];
+    d.nbr_cnt[i] = n;
+    if (d.pq) {
+        d.sref[i] = qi;
+    } else {
+        const double2 u = ldm<PERSIST>(&cur_u<PERSIST>(d)[i]);
+        d.sref[i] = make_float4((float)u.x, (float)u.y, 0.f, 0.f);
+    }
+    if (over) atomicAdd(&d.status[PD_STATUS_OVERFLOW], 1);
 }
 
 // Acceleration and velocity update of node i (Algorithm 1) plus the optional
@@ -929,8 +1071,8 @@ __device__ __forceinline__ void finish_node(const DevPtrs &d, const KParams &k, 
 // update phase, which would have read u, v and a back from memory.
 template <bool PERSIST>
 __device__ __forceinline__ void finish_node32_total(const DevPtrs &d, const KParams &k, int i, int vin, int update_v,
-                                                    double2 vi, float2 ao, float fx, float fy, bool walls,
-                                                    double Fwx, double Fwy, float inv_m, double2 ui = {}) {
+                                                    const Update32 &n, float fx, float fy, bool walls, double Fwx,
+                                                    double Fwy, float inv_m) {
     float ax, ay;
     if (walls) {
         ax = fmaf(__double2float_rn(f2d_bits(fx) + Fwx), inv_m, k.gxf);
@@ -941,10 +1083,10 @@ __device__ __forceinline__ void finish_node32_total(const DevPtrs &d, const KPar
     }
     if (update_v) {
         const float hdt = 0.5f * k.dtf;
-        const double2 vn = make_double2(vi.x + f2d_bits(hdt * (ao.x + ax)), vi.y + f2d_bits(hdt * (ao.y + ay)));
+        const double2 vn = make_double2(n.v.x + f2d_bits(hdt * (n.a.x + ax)), n.v.y + f2d_bits(hdt * (n.a.y + ay)));
         d.v[vin ^ 1][i] = vn;
         if constexpr (PERSIST) {
-            if (advance_node32<PERSIST>(d, k, i, ui, vn, ax, ay, d.ub[vin], d.pqb[vin]))
+            if (advance_node32(d, k, i, n.u, vn, ax, ay, n.xs, n.sref, d.ub[vin], d.pqb[vin]))
                 *(volatile int *)d.rebuild_next = 1;
         }
     }
@@ -977,6 +1119,70 @@ __device__ __forceinline__ T lane_sum(T v) {
     return v;
 }
 
+// Bond tile: the bonds of a run of consecutive nodes, each evaluated once.
+//
+// The bond loop is bound by instruction issue (FP32 split) or by the FP64 pipe
+// (FP64 path), and a bond's force on its two nodes differs in sign only: both
+// paths' arithmetic is odd in d, so the second evaluation gives the same bits.
+// With one thread per node a block therefore takes its run of nodes in tiles of
+// BLOCK consecutive ones: every thread evaluates the forward half of its node's
+// stencil (offsets 12..23, towards higher node indices) into shared memory,
+// and after a block barrier sums its backward half from the slots of the nodes
+// that evaluated it.  Nodes of a grain are numbered row by row, so those lie
+// at most two lattice rows back; what a tile needs of the one before it is
+// carried over (the last kCarry nodes' slots; KParams::pair says that no row
+// is longer), and the first tile of a run is preceded by a pass that forms the
+// slots of the kCarry nodes before the run.  Each node still adds its bonds in
+// the order of the stencil, so a sum does not depend on where tiles begin and
+// the results of every path and block size agree.
+//
+// A slot whose force was not formed holds a marker (a NaN no operation makes):
+// kPairNone (no such bond in the evaluating node's list, its bonds are not
+// stencil bonds, or it is broken there), kPairBroken (breaks at this
+// evaluation), kPairGuard (FP32 split: in the guard band, each node decides it
+// in FP64).  Any NaN sends the reader to its general loop.
+constexpr unsigned kPairNone = 0x7FC0D000u, kPairBroken = 0x7FC0D001u, kPairGuard = 0x7FC0D002u;
+constexpr int kPairHalf = 12;     // forward offsets of the stencil
+// What a node's bond pass leaves to do: bonds in the guard band to decide, and
+// that one of its bonds broke at this evaluation.
+constexpr unsigned kNoteGuard = 1u, kNoteBroke = 2u;
+template <class Slot, int BLOCK>
+struct PairTile {
+    static constexpr int kStride = kCarry + BLOCK;      // carried slots, then the tile's
+    static constexpr int kBytes = kPairHalf * kStride * (int)sizeof(Slot);
+    static_assert(kCarry <= BLOCK, "the carried slots must not overlap their source");
+    static __device__ __forceinline__ void carry(Slot *slot) {
+        for (int e = threadIdx.x; e < kPairHalf * kCarry; e += BLOCK) {
+            const int o = e / kCarry, q = e % kCarry;
+            slot[o * kStride + q] = slot[o * kStride + BLOCK + q];
+        }
+    }
+};
+
+// Asynchronous copies of 4, 8 or 16 bytes into the calling thread's own places
+// in shared memory; commit closes a group, wait<n> returns when all but the
+// last n groups of the thread have arrived.
+template <class T>
+__device__ __forceinline__ void copy_async(T *dst, const T *src) {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(dst);
+    if constexpr (sizeof(T) == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(a), "l"(src), "n"(sizeof(T)) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// The broken-bond bit of offset o.
+__device__ __forceinline__ uint32_t stn_bit(uint32_t mask, int o) { return 1u << __popc(mask & ((1u << o) - 1u)); }
+
+// Whether some thread of the node's LANES says so.
+template <int LANES>
+__device__ __forceinline__ bool any_lane(bool v) {
+    if constexpr (LANES == 1) return v;
+    const unsigned all = __ballot_sync(0xffffffffu, v);
+    return (all >> ((threadIdx.x & 31) / LANES * LANES)) & ((1u << LANES) - 1u);
+}
+
 // FP64 forces of node i (eq:full, Algorithm 1), LANES threads per node: lane l
 // takes bonds l, l + LANES, ... and grid cells l, l + LANES, ...; partial sums
 // meet in a fixed xor-butterfly (deterministic).  With LANES = 1 every sum is
@@ -992,34 +1198,270 @@ struct Sums32 {
     float bx, by, sx, sy, nx, ny;
 };
 
+// One FP64 bond (eq:peri, eq:pmb, Sec. 3.1) of a node at pi towards pj with
+// reference length xi: false when it breaks at this evaluation, else its force
+// (fx, fy) on the node.  The stretch's cancelling difference L - |xi| is formed
+// exactly as the FP64 definition rounds it: dx, dy and |d|^2 in FP64, L =
+// sqrt(|d|^2) correctly rounded (integer square root), L - |xi| in FP64.  The
+// quotient by |xi|, the break decision away from the threshold and the bond
+// force c_w w s V_x V_y (d / L) are float-float (relative error ~1e-14; a bond
+// whose stretch lies within 1e-6 of s0 is decided by the FP64 quotient).
+// cwVV = c_w V^2 (one grain: V_y = V_x).
+__device__ __forceinline__ bool bond_force64(double2 pi, double2 pj, double xi, ff cwVV, ff inv_eps, float s0f,
+                                             double s0, int micro, ff &fx, ff &fy) {
+    const double dx = __dsub_rn(pj.x, pi.x), dy = __dsub_rn(pj.y, pi.y);
+    const double L = sqrt_rn_int(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
+    const double diff = __dsub_rn(L, xi);                       // |xi| s, exact as in FP64
+    const ff dff = to_ff(diff), xff = to_ff(xi);
+    // break test |diff| > s0 |xi| in float, the FP64 quotient near the threshold
+    const float lhs = fabsf(dff.hi), rhs = s0f * xff.hi;
+    bool brk = lhs > rhs;
+    if (fabsf(lhs - rhs) <= 1e-6f * rhs) brk = fabs(__ddiv_rn(diff, xi)) > s0;
+    if (brk) return false;
+    // c_w w V_x V_y (diff / |xi|) / L  (w = 1 - |xi| / eps for the conic micromodulus)
+    ff c = cwVV;
+    if (micro) c = ff_mul(c, ff_add({1.0f, 0.f}, ff_mul({-xff.hi, -xff.lo}, inv_eps)));
+    const ff t = ff_mul(ff_mul(c, dff), ff_rcp(ff_mul(xff, to_ff(L))));
+    fx = ff_mul(t, to_ff(dx));
+    fy = ff_mul(t, to_ff(dy));
+    return true;
+}
+
+// The forward half of node ii's stencil bonds (alive: the intact ones), FP64
+// path, into the thread's slots; returns the offsets whose force is there.
+// OWN: the block owns the node and records its broken bonds.
+template <bool PERSIST, int BLOCK, bool OWN>
+__device__ __forceinline__ uint32_t tile_forward64(const DevPtrs &d, const KParams &k, int ii, uint32_t alive,
+                                                   const uint4 &st, double2 pi, ff cwVV, ff inv_eps, float s0f,
+                                                   double s0, float4 *slot, unsigned &note) {
+    constexpr int S = PairTile<float4, BLOCK>::kStride;
+    const int at = kCarry + (int)threadIdx.x;
+    uint32_t formed = 0u;
+    constexpr int kBatch = 4;
+#pragma unroll
+    for (int m0 = 0; m0 < kPairHalf; m0 += kBatch) {
+        double2 pb[kBatch];
+        double xb[kBatch];
+#pragma unroll
+        for (int m = 0; m < kBatch; ++m) {
+            const int o = kPairHalf + m0 + m;
+            const bool live = (alive >> o) & 1u;
+            pb[m] = ldm<PERSIST>(&d.p[live ? ii + stn_di(o) + stn_row(st, stn_dj(o)) : ii]);
+            xb[m] = live ? __ldg(&d.xif[(size_t)(m0 + m) * k.N + ii]) : 1.0;
+        }
+#pragma unroll
+        for (int m = 0; m < kBatch; ++m) {
+            const int o = kPairHalf + m0 + m;
+            unsigned mark = kPairNone;
+            ff fx = {0.f, 0.f}, fy = fx;
+            if ((alive >> o) & 1u) {
+                if (bond_force64(pi, pb[m], xb[m], cwVV, inv_eps, s0f, s0, k.micro, fx, fy)) {
+                    mark = 0u;
+                    formed |= 1u << o;
+                } else {
+                    mark = kPairBroken;
+                    if (OWN) atomicOr(&d.bits[(size_t)ii * k.wpn], stn_bit(st.x, o));
+                    note |= kNoteBroke;
+                }
+            }
+            slot[(m0 + m) * S + at] = make_float4(mark ? __uint_as_float(mark) : fx.hi, fx.lo, fy.hi, fy.lo);
+        }
+    }
+    return formed;
+}
+
+// The bond sum of node ii, FP64 path: the backward half from the slots of the
+// nodes that formed it, then the node's own forward slots.
+template <bool PERSIST, int BLOCK>
+__device__ __forceinline__ void tile_sum64(const DevPtrs &d, const KParams &k, int ii, uint32_t alive, uint32_t formed,
+                                           const uint4 &st, double2 pi, ff cwVV, ff inv_eps, float s0f, double s0,
+                                           const float4 *slot, ff &Fx, ff &Fy, unsigned &note) {
+    constexpr int S = PairTile<float4, BLOCK>::kStride;
+    const int at = kCarry + (int)threadIdx.x;
+    const uint32_t back = alive & ((1u << kPairHalf) - 1u);
+    uint32_t got = 0u;
+#pragma unroll
+    for (int o = 0; o < kPairHalf; ++o) {
+        const bool in = (back >> o) & 1u;
+        const float4 v = slot[(kPairHalf - 1 - o) * S + (in ? at + stn_di(o) + stn_row(st, stn_dj(o)) : at)];
+        const bool ok = in && v.x == v.x;
+        if (ok) got |= 1u << o;
+        Fx = ff_add(Fx, ok ? ff{-v.x, -v.y} : ff{0.f, 0.f});
+        Fy = ff_add(Fy, ok ? ff{-v.z, -v.w} : ff{0.f, 0.f});
+    }
+    if (back != got) {
+        // some slot holds a marker: the half again, in order
+        Fx = Fy = {0.f, 0.f};
+        for (uint32_t m = back; m; m &= m - 1u) {
+            const int o = __ffs(m) - 1;
+            const int off = stn_di(o) + stn_row(st, stn_dj(o));
+            const float4 v = slot[(kPairHalf - 1 - o) * S + at + off];
+            unsigned mark = __float_as_uint(v.x);
+            if (mark == kPairNone) {
+                ff fx, fy;
+                const int b = (int)st.w + __popc(st.x & ((1u << o) - 1u));
+                if (bond_force64(pi, ldm<PERSIST>(&d.p[ii + off]), __ldg(&d.xi[b]), cwVV, inv_eps, s0f, s0, k.micro,
+                                 fx, fy)) {
+                    Fx = ff_add(Fx, fx);
+                    Fy = ff_add(Fy, fy);
+                    continue;
+                }
+                mark = kPairBroken;
+            }
+            if (mark == kPairBroken) {
+                atomicOr(&d.bits[(size_t)ii * k.wpn], stn_bit(st.x, o));
+                note |= kNoteBroke;
+                continue;
+            }
+            Fx = ff_add(Fx, ff{-v.x, -v.y});
+            Fy = ff_add(Fy, ff{-v.z, -v.w});
+        }
+    }
+#pragma unroll
+    for (int o = kPairHalf; o < 2 * kPairHalf; ++o) {
+        const float4 v = slot[(o - kPairHalf) * S + at];
+        const bool ok = (formed >> o) & 1u;
+        Fx = ff_add(Fx, ok ? ff{v.x, v.y} : ff{0.f, 0.f});
+        Fy = ff_add(Fy, ok ? ff{v.z, v.w} : ff{0.f, 0.f});
+    }
+}
+
+// Contact force of candidate j on node ii, FP64 path: self-contact (Sec. 4.4)
+// into fs, inter-grain contact (Secs. 4.1-4.3) into fn, zero beyond R_c.
+template <bool PERSIST>
+__device__ __forceinline__ void contact_pair64(const DevPtrs &d, const KParams &k, const AggParams &A, int ii, int j,
+                                               int vin, int gi, int r0, int r1, double2 pi, double2 pj, double2 vi,
+                                               double &fsx, double &fsy, double &fnx, double &fny) {
+    fsx = fsy = fnx = fny = 0.0;
+    const double Rc = A.Rc;
+    // |d|^2 above R_c^2 (1 + 1e-12) means sqrt(|d|^2) rounds to R_c or more:
+    // candidates that far are dropped before the square root
+    const double rc2_out = Rc * Rc * (1.0 + 1e-12);
+    double dx = pj.x - pi.x, dy = pj.y - pi.y;
+    const double dd2 = dx * dx + dy * dy;
+    if (!(dd2 <= rc2_out)) return;
+    double dd = dd2 > 0.0 ? sqrt_rn_int(dd2) : 0.0;
+    if (!(dd < Rc)) return;
+    if (dd == 0.0) {
+        atomicAdd(&d.status[PD_STATUS_COINCIDENT], 1);
+        return;
+    }
+    const double Vi = __ldg(&d.V[ii]), cw = __ldg(&d.g_cw[gi]);
+    const double2 Xi = __ldg(&d.X[ii]);
+    const double rho_i = k.mat ? __ldg(&d.g_rho[gi]) : k.rho;
+    double ex = dx / dd, ey = dy / dd;
+    const double Vj = __ldg(&d.V[j]);
+    const double2 vj = ldm<PERSIST>(&d.v[vin][j]);
+    double vrx = vi.x - vj.x, vry = vi.y - vj.y;
+    const int gj = __ldg(&d.grain[j]);
+    if (gj == gi) {
+        if (bonded_intact(d, k, ii, r0, r1, j)) return;
+        const double2 Xj = __ldg(&d.X[j]);
+        double xix = Xj.x - Xi.x, xiy = Xj.y - Xi.y;
+        double xi = sqrt(xix * xix + xiy * xiy);
+        double m;
+        if (xi < Rc)
+            m = (dd < xi) ? cw * (dd - xi) / xi : 0.0;
+        else
+            m = cw * (dd - Rc) / Rc;
+        if (m == 0.0) return;
+        double f = m * Vi * Vj;
+        double gx = f * ex, gy = f * ey;
+        const double Kn = k.mat ? 18.0 * __ldg(&d.g_k[gi]) / A.pe5 : A.Kn;
+        damping_friction64(k, Kn, rho_i, rho_i, ex, ey, vrx, vry, -f, Vi, Vj, gx, gy);
+        fsx = gx;
+        fsy = gy;
+    } else {
+        double Kn = A.Kn, rho_d = rho_i;
+        if (k.mat) {
+            Kn = 18.0 * harmonic64(__ldg(&d.g_k[gi]), __ldg(&d.g_k[gj])) / A.pe5;
+            rho_d = harmonic64(rho_i, __ldg(&d.g_rho[gj]));
+        }
+        double Fr = Kn * (Rc - dd) * Vi * Vj;
+        double gx = -Fr * ex, gy = -Fr * ey;
+        damping_friction64(k, Kn, rho_d, rho_i, ex, ey, vrx, vry, Fr, Vi, Vj, gx, gy);
+        fnx = gx;
+        fny = gy;
+    }
+}
+
+// Candidate q of node ii: the nc of its list (ascending node index), then the
+// partners of the bonds broken since the rebuild; together every pair closer
+// than R_c without an intact bond.
+template <bool PERSIST>
+__device__ __forceinline__ int candidate(const DevPtrs &d, const KParams &k, int ii, int nc, int r0, int q) {
+    return q < nc ? ldm<PERSIST>(&d.nbr[(size_t)q * k.N + ii]) : fresh_partner(d, k, ii, r0, q - nc);
+}
+
+// Contact forces of node ii, FP64 path: every LANES-th of its nc + nb candidates.
 template <bool PERSIST, int LANES>
+__device__ __forceinline__ void contacts64(const DevPtrs &d, const KParams &k, int ii, int lane, int vin, int gi, int nc,
+                                           int nb, int r0, int r1, double2 pi, double &Fsx, double &Fsy, double &Fnx,
+                                           double &Fny) {
+    const AggParams &A = d.agg[__ldg(&d.g_agg[gi])];
+    const double2 vi = ldm<PERSIST>(&d.v[vin][ii]);
+    for (int q = lane; q < nc + nb; q += LANES) {
+        const int j = candidate<PERSIST>(d, k, ii, nc, r0, q);
+        double a, b, c, e;
+        contact_pair64<PERSIST>(d, k, A, ii, j, vin, gi, r0, r1, pi, ldm<PERSIST>(&d.p[j]), vi, a, b, c, e);
+        Fsx += a;
+        Fsy += b;
+        Fnx += c;
+        Fny += e;
+    }
+}
+
+// (slot: the bond tile of a block of BLOCK threads with one thread per node,
+// and warm the pass before a run, which forms slots only and leaves `out`;
+// with more threads per node BLOCK is 0 and there is no tile.  contact: the node
+// has contact candidates; without INLINE its contact forces are left to a later
+// pass.)
+template <bool PERSIST, int LANES, int BLOCK, bool INLINE = true>
 __device__ __forceinline__ void force_node64(const DevPtrs &d, const KParams &k, int i, int lane, bool active,
-                                             int vin, Sums64 &out) {
+                                             int vin, Sums64 &out, float4 *slot, bool warm, bool &contact) {
+    contact = false;
     const int ii = active ? i : 0;
     const double2 pi = ldm<PERSIST>(&d.p[ii]);
-    const double2 Xi = __ldg(&d.X[ii]);
     const double Vi = __ldg(&d.V[ii]);
     const int gi = __ldg(&d.grain[ii]);
-    const int ag = __ldg(&d.g_agg[gi]);
-    const AggParams &A = d.agg[ag];
     const double cw = __ldg(&d.g_cw[gi]), s0 = __ldg(&d.g_s0[gi]), eps = __ldg(&d.g_eps[gi]);
-    const int r0 = active ? __ldg(&d.row_ptr[ii]) : 0, r1 = active ? __ldg(&d.row_ptr[ii + 1]) : 0;
     uint32_t *bw = d.bits + (size_t)ii * k.wpn;
 
-    // peridynamic bonds with breaking (eq:peri, eq:pmb, Sec. 3.1).  The
-    // stretch's cancelling difference L - |xi| is formed exactly as the FP64
-    // definition rounds it: dx, dy and |d|^2 in FP64, L = sqrt(|d|^2) correctly
-    // rounded (integer square root), L - |xi| in FP64.  The quotient by |xi|,
-    // the break decision away from the threshold and the bond force
-    // c_w w s V_x V_y (d / L) are float-float (relative error ~1e-14; a bond
-    // whose stretch lies within 1e-6 of s0 is decided by the FP64 quotient).
     ff Fbx = {0.f, 0.f}, Fby = {0.f, 0.f};
     const uint32_t w0 = active ? __ldcg(bw) : 0u;      // the row's first 32 broken bits (own bonds only)
     const float s0f = (float)s0;
     const ff cwVV = to_ff(cw * Vi * Vi);                // one grain: V_y = V_x
     const ff inv_eps = ff_rcp(to_ff(eps));
+    bool csr = true;           // bonds from the CSR columns
+    unsigned note = 0u;
+    int r0, r1;
+    if constexpr (LANES == 1) {
+        const uint4 st = (k.stencil && active) ? __ldg(&d.stn[ii]) : make_uint4(kStnIrregular, 0u, 0u, 0u);
+        csr = (st.x & kStnIrregular) != 0u || !k.pair;
+        r0 = (int)st.w;
+        r1 = r0 + __popc(st.x);
+        if (csr) {
+            r0 = active ? __ldg(&d.row_ptr[ii]) : 0;
+            r1 = active ? __ldg(&d.row_ptr[ii + 1]) : 0;
+        }
+        if (k.pair) {
+            const uint32_t alive = csr ? 0u : stn_alive(st.x, w0);
+            if (warm) {
+                tile_forward64<PERSIST, BLOCK, false>(d, k, ii, alive, st, pi, cwVV, inv_eps, s0f, s0, slot, note);
+                return;
+            }
+            const uint32_t formed =
+                tile_forward64<PERSIST, BLOCK, true>(d, k, ii, alive, st, pi, cwVV, inv_eps, s0f, s0, slot, note);
+            __syncthreads();
+            tile_sum64<PERSIST, BLOCK>(d, k, ii, alive, formed, st, pi, cwVV, inv_eps, s0f, s0, slot, Fbx, Fby,
+                                       note);
+        }
+    } else {
+        r0 = active ? __ldg(&d.row_ptr[ii]) : 0;
+        r1 = active ? __ldg(&d.row_ptr[ii + 1]) : 0;
+    }
     constexpr int kBondBatch64 = 4;
-    for (int b0 = r0 + lane; b0 < r1; b0 += kBondBatch64 * LANES) {
+    for (int b0 = r0 + lane; b0 < r1 && csr; b0 += kBondBatch64 * LANES) {
         int jb[kBondBatch64];
         uint32_t wb[kBondBatch64];
         double xb[kBondBatch64];
@@ -1037,87 +1479,24 @@ __device__ __forceinline__ void force_node64(const DevPtrs &d, const KParams &k,
         for (int m = 0; m < kBondBatch64; ++m) {
             const int kk = b0 + m * LANES - r0;
             if (jb[m] < 0 || ((wb[m] >> (kk & 31)) & 1u)) continue;
-            const double xi = xb[m];
-            const double dx = __dsub_rn(pb[m].x, pi.x), dy = __dsub_rn(pb[m].y, pi.y);
-            const double L = sqrt_rn_int(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
-            const double diff = __dsub_rn(L, xi);                       // |xi| s, exact as in FP64
-            const ff dff = to_ff(diff), xff = to_ff(xi);
-            // break test |diff| > s0 |xi| in float, the FP64 quotient near the threshold
-            const float lhs = fabsf(dff.hi), rhs = s0f * xff.hi;
-            bool brk = lhs > rhs;
-            if (fabsf(lhs - rhs) <= 1e-6f * rhs) brk = fabs(__ddiv_rn(diff, xi)) > s0;
-            if (brk) {
+            ff fx, fy;
+            if (!bond_force64(pi, pb[m], xb[m], cwVV, inv_eps, s0f, s0, k.micro, fx, fy)) {
                 atomicOr(&bw[kk >> 5], 1u << (kk & 31));
+                note |= kNoteBroke;
                 continue;
             }
-            // c_w w V_x V_y (diff / |xi|) / L  (w = 1 - |xi| / eps for the conic micromodulus)
-            ff c = cwVV;
-            if (k.micro) c = ff_mul(c, ff_add({1.0f, 0.f}, ff_mul({-xff.hi, -xff.lo}, inv_eps)));
-            const ff t = ff_mul(ff_mul(c, dff), ff_rcp(ff_mul(xff, to_ff(L))));
-            Fbx = ff_add(Fbx, ff_mul(t, to_ff(dx)));
-            Fby = ff_add(Fby, ff_mul(t, to_ff(dy)));
+            Fbx = ff_add(Fbx, fx);
+            Fby = ff_add(Fby, fy);
         }
     }
     __syncwarp();
 
-    // contact candidates (the node's list: every pair closer than R_c is in it,
-    // ascending node index), self-contact (Sec. 4.4), inter-grain contact
-    // (Secs. 4.1-4.3)
-    const double Rc = A.Rc;
-    // |d|^2 above R_c^2 (1 + 1e-12) means sqrt(|d|^2) rounds to R_c or more:
-    // candidates that far are dropped before the square root
-    const double rc2_out = Rc * Rc * (1.0 + 1e-12);
-    const double rho_i = k.mat ? __ldg(&d.g_rho[gi]) : k.rho;
     const int nc = active ? ldm<PERSIST>(&d.nbr_cnt[ii]) : 0;
-    const double2 vi = ldm<PERSIST>(&d.v[vin][ii]);
+    const int nb = fresh_bonds(d, k, ii, any_lane<LANES>(w0 != 0u || (note & kNoteBroke) || (active && k.wpn > 1)));
     double Fsx = 0.0, Fsy = 0.0, Fnx = 0.0, Fny = 0.0;
-    for (int q = lane; q < nc; q += LANES) {
-        const int j = ldm<PERSIST>(&d.nbr[(size_t)q * k.N + ii]);
-        const double2 pj = ldm<PERSIST>(&d.p[j]);
-        double dx = pj.x - pi.x, dy = pj.y - pi.y;
-        const double dd2 = dx * dx + dy * dy;
-        if (!(dd2 <= rc2_out)) continue;
-        double dd = dd2 > 0.0 ? sqrt_rn_int(dd2) : 0.0;
-        if (!(dd < Rc)) continue;
-        if (dd == 0.0) {
-            atomicAdd(&d.status[PD_STATUS_COINCIDENT], 1);
-            continue;
-        }
-        double ex = dx / dd, ey = dy / dd;
-        const double Vj = __ldg(&d.V[j]);
-        const double2 vj = ldm<PERSIST>(&d.v[vin][j]);
-        double vrx = vi.x - vj.x, vry = vi.y - vj.y;
-        const int gj = __ldg(&d.grain[j]);
-        if (gj == gi) {
-            if (bonded_intact(d, k, ii, r0, r1, j)) continue;
-            const double2 Xj = __ldg(&d.X[j]);
-            double xix = Xj.x - Xi.x, xiy = Xj.y - Xi.y;
-            double xi = sqrt(xix * xix + xiy * xiy);
-            double m;
-            if (xi < Rc)
-                m = (dd < xi) ? cw * (dd - xi) / xi : 0.0;
-            else
-                m = cw * (dd - Rc) / Rc;
-            if (m == 0.0) continue;
-            double f = m * Vi * Vj;
-            double gx = f * ex, gy = f * ey;
-            const double Kn = k.mat ? 18.0 * __ldg(&d.g_k[gi]) / A.pe5 : A.Kn;
-            damping_friction64(k, Kn, rho_i, rho_i, ex, ey, vrx, vry, -f, Vi, Vj, gx, gy);
-            Fsx += gx;
-            Fsy += gy;
-        } else {
-            double Kn = A.Kn, rho_d = rho_i;
-            if (k.mat) {
-                Kn = 18.0 * harmonic64(__ldg(&d.g_k[gi]), __ldg(&d.g_k[gj])) / A.pe5;
-                rho_d = harmonic64(rho_i, __ldg(&d.g_rho[gj]));
-            }
-            double Fr = Kn * (Rc - dd) * Vi * Vj;
-            double gx = -Fr * ex, gy = -Fr * ey;
-            damping_friction64(k, Kn, rho_d, rho_i, ex, ey, vrx, vry, Fr, Vi, Vj, gx, gy);
-            Fnx += gx;
-            Fny += gy;
-        }
-    }
+    contact = nc + nb > 0;
+    if (INLINE && contact) contacts64<PERSIST, LANES>(d, k, ii, lane, vin, gi, nc, nb, r0, r1, pi, Fsx, Fsy, Fnx, Fny);
+    __syncwarp();
     out.bx = lane_sum<LANES>(f2d_bits(Fbx.hi) + f2d_bits(Fbx.lo));
     out.by = lane_sum<LANES>(f2d_bits(Fby.hi) + f2d_bits(Fby.lo));
     out.sx = lane_sum<LANES>(Fsx);
@@ -1163,62 +1542,77 @@ __device__ __forceinline__ void node_epilogue64(const DevPtrs &d, const KParams 
 
 // FP32-split geometry of one bond to a neighbour at qj (float-float shifted
 // position), lattice offset code nn = di^2 + dj^2 and sqn = sqrt(nn):
-// num = |d|^2 - |xi|^2 (float-float difference, |xi|^2 = n h^2 exact to
-// float-float), den = |xi| (L + |xi|), so that s = num / den.  Returns 0 =
-// intact, 1 = broken at this evaluation (|s| > s0), 2 = |s| in the guard band
-// around s0 (decided in FP64 after the loop).  The tests compare |num| with
-// s0 den: no division.
+// num = |d|^2 - |xi|^2 (|xi|^2 = n h^2 exact to float-float), den = |xi| (L + |xi|),
+// so that s = num / den.  The square |d|^2 is (s, r): s the rounded sum of the
+// squared high parts and r everything below it.  With a >= b the magnitudes of
+// the high parts, p = RN(a^2) and s = RN(b^2 + p) satisfy s/2 <= p <= s (one
+// last place aside), so p - s is exact and fma(b, b, p - s) is the rounding
+// error of s: eight operations where two exact products and an exact sum take
+// ten.  r keeps the low parts' own squares too (see len2_ff) and stays apart
+// from s until |xi|^2 has been taken off: s - n h^2 is exact for moderate
+// stretches, so nothing is renormalised first.  Every operation is even in d,
+// so both nodes of a bond get the same num and den.
 struct BondGeom32 {
     float dx, dy, L, num, den, xi;
 };
 // (pow2: n is a power of two, so n h^2 is exact in float-float without a
 // product residual; callers that know n at compile time pass it as a constant)
-__device__ __forceinline__ int bond_classify32(float4 qj, float2 phi, float2 pli, float nn, float sqn, float4 gq,
-                                               float s0_lo, float s0_hi, BondGeom32 &g, bool pow2 = false) {
-    const float dxh = __fsub_rn(qj.x, phi.x), dxl = qj.z - pli.x;
-    const float dyh = __fsub_rn(qj.y, phi.y), dyl = qj.w - pli.y;
-    float L2h, L2l;
-    len2_ff(dxh, dxl, dyh, dyl, L2h, L2l);
+__device__ __forceinline__ void bond_geom32(float4 qj, float2 phi, float2 pli, float nn, float sqn, float4 gq,
+                                            BondGeom32 &g, bool pow2 = false) {
+    const float dxh = __fsub_rn(qj.x, phi.x), dxl = __fsub_rn(qj.z, pli.x);
+    const float dyh = __fsub_rn(qj.y, phi.y), dyl = __fsub_rn(qj.w, pli.y);
+    const float a = fmaxf(fabsf(dxh), fabsf(dyh)), b = fminf(fabsf(dxh), fabsf(dyh));
+    const float p = __fmul_rn(a, a), ep = fmaf(a, a, -p);
+    const float s = fmaf(b, b, p), es = fmaf(b, b, __fsub_rn(p, s));
+    // ep + es + dxl (2 dxh + dxl) + dyl (2 dyh + dyl)
+    const float r = __fadd_rn(es, fmaf(dxl, fmaf(2.f, dxh, dxl), fmaf(dyl, fmaf(2.f, dyh, dyl), ep)));
     float q, eq;                                         // |xi|^2 = n h^2 as a float-float pair
     if (pow2) {
-        q = nn * gq.y;
-        eq = nn * gq.z;
+        q = __fmul_rn(nn, gq.y);
+        eq = __fmul_rn(nn, gq.z);
     } else {
         two_prod(nn, gq.y, q, eq);
         eq = fmaf(nn, gq.z, eq);
     }
-    g.num = ff_diff(L2h, L2l, q, eq);
-    g.xi = gq.x * sqn;
-    g.L = sqrt_approx(L2h);
-    g.den = g.xi * (g.L + g.xi);
-    g.dx = dxh + dxl;
-    g.dy = dyh + dyl;
-    // intact and clear of the guard band (the common case): one comparison; a
-    // NaN stretch counts as intact, as in the band tests
-    const float an = fabsf(g.num);
-    if (!(an > s0_lo * g.den)) return 0;
-    return an < s0_hi * g.den ? 2 : 1;
+    g.num = __fadd_rn(__fsub_rn(s, q), __fsub_rn(r, eq));
+    g.xi = __fmul_rn(gq.x, sqn);
+    g.L = sqrt_approx(__fadd_rn(s, r));
+    g.den = fmaf(g.xi, g.L, q);                          // |xi| L + |xi|^2
+    g.dx = __fadd_rn(dxh, dxl);
+    g.dy = __fadd_rn(dyh, dyl);
+}
+// Break decision of a bond: 0 = intact, 1 = broken at this evaluation (|s| >
+// s0), 2 = |s| in the guard band around s0 (decided in FP64 after the loop).
+// The tests compare |num| with s0 den: no division.  A NaN stretch counts as
+// intact.
+__device__ __forceinline__ float bond_excess32(const BondGeom32 &g, float s0_lo) {
+    return fmaf(-s0_lo, g.den, fabsf(g.num));           // > 0: not clearly intact
+}
+__device__ __forceinline__ int bond_state32(const BondGeom32 &g, float s0_lo, float s0_hi) {
+    if (!(bond_excess32(g, s0_lo) > 0.f)) return 0;
+    return fabsf(g.num) < __fmul_rn(s0_hi, g.den) ? 2 : 1;
+}
+__device__ __forceinline__ int bond_classify32(float4 qj, float2 phi, float2 pli, float nn, float sqn, float4 gq,
+                                               float s0_lo, float s0_hi, BondGeom32 &g, bool pow2 = false) {
+    bond_geom32(qj, phi, pli, nn, sqn, gq, g, pow2);
+    return bond_state32(g, s0_lo, s0_hi);
 }
 
-// Adds the bond force c_w w V^2 s (d / L) of an intact bond (w = 1 - |xi| / eps
-// for the conic micromodulus).
-__device__ __forceinline__ void bond_add32(const BondGeom32 &g, float cw, float eps, float VV, int micro, float &Fbx,
-                                           float &Fby) {
-    const float c = micro ? cw * (1.0f - __fdividef(g.xi, eps)) : cw;
-    const float qf = __fdividef(c * VV * g.num, g.den * g.L);
-    Fbx += qf * g.dx;
-    Fby += qf * g.dy;
+// Bond force c_w w V^2 s (d / L) of an intact bond (w = 1 - |xi| / eps for the
+// conic micromodulus).  The products are rounded by themselves (no FMA into a
+// running sum): a bond's force on its other node is then the exact negative,
+// whichever of the two nodes evaluates it.
+__device__ __forceinline__ float2 bond_force32(const BondGeom32 &g, float cw, float inv_eps, float VV, int micro) {
+    const float c = micro ? cw * fmaf(-g.xi, inv_eps, 1.0f) : cw;
+    const float qf = __fmul_rn(__fmul_rn(__fmul_rn(c, VV), g.num), rcp_approx(__fmul_rn(g.den, g.L)));
+    return make_float2(__fmul_rn(qf, g.dx), __fmul_rn(qf, g.dy));
 }
-
-// sqrt(di^2 + dj^2) of the stencil offsets (compile-time for a fixed offset)
-__host__ __device__ constexpr float stn_sqrt_n(int n) {
-    return n == 1 ? 1.0f : (n == 2 ? 1.41421356f : (n == 4 ? 2.0f : (n == 5 ? 2.23606798f : 2.82842712f)));
+__device__ __forceinline__ void bond_add32(const BondGeom32 &g, float cw, float inv_eps, float VV, int micro,
+                                           float &Fbx, float &Fby) {
+    const float2 f = bond_force32(g, cw, inv_eps, VV, micro);
+    Fbx = __fadd_rn(Fbx, f.x);
+    Fby = __fadd_rn(Fby, f.y);
 }
-
-// Offset o (0..23) of the bond stencil: the 5 x 5 lattice block without its
-// centre, in (dj, di) order.
-__host__ __device__ constexpr int stn_di(int o) { return (o + (o >= 12 ? 1 : 0)) % 5 - 2; }
-__host__ __device__ constexpr int stn_dj(int o) { return (o + (o >= 12 ? 1 : 0)) / 5 - 2; }
 
 // FP32-split forces of node i: the same laws and lane layout, with the bond,
 // self-contact and contact arithmetic on the FP32 pipe.  Positions are
@@ -1238,99 +1632,281 @@ __device__ __forceinline__ bool sur_healthy(const DevPtrs &d) {
     return __ldcg(&d.status[PD_STATUS_TIMEOUT]) == 0 && (d.mlp_err == nullptr || __ldcg(d.mlp_err) == 0);
 }
 
-template <bool PERSIST, int LANES>
-__device__ __forceinline__ void force_node32(const DevPtrs &d, const KParams &k, int i, int lane, bool active,
-                                             int vin, Sums32 &out) {
-    const int ii = active ? i : 0;
-    const float4 qi = ldm<PERSIST>(&cur_pq<PERSIST>(d)[ii]);
-    const float2 phi = make_float2(qi.x, qi.y), pli = make_float2(qi.z, qi.w);
-    const int gi = __ldg(&d.grain[ii]);
-    const int ag = __ldg(&d.g_agg[gi]);
-    const AggParams &A = d.agg[ag];
-    const float4 gq = __ldg(&d.gq[gi]);                   // (h, h^2 hi, h^2 lo, V)
-    const float Vi = gq.w;
-    const float4 gc = __ldg(&d.gc[gi]);                   // (c_w, s0, eps) as floats
-    const float cw = gc.x, s0 = gc.y, eps = gc.z;
-    const float s0_lo = s0 * (1.0f - k.guard), s0_hi = s0 * (1.0f + k.guard);
-    // lattice stencil of the node's bonds (regular nodes: the neighbour at
-    // offset o is node ii + di + D[dj], no column load), else the CSR columns
-    const uint4 st = (k.stencil && active) ? __ldg(&d.stn[ii]) : make_uint4(kStnIrregular, 0u, 0u, 0u);
-    const bool stencil = !(st.x & kStnIrregular);
-    int r0 = 0, r1 = 0;
-    if (stencil) {
-        r0 = (int)st.w;
-        r1 = r0 + __popc(st.x);
-    } else if (active) {
-        r0 = __ldg(&d.row_ptr[ii]);
-        r1 = __ldg(&d.row_ptr[ii + 1]);
-    }
-    uint32_t *bw = d.bits + (size_t)ii * k.wpn;
-    const float Rc = A.rcf, Kn = A.knf;
+// Shared memory of an FP32-split tile: the bond slots, the positions of the
+// tile and of the one after it (by tile parity; the even tile's first ones again
+// behind the odd tile, so that no index wraps), and the streams of the tile's
+// nodes.  A step reads about 180 bytes a node in a chain of dependent loads,
+// and with the bonds evaluated once the warps that fit no longer hide that
+// chain: with every load on the spot the same loop took 347 us on 2.28M nodes
+// (16 warps an SM, 60 % of their time waiting for memory).  So every thread
+// copies its next node's streams asynchronously while it works on the present
+// one, and the bond loop's gathers are shared-memory reads.  A step of that
+// ensemble (kernel alone) went from 226 us, with the loop that evaluates each
+// bond twice from L1-cached gathers, to about 140 us; 1,119 instead of 2,350
+// thread instructions a node.
+template <int BLOCK>
+struct Tile32 {
+    float2 slot[kPairHalf * PairTile<float2, BLOCK>::kStride];
+    static constexpr int kAhead = kCarry + 8;           // farthest forward place read, absent bonds included
+    float4 q[2 * BLOCK + kAhead];
+    uint4 st[BLOCK];
+    double2 v[BLOCK], u[BLOCK], xs[BLOCK];
+    float4 sref[BLOCK];
+    float2 a[BLOCK];
+    int2 cell[BLOCK];
+    int gi[BLOCK], nc[BLOCK];
+    uint32_t bits[BLOCK];
+};
 
-    float Fbx = 0.f, Fby = 0.f;
-    const float VV = Vi * Vi;
-    // learned modal surrogate: between judge steps an active grain skips the
-    // bond loop; the epilogue adds its surrogate bond force instead
-    bool sur = false, judge = false;
-    if constexpr (!PERSIST) {
-        if (k.sur && active) {
-            sur = d.sur_active[gi] != 0 && sur_healthy(d);
-            judge = (*d.step) % k.judge_every == 0;
+// What the bond loop takes from a node's grain and list.
+struct BondNode32 {
+    float4 qi, gq, gc;      // position; (h, h^2 hi, h^2 lo, V); (c_w, s0, eps, rho)
+    uint4 st;               // stencil record
+};
+
+// The forward half of a node's stencil bonds: their forces into the thread's
+// slots and their sum in (Fx, Fy).  alive: the intact ones of st.x.  win: the
+// node's place in the position window.  Straight-line code over all twelve
+// offsets: a slot of an absent bond holds what the arithmetic makes of the
+// wrong position (nobody reads it: bonds are in both nodes' lists), and one
+// comparison over the largest excess of a stretch tells whether the general
+// pass after it is needed.  OWN: the block owns the node (broken-bond word bw)
+// and records its broken bonds.
+template <int BLOCK, bool OWN, bool MICRO>
+__device__ __forceinline__ void tile_forward32(const KParams &k, uint32_t alive, const BondNode32 &nd, const float4 *win,
+                                               float2 *mine, uint32_t *bw, float &Fx, float &Fy, unsigned &note) {
+    constexpr int S = PairTile<float2, BLOCK>::kStride;
+    const float2 phi = make_float2(nd.qi.x, nd.qi.y), pli = make_float2(nd.qi.z, nd.qi.w);
+    const float VV = nd.gq.w * nd.gq.w, inv_eps = MICRO ? 1.0f / nd.gc.z : 0.f;
+    const float s0_lo = nd.gc.y * (1.0f - k.guard);
+    const float4 *const row[3] = {win, win + stn_row(nd.st, 1), win + stn_row(nd.st, 2)};
+    float excess = 0.f;
+    Fx = Fy = 0.f;
+    constexpr int kBatch = 4;
+#pragma unroll
+    for (int m0 = 0; m0 < kPairHalf; m0 += kBatch) {
+        float4 qb[kBatch];
+#pragma unroll
+        for (int m = 0; m < kBatch; ++m) {
+            const int o = kPairHalf + m0 + m;
+            qb[m] = row[stn_dj(o)][stn_di(o)];
+        }
+#pragma unroll
+        for (int m = 0; m < kBatch; ++m) {
+            const int o = kPairHalf + m0 + m, di = stn_di(o), dj = stn_dj(o), n = di * di + dj * dj;
+            BondGeom32 g;
+            bond_geom32(qb[m], phi, pli, (float)n, stn_sqrt_n(n), nd.gq, g, (n & (n - 1)) == 0);
+            const float2 f = bond_force32(g, nd.gc.x, inv_eps, VV, MICRO);
+            mine[(m0 + m) * S] = f;
+            if ((alive >> o) & 1u) {
+                excess = fmaxf(excess, bond_excess32(g, s0_lo));      // (a NaN stretch counts as intact)
+                Fx = __fadd_rn(Fx, f.x);
+                Fy = __fadd_rn(Fy, f.y);
+            }
         }
     }
-    // broken-bond bits of the node's first 32 bonds: only the node's own threads
-    // set them, each for its own bonds, so one load at the start serves the loop
-    const uint32_t w0 = active ? __ldcg(bw) : 0u;
-    bool pending = false;      // a bond of this lane lies in the guard band
-    // bonds in batches of kBondBatch per lane: the column indices, broken words and
-    // neighbour positions of a batch are all in flight before any is used (the
-    // per-lane summation order is unchanged: bonds lane, lane + LANES, ...)
-    constexpr int kBondBatch = 4;
-    if (stencil && !(sur && !judge)) {
-        const uint32_t mask = st.x;
-        // the intact bonds by stencil offset: the broken-bond bits follow the
-        // order of the node's bonds (the rank of the offset among the stencil
-        // bits), so each set bit clears the stencil bit of that rank (a node
-        // seldom has a broken bond: the loop is skipped)
-        uint32_t alive = mask;
-        for (uint32_t wb = w0; wb; wb &= wb - 1u) {
-            uint32_t m = mask;
-            for (int t = __ffs(wb) - 1; t > 0; --t) m &= m - 1u;
-            alive &= ~(m & (0u - m));
-        }
-        const int Dm2 = (int)(short)(st.y & 0xFFFFu), Dm1 = (int)(short)(st.y >> 16);
-        const int Dp1 = (int)(short)(st.z & 0xFFFFu), Dp2 = (int)(short)(st.z >> 16);
-        constexpr int kPerLane = (24 + LANES - 1) / LANES;
-        // fully unrolled: offsets, lattice codes and sqrt(n) are constants for one
-        // lane per node (a loop over the batches was 30 % slower on the compaction)
-#pragma unroll
-        for (int m0 = 0; m0 < kPerLane; m0 += kBondBatch) {
-            float4 qb[kBondBatch];
-            bool live[kBondBatch];
-#pragma unroll
-            for (int m = 0; m < kBondBatch; ++m) {
-                const int o = (m0 + m) * LANES + lane;
-                const int dj = stn_dj(o), di = stn_di(o);
-                const int D = dj == -2 ? Dm2 : (dj == -1 ? Dm1 : (dj == 0 ? 0 : (dj == 1 ? Dp1 : Dp2)));
-                live[m] = (m0 + m) < kPerLane && o < 24 && ((alive >> o) & 1u);
-                qb[m] = ldm<PERSIST>(&cur_pq<PERSIST>(d)[live[m] ? ii + di + D : ii]);
+    if (excess > 0.f || alive != nd.st.x) {
+        // a bond breaks, lies in the guard band or is broken: markers and the sum again
+        Fx = Fy = 0.f;
+        for (uint32_t m = nd.st.x & ~((1u << kPairHalf) - 1u); m; m &= m - 1u) {
+            const int o = __ffs(m) - 1, di = stn_di(o), dj = stn_dj(o), n = di * di + dj * dj;
+            float2 *const at = &mine[(o - kPairHalf) * S];
+            unsigned mark = kPairNone;
+            if ((alive >> o) & 1u) {
+                BondGeom32 g;
+                const int r = bond_classify32(win[di + stn_row(nd.st, dj)], phi, pli, (float)n, stn_sqrt_n(n), nd.gq, s0_lo,
+                                              nd.gc.y * (1.0f + k.guard), g);
+                if (r == 0) {
+                    Fx = __fadd_rn(Fx, at->x);
+                    Fy = __fadd_rn(Fy, at->y);
+                    continue;
+                }
+                mark = r == 1 ? kPairBroken : kPairGuard;
+                if (r == 2) {
+                    note |= kNoteGuard;
+                } else if (OWN) {
+                    atomicOr(bw, stn_bit(nd.st.x, o));
+                    note |= kNoteBroke;
+                }
             }
+            at->x = __uint_as_float(mark);
+        }
+    }
+}
+
+// The backward half of node ii's bonds, from the slots of the nodes that formed
+// them: its sum in (Fx, Fy).
+template <bool PERSIST, int BLOCK>
+__device__ __forceinline__ void tile_backward32(const DevPtrs &d, const KParams &k, int ii, uint32_t alive,
+                                                const BondNode32 &nd, const float2 *mine, float &Fx, float &Fy,
+                                                unsigned &note) {
+    constexpr int S = PairTile<float2, BLOCK>::kStride;
+    const float2 *const row[3] = {mine + stn_row(nd.st, -2), mine + stn_row(nd.st, -1), mine};
+    Fx = Fy = 0.f;
 #pragma unroll
-            for (int m = 0; m < kBondBatch; ++m) {
-                if (!live[m]) continue;
-                const int o = (m0 + m) * LANES + lane;
-                const int dj = stn_dj(o), di = stn_di(o);
+    for (int o = 0; o < kPairHalf; ++o) {
+        // (a row without bonds has offset 0: some slot of the tile)
+        const float2 v = row[stn_dj(o) + 2][(kPairHalf - 1 - o) * S + stn_di(o)];
+        if ((alive >> o) & 1u) {
+            Fx = __fsub_rn(Fx, v.x);
+            Fy = __fsub_rn(Fy, v.y);
+        }
+    }
+    if (Fx != Fx) {
+        // some slot holds a marker (or a force is not finite): the half again
+        const float2 phi = make_float2(nd.qi.x, nd.qi.y), pli = make_float2(nd.qi.z, nd.qi.w);
+        Fx = Fy = 0.f;
+        for (uint32_t m = alive & ((1u << kPairHalf) - 1u); m; m &= m - 1u) {
+            const int o = __ffs(m) - 1, di = stn_di(o), dj = stn_dj(o), off = di + stn_row(nd.st, dj);
+            const float2 v = mine[(kPairHalf - 1 - o) * S + off];
+            unsigned mark = __float_as_uint(v.x);
+            if (mark == kPairNone) {
                 const int n = di * di + dj * dj;
-                BondGeom32 bg;
-                const int r = bond_classify32(qb[m], phi, pli, (float)n, stn_sqrt_n(n), gq, s0_lo, s0_hi, bg,
-                                              (n & (n - 1)) == 0);
-                if (r == 0) bond_add32(bg, cw, eps, VV, k.micro, Fbx, Fby);
-                else if (r == 2) pending = true;
-                else atomicOr(bw, 1u << __popc(mask & ((1u << o) - 1u)));
+                BondGeom32 g;
+                const int r = bond_classify32(ldm<PERSIST>(&cur_pq<PERSIST>(d)[ii + off]), phi, pli, (float)n,
+                                              stn_sqrt_n(n), nd.gq, nd.gc.y * (1.0f - k.guard),
+                                              nd.gc.y * (1.0f + k.guard), g);
+                if (r == 0) {
+                    bond_add32(g, nd.gc.x, 1.0f / nd.gc.z, nd.gq.w * nd.gq.w, k.micro, Fx, Fy);
+                    continue;
+                }
+                mark = r == 1 ? kPairBroken : kPairGuard;
+            }
+            if (mark == kPairBroken) {
+                atomicOr(&d.bits[(size_t)ii * k.wpn], stn_bit(nd.st.x, o));
+                note |= kNoteBroke;
+            } else if (mark == kPairGuard) {
+                note |= kNoteGuard;
+            } else {
+                Fx = __fsub_rn(Fx, v.x);
+                Fy = __fsub_rn(Fy, v.y);
             }
         }
     }
-    for (int b0 = r0 + lane; b0 < r1 && !stencil && !(sur && !judge); b0 += kBondBatch * LANES) {
+}
+
+// The bonds of a node that lie in the guard band, in the order of its list
+// (every step-th from lane): FP64 break decision, else the FP32 force.
+template <bool PERSIST>
+__device__ __forceinline__ void guard_bonds32(const DevPtrs &d, const KParams &k, int ii, int r0, int r1, int lane, int step,
+                                           bool stencil, float2 phi, float2 pli, float4 gq, float4 gc, int gi,
+                                           float s0_lo, float s0_hi, uint32_t *bw, float &Fbx, float &Fby,
+                                              unsigned &note) {
+    for (int b = r0 + lane; b < r1; b += step) {
+        const int kk = b - r0;
+        if ((__ldcg(&bw[kk >> 5]) >> (kk & 31)) & 1u) continue;
+        const uint32_t c = __ldg(&d.colx[b]);
+        const int j = (int)(c & kColMask);
+        const float4 qj = ldm<PERSIST>(&cur_pq<PERSIST>(d)[j]);
+        const float nn = (float)(c >> kColBits);
+        // the same classification as the loop (stencil: sqrt(n) from the table)
+        const float sqn = stencil ? stn_sqrt_n((int)nn) : sqrt_approx(nn);
+        BondGeom32 bg;
+        if (bond_classify32(qj, phi, pli, nn, sqn, gq, s0_lo, s0_hi, bg) != 2) continue;
+        const double2 pi = position64<PERSIST>(d, ii), pj = position64<PERSIST>(d, j);
+        const double ddx = __dsub_rn(pj.x, pi.x), ddy = __dsub_rn(pj.y, pi.y);
+        const double L64 = __dsqrt_rn(__dadd_rn(__dmul_rn(ddx, ddx), __dmul_rn(ddy, ddy)));
+        const double xi64 = __ldg(&d.xi[b]);
+        if (fabs(__ddiv_rn(__dsub_rn(L64, xi64), xi64)) > __ldg(&d.g_s0[gi])) {
+            atomicOr(&bw[kk >> 5], 1u << (kk & 31));
+            note |= kNoteBroke;
+            continue;
+        }
+        bond_add32(bg, gc.x, 1.0f / gc.z, gq.w * gq.w, k.micro, Fbx, Fby);
+    }
+}
+
+// Contact force of candidate j on node ii, FP32 split: self-contact into fs,
+// inter-grain contact into fn, zero beyond R_c (exact in float-float).
+template <bool PERSIST>
+__device__ __forceinline__ void contact_pair32(const DevPtrs &d, const KParams &k, const AggParams &A, int ii, int j,
+                                               int vin, int gi, int r0, int r1, float2 phi, float2 pli, float4 gq,
+                                               float4 gc, float4 qj, double2 vi64, float &fsx, float &fsy, float &fnx,
+                                               float &fny) {
+    fsx = fsy = fnx = fny = 0.f;
+    const float Rc = A.rcf, Kn = A.knf, Vi = gq.w, cw = gc.x;
+    const float rd = k.rdf, rho = gc.w, dt = k.dtf, mu = k.muf;     // rho: this grain's density
+    const float dxh = __fsub_rn(qj.x, phi.x), dxl = qj.z - pli.x;
+    const float dyh = __fsub_rn(qj.y, phi.y), dyl = qj.w - pli.y;
+    float L2h, L2l;
+    len2_ff(dxh, dxl, dyh, dyl, L2h, L2l);
+    if (!(ff_diff(A.rc2_hi, A.rc2_lo, L2h, L2l) > 0.f)) return;
+    const float dd = sqrtf(L2h);
+    if (dd == 0.f) {
+        atomicAdd(&d.status[PD_STATUS_COINCIDENT], 1);
+        return;
+    }
+    const float ex = (dxh + dxl) / dd, ey = (dyh + dyl) / dd;
+    const float overlap = ff_diff(A.rc2_hi, A.rc2_lo, L2h, L2l) / (Rc + dd);   // R_c - |d|
+    const int gj = __ldg(&d.grain[j]);
+    const float Vj = __ldg(&d.gq[gj]).w;
+    // v(x) - v(y) in FP64, rounded once to float (nearby nodes move alike:
+    // a float difference of float velocities would cancel)
+    const double2 vj64 = ldm<PERSIST>(&d.v[vin][j]);
+    const float vrx = (float)__dsub_rn(vi64.x, vj64.x), vry = (float)__dsub_rn(vi64.y, vj64.y);
+    if (gj == gi) {
+        if (bonded_intact(d, k, ii, r0, r1, j)) return;
+        const int2 li = __ldg(&d.lat[ii]), lj = __ldg(&d.lat[j]);
+        const int di = lj.x - li.x, dj = lj.y - li.y;
+        const float nn = (float)(di * di + dj * dj);
+        const float xi = gq.x * sqrtf(nn);
+        float m;
+        if (xi < Rc) {
+            float q2, eq2;
+            two_prod(nn, gq.y, q2, eq2);
+            const float dl = ff_diff(L2h, L2l, q2, eq2 + nn * gq.z) / (dd + xi);   // |d| - |xi|
+            m = (dl < 0.f) ? cw * dl / xi : 0.f;
+        } else {
+            m = -cw * overlap / Rc;
+        }
+        if (m == 0.f) return;
+        const float f = m * Vi * Vj;
+        float gx = f * ex, gy = f * ey;
+        const float Kns = k.mat ? __ldg(&d.g_kf[gi]) : Kn;
+        damping_friction32(rd, Kns, rho, rho, dt, mu, ex, ey, vrx, vry, -f, Vi, Vj, gx, gy);
+        fsx = gx;
+        fsy = gy;
+    } else {
+        // the harmonic mean of the grains' own K_n is K_n of the harmonic-mean modulus
+        const float Knp = k.mat ? harmonic32(__ldg(&d.g_kf[gi]), __ldg(&d.g_kf[gj])) : Kn;
+        const float Fr = Knp * overlap * Vi * Vj;
+        float gx = -Fr * ex, gy = -Fr * ey;
+        damping_friction32(rd, Knp, harmonic32(rho, __ldg(&d.gc[gj]).w), rho, dt, mu, ex, ey, vrx, vry, Fr, Vi,
+                           Vj, gx, gy);
+        fnx = gx;
+        fny = gy;
+    }
+}
+
+// Contact forces of node ii, FP32 split: every LANES-th of its nc + nb candidates.
+template <bool PERSIST, int LANES>
+__device__ __forceinline__ void contacts32(const DevPtrs &d, const KParams &k, int ii, int lane, int vin, int gi, int nc,
+                                           int nb, int r0, int r1, float2 phi, float2 pli, float4 gq, float4 gc, float &Fsx,
+                                           float &Fsy, float &Fnx, float &Fny) {
+    const AggParams &A = d.agg[__ldg(&d.g_agg[gi])];
+    const double2 vi64 = ldm<PERSIST>(&d.v[vin][ii]);      // start-of-step velocity
+    for (int q = lane; q < nc + nb; q += LANES) {
+        const int j = candidate<PERSIST>(d, k, ii, nc, r0, q);
+        float a, b, c, e;
+        contact_pair32<PERSIST>(d, k, A, ii, j, vin, gi, r0, r1, phi, pli, gq, gc, ldm<PERSIST>(&cur_pq<PERSIST>(d)[j]),
+                                vi64, a, b, c, e);
+        Fsx += a;
+        Fsy += b;
+        Fnx += c;
+        Fny += e;
+    }
+}
+
+// The bonds of node ii from its CSR columns (a row with a gap, a horizon
+// without the stencil): every LANES-th from lane.
+template <bool PERSIST, int LANES>
+__device__ __forceinline__ void csr_bonds32(const DevPtrs &d, const KParams &k, int ii, int lane, int r0, int r1,
+                                            float2 phi, float2 pli, float4 gq, float4 gc, float s0_lo, float s0_hi,
+                                            uint32_t w0, float &Fbx, float &Fby, unsigned &note) {
+    constexpr int kBondBatch = 4;
+    uint32_t *bw = d.bits + (size_t)ii * k.wpn;
+    const float cw = gc.x, VV = gq.w * gq.w, inv_eps = 1.0f / gc.z;
+    for (int b0 = r0 + lane; b0 < r1; b0 += kBondBatch * LANES) {
         uint32_t cb[kBondBatch], wb[kBondBatch];
 #pragma unroll
         for (int m = 0; m < kBondBatch; ++m) {
@@ -1353,99 +1929,108 @@ __device__ __forceinline__ void force_node32(const DevPtrs &d, const KParams &k,
             const float nn = (float)(cb[m] >> kColBits);         // lattice offset di^2 + dj^2
             BondGeom32 bg;
             const int r = bond_classify32(qb[m], phi, pli, nn, sqrt_approx(nn), gq, s0_lo, s0_hi, bg);
-            if (r == 0) bond_add32(bg, cw, eps, VV, k.micro, Fbx, Fby);
-            else if (r == 2) pending = true;
-            else atomicOr(&bw[kk >> 5], 1u << (kk & 31));
-        }
-    }
-    if (pending) {
-        // the lane's bonds in the guard band, in its order: FP64 break decision,
-        // else the FP32 force
-        for (int b = r0 + lane; b < r1; b += LANES) {
-            const int kk = b - r0;
-            if ((__ldcg(&bw[kk >> 5]) >> (kk & 31)) & 1u) continue;
-            const uint32_t c = __ldg(&d.colx[b]);
-            const int j = (int)(c & kColMask);
-            const float4 qj = ldm<PERSIST>(&cur_pq<PERSIST>(d)[j]);
-            const float nn = (float)(c >> kColBits);
-            // the same classification as the loop (stencil: sqrt(n) from the table)
-            const float sqn = stencil ? stn_sqrt_n((int)nn) : sqrt_approx(nn);
-            BondGeom32 bg;
-            if (bond_classify32(qj, phi, pli, nn, sqn, gq, s0_lo, s0_hi, bg) != 2) continue;
-            const double2 pi = position64<PERSIST>(d, ii), pj = position64<PERSIST>(d, j);
-            const double ddx = __dsub_rn(pj.x, pi.x), ddy = __dsub_rn(pj.y, pi.y);
-            const double L64 = __dsqrt_rn(__dadd_rn(__dmul_rn(ddx, ddx), __dmul_rn(ddy, ddy)));
-            const double xi64 = __ldg(&d.xi[b]);
-            if (fabs(__ddiv_rn(__dsub_rn(L64, xi64), xi64)) > __ldg(&d.g_s0[gi])) {
-                atomicOr(&bw[kk >> 5], 1u << (kk & 31));
-                continue;
-            }
-            bond_add32(bg, cw, eps, VV, k.micro, Fbx, Fby);
-        }
-    }
-    __syncwarp();
-
-    // contact candidates from the node's list (ascending node index); the
-    // R_c test is exact in float-float
-    const int nc = active ? ldm<PERSIST>(&d.nbr_cnt[ii]) : 0;
-    // start-of-step velocity (FP64; read only by nodes with candidates)
-    const double2 vi64 = nc > 0 ? ldm<PERSIST>(&d.v[vin][ii]) : make_double2(0.0, 0.0);
-    const float rd = k.rdf, rho = gc.w, dt = k.dtf, mu = k.muf;     // rho: this grain's density
-    float Fsx = 0.f, Fsy = 0.f, Fnx = 0.f, Fny = 0.f;
-    for (int q = lane; q < nc; q += LANES) {
-        const int j = ldm<PERSIST>(&d.nbr[(size_t)q * k.N + ii]);
-        const float4 qj = ldm<PERSIST>(&cur_pq<PERSIST>(d)[j]);
-        const float dxh = __fsub_rn(qj.x, phi.x), dxl = qj.z - pli.x;
-        const float dyh = __fsub_rn(qj.y, phi.y), dyl = qj.w - pli.y;
-        float L2h, L2l;
-        len2_ff(dxh, dxl, dyh, dyl, L2h, L2l);
-        if (!(ff_diff(A.rc2_hi, A.rc2_lo, L2h, L2l) > 0.f)) continue;
-        const float dd = sqrtf(L2h);
-        if (dd == 0.f) {
-            atomicAdd(&d.status[PD_STATUS_COINCIDENT], 1);
-            continue;
-        }
-        const float ex = (dxh + dxl) / dd, ey = (dyh + dyl) / dd;
-        const float overlap = ff_diff(A.rc2_hi, A.rc2_lo, L2h, L2l) / (Rc + dd);   // R_c - |d|
-        const int gj = __ldg(&d.grain[j]);
-        const float Vj = __ldg(&d.gq[gj]).w;
-        // v(x) - v(y) in FP64, rounded once to float (nearby nodes move alike:
-        // a float difference of float velocities would cancel)
-        const double2 vj64 = ldm<PERSIST>(&d.v[vin][j]);
-        const float vrx = (float)__dsub_rn(vi64.x, vj64.x), vry = (float)__dsub_rn(vi64.y, vj64.y);
-        if (gj == gi) {
-            if (bonded_intact(d, k, ii, r0, r1, j)) continue;
-            const int2 li = __ldg(&d.lat[ii]), lj = __ldg(&d.lat[j]);
-            const int di = lj.x - li.x, dj = lj.y - li.y;
-            const float nn = (float)(di * di + dj * dj);
-            const float xi = gq.x * sqrtf(nn);
-            float m;
-            if (xi < Rc) {
-                float q2, eq2;
-                two_prod(nn, gq.y, q2, eq2);
-                const float dl = ff_diff(L2h, L2l, q2, eq2 + nn * gq.z) / (dd + xi);   // |d| - |xi|
-                m = (dl < 0.f) ? cw * dl / xi : 0.f;
+            if (r == 0) {
+                bond_add32(bg, cw, inv_eps, VV, k.micro, Fbx, Fby);
+            } else if (r == 2) {
+                note |= kNoteGuard;
             } else {
-                m = -cw * overlap / Rc;
+                atomicOr(&bw[kk >> 5], 1u << (kk & 31));
+                note |= kNoteBroke;
             }
-            if (m == 0.f) continue;
-            const float f = m * Vi * Vj;
-            float gx = f * ex, gy = f * ey;
-            const float Kns = k.mat ? __ldg(&d.g_kf[gi]) : Kn;
-            damping_friction32(rd, Kns, rho, rho, dt, mu, ex, ey, vrx, vry, -f, Vi, Vj, gx, gy);
-            Fsx += gx;
-            Fsy += gy;
-        } else {
-            // the harmonic mean of the grains' own K_n is K_n of the harmonic-mean modulus
-            const float Knp = k.mat ? harmonic32(__ldg(&d.g_kf[gi]), __ldg(&d.g_kf[gj])) : Kn;
-            const float Fr = Knp * overlap * Vi * Vj;
-            float gx = -Fr * ex, gy = -Fr * ey;
-            damping_friction32(rd, Knp, harmonic32(rho, __ldg(&d.gc[gj]).w), rho, dt, mu, ex, ey, vrx, vry, Fr, Vi,
-                               Vj, gx, gy);
-            Fnx += gx;
-            Fny += gy;
         }
     }
+}
+
+template <bool PERSIST, int LANES>
+__device__ __forceinline__ void force_node32(const DevPtrs &d, const KParams &k, int i, int lane, bool active,
+                                             int vin, Sums32 &out) {
+    const int ii = active ? i : 0;
+    const float4 qi = ldm<PERSIST>(&cur_pq<PERSIST>(d)[ii]);
+    const float2 phi = make_float2(qi.x, qi.y), pli = make_float2(qi.z, qi.w);
+    const int gi = __ldg(&d.grain[ii]);
+    const int ag = __ldg(&d.g_agg[gi]);
+    const float4 gq = __ldg(&d.gq[gi]);                   // (h, h^2 hi, h^2 lo, V)
+    const float4 gc = __ldg(&d.gc[gi]);                   // (c_w, s0, eps) as floats
+    const float cw = gc.x, s0 = gc.y, inv_eps = 1.0f / gc.z;
+    const float s0_lo = s0 * (1.0f - k.guard), s0_hi = s0 * (1.0f + k.guard);
+    // lattice stencil of the node's bonds (regular nodes: the neighbour at
+    // offset o is node ii + di + D[dj], no column load), else the CSR columns
+    const uint4 st = (k.stencil && active) ? __ldg(&d.stn[ii]) : make_uint4(kStnIrregular, 0u, 0u, 0u);
+    const bool stencil = !(st.x & kStnIrregular);
+    int r0 = 0, r1 = 0;
+    if (stencil) {
+        r0 = (int)st.w;
+        r1 = r0 + __popc(st.x);
+    } else if (active) {
+        r0 = __ldg(&d.row_ptr[ii]);
+        r1 = __ldg(&d.row_ptr[ii + 1]);
+    }
+    uint32_t *bw = d.bits + (size_t)ii * k.wpn;
+    float Fbx = 0.f, Fby = 0.f;
+    const float VV = gq.w * gq.w;
+    // learned modal surrogate: between judge steps an active grain skips the
+    // bond loop; the epilogue adds its surrogate bond force instead
+    bool sur = false, judge = false;
+    if constexpr (!PERSIST) {
+        if (k.sur && active) {
+            sur = d.sur_active[gi] != 0 && sur_healthy(d);
+            judge = (*d.step) % k.judge_every == 0;
+        }
+    }
+    const bool bonds = !(sur && !judge);
+    // broken-bond bits of the node's first 32 bonds: only the node's own threads
+    // set them, each for its own bonds, so one load at the start serves the loop
+    const uint32_t w0 = active ? __ldcg(bw) : 0u;
+    unsigned note = 0u;
+    // bonds in batches of kBondBatch per lane: the column indices, broken words and
+    // neighbour positions of a batch are all in flight before any is used (the
+    // per-lane summation order is unchanged: bonds lane, lane + LANES, ...)
+    constexpr int kBondBatch = 4;
+    if (stencil && bonds) {
+        const uint32_t mask = st.x, alive = stn_alive(mask, w0);
+        constexpr int kPerLane = (24 + LANES - 1) / LANES;
+        // fully unrolled (a loop over the batches was 30 % slower on the compaction)
+#pragma unroll
+        for (int m0 = 0; m0 < kPerLane; m0 += kBondBatch) {
+            float4 qb[kBondBatch];
+            bool live[kBondBatch];
+#pragma unroll
+            for (int m = 0; m < kBondBatch; ++m) {
+                const int o = (m0 + m) * LANES + lane;
+                live[m] = (m0 + m) < kPerLane && o < 24 && ((alive >> o) & 1u);
+                qb[m] = ldm<PERSIST>(&cur_pq<PERSIST>(d)[live[m] ? ii + stn_di(o) + stn_row(st, stn_dj(o)) : ii]);
+            }
+#pragma unroll
+            for (int m = 0; m < kBondBatch; ++m) {
+                if (!live[m]) continue;
+                const int o = (m0 + m) * LANES + lane;
+                const int dj = stn_dj(o), di = stn_di(o);
+                const int n = di * di + dj * dj;
+                BondGeom32 bg;
+                const int r = bond_classify32(qb[m], phi, pli, (float)n, stn_sqrt_n(n), gq, s0_lo, s0_hi, bg);
+                if (r == 0) {
+                    bond_add32(bg, cw, inv_eps, VV, k.micro, Fbx, Fby);
+                } else if (r == 2) {
+                    note |= kNoteGuard;
+                } else {
+                    atomicOr(bw, stn_bit(mask, o));
+                    note |= kNoteBroke;
+                }
+            }
+        }
+    }
+    if (!stencil && bonds)
+        csr_bonds32<PERSIST, LANES>(d, k, ii, lane, r0, r1, phi, pli, gq, gc, s0_lo, s0_hi, w0, Fbx, Fby, note);
+    if (note & kNoteGuard)
+        guard_bonds32<PERSIST>(d, k, ii, r0, r1, lane, LANES, stencil, phi, pli, gq, gc, gi, s0_lo, s0_hi, bw, Fbx, Fby,
+                                note);
+    __syncwarp();
+    float Fsx = 0.f, Fsy = 0.f, Fnx = 0.f, Fny = 0.f;
+    const int nc = active ? ldm<PERSIST>(&d.nbr_cnt[ii]) : 0;
+    const int nb = fresh_bonds(d, k, ii, any_lane<LANES>(w0 != 0u || (note & kNoteBroke) || (active && k.wpn > 1)));
+    if (nc + nb > 0)
+        contacts32<PERSIST, LANES>(d, k, ii, lane, vin, gi, nc, nb, r0, r1, phi, pli, gq, gc, Fsx, Fsy, Fnx, Fny);
+    __syncwarp();
     out.bx = lane_sum<LANES>(Fbx);
     out.by = lane_sum<LANES>(Fby);
     out.sx = lane_sum<LANES>(Fsx);
@@ -1455,20 +2040,174 @@ __device__ __forceinline__ void force_node32(const DevPtrs &d, const KParams &k,
     if (sur && judge && lane == 0) d.sur_fb[i] = make_float2(out.bx, out.by);   // full bond force for the judge
 }
 
+// FP32 split, one thread per node: forces of the nodes [lo, hi) by the calling
+// block, in tiles (see PairTile, Tile32).  All threads call out(i, sums, place,
+// active, contact) with each node's sums, its update streams in shared memory at
+// `place` when `update`; without INLINE the contact forces are left to a later
+// pass (contact: the node has candidates).
+template <bool PERSIST, int BLOCK, bool INLINE, class Out>
+__device__ __forceinline__ void tile_nodes32(const DevPtrs &d, const KParams &k, int lo, int hi, int vin, bool update,
+                                             Tile32<BLOCK> &sm, Out out) {
+    if (lo >= hi) return;
+    const int tid = threadIdx.x;
+    const float4 *const pq = cur_pq<PERSIST>(d);
+    const double2 *const cu = cur_u<PERSIST>(d);
+    // positions are read up to kCarry nodes past the run
+    const int qend = min(hi + kCarry, k.N);
+    auto copy_q = [&](int i, int half) {
+        if (i >= qend) return;
+        copy_async(&sm.q[half * BLOCK + tid], &pq[i]);
+        if (half == 0 && tid < Tile32<BLOCK>::kAhead) copy_async(&sm.q[2 * BLOCK + tid], &pq[i]);
+    };
+    auto copy_list = [&](int i) {
+        if (i >= hi) return;
+        copy_async(&sm.st[tid], &d.stn[i]);
+        copy_async(&sm.gi[tid], &d.grain[i]);
+        copy_async(&sm.nc[tid], &d.nbr_cnt[i]);
+        copy_async(&sm.bits[tid], &d.bits[(size_t)i * k.wpn]);
+    };
+    auto copy_update = [&](int i) {
+        if (i >= hi || !update) return;
+        copy_async(&sm.v[tid], &d.v[vin][i]);
+        copy_async(&sm.a[tid], &d.af[i]);
+        copy_async(&sm.cell[tid], &d.cell[i]);
+        copy_async(&sm.u[tid], &cu[i]);
+        copy_async(&sm.xs[tid], &d.xs[i]);
+        copy_async(&sm.sref[tid], &d.sref[i]);
+    };
+    // the pass before the run takes the nodes [lo - BLOCK, lo), of which the last kCarry have slots
+    const int first = lo > 0 ? lo - BLOCK : lo;
+    const int skip = lo > 0 ? BLOCK - kCarry : 0;      // threads without a node in the first pass
+    int half = 0;                                      // the tile's half of the position window
+    if (tid >= skip && first + tid >= 0) {
+        copy_q(first + tid, 0);
+        copy_list(first + tid);
+    }
+    copy_q(first + BLOCK + tid, 1);
+    copy_commit();
+    if (first == lo) copy_update(lo + tid);
+    copy_commit();
+    copy_wait<1>();
+    __syncthreads();
+    for (int node0 = first; node0 < hi; node0 += BLOCK, half ^= 1) {
+        const int i = node0 + tid;
+        const bool warm = node0 < lo;
+        const bool active = i < hi && !(warm && (tid < skip || i < 0));
+        const float4 *const win = sm.q + half * BLOCK + tid;
+        float2 *const mine = sm.slot + kCarry + tid;
+        BondNode32 nd;
+        nd.st = make_uint4(kStnIrregular, 0u, 0u, 0u);
+        nd.qi = *win;
+        int gi = 0, nc = 0;
+        uint32_t w0 = 0u;
+        if (active) {
+            nd.st = sm.st[tid];
+            gi = sm.gi[tid];
+            nc = sm.nc[tid];
+            w0 = sm.bits[tid];
+        }
+        nd.gq = __ldg(&d.gq[gi]);
+        nd.gc = __ldg(&d.gc[gi]);
+        const bool stencil = !(nd.st.x & kStnIrregular);
+        // learned modal surrogate: between judge steps an active grain skips the
+        // bond loop; the epilogue adds its surrogate bond force instead
+        bool sur = false, judge = false;
+        if constexpr (!PERSIST) {
+            if (k.sur && active) {
+                sur = d.sur_active[gi] != 0 && sur_healthy(d);
+                judge = (*d.step) % k.judge_every == 0;
+            }
+        }
+        const bool bonds = active && !(sur && !judge);
+        const uint32_t alive = bonds && stencil ? stn_alive(nd.st.x, w0) : 0u;
+        unsigned note = 0u;
+        uint32_t *bw = &d.bits[(size_t)(active ? i : 0) * k.wpn];
+        float fx = 0.f, fy = 0.f;
+        if (bonds && stencil) {
+            if (k.micro) {
+                if (warm) tile_forward32<BLOCK, false, true>(k, alive, nd, win, mine, bw, fx, fy, note);
+                else tile_forward32<BLOCK, true, true>(k, alive, nd, win, mine, bw, fx, fy, note);
+            } else {
+                if (warm) tile_forward32<BLOCK, false, false>(k, alive, nd, win, mine, bw, fx, fy, note);
+                else tile_forward32<BLOCK, true, false>(k, alive, nd, win, mine, bw, fx, fy, note);
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < kPairHalf; ++q)
+                mine[q * PairTile<float2, BLOCK>::kStride].x = __uint_as_float(kPairNone);
+        }
+        __syncthreads();
+        // the tile's positions and lists have been read: the next ones' take their places
+        copy_q(i + 2 * BLOCK, half);
+        copy_list(i + BLOCK);
+        copy_commit();
+        if (!warm) {
+            Sums32 f{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            bool contact = false;
+            if (active) {
+                tile_backward32<PERSIST, BLOCK>(d, k, i, alive, nd, mine, f.bx, f.by, note);
+                f.bx = __fadd_rn(f.bx, fx);
+                f.by = __fadd_rn(f.by, fy);
+                const float2 phi = make_float2(nd.qi.x, nd.qi.y), pli = make_float2(nd.qi.z, nd.qi.w);
+                int r0 = (int)nd.st.w, r1 = r0 + __popc(nd.st.x);
+                if (!stencil || note) {
+                    const float s0_lo = nd.gc.y * (1.0f - k.guard), s0_hi = nd.gc.y * (1.0f + k.guard);
+                    if (!stencil) {
+                        r0 = __ldg(&d.row_ptr[i]);
+                        r1 = __ldg(&d.row_ptr[i + 1]);
+                        if (bonds)
+                            csr_bonds32<PERSIST, 1>(d, k, i, 0, r0, r1, phi, pli, nd.gq, nd.gc, s0_lo, s0_hi, w0, f.bx,
+                                                    f.by, note);
+                    }
+                    if (note & kNoteGuard)
+                        guard_bonds32<PERSIST>(d, k, i, r0, r1, 0, 1, stencil, phi, pli, nd.gq, nd.gc, gi, s0_lo, s0_hi,
+                                               bw, f.bx, f.by, note);
+                }
+                const int nb = fresh_bonds(d, k, i, w0 != 0u || (note & kNoteBroke));
+                contact = nc + nb > 0;
+                if (INLINE && contact)
+                    contacts32<PERSIST, 1>(d, k, i, 0, vin, gi, nc, nb, r0, r1, phi, pli, nd.gq, nd.gc, f.sx, f.sy, f.nx,
+                                           f.ny);
+                if (sur && judge) d.sur_fb[i] = make_float2(f.bx, f.by);   // full bond force for the judge
+            }
+            copy_wait<1>();              // the node's update streams
+            out(i, f, tid, active, contact);
+        }
+        copy_update(i + BLOCK);
+        copy_commit();
+        copy_wait<1>();                  // the next tile's positions and lists
+        __syncthreads();
+        PairTile<float2, BLOCK>::carry(sm.slot);
+        __syncthreads();
+    }
+    copy_wait<0>();
+}
+
+// The update streams of node i from memory, all in flight together.
 template <bool PERSIST>
-__device__ __forceinline__ void node_epilogue32(const DevPtrs &d, const KParams &k, int i, int vin, int update_v,
-                                                const Sums32 &fin, bool total = false) {
-    // the node's independent loads first, all in flight together (the pass is
-    // bound by memory latency): velocity, previous acceleration, grain, cell
-    const double2 vi = ldm<PERSIST>(&d.v[vin][i]);
-    const float2 ao = update_v ? ldm<PERSIST>(&d.af[i]) : make_float2(0.f, 0.f);
-    const int gi = __ldg(&d.grain[i]);
-    const int2 cell = ldm<PERSIST>(&d.cell[i]);
+__device__ __forceinline__ Update32 load_update32(const DevPtrs &d, int i, int vin, int update_v) {
+    Update32 n{};
+    n.v = ldm<PERSIST>(&d.v[vin][i]);
+    n.cell = ldm<PERSIST>(&d.cell[i]);
+    if (update_v) {
+        n.a = ldm<PERSIST>(&d.af[i]);
+        if (PERSIST) {
+            // for the next step's displacement update
+            n.u = ldm<PERSIST>(&cur_u<PERSIST>(d)[i]);
+            n.xs = __ldg(&d.xs[i]);
+            n.sref = ldm<PERSIST>(&d.sref[i]);
+        }
+    }
+    return n;
+}
+
+template <bool PERSIST>
+__device__ __forceinline__ void node_epilogue32(const DevPtrs &d, const KParams &k, int i, int gi, int vin, int update_v,
+                                                const Sums32 &fin, const Update32 &n, bool total = false) {
+    const double2 vi = n.v;
     const int ag = __ldg(&d.g_agg[gi]);
     const float inv_m = __ldg(&d.g_invmf[gi]);
     const int4 wc = ldm<PERSIST>(&d.wall_cell[ag]);
-    // the displacement for the next step's update (persistent kernel)
-    const double2 ui = PERSIST && update_v ? ldm<PERSIST>(&cur_u<PERSIST>(d)[i]) : double2{};
     Sums32 f = fin;
     if constexpr (!PERSIST) {
         // learned modal surrogate: between judge steps an active grain's bond force
@@ -1483,7 +2222,7 @@ __device__ __forceinline__ void node_epilogue32(const DevPtrs &d, const KParams 
         }
     }
     double Fwx = 0.0, Fwy = 0.0;
-    const bool walls = !cells_far_from_walls(cell, wc);
+    const bool walls = !cells_far_from_walls(n.cell, wc);
     if (walls) {
         const double2 pi = position64<PERSIST>(d, i);
         const AggParams &A = d.agg[ag];
@@ -1503,7 +2242,133 @@ __device__ __forceinline__ void node_epilogue32(const DevPtrs &d, const KParams 
         d.parts[2 * (size_t)k.N + i] = make_double2((double)f.nx, (double)f.ny);
         d.parts[3 * (size_t)k.N + i] = make_double2(Fwx, Fwy);
     }
-    finish_node32_total<PERSIST>(d, k, i, vin, update_v, vi, ao, fx, fy, walls, Fwx, Fwy, inv_m, ui);
+    finish_node32_total<PERSIST>(d, k, i, vin, update_v, n, fx, fy, walls, Fwx, Fwy, inv_m);
+}
+
+// ---------------------------------------------------------------------------
+// special nodes of the persistent kernel with one thread per node: those with
+// contact candidates or near a wall.  They are few, but each takes several
+// times as long as a plain node, and a block's run of nodes can hold many: in
+// place, the blocks whose grains touch set the time of the step.  So the tile
+// pass puts such a node's bond sum aside and the node on a list (one atomic per
+// warp), and after a grid barrier all threads share the list.
+
+// Appends the calling warp's nodes i with `take` set to the list.
+__device__ __forceinline__ void list_special(const DevPtrs &d, int which, int i, bool take) {
+    const unsigned m = __ballot_sync(0xffffffffu, take);
+    if (m == 0u) return;
+    const int lane = threadIdx.x & 31, lead = __ffs(m) - 1;
+    int at = 0;
+    if (lane == lead) at = atomicAdd(&d.spec_n[which], __popc(m));
+    at = __shfl_sync(0xffffffffu, at, lead);
+    if (take) d.spec[at + __popc(m & ((1u << lane) - 1u))] = i;
+}
+
+// A group of kSpecialLanes threads takes one special node: each thread a
+// candidate (and, FP64 path, a wall or a corner), whose forces are then added
+// in the candidates' order, so the sums are those of one thread working through
+// them.  A contact is a chain of divisions and square roots -- on the 2-lane
+// FP64 pipe about 4 us -- and a node has up to a dozen.
+constexpr int kSpecialLanes = 8;
+
+// Adds the group's v, lane by lane, to the running sum `acc` of all its threads.
+template <class T>
+__device__ __forceinline__ T add_in_order(T acc, T v, int n) {
+#pragma unroll
+    for (int l = 0; l < kSpecialLanes; ++l) {
+        const T w = __shfl_sync(0xffffffffu, v, l, kSpecialLanes);
+        if (l < n) acc += w;
+    }
+    return acc;
+}
+
+// (node: the group has one; every thread of the warp calls it)
+template <bool PERSIST>
+__device__ __forceinline__ void special_node32(const DevPtrs &d, const KParams &k, int i, bool node, int vin) {
+    const int lane = threadIdx.x & (kSpecialLanes - 1);
+    const int ii = node ? i : 0;
+    const float2 b = reinterpret_cast<const float2 *>(d.fsum)[ii];
+    const float4 qi = ldm<PERSIST>(&cur_pq<PERSIST>(d)[ii]);
+    const int gi = __ldg(&d.grain[ii]), nc = node ? ldm<PERSIST>(&d.nbr_cnt[ii]) : 0;
+    const int r0 = __ldg(&d.row_ptr[ii]), r1 = __ldg(&d.row_ptr[ii + 1]);
+    const Update32 n = load_update32<PERSIST>(d, ii, vin, 1);
+    const int nb = node ? fresh_bonds(d, k, ii, true) : 0;
+    const AggParams &A = d.agg[__ldg(&d.g_agg[gi])];
+    const float4 gq = __ldg(&d.gq[gi]), gc = __ldg(&d.gc[gi]);
+    Sums32 f{b.x, b.y, 0.f, 0.f, 0.f, 0.f};
+    for (int q0 = 0; __any_sync(0xffffffffu, q0 < nc + nb); q0 += kSpecialLanes) {
+        float sx = 0.f, sy = 0.f, nx = 0.f, ny = 0.f;
+        if (q0 + lane < nc + nb) {
+            const int j = candidate<PERSIST>(d, k, ii, nc, r0, q0 + lane);
+            contact_pair32<PERSIST>(d, k, A, ii, j, vin, gi, r0, r1, make_float2(qi.x, qi.y), make_float2(qi.z, qi.w), gq,
+                                    gc, ldm<PERSIST>(&cur_pq<PERSIST>(d)[j]), n.v, sx, sy, nx, ny);
+        }
+        const int m = nc + nb - q0;
+        f.sx = add_in_order(f.sx, sx, m);
+        f.sy = add_in_order(f.sy, sy, m);
+        f.nx = add_in_order(f.nx, nx, m);
+        f.ny = add_in_order(f.ny, ny, m);
+    }
+    if (node && lane == 0) node_epilogue32<PERSIST>(d, k, ii, gi, vin, 1, f, n);
+}
+
+template <bool PERSIST>
+__device__ __forceinline__ void special_node64(const DevPtrs &d, const KParams &k, int i, bool node, int vin) {
+    const int lane = threadIdx.x & (kSpecialLanes - 1);
+    const int ii = node ? i : 0;
+    const double2 b = reinterpret_cast<const double2 *>(d.fsum)[ii];
+    const double2 pi = ldm<PERSIST>(&d.p[ii]), vi = ldm<PERSIST>(&d.v[vin][ii]), ao = ldm<PERSIST>(&d.a[ii]);
+    const int gi = __ldg(&d.grain[ii]), nc = node ? ldm<PERSIST>(&d.nbr_cnt[ii]) : 0;
+    const int r0 = __ldg(&d.row_ptr[ii]), r1 = __ldg(&d.row_ptr[ii + 1]);
+    const int2 cell = ldm<PERSIST>(&d.cell[ii]);
+    const int nb = node ? fresh_bonds(d, k, ii, true) : 0;
+    const int ag = __ldg(&d.g_agg[gi]);
+    const AggParams &A = d.agg[ag];
+    Sums64 f{b.x, b.y, 0.0, 0.0, 0.0, 0.0};
+    for (int q0 = 0; __any_sync(0xffffffffu, q0 < nc + nb); q0 += kSpecialLanes) {
+        double sx = 0.0, sy = 0.0, nx = 0.0, ny = 0.0;
+        if (q0 + lane < nc + nb) {
+            const int j = candidate<PERSIST>(d, k, ii, nc, r0, q0 + lane);
+            contact_pair64<PERSIST>(d, k, A, ii, j, vin, gi, r0, r1, pi, ldm<PERSIST>(&d.p[j]), vi, sx, sy, nx, ny);
+        }
+        const int m = nc + nb - q0;
+        f.sx = add_in_order(f.sx, sx, m);
+        f.sy = add_in_order(f.sy, sy, m);
+        f.nx = add_in_order(f.nx, nx, m);
+        f.ny = add_in_order(f.ny, ny, m);
+    }
+    // walls: thread l takes wall l, thread 4 + c corner c
+    const bool walls = node && !cells_far_from_walls(cell, ldm<PERSIST>(&d.wall_cell[ag]));
+    double Fwx = 0.0, Fwy = 0.0;
+    if (__any_sync(0xffffffffu, walls)) {
+        double gx = 0.0, gy = 0.0;
+        if (walls) {
+            const double rho = k.mat ? __ldg(&d.g_rho[gi]) : k.rho;
+            const double Kn = k.mat ? 18.0 * __ldg(&d.g_k[gi]) / A.pe5 : A.Kn;
+            const double t = ldm<PERSIST>(d.t_now), V = __ldg(&d.V[ii]);
+            bool past, past2;
+            if (lane < 4) {
+                const double dl = wall_distance(A, lane, t, pi.x, pi.y, past);
+                if (past) atomicAdd(&d.status[PD_STATUS_PENETRATION], 1);
+                wall_single64(k, A, Kn, rho, lane, dl, vi.x, vi.y, V, gx, gy);
+            } else {
+                const int c = lane - 4;
+                wall_corner64(k, A, Kn, rho, c, wall_distance(A, c >> 1, t, pi.x, pi.y, past),
+                              wall_distance(A, 2 + (c & 1), t, pi.x, pi.y, past2), vi.x, vi.y, V, gx, gy);
+                gx = -gx;
+                gy = -gy;
+            }
+        }
+        Fwx = add_in_order(0.0, gx, kSpecialLanes);
+        Fwy = add_in_order(0.0, gy, kSpecialLanes);
+    }
+    if (!node || lane != 0) return;
+    const double inv_m = __ldg(&d.g_invm[gi]);
+    if (k.store)
+        finish_node<PERSIST, true>(d, k, ii, vin, 1, vi, 0.0, f.bx, f.by, f.sx, f.sy, f.nx, f.ny, Fwx, Fwy, inv_m);
+    else
+        finish_node64_total<PERSIST>(d, k, ii, vin, 1, vi, ao, __dadd_rn(__dadd_rn(f.bx, f.sx), f.nx),
+                                     __dadd_rn(__dadd_rn(f.by, f.sy), f.ny), walls, Fwx, Fwy, inv_m);
 }
 
 }  // namespace pd

@@ -236,7 +236,7 @@ constexpr double kPiAgg = 3.14159265358979323846;
 
 // Per-aggregate contact constants (Sec. 4.1): R_c = rc_ratio h_min and
 // K_n = 18 k / (pi eps_c^5) with eps_c = horizon_ratio h_min, h_min the
-// smallest lattice spacing of the aggregate's grains; hash grid anchored at
+// smallest lattice spacing of the aggregate's grains; contact grid anchored at
 // the aggregate's lower-left wall corner with cells of side R_c.
 void compute_aggregates(pd_ctx *c) {
     const pd_params &p = c->prm;
@@ -282,6 +282,31 @@ void compute_aggregates(pd_ctx *c) {
     c->Kn = c->aggp[0].Kn;
 }
 
+// Contact grid of every aggregate: cells over its wall box at t = 0 and one
+// around it, at least 3 each way and, by shrinking both ways alike, at most
+// four per node (two beyond 2^28 nodes, for 32-bit cell indices), 64 at least.
+void compute_grid(pd_ctx *c) {
+    std::vector<int64_t> nodes(c->n_agg, 0);
+    for (int g = 0; g < c->G; ++g) nodes[c->g_agg[g]] += c->g_start[g + 1] - c->g_start[g];
+    int64_t total = 0;
+    for (int a = 0; a < c->n_agg; ++a) {
+        pd::AggParams &A = c->aggp[a];
+        const double *w = &c->agg_walls[8 * (size_t)a];
+        double gw = std::ceil((w[1] - w[0]) / A.cell) + 2, gh = std::ceil((w[3] - w[2]) / A.cell) + 2;
+        const double most = std::max(64.0, (c->N > (int64_t(1) << 28) ? 2.0 : 4.0) * (double)nodes[a]);
+        if (gw * gh > most) {
+            const double f = std::sqrt(most / (gw * gh));
+            gw = std::max(3.0, std::min(std::floor(gw * f), std::floor(most / 3)));
+            gh = std::max(3.0, std::floor(most / gw));
+        }
+        A.gw = (int)std::max(gw, 3.0);
+        A.gh = (int)std::max(gh, 3.0);
+        A.gbase = (int)total;
+        total += (int64_t)A.gw * A.gh;
+    }
+    c->T = (unsigned)((total + 3) / 4 * 4);
+}
+
 }  // namespace
 
 namespace {
@@ -323,6 +348,12 @@ void carve(char *base, size_t &off, T *&ptr, size_t count) {
     off = align_up(off + sizeof(T) * std::max<size_t>(count, 1));
 }
 
+// Horizons whose neighbourhood is exactly the 24 offsets of the 5 x 5 block.
+bool has_stencil(const pd_ctx *c) {
+    const double hr2 = c->prm.horizon_ratio * c->prm.horizon_ratio;
+    return hr2 > 8.0 && hr2 <= 9.0;
+}
+
 size_t layout(pd_ctx *c, char *base) {
     size_t off = 0;
     pd::DevPtrs &d = c->d;
@@ -347,6 +378,7 @@ size_t layout(pd_ctx *c, char *base) {
     carve(base, off, d.col, nb);
     carve(base, off, d.xi, nb);
     carve(base, off, d.bits, N * (size_t)c->wpn);
+    carve(base, off, d.bref, N * (size_t)c->wpn);
     carve(base, off, d.g_cw, G);
     carve(base, off, d.g_s0, G);
     carve(base, off, d.g_eps, G);
@@ -360,7 +392,7 @@ size_t layout(pd_ctx *c, char *base) {
     carve(base, off, d.wall_cell, (size_t)c->n_agg);
     carve(base, off, d.count, c->T);
     carve(base, off, d.start, (size_t)c->T + 1);
-    carve(base, off, d.cursor, c->T);
+    carve(base, off, d.rank, N);
     carve(base, off, d.sorted, N);
     carve(base, off, d.srec, N);
     carve(base, off, d.nbr_cnt, N);
@@ -370,6 +402,8 @@ size_t layout(pd_ctx *c, char *base) {
     carve(base, off, d.pred_done, 1);
     carve(base, off, d.rebuild_next, 1);
     carve(base, off, d.pred_ok, 1);
+    carve(base, off, d.spec, N);
+    carve(base, off, d.spec_n, 2);
     carve(base, off, d.fsum, 6 * N * (c->prm.precision == PD_FP32_SPLIT ? 4 : 8));
     // block sums of the scan: one per scan tile (multi-kernel path) or per
     // block of the persistent kernel (at most 16 blocks per SM)
@@ -390,17 +424,18 @@ size_t layout(pd_ctx *c, char *base) {
         carve(base, off, d.pqb[1], N);
         carve(base, off, d.xs, N);
         carve(base, off, d.colx, nb);
-        carve(base, off, d.stn, N);
         carve(base, off, d.gc, G);
+        d.xif = nullptr;
     } else {
         d.lat = nullptr;
         d.gq = nullptr;
         d.pqb[0] = d.pqb[1] = nullptr;
         d.xs = nullptr;
         d.colx = nullptr;
-        d.stn = nullptr;
         d.gc = nullptr;
+        carve(base, off, d.xif, has_stencil(c) ? 12 * N : 0);
     }
+    carve(base, off, d.stn, has_stencil(c) ? N : 0);
     carve(base, off, d.g_invm, G);
     carve(base, off, d.g_invmf, G);
     carve(base, off, d.bu, N);
@@ -937,11 +972,8 @@ int pd_build_bonds(pd_ctx *c, int64_t *n_bonds_out) {
         c->g_slot[g] = c->tmpl_count[c->g_tmpl[g]]++;
     }
     c->n_tmpl = (int)c->tmpl_first.size();
-    // contact hash: power of two >= 2N buckets
     if (c->N > (int64_t(1) << 29)) return fail(PD_EINVAL, "too many nodes for the contact grid (at most 2^29)");
-    unsigned T = 1024;
-    while ((int64_t)T < 2 * c->N) T <<= 1;
-    c->T = T;
+    compute_grid(c);
     c->state = 2;
     if (n_bonds_out) *n_bonds_out = (int64_t)c->col.size();
     return PD_OK;
@@ -950,6 +982,7 @@ int pd_build_bonds(pd_ctx *c, int64_t *n_bonds_out) {
 int pd_arena_bytes(pd_ctx *c, size_t *bytes) {
     if (int r = check_ctx(c, 2)) return r;
     if (!bytes) return fail(PD_EINVAL, "null bytes");
+    compute_grid(c);
     c->kp.n_diag_blocks = (int)std::min<int64_t>(1024, (c->N + pd::kBlock - 1) / pd::kBlock);
     *bytes = layout(c, nullptr);
     return PD_OK;
@@ -959,6 +992,7 @@ int pd_bind_arena(pd_ctx *c, void *arena, size_t bytes) {
     if (int r = check_ctx(c, 2)) return r;
     if (c->state != 2) return fail(PD_ESTATE, "arena already bound");
     if (!arena || ((uintptr_t)arena & 255)) return fail(PD_EINVAL, "arena null or not 256-byte aligned");
+    compute_grid(c);
     c->kp.n_diag_blocks = (int)std::min<int64_t>(1024, (c->N + pd::kBlock - 1) / pd::kBlock);
     size_t need = layout(c, nullptr);
     if (bytes < need) return fail(PD_EINVAL, "arena too small");
@@ -1043,14 +1077,16 @@ int pd_bind_arena(pd_ctx *c, void *arena, size_t bytes) {
     PD_CUDA(cudaMemcpyAsync(d.agg, c->aggp.data(), sizeof(pd::AggParams) * c->aggp.size(), cudaMemcpyHostToDevice, s));
     PD_CUDA(cudaMemsetAsync(d.bar, 0, 2 * sizeof(unsigned), s));
     PD_CUDA(cudaMemsetAsync(d.t_now, 0, sizeof(double), s));
-    // bucket counts are zero between rebuilds; the first force evaluation rebuilds
+    // cell counts are zero between rebuilds; the first force evaluation rebuilds
     PD_CUDA(cudaMemsetAsync(d.count, 0, sizeof(int) * c->T, s));
     PD_CUDA(cudaMemsetAsync(d.nbr_cnt, 0, 4 * N, s));
+    PD_CUDA(cudaMemsetAsync(d.bref, 0, 4 * N * c->wpn, s));
     PD_CUDA(cudaMemsetAsync(d.sref, 0, 16 * N, s));
     PD_CUDA(cudaMemsetAsync(d.rebuild, 1, sizeof(int), s));
     PD_CUDA(cudaMemsetAsync(d.pred_done, 0, sizeof(unsigned), s));
     PD_CUDA(cudaMemsetAsync(d.rebuild_next, 0, sizeof(int), s));
     PD_CUDA(cudaMemsetAsync(d.pred_ok, 0, sizeof(int), s));
+    PD_CUDA(cudaMemsetAsync(d.spec_n, 0, 2 * sizeof(int), s));
     std::vector<int32_t> gstart32(c->g_start.begin(), c->g_start.end()), tnode, tslot;
     PD_CUDA(cudaMemcpyAsync(d.g_start, gstart32.data(), 4 * (G + 1), cudaMemcpyHostToDevice, s));
     std::vector<float> fc;
@@ -1115,7 +1151,8 @@ int pd_bind_arena(pd_ctx *c, void *arena, size_t bytes) {
     std::vector<double> invm;
     std::vector<uint32_t> colx;
     std::vector<uint4> stn;
-    std::vector<double> xs;
+    std::vector<double> xs, xif;
+    PD_CUDA(k.fp32 ? pd::init_tiles32() : pd::init_tiles64());
     if (p.precision == PD_FP32_SPLIT) {
         // per grain: h, h^2 as a float-float pair, V as float
         gq.resize(4 * G);
@@ -1142,43 +1179,6 @@ int pd_bind_arena(pd_ctx *c, void *arena, size_t bytes) {
                 colx[b] = (uint32_t)j | ((uint32_t)n << pd::kColBits);
             }
         if (nb) PD_CUDA(cudaMemcpyAsync(d.colx, colx.data(), 4 * nb, cudaMemcpyHostToDevice, s));
-        // lattice stencil of the bonds (horizons with exactly the 24 offsets of the 5 x 5 block)
-        const double hr2 = p.horizon_ratio * p.horizon_ratio;
-        c->kp.stencil = (hr2 > 8.0 && hr2 <= 9.0) ? 1 : 0;
-        if (c->kp.stencil) {
-            stn.assign(N, make_uint4(pd::kStnIrregular, 0u, 0u, 0u));
-            size_t irregular = 0;
-            for (size_t x = 0; x < N; ++x) {
-                uint32_t mask = 0;
-                int D[5] = {0, 0, 0, 0, 0};
-                bool seen[5] = {false, false, false, false, false}, ok = true;
-                int last = -1;
-                for (int b = c->row_ptr[x]; b < c->row_ptr[x + 1] && ok; ++b) {
-                    const int j = c->col[b];
-                    const int di = c->lat[2 * (size_t)j] - c->lat[2 * x], dj = c->lat[2 * (size_t)j + 1] - c->lat[2 * x + 1];
-                    if (di < -2 || di > 2 || dj < -2 || dj > 2) { ok = false; break; }
-                    const int oo = (dj + 2) * 5 + (di + 2), o = oo < 12 ? oo : oo - 1;
-                    const long long base = (long long)j - (long long)x - di;
-                    if (o <= last) ok = false;                      // CSR order must be the offset order
-                    last = o;
-                    if (!seen[dj + 2]) { seen[dj + 2] = true; D[dj + 2] = (int)std::max<long long>(-40000, std::min<long long>(40000, base)); }
-                    else if (D[dj + 2] != base) ok = false;
-                    if (dj == 0 && base != 0) ok = false;
-                    if (D[dj + 2] < -32768 || D[dj + 2] > 32767) ok = false;
-                    mask |= 1u << o;
-                }
-                if (!ok) {
-                    stn[x] = make_uint4(pd::kStnIrregular, 0u, 0u, (unsigned)c->row_ptr[x]);
-                    ++irregular;
-                    continue;
-                }
-                auto u16 = [](int v) { return (uint32_t)(uint16_t)(int16_t)v; };
-                stn[x] = make_uint4(mask, u16(D[0]) | (u16(D[1]) << 16), u16(D[3]) | (u16(D[4]) << 16),
-                                    (unsigned)c->row_ptr[x]);
-            }
-            c->stn_irregular = irregular;
-            PD_CUDA(cudaMemcpyAsync(d.stn, stn.data(), 16 * N, cudaMemcpyHostToDevice, s));
-        }
         // X + the aggregate's shift (FP64): the FP32-split positions are (X + shift) + u
         xs.resize(2 * N);
         for (size_t x = 0; x < N; ++x) {
@@ -1196,6 +1196,69 @@ int pd_bind_arena(pd_ctx *c, void *arena, size_t bytes) {
             gcf[4 * g + 3] = (float)c->g_rho[g];
         }
         PD_CUDA(cudaMemcpyAsync(d.gc, gcf.data(), 16 * G, cudaMemcpyHostToDevice, s));
+    }
+    // lattice stencil of the bonds (FP64 path: with the forward bonds' reference lengths)
+    c->kp.stencil = has_stencil(c) ? 1 : 0;
+    k.pair = 0;
+    if (c->kp.stencil) {
+        stn.assign(N, make_uint4(pd::kStnIrregular, 0u, 0u, 0u));
+        if (!k.fp32) xif.assign(12 * N, 1.0);
+        size_t irregular = 0;
+        int reach = 0;             // farthest bond along the node numbering
+        for (size_t x = 0; x < N; ++x) {
+            uint32_t mask = 0;
+            int D[5] = {0, 0, 0, 0, 0};
+            bool seen[5] = {false, false, false, false, false}, ok = true;
+            int last = -1;
+            for (int b = c->row_ptr[x]; b < c->row_ptr[x + 1] && ok; ++b) {
+                const int j = c->col[b];
+                const int di = c->lat[2 * (size_t)j] - c->lat[2 * x], dj = c->lat[2 * (size_t)j + 1] - c->lat[2 * x + 1];
+                if (di < -2 || di > 2 || dj < -2 || dj > 2) { ok = false; break; }
+                const int oo = (dj + 2) * 5 + (di + 2), o = oo < 12 ? oo : oo - 1;
+                const long long base = (long long)j - (long long)x - di;
+                if (o <= last) ok = false;                      // CSR order must be the offset order
+                last = o;
+                if (!seen[dj + 2]) { seen[dj + 2] = true; D[dj + 2] = (int)std::max<long long>(-40000, std::min<long long>(40000, base)); }
+                else if (D[dj + 2] != base) ok = false;
+                if (dj == 0 && base != 0) ok = false;
+                if (D[dj + 2] < -32768 || D[dj + 2] > 32767) ok = false;
+                mask |= 1u << o;
+                reach = std::max(reach, std::abs(j - (int)x));
+            }
+            if (!ok) {
+                stn[x] = make_uint4(pd::kStnIrregular, 0u, 0u, (unsigned)c->row_ptr[x]);
+                ++irregular;
+                continue;
+            }
+            auto u16 = [](int v) { return (uint32_t)(uint16_t)(int16_t)v; };
+            stn[x] = make_uint4(mask, u16(D[0]) | (u16(D[1]) << 16), u16(D[3]) | (u16(D[4]) << 16),
+                                (unsigned)c->row_ptr[x]);
+            if (!k.fp32) {
+                int b = c->row_ptr[x];
+                for (int o = 0; o < 24; ++o) {
+                    if (!((mask >> o) & 1u)) continue;
+                    if (o >= 12) xif[(size_t)(o - 12) * N + x] = c->xi[b];
+                    ++b;
+                }
+            }
+        }
+        c->stn_irregular = irregular;
+        k.pair = reach <= pd::kCarry ? 1 : 0;
+        // a node that forms a bond relies on the other node's list having it too
+        for (size_t x = 0; x < N && k.pair; ++x) {
+            const uint4 &a = stn[x];
+            if (a.x & pd::kStnIrregular) continue;
+            for (int o = 0; o < 24; ++o) {
+                if (!((a.x >> o) & 1u)) continue;
+                const int oo = o < 12 ? o : o + 1, dj = oo / 5 - 2, di = oo % 5 - 2;
+                const uint32_t w = dj < 0 ? a.y : a.z;
+                const int row = dj == 0 ? 0 : (int)(int16_t)(uint16_t)((dj == -2 || dj == 1) ? w & 0xFFFFu : w >> 16);
+                const uint32_t other = stn[x + di + row].x;
+                if (!(other & pd::kStnIrregular) && !((other >> (23 - o)) & 1u)) k.pair = 0;
+            }
+        }
+        PD_CUDA(cudaMemcpyAsync(d.stn, stn.data(), 16 * N, cudaMemcpyHostToDevice, s));
+        if (!k.fp32) PD_CUDA(cudaMemcpyAsync(d.xif, xif.data(), 8 * xif.size(), cudaMemcpyHostToDevice, s));
     }
     // per grain 1 / (rho V): the update multiplies by it (an FP64 division per
     // node and component costs about nine FP64 operations on GB300)
@@ -1469,7 +1532,7 @@ int pd_clear_status(pd_ctx *c) {
     PD_CUDA(cudaMemsetAsync(d.pred_done, 0, sizeof(unsigned), s));
     PD_CUDA(cudaMemsetAsync(d.pred_ok, 0, sizeof(int), s));
     PD_CUDA(cudaMemsetAsync(d.rebuild_next, 0, sizeof(int), s));
-    // a step that gave up inside a rebuild leaves bucket counts behind; they are
+    // a step that gave up inside a rebuild leaves cell counts behind; they are
     // zero between rebuilds, and the next step rebuilds the candidate lists
     PD_CUDA(cudaMemsetAsync(d.count, 0, sizeof(int) * c->T, s));
     PD_CUDA(cudaMemsetAsync(d.rebuild, 1, sizeof(int), s));

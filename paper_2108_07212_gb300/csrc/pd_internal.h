@@ -8,10 +8,11 @@
 namespace pd {
 
 // Contact candidate list (Verlet list with a skin): every node keeps the nodes
-// y of its aggregate with |p(y) - p(x)| < R_c + skin at the last rebuild, at
-// most kMaxList of them, in ascending index.  A rebuild runs when some node
+// y of its aggregate with |p(y) - p(x)| < R_c + skin at the last rebuild that it
+// had no intact bond with, at most kMaxList of them, in ascending index.  A rebuild runs when some node
 // has moved more than kSkinTrigger * skin since the last one, so every pair
-// closer than R_c is always in the list (the force phase tests R_c exactly).
+// closer than R_c is in the list, or its bond has broken since (the force phase
+// takes those from the broken bits, and tests R_c exactly).
 constexpr int kMaxList = 24;
 constexpr double kSkinRatio = 0.10;     // skin = kSkinRatio * R_c
 constexpr double kSkinTrigger = 0.45;   // < 1/2: margin for the float displacement test
@@ -25,7 +26,7 @@ constexpr size_t kPrefetchMaxBytes = 24u << 20;
 // lattice offset di^2 + dj^2 (< 16 for horizons up to 4 h) in the top bits.
 constexpr int kColBits = 28;
 constexpr uint32_t kColMask = (1u << kColBits) - 1u;
-// FP32-split bond stencil (horizon 3 h: the 24 offsets (di, dj) of the 5 x 5
+// Bond stencil (horizon 3 h: the 24 offsets (di, dj) of the 5 x 5
 // lattice block without its centre, numbered o = 0..23 in (dj, di) order).
 // Nodes of a grain are numbered row by row (j, then i), so for a node whose
 // neighbour rows are contiguous runs near it the neighbour at offset o is node
@@ -35,6 +36,10 @@ constexpr uint32_t kColMask = (1u << kColBits) - 1u;
 //   y: D[-2] | D[-1] << 16, z: D[1] | D[2] << 16 (16-bit two's complement)
 //   w: first bond of the node's CSR row
 constexpr uint32_t kStnIrregular = 0x80000000u;
+// Nodes before a run of nodes whose bond forces it can use (see PairTile): two
+// lattice rows of a grain of up to 32 lattice spacings a radius (the finest
+// workloads have 23).
+constexpr int kCarry = 128;
 // Threads per block of the node-parallel multi-kernel path.
 constexpr int kBlock = 128;
 // Scan tile: threads x items per thread.
@@ -51,7 +56,7 @@ struct AggParams {
     double Rc, Kn;
     double pe5;            // pi eps_c^5: K_n = 18 k / pe5 for a pair's bulk modulus k (materials)
     double w0[4], wv[4];   // walls x_lo, x_hi, y_lo, y_hi at t = 0 and their normal velocities
-    double ox, oy, cell;   // hash-grid origin and cell side (>= R_c)
+    double ox, oy, cell;   // contact grid origin and cell side (>= R_c + skin)
     double inv_cell;       // 1 / cell
     double sx, sy;         // FP32-split shift: coordinates of the box map to [L, 2L)
     float rc2_hi, rc2_lo;  // R_c^2 as a float-float pair
@@ -59,6 +64,7 @@ struct AggParams {
     float oxs, oys, inv_cell_f;  // FP32 split: grid origin in shifted coordinates, 1 / cell
     float rs2;             // (R_c + skin)^2 as a float: radius of the candidate lists
     float dmax2;           // (kSkinTrigger skin)^2: displacement since the last rebuild that triggers the next
+    int gw, gh, gbase;     // contact grid: cells in x and y (at least 3), index of its first cell
 };
 
 // Device pointers carved out of the caller's arena.
@@ -77,7 +83,9 @@ struct DevPtrs {
     // bonds: CSR, reference lengths |xi|, broken bits (wpn words per node)
     int *row_ptr, *col;
     double *xi;
+    double *xif;        // FP64 path with the stencil: |xi| of the forward bonds, offset 12 + q of node i at xif[q N + i]
     uint32_t *bits;
+    uint32_t *bref;     // the broken bits at the last rebuild of the candidate lists
     // per-grain constants and aggregate of each grain
     double *g_cw, *g_s0, *g_eps;
     int *g_agg;
@@ -86,9 +94,9 @@ struct DevPtrs {
     // contact stiffness 18 k / (pi eps_c^5) as a float (FP32-split contact laws)
     double *g_rho, *g_k;
     float *g_kf;
-    // contact hash grid (T buckets)
-    int *key, *count, *start, *cursor, *sorted, *blocksums;
-    int2 *cell;         // hash-grid cell (x, y) of every node at the last rebuild
+    // contact grid (T cells)
+    int *key, *rank, *count, *start, *sorted, *blocksums;   // a node's cell and its rank in it; counting sort
+    int2 *cell;         // grid cell (x, y) of every node at the last rebuild
     // contact candidate lists (rebuilt when a node has moved kSkinTrigger * skin)
     int *nbr_cnt;       // list length of every node
     int *nbr;           // list entry q of node i at nbr[q N + i] (kMaxList slots), ascending node index
@@ -97,8 +105,11 @@ struct DevPtrs {
     unsigned *pred_done;  // blocks of the displacement update that have finished (last-block election)
     int *rebuild_next;  // FP32-split persistent kernel: the next step's rebuild flag, raised in the velocity update
     int *pred_ok;       // nonzero: ub / pqb of the other parity hold the next step's u and pq (persistent kernel)
-    uint4 *srec;        // position of sorted[t] in bucket order: FP32 split pq, FP64 p (16 bytes)
+    uint4 *srec;        // position of sorted[t] in cell order: FP32 split pq, FP64 p (16 bytes)
     void *fsum;         // split force phase: per-node lane sums, six components of N floats (FP32) or doubles
+                        // (persistent kernel, one thread per node: special nodes' bond sums, N pairs)
+    int *spec;          // special nodes of the step (see list_special)
+    int *spec_n;        // their number, by step parity
     // globals
     long long *step;
     double *t_now;      // time of the force evaluation that follows the predict phase
@@ -115,11 +126,11 @@ struct DevPtrs {
     float4 *pqb[2];     // its two buffers (see ub)
     double2 *xs;        // X + the aggregate's shift (FP64)
     uint32_t *colx;     // bond columns with the lattice offset n = di^2 + dj^2 in the top 4 bits
-    uint4 *stn;         // lattice stencil of every node's bonds (see kStnIrregular), when KParams::stencil
+    uint4 *stn;         // lattice stencil of every node's bonds (see kStnIrregular), when KParams::stencil (both paths)
     float4 *gc;         // per grain: (c_w, s0, eps, rho) as floats
     double *g_invm;     // per grain: 1 / (rho V)
     float *g_invmf;     // the same as floats (FP32-split contexts)
-    int4 *wall_cell;    // per aggregate: hash-grid cells of its walls x_lo, x_hi, y_lo, y_hi at the current time
+    int4 *wall_cell;    // per aggregate: grid cells of its walls x_lo, x_hi, y_lo, y_hi at the current time
     // autotuner backup of the state
     double2 *bu, *bv, *ba;
     float2 *af;         // FP32-split contexts: the acceleration, a = F / m + g rounded to float (d.a unused)
@@ -160,7 +171,7 @@ struct DevPtrs {
 // By-value kernel parameters (baked into captured graphs).
 struct KParams {
     int N, G, wpn, n_diag_blocks, n_agg;
-    unsigned T;         // hash buckets (power of two)
+    unsigned T;         // contact grid cells of all aggregates, rounded up to a multiple of 4
     double rho, rd, mu, gx, gy, dt, half_dt, half_dt2;
     float rhof, rdf, muf, dtf;   // the same as floats (FP32-split contact laws)
     float gxf, gyf;              // gravity as floats (FP32-split acceleration)
@@ -172,7 +183,8 @@ struct KParams {
     int split;          // 1: lane sums through global memory and a separate epilogue pass
     int fp32;           // precision of the force phase
     int pf_bonds;       // > 0: prefetch the force phase's read-only arrays (this many bonds) into L2
-    int stencil;        // FP32 split: bonds from the lattice stencil (DevPtrs::stn) instead of the columns
+    int stencil;        // bonds from the lattice stencil (DevPtrs::stn) instead of the columns
+    int pair;           // one thread per node: each stencil bond evaluated once (no row reaches past kCarry nodes)
     // surrogate
     int sur;            // surrogate on
     int n_modes;        // modes of the basis (32)
@@ -278,5 +290,8 @@ cudaError_t launch_observables(const DevPtrs &d, const KParams &k, int vcur, dou
 cudaError_t launch_persistent(const DevPtrs &d, const KParams &k, int vin, int nsteps, int block, cudaStream_t s);
 cudaError_t launch_persistent64(const DevPtrs &d, const KParams &k, int vin, int nsteps, int block, cudaStream_t s);
 cudaError_t launch_persistent32(const DevPtrs &d, const KParams &k, int vin, int nsteps, int block, cudaStream_t s);
+// Shared-memory limits of the kernels with bond tiles (not capturable).
+cudaError_t init_tiles64();
+cudaError_t init_tiles32();
 
 }  // namespace pd

@@ -22,4 +22,16 @@ cudaError_t launch_persistent_lanes(const DevPtrs &d, const KParams &k, int vin,
 template cudaError_t launch_persistent_lanes<PD_PERSIST_FP32 != 0, PD_PERSIST_LANES>(const DevPtrs &, const KParams &,
                                                                                      int, int, int, cudaStream_t);
 
+#if PD_PERSIST_LANES == 1
+template <>
+cudaError_t init_persistent_tiles<PD_PERSIST_FP32 != 0>() {
+    constexpr bool kFp32 = PD_PERSIST_FP32 != 0;
+    const cudaError_t e = cudaFuncSetAttribute(k_persistent<kFp32, 1, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               run_smem<kFp32, 128>());
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_persistent<kFp32, 1, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                run_smem<kFp32, 256>());
+}
+#endif
+
 }  // namespace pd

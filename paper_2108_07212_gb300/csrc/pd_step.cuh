@@ -15,18 +15,22 @@ namespace pd {
 // integrates (FP64, converged warps).  Every thread of the block must call it.
 template <bool FP32, bool PERSIST, int LANES, int BLOCK>
 __device__ __forceinline__ void force_block(const DevPtrs &d, const KParams &k, int node0, int vin, int update_v) {
+    static_assert(LANES > 1, "one thread per node: tile_nodes");
     constexpr int NB = BLOCK / LANES;
     using Sums = typename std::conditional<FP32, Sums32, Sums64>::type;
     __shared__ Sums sm[NB];
     const int local = threadIdx.x / LANES, lane = threadIdx.x % LANES;
     const int i = node0 + local;
     Sums f;
+    [[maybe_unused]] bool contact;
     if constexpr (FP32) force_node32<PERSIST, LANES>(d, k, i, lane, i < k.N, vin, f);
-    else force_node64<PERSIST, LANES>(d, k, i, lane, i < k.N, vin, f);
+    else force_node64<PERSIST, LANES, 0>(d, k, i, lane, i < k.N, vin, f, nullptr, false, contact);
     if (lane == 0) sm[local] = f;
     __syncthreads();
     if ((int)threadIdx.x < NB && node0 + (int)threadIdx.x < k.N) {
-        if constexpr (FP32) node_epilogue32<PERSIST>(d, k, node0 + threadIdx.x, vin, update_v, sm[threadIdx.x]);
+        if constexpr (FP32)
+            node_epilogue32<PERSIST>(d, k, node0 + threadIdx.x, __ldg(&d.grain[node0 + threadIdx.x]), vin, update_v,
+                                     sm[threadIdx.x], load_update32<PERSIST>(d, node0 + threadIdx.x, vin, update_v));
         else node_epilogue64<PERSIST>(d, k, node0 + threadIdx.x, vin, update_v, sm[threadIdx.x]);
     }
     __syncthreads();
@@ -38,46 +42,173 @@ __device__ __forceinline__ void clear_rebuild(const DevPtrs &d) {
     if (blockIdx.x == 0 && threadIdx.x == 0) *d.rebuild = 0;
 }
 
-// Multi-kernel path: one block per BLOCK / LANES nodes.
+// The lane sums of node i into global memory (split force phase; structure of
+// arrays): six components with per-part output, else only their total (F_b +
+// F_s) + F_n, as the epilogue would form it.
+template <bool FP32, class Sums>
+__device__ __forceinline__ void store_sums(const DevPtrs &d, const KParams &k, int i, const Sums &f) {
+    const size_t N = (size_t)k.N;
+    using T = typename std::conditional<FP32, float, double>::type;
+    T *o = static_cast<T *>(d.fsum);
+    if (k.store) {
+        o[i] = f.bx, o[N + i] = f.by, o[2 * N + i] = f.sx, o[3 * N + i] = f.sy, o[4 * N + i] = f.nx, o[5 * N + i] = f.ny;
+    } else if constexpr (FP32) {
+        reinterpret_cast<float2 *>(o)[i] = make_float2((f.bx + f.sx) + f.nx, (f.by + f.sy) + f.ny);
+    } else {
+        reinterpret_cast<double2 *>(o)[i] =
+            make_double2(__dadd_rn(__dadd_rn(f.bx, f.sx), f.nx), __dadd_rn(__dadd_rn(f.by, f.sy), f.ny));
+    }
+}
+
+extern __shared__ __align__(16) unsigned char tile_smem[];
+
+// One thread per node, FP64 path: the nodes [lo, hi) in bond tiles of BLOCK
+// nodes (see PairTile).  All threads call out(i, sums, active, contact) as
+// tile_nodes32 does.  Every thread of the block calls it with the same range.
+template <bool PERSIST, int BLOCK, bool INLINE, class Out>
+__device__ __forceinline__ void tile_nodes64(const DevPtrs &d, const KParams &k, int lo, int hi, int vin, Out out) {
+    float4 *slot = reinterpret_cast<float4 *>(tile_smem);
+    // the pass before the run takes the nodes [lo - BLOCK, lo), of which the last kCarry have slots
+    for (int node0 = lo > 0 && lo < hi && k.pair ? lo - BLOCK : lo; node0 < hi; node0 += BLOCK) {
+        const int i = node0 + (int)threadIdx.x;
+        const bool warm = node0 < lo;
+        const bool active = warm ? i >= max(0, lo - kCarry) : i < hi;
+        Sums64 f;
+        bool contact;
+        force_node64<PERSIST, 1, BLOCK, INLINE>(d, k, i, 0, active, vin, f, slot, warm, contact);
+        if (!warm) out(i, f, active, contact);
+        __syncthreads();                   // the tile's slots have been read (or formed)
+        if (k.pair) PairTile<float4, BLOCK>::carry(slot);
+        __syncthreads();
+    }
+}
+
+// Nodes per block when N nodes are dealt to n of them: a multiple of the warp.
+__host__ __device__ __forceinline__ int run_length(int N, int n) {
+    return (int)((((long long)N + n - 1) / n + 31) / 32 * 32);
+}
+
+// The forces of the nodes [lo, hi), one thread per node, by the calling block:
+// sums stored (split force phase), or each node's walls and update behind them.
+// Grains with rows too long for the carried slots (k.pair clear) take the
+// general bond loop.
+template <bool FP32, bool PERSIST, int BLOCK>
+__device__ __forceinline__ void run_nodes(const DevPtrs &d, const KParams &k, int lo, int hi, int vin, int update_v,
+                                          bool fused) {
+    if constexpr (FP32) {
+        auto out = [&](int i, const Sums32 &f, int, bool active, bool) {
+            if (!active) return;
+            if (fused) node_epilogue32<PERSIST>(d, k, i, __ldg(&d.grain[i]), vin, update_v, f,
+                                                load_update32<PERSIST>(d, i, vin, update_v));
+            else store_sums<true>(d, k, i, f);
+        };
+        if (k.pair) {
+            tile_nodes32<PERSIST, BLOCK, true>(d, k, lo, hi, vin, false, *reinterpret_cast<Tile32<BLOCK> *>(tile_smem), out);
+            return;
+        }
+        for (int g = lo; g < hi; g += BLOCK) {
+            const int i = g + (int)threadIdx.x;
+            Sums32 f;
+            force_node32<PERSIST, 1>(d, k, i, 0, i < hi, vin, f);
+            out(i, f, 0, i < hi, false);
+        }
+    } else {
+        tile_nodes64<PERSIST, BLOCK, true>(d, k, lo, hi, vin, [&](int i, const Sums64 &f, bool active, bool) {
+            if (!active) return;
+            if (fused) node_epilogue64<PERSIST>(d, k, i, vin, update_v, f);
+            else store_sums<false>(d, k, i, f);
+        });
+    }
+}
+
+// The same for the persistent kernel's fused force phase: plain nodes are
+// updated at once, special ones (see list_special) put on list `which`.
+template <bool FP32, int BLOCK>
+__device__ __forceinline__ void run_plain_nodes(const DevPtrs &d, const KParams &k, int lo, int hi, int vin, int which) {
+    if constexpr (FP32) {
+        Tile32<BLOCK> &sm = *reinterpret_cast<Tile32<BLOCK> *>(tile_smem);
+        tile_nodes32<true, BLOCK, false>(d, k, lo, hi, vin, true, sm,
+                                         [&](int i, const Sums32 &f, int at, bool active, bool contact) {
+            bool special = false;
+            if (active) {
+                const Update32 n{sm.v[at], sm.u[at], sm.xs[at], sm.sref[at], sm.a[at], sm.cell[at]};
+                const int gi = __ldg(&d.grain[i]);
+                special = contact || k.store || !cells_far_from_walls(n.cell, ldm<true>(&d.wall_cell[__ldg(&d.g_agg[gi])]));
+                if (special) reinterpret_cast<float2 *>(d.fsum)[i] = make_float2(f.bx, f.by);
+                else finish_node32_total<true>(d, k, i, vin, 1, n, f.bx, f.by, false, 0.0, 0.0, __ldg(&d.g_invmf[gi]));
+            }
+            list_special(d, which, i, special);
+        });
+    } else {
+        tile_nodes64<true, BLOCK, false>(d, k, lo, hi, vin, [&](int i, const Sums64 &f, bool active, bool contact) {
+            bool special = false;
+            if (active) {
+                const int gi = __ldg(&d.grain[i]);
+                const double2 v = ldm<true>(&d.v[vin][i]), a = ldm<true>(&d.a[i]);
+                special = contact || k.store ||
+                          !cells_far_from_walls(ldm<true>(&d.cell[i]), ldm<true>(&d.wall_cell[__ldg(&d.g_agg[gi])]));
+                if (special) reinterpret_cast<double2 *>(d.fsum)[i] = make_double2(f.bx, f.by);
+                else finish_node64_total<true>(d, k, i, vin, 1, v, a, f.bx, f.by, false, 0.0, 0.0, __ldg(&d.g_invm[gi]));
+            }
+            list_special(d, which, i, special);
+        });
+    }
+}
+
+// The special nodes of list `which`, dealt to the warps of all blocks in turn
+// (one each before any takes a second into its other groups of threads).
+template <bool FP32, int BLOCK>
+__device__ __forceinline__ void run_special_nodes(const DevPtrs &d, const KParams &k, int vin, int which) {
+    const int n = __ldcg(&d.spec_n[which]);
+    constexpr int kGroups = 32 / kSpecialLanes;
+    const int warps = gridDim.x * (BLOCK / 32), warp = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    const int group = (threadIdx.x & 31) / kSpecialLanes;
+    for (int g = 0; g + warp < n; g += warps * kGroups) {
+        const int q = g + group * warps + warp;
+        const bool node = q < n;
+        const int i = node ? __ldcg(&d.spec[q]) : 0;
+        if constexpr (FP32) special_node32<true>(d, k, i, node, vin);
+        else special_node64<true>(d, k, i, node, vin);
+    }
+}
+template <bool FP32, int BLOCK>
+constexpr int run_smem() {
+    return FP32 ? (int)sizeof(Tile32<BLOCK>) : PairTile<float4, BLOCK>::kBytes;
+}
+// Blocks of BLOCK threads per SM of the kernels with tiles: 512 threads of up to
+// 128 registers.  (FP32 split: three blocks of 256 at 80 registers spilled in
+// the tile loop, 211 us against 183 us on 2.28M nodes.)
+constexpr int run_blocks(int block) { return 512 / block; }
+
+// Multi-kernel path, one thread per node: four tiles of nodes a block (long
+// enough that the pass before a run costs little, short enough that blocks with
+// many contacts do not set the kernel's time).
+constexpr int kRunBlock = 256, kRunNodes = 4 * kRunBlock;
+template <bool FP32>
+__global__ void __launch_bounds__(kRunBlock, run_blocks(kRunBlock))
+    k_force_run(DevPtrs d, KParams k, int vin, int update_v, int fused) {
+    clear_rebuild(d);
+    const int lo = blockIdx.x * kRunNodes;
+    run_nodes<FP32, false, kRunBlock>(d, k, lo, min(lo + kRunNodes, k.N), vin, update_v, fused != 0);
+}
+
+// Multi-kernel path, several threads per node: one block per BLOCK / LANES nodes.
 template <bool FP32, int LANES>
-__global__ void __launch_bounds__(kBlock, FP32 ? (LANES == 1 ? 8 : 5) : 4) k_force(DevPtrs d, KParams k, int vin, int update_v) {
+__global__ void __launch_bounds__(kBlock, FP32 ? 5 : 4) k_force(DevPtrs d, KParams k, int vin, int update_v) {
     clear_rebuild(d);
     force_block<FP32, false, LANES, kBlock>(d, k, blockIdx.x * (kBlock / LANES), vin, update_v);
 }
 
-// Split variant: the lane sums of node i go to global memory (structure of
-// arrays, six components) and a second pass adds walls and integrates.
+// Split variant: the lane sums of node i go to global memory and a second pass
+// adds walls and integrates.
 template <bool FP32, bool PERSIST, int LANES>
 __device__ __forceinline__ void sums_node(const DevPtrs &d, const KParams &k, int i, int lane, int vin) {
     const bool active = i < k.N;
-    const size_t N = (size_t)k.N;
-    if constexpr (FP32) {
-        Sums32 f;
-        force_node32<PERSIST, LANES>(d, k, i, lane, active, vin, f);
-        if (active && lane == 0) {
-            float *o = static_cast<float *>(d.fsum);
-            if (k.store) {
-                o[i] = f.bx, o[N + i] = f.by, o[2 * N + i] = f.sx, o[3 * N + i] = f.sy, o[4 * N + i] = f.nx,
-                o[5 * N + i] = f.ny;
-            } else {
-                // only the total is needed: (F_b + F_s) + F_n, as the epilogue would form it
-                reinterpret_cast<float2 *>(o)[i] = make_float2((f.bx + f.sx) + f.nx, (f.by + f.sy) + f.ny);
-            }
-        }
-    } else {
-        Sums64 f;
-        force_node64<PERSIST, LANES>(d, k, i, lane, active, vin, f);
-        if (active && lane == 0) {
-            double *o = static_cast<double *>(d.fsum);
-            if (k.store) {
-                o[i] = f.bx, o[N + i] = f.by, o[2 * N + i] = f.sx, o[3 * N + i] = f.sy, o[4 * N + i] = f.nx,
-                o[5 * N + i] = f.ny;
-            } else {
-                reinterpret_cast<double2 *>(o)[i] =
-                    make_double2(__dadd_rn(__dadd_rn(f.bx, f.sx), f.nx), __dadd_rn(__dadd_rn(f.by, f.sy), f.ny));
-            }
-        }
-    }
+    typename std::conditional<FP32, Sums32, Sums64>::type f;
+    [[maybe_unused]] bool contact;
+    if constexpr (FP32) force_node32<PERSIST, LANES>(d, k, i, lane, active, vin, f);
+    else force_node64<PERSIST, LANES, 0>(d, k, i, lane, active, vin, f, nullptr, false, contact);
+    if (active && lane == 0) store_sums<FP32>(d, k, i, f);
 }
 
 template <bool FP32, bool PERSIST>
@@ -86,13 +217,15 @@ __device__ __forceinline__ void epilogue_node(const DevPtrs &d, const KParams &k
     // per-part sums (k.store) or the total of the parts
     if constexpr (FP32) {
         const float *o = static_cast<const float *>(d.fsum);
+        const Update32 n = load_update32<PERSIST>(d, i, vin, update_v);
         if (k.store) {
             const Sums32 f{ldm<PERSIST>(o + i), ldm<PERSIST>(o + N + i), ldm<PERSIST>(o + 2 * N + i),
                            ldm<PERSIST>(o + 3 * N + i), ldm<PERSIST>(o + 4 * N + i), ldm<PERSIST>(o + 5 * N + i)};
-            node_epilogue32<PERSIST>(d, k, i, vin, update_v, f);
+            node_epilogue32<PERSIST>(d, k, i, __ldg(&d.grain[i]), vin, update_v, f, n);
         } else {
             const float2 t = ldm<PERSIST>(reinterpret_cast<const float2 *>(o) + i);
-            node_epilogue32<PERSIST>(d, k, i, vin, update_v, Sums32{t.x, t.y, 0.f, 0.f, 0.f, 0.f}, true);
+            node_epilogue32<PERSIST>(d, k, i, __ldg(&d.grain[i]), vin, update_v,
+                                     Sums32{t.x, t.y, 0.f, 0.f, 0.f, 0.f}, n, true);
         }
     } else {
         const double *o = static_cast<const double *>(d.fsum);
@@ -120,6 +253,18 @@ __global__ void __launch_bounds__(256, 6) k_epilogue(DevPtrs d, KParams k, int v
     if (i < k.N) epilogue_node<FP32, false>(d, k, i, vin, update_v);
 }
 
+template <bool FP32>
+cudaError_t launch_force_run(const DevPtrs &d, const KParams &k, int vin, int update_v, cudaStream_t s, int fused) {
+    k_force_run<FP32><<<(k.N + kRunNodes - 1) / kRunNodes, kRunBlock, run_smem<FP32, kRunBlock>(), s>>>(d, k, vin,
+                                                                                                     update_v, fused);
+    return cudaGetLastError();
+}
+template <bool FP32>
+cudaError_t init_force_run() {
+    return cudaFuncSetAttribute(k_force_run<FP32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                run_smem<FP32, kRunBlock>());
+}
+
 // phase (split force phase only): 0 both passes, 1 the lane sums, 2 the epilogue.
 template <bool FP32>
 cudaError_t launch_force_impl(const DevPtrs &d, const KParams &k, int vin, int update_v, cudaStream_t s, int phase) {
@@ -130,7 +275,7 @@ cudaError_t launch_force_impl(const DevPtrs &d, const KParams &k, int vin, int u
             if (k.lanes == 8) k_sums<FP32, 8><<<grid, kBlock, 0, s>>>(d, k, vin);
             else if (k.lanes == 4) k_sums<FP32, 4><<<grid, kBlock, 0, s>>>(d, k, vin);
             else if (k.lanes == 2) k_sums<FP32, 2><<<grid, kBlock, 0, s>>>(d, k, vin);
-            else k_sums<FP32, 1><<<grid, kBlock, 0, s>>>(d, k, vin);
+            else if (const cudaError_t e = launch_force_run<FP32>(d, k, vin, 0, s, 0)) return e;
         }
         if (phase != 1) k_epilogue<FP32><<<(unsigned)((k.N + 255) / 256), 256, 0, s>>>(d, k, vin, update_v);
         return cudaGetLastError();
@@ -139,7 +284,7 @@ cudaError_t launch_force_impl(const DevPtrs &d, const KParams &k, int vin, int u
     if (k.lanes == 8) k_force<FP32, 8><<<grid, kBlock, 0, s>>>(d, k, vin, update_v);
     else if (k.lanes == 4) k_force<FP32, 4><<<grid, kBlock, 0, s>>>(d, k, vin, update_v);
     else if (k.lanes == 2) k_force<FP32, 2><<<grid, kBlock, 0, s>>>(d, k, vin, update_v);
-    else k_force<FP32, 1><<<grid, kBlock, 0, s>>>(d, k, vin, update_v);
+    else return launch_force_run<FP32>(d, k, vin, update_v, s, 1);
     return cudaGetLastError();
 }
 
@@ -235,14 +380,14 @@ __device__ __forceinline__ int block_scan1(int &v, int *sm) {
 //      (FP32 split: taken by the previous step's velocity update instead,
 //      except in the first step of a launch that finds no valid prediction)
 //   when some node moved kSkinTrigger * skin since the last rebuild:
-//     R1 bucket counts
-//     R2 per-block sums of the bucket counts
+//     R1 cell counts
+//     R2 per-block sums of the cell counts
 //     R3 exclusive scan of the counts -> cell starts (counts cleared)
 //     R4 counting-sort scatter of the node indices
 //     R5 candidate lists
 //   E  forces, acceleration and velocity update
 // s_cur_u / s_cur_pq hold this step's current displacement and positions
-// (parity vin ^ 1).  Bucket counts are zero on entry and on exit.  False when a
+// (parity vin ^ 1).  Cell counts are zero on entry and on exit.  False when a
 // grid barrier gave up (the kernel then returns).
 template <bool FP32, int LANES, int BLOCK>
 __device__ __forceinline__ bool persistent_step(const DevPtrs &d, const KParams &k, int vin, int st, int nsteps,
@@ -250,7 +395,7 @@ __device__ __forceinline__ bool persistent_step(const DevPtrs &d, const KParams 
     const int nthreads = gridDim.x * BLOCK;
     const int gtid = blockIdx.x * BLOCK + threadIdx.x;
     const unsigned T = k.T;
-    const unsigned slice = (T + gridDim.x - 1) / gridDim.x;
+    const unsigned slice = (T / 4 + gridDim.x - 1) / gridDim.x * 4;
     const unsigned lo = min(T, blockIdx.x * slice), hi = min(T, lo + slice);
     // A (the step counter's load is issued first, so that its latency
     // overlaps the displacement update of block 0's nodes)
@@ -266,6 +411,7 @@ __device__ __forceinline__ bool persistent_step(const DevPtrs &d, const KParams 
             *d.step = s;
             *d.t_now = (double)s * k.dt;
             s_step = s;
+            if (st == 0) d.spec_n[0] = d.spec_n[1] = 0;
             if constexpr (FP32) {
                 // the previous velocity update's rebuild test becomes this step's
                 // flag (no block reads the flag before the barrier below)
@@ -279,11 +425,14 @@ __device__ __forceinline__ bool persistent_step(const DevPtrs &d, const KParams 
     if (!grid_barrier(d, k.bar_spins)) return false;
     if (__ldcg(d.rebuild)) {
         // R1
-        for (int i = gtid; i < k.N; i += nthreads) bin_node<true>(d, k, i);
+        for (int i = gtid; i < k.N; i += kBinBatch * nthreads) bin_nodes<true>(d, k, i, nthreads);
         if (!grid_barrier(d, k.bar_spins)) return false;
-        // R2
+        // R2 (four cells a thread; T is a multiple of 4)
         int part = 0;
-        for (unsigned b = lo + threadIdx.x; b < hi; b += BLOCK) part += __ldcg(&d.count[b]);
+        for (unsigned b = lo + 4 * threadIdx.x; b < hi; b += 4 * BLOCK) {
+            const int4 c = __ldcg(reinterpret_cast<const int4 *>(&d.count[b]));
+            part += (c.x + c.y) + (c.z + c.w);
+        }
         part = block_sum<BLOCK>(part, sm);
         if (threadIdx.x == 0) d.blocksums[blockIdx.x] = part;
         if (!grid_barrier(d, k.bar_spins)) return false;
@@ -291,21 +440,23 @@ __device__ __forceinline__ bool persistent_step(const DevPtrs &d, const KParams 
         int off = 0;
         for (int b = threadIdx.x; b < (int)blockIdx.x; b += BLOCK) off += __ldcg(&d.blocksums[b]);
         off = block_sum<BLOCK>(off, sm);
-        for (unsigned b0 = lo; b0 < hi; b0 += BLOCK) {
-            const unsigned b = b0 + threadIdx.x;
-            int c = (b < hi) ? __ldcg(&d.count[b]) : 0;
-            if (b < hi) d.count[b] = 0;
-            const int tot = block_scan1<BLOCK>(c, sm);
+        for (unsigned b0 = lo; b0 < hi; b0 += 4 * BLOCK) {
+            const unsigned b = b0 + 4 * threadIdx.x;
+            int4 c = make_int4(0, 0, 0, 0);
             if (b < hi) {
-                d.start[b] = off + c;
-                d.cursor[b] = off + c;
+                c = __ldcg(reinterpret_cast<const int4 *>(&d.count[b]));
+                *reinterpret_cast<int4 *>(&d.count[b]) = make_int4(0, 0, 0, 0);
             }
+            int at = (c.x + c.y) + (c.z + c.w);
+            const int tot = block_scan1<BLOCK>(at, sm);
+            at += off;
+            if (b < hi) *reinterpret_cast<int4 *>(&d.start[b]) = make_int4(at, at + c.x, at + c.x + c.y, at + c.x + c.y + c.z);
             off += tot;
         }
         if (gtid == 0) d.start[T] = k.N;
         if (!grid_barrier(d, k.bar_spins)) return false;
         // R4
-        for (int i = gtid; i < k.N; i += nthreads) scatter_node<true>(d, k, i);
+        for (int i = gtid; i < k.N; i += kBinBatch * nthreads) scatter_nodes<true>(d, k, i, nthreads);
         if (!grid_barrier(d, k.bar_spins)) return false;
         // R5 (every block has read the flag: clear it for the next step)
         if (gtid == 0) {
@@ -316,7 +467,22 @@ __device__ __forceinline__ bool persistent_step(const DevPtrs &d, const KParams 
         if (!grid_barrier(d, k.bar_spins)) return false;
     }
     // E
-    if (k.split) {
+    if constexpr (LANES == 1) {
+        const int len = run_length(k.N, gridDim.x);
+        const int lo0 = (int)min((long long)k.N, (long long)blockIdx.x * len), hi0 = min(lo0 + len, k.N);
+        if (k.split || !k.pair) {
+            run_nodes<FP32, true, BLOCK>(d, k, lo0, hi0, vin, 1, !k.split);
+            if (k.split) {
+                if (!grid_barrier(d, k.bar_spins)) return false;
+                for (int i = gtid; i < k.N; i += nthreads) epilogue_node<FP32, true>(d, k, i, vin, 1);
+            }
+        } else {
+            run_plain_nodes<FP32, BLOCK>(d, k, lo0, hi0, vin, st & 1);
+            if (!grid_barrier(d, k.bar_spins)) return false;
+            if (gtid == 0) d.spec_n[(st + 1) & 1] = 0;
+            run_special_nodes<FP32, BLOCK>(d, k, vin, st & 1);
+        }
+    } else if (k.split) {
         const long long total = (((long long)LANES * k.N + 31) / 32) * 32;
         for (long long t = gtid; t < total; t += nthreads) sums_node<FP32, true, LANES>(d, k, (int)(t / LANES), (int)(t % LANES), vin);
         if (!grid_barrier(d, k.bar_spins)) return false;
@@ -333,13 +499,9 @@ __device__ __forceinline__ bool persistent_step(const DevPtrs &d, const KParams 
 // grid barriers.  Every step reads its current displacement and positions
 // through s_cur_u / s_cur_pq, the buffers of its parity (the FP32 split keeps
 // two of each; the FP64 path one).
-// (FP32 split, one thread per node: capped at 64 registers, eight blocks of 128
-// per SM, as the lane-sum kernel of the graph path; the phases that need more
-// spill a few hundred bytes, which costs less than the halved occupancy.  Two
-// or more threads per node, and the FP64 path: capped at 128 registers, four
-// blocks of 128.)
+// (Capped at 128 registers, four blocks of 128 threads per SM.)
 template <bool FP32, int LANES, int BLOCK>
-__global__ void __launch_bounds__(BLOCK, (FP32 && LANES == 1 ? 1024 : 512) / BLOCK)
+__global__ void __launch_bounds__(BLOCK, run_blocks(BLOCK))
     k_persistent(DevPtrs d, KParams k, int vin, int nsteps) {
     __shared__ int sm[33];
     __shared__ long long s_step;
@@ -369,13 +531,15 @@ cudaError_t launch_persistent_cfg(const DevPtrs &d, const KParams &k, int vin, i
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BLOCK, 0)) != cudaSuccess) return e;
+    const size_t smem = LANES == 1 ? run_smem<FP32, BLOCK>() : 0;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BLOCK, smem)) != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     const long long need = ((long long)LANES * k.N + BLOCK - 1) / BLOCK;
     const int grid = (int)std::max(1LL, std::min<long long>((long long)per_sm * sms, need));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(BLOCK);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -391,6 +555,10 @@ cudaError_t launch_persistent_cfg(const DevPtrs &d, const KParams &k, int vin, i
 template <bool FP32, int LANES>
 cudaError_t launch_persistent_lanes(const DevPtrs &d, const KParams &k, int vin, int nsteps, int block,
                                     cudaStream_t s);
+
+// Shared-memory limits of the kernels with bond tiles (once, outside captures).
+template <bool FP32>
+cudaError_t init_persistent_tiles();
 
 template <bool FP32>
 cudaError_t launch_persistent_impl(const DevPtrs &d, const KParams &k, int vin, int nsteps, int block, cudaStream_t s) {

@@ -13,4 +13,9 @@ cudaError_t launch_persistent32(const DevPtrs &d, const KParams &k, int vin, int
     return launch_persistent_impl<true>(d, k, vin, nsteps, block, s);
 }
 
+cudaError_t init_tiles32() {
+    const cudaError_t e = init_force_run<true>();
+    return e != cudaSuccess ? e : init_persistent_tiles<true>();
+}
+
 }  // namespace pd

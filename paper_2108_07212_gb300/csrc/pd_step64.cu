@@ -14,4 +14,9 @@ cudaError_t launch_persistent64(const DevPtrs &d, const KParams &k, int vin, int
     return launch_persistent_impl<false>(d, k, vin, nsteps, block, s);
 }
 
+cudaError_t init_tiles64() {
+    const cudaError_t e = init_force_run<false>();
+    return e != cudaSuccess ? e : init_persistent_tiles<false>();
+}
+
 }  // namespace pd
