@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(kBlock) k_predict(DevPtrs d, KParams k, int vi
             // the persistent kernel's prediction of the next step no longer holds
             *d.pred_ok = 0;
         }
-        wall_cells(d, k, (double)st * k.dt);
+        wall_cells(d, k, (double)st * k.dt, d.wall_cell);
     }
     const bool need = i < k.N && predict_node<false>(d, k, i, vin, advance);
     if (__any_sync(0xffffffffu, need) && (threadIdx.x & 31) == 0) {

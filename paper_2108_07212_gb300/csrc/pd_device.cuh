@@ -582,6 +582,10 @@ __device__ __forceinline__ float d2f_hi_bits(double x) {
 // (one kernel body serves both parities).
 __shared__ double2 *s_cur_u;
 __shared__ float4 *s_cur_pq;
+// Likewise its time, its wall cells and the word its rebuild test raises.
+__shared__ double s_cur_t;
+__shared__ int4 *s_cur_wall;
+__shared__ int *s_raise;
 
 // Current displacement / positions of the kernel: the device pointers' own on
 // the multi-kernel path (the host sets them per launch), the persistent
@@ -604,6 +608,17 @@ struct Update32 {
     float2 a;               // previous acceleration
     int2 cell;
 };
+
+template <bool PERSIST>
+__device__ __forceinline__ const int4 *cur_wall(const DevPtrs &d) {
+    if constexpr (PERSIST) return s_cur_wall;
+    else return d.wall_cell;
+}
+template <bool PERSIST>
+__device__ __forceinline__ double cur_time(const DevPtrs &d) {
+    if constexpr (PERSIST) return s_cur_t;
+    else return *d.t_now;
+}
 
 // Shifted position xs + u of node i as a float-float pair into q_out[i], and
 // the rebuild test: the displacement since the last rebuild from the float-float
@@ -751,7 +766,7 @@ __device__ __forceinline__ void prefetch_force_inputs(const DevPtrs &d, const KP
     prefetch_range(d.step, sizeof(long long), g, nt);
     prefetch_range(d.rebuild, sizeof(int), g, nt);
     prefetch_range(d.status, sizeof(int) * PD_STATUS_COUNT, g, nt);
-    prefetch_range(d.bar, 2 * sizeof(unsigned), g, nt);
+    prefetch_range(d.bar, 3 * sizeof(unsigned), g, nt);
     prefetch_range(d.g_agg, 4 * G, g, nt);
     prefetch_range(d.agg, sizeof(AggParams) * (size_t)k.n_agg, g, nt);
     if (d.pq) {
@@ -785,10 +800,10 @@ __device__ __forceinline__ void prefetch_force_inputs(const DevPtrs &d, const KP
 // per force evaluation by the threads of one block, one aggregate each): a node
 // two or more cells away from all of them is farther than R_c from every wall
 // and feels no wall force.
-__device__ __forceinline__ void wall_cells(const DevPtrs &d, const KParams &k, double t) {
+__device__ __forceinline__ void wall_cells(const DevPtrs &d, const KParams &k, double t, int4 *out) {
     for (int a = threadIdx.x; a < k.n_agg; a += blockDim.x) {
         const AggParams &A = d.agg[a];
-        d.wall_cell[a] = make_int4(cell_coord(A.w0[0] + A.wv[0] * t, A.ox, A.inv_cell),
+        out[a] = make_int4(cell_coord(A.w0[0] + A.wv[0] * t, A.ox, A.inv_cell),
                                    cell_coord(A.w0[1] + A.wv[1] * t, A.ox, A.inv_cell),
                                    cell_coord(A.w0[2] + A.wv[2] * t, A.oy, A.inv_cell),
                                    cell_coord(A.w0[3] + A.wv[3] * t, A.oy, A.inv_cell));
@@ -801,7 +816,7 @@ __device__ __forceinline__ void wall_cells(const DevPtrs &d, const KParams &k, d
 template <bool PERSIST>
 __device__ __forceinline__ bool far_from_walls(const DevPtrs &d, int i, int ag) {
     const int2 c = ldm<PERSIST>(&d.cell[i]);
-    const int4 w = ldm<PERSIST>(&d.wall_cell[ag]);
+    const int4 w = ldm<PERSIST>(&cur_wall<PERSIST>(d)[ag]);
     return c.x - w.x >= 2 && w.y - c.x >= 2 && c.y - w.z >= 2 && w.w - c.y >= 2;
 }
 
@@ -879,17 +894,16 @@ __device__ __forceinline__ bool stn_bonded(const uint4 &st, uint32_t alive, int 
     return hit;
 }
 
-// Is the bond x -> j intact?  (row columns ascending: binary search; broken
-// flags read past L1, since other lanes may have just set them.)
+// Is the bond i -> j (rows r0..r1) intact?  (eight columns in flight at a time:
+// a search would be a chain of loads; broken flags read past L1, since other
+// lanes may have just set them.)
 __device__ __forceinline__ bool bonded_intact(const DevPtrs &d, const KParams &k, int i, int r0, int r1, int j) {
-    int lo = r0, hi = r1;
-    while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if (__ldg(&d.col[mid]) < j) lo = mid + 1; else hi = mid;
-    }
-    if (lo < r1 && __ldg(&d.col[lo]) == j) {
-        const int kk = lo - r0;
-        return !((__ldcg(&d.bits[(size_t)i * k.wpn + (kk >> 5)]) >> (kk & 31)) & 1u);
+    for (int b0 = r0; b0 < r1; b0 += 8) {
+        int hit = -1;
+#pragma unroll
+        for (int m = 0; m < 8; ++m)
+            if (b0 + m < r1 && __ldg(&d.col[b0 + m]) == j) hit = b0 + m - r0;
+        if (hit >= 0) return !((__ldcg(&d.bits[(size_t)i * k.wpn + (hit >> 5)]) >> (hit & 31)) & 1u);
     }
     return false;
 }
@@ -932,33 +946,34 @@ __device__ __forceinline__ int fresh_partner(const DevPtrs &d, const KParams &k,
 template <bool PERSIST>
 __device__ __forceinline__ void build_list_node(const DevPtrs &d, const KParams &k, int i) {
     const int gi = __ldg(&d.grain[i]);
-    const AggParams &A = d.agg[__ldg(&d.g_agg[gi])];
     const int2 cc = ldm<PERSIST>(&d.cell[i]);
-    const int wx = wrap_cell(cc.x, A.gw);
+    const int rank = ldm<PERSIST>(&d.rank[i]), key = ldm<PERSIST>(&d.key[i]);
+    const uint4 st = k.stencil ? __ldg(&d.stn[i]) : make_uint4(kStnIrregular, 0u, 0u, 0u);
+    const uint32_t w0 = __ldcg(&d.bits[(size_t)i * k.wpn]);
+    float4 qi = make_float4(0.f, 0.f, 0.f, 0.f);
+    double2 pi = make_double2(0.0, 0.0), ui = pi;
+    if (d.pq) {
+        qi = ldm<PERSIST>(&cur_pq<PERSIST>(d)[i]);
+    } else {
+        pi = ldm<PERSIST>(&d.p[i]);
+        ui = ldm<PERSIST>(&cur_u<PERSIST>(d)[i]);
+    }
+    const AggParams &A = d.agg[__ldg(&d.g_agg[gi])];
+    const int s0 = __ldg(&d.g_start[gi]), s1 = __ldg(&d.g_start[gi + 1]);
+    const int own = ldm<PERSIST>(&d.start[key]) + rank;          // the node's own record
     // the block's rows, each one range of records unless it wraps around
+    const int wx = wrap_cell(cc.x, A.gw);
     const bool whole = wx > 0 && wx < A.gw - 1;
-    int row[3], t0[3] = {0, 0, 0}, t1[3] = {0, 0, 0};
+    int row[3], t0[3], m[3];
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
         row[r] = A.gbase + wrap_cell(cc.y + r - 1, A.gh) * A.gw;
-        if (whole) {
-            t0[r] = ldm<PERSIST>(&d.start[row[r] + wx - 1]);
-            t1[r] = ldm<PERSIST>(&d.start[row[r] + wx + 2]);
-        }
+        t0[r] = ldm<PERSIST>(&d.start[row[r] + max(wx - 1, 0)]);
+        m[r] = whole ? ldm<PERSIST>(&d.start[row[r] + wx + 2]) - t0[r] : 0;
     }
-    const int s0 = __ldg(&d.g_start[gi]), s1 = __ldg(&d.g_start[gi + 1]);
-    const uint4 st = k.stencil ? __ldg(&d.stn[i]) : make_uint4(kStnIrregular, 0u, 0u, 0u);
-    const uint32_t w0 = __ldcg(&d.bits[(size_t)i * k.wpn]);
-    d.bref[(size_t)i * k.wpn] = w0;
-    for (int w = 1; w < k.wpn; ++w) d.bref[(size_t)i * k.wpn + w] = __ldcg(&d.bits[(size_t)i * k.wpn + w]);
-    float4 qi = make_float4(0.f, 0.f, 0.f, 0.f);
-    double2 pi = make_double2(0.0, 0.0);
-    if (d.pq) qi = ldm<PERSIST>(&cur_pq<PERSIST>(d)[i]);
-    else pi = ldm<PERSIST>(&d.p[i]);
     int lst[kMaxList];
     int n = 0, over = 0;
-    auto visit = [&](int t) {
-        const uint4 rec = ldm<PERSIST>(&d.srec[t]);
+    auto inside = [&](const uint4 &rec) {
         float dx, dy;
         if (d.pq) {
             dx = (__uint_as_float(rec.x) - qi.x) + (__uint_as_float(rec.z) - qi.z);
@@ -967,9 +982,9 @@ __device__ __forceinline__ void build_list_node(const DevPtrs &d, const KParams 
             dx = (float)(__hiloint2double((int)rec.y, (int)rec.x) - pi.x);
             dy = (float)(__hiloint2double((int)rec.w, (int)rec.z) - pi.y);
         }
-        if (!(dx * dx + dy * dy < A.rs2)) return;
-        const int j = ldm<PERSIST>(&d.sorted[t]);
-        if (j == i) return;
+        return dx * dx + dy * dy < A.rs2;
+    };
+    auto take = [&](int j) {
         if (j >= s0 && j < s1) {
             if (st.x & kStnIrregular) {
                 if (bonded_intact(d, k, i, __ldg(&d.row_ptr[i]), __ldg(&d.row_ptr[i + 1]), j)) return;
@@ -988,26 +1003,43 @@ __device__ __forceinline__ void build_list_node(const DevPtrs &d, const KParams 
             over = 1;
         }
     };
-    if (whole) {
+    // kListBatch records in flight together, then the node numbers of those inside
+    constexpr int kListBatch = 6;
+    const int tot = m[0] + m[1] + m[2];
+    for (int e0 = 0; e0 < tot; e0 += kListBatch) {
+        int t[kListBatch];
+        uint4 rec[kListBatch];
 #pragma unroll
-        for (int r = 0; r < 3; ++r)
-            for (int t = t0[r]; t < t1[r]; ++t) visit(t);
-    } else {
-        // (a grid has at least three cells each way: the nine are different)
-        for (int r = 0; r < 3; ++r)
-            for (int c = -1; c <= 1; ++c) {
-                const int cell = row[r] + wrap_cell(cc.x + c, A.gw);
-                for (int t = ldm<PERSIST>(&d.start[cell]), e = ldm<PERSIST>(&d.start[cell + 1]); t < e; ++t) visit(t);
-            }
+        for (int q = 0; q < kListBatch; ++q) {
+            const int e = e0 + q;
+            t[q] = e < m[0] ? t0[0] + e : (e < m[0] + m[1] ? t0[1] + (e - m[0]) : t0[2] + (e - m[0] - m[1]));
+            if (e >= tot || t[q] == own) t[q] = -1;
+            rec[q] = ldm<PERSIST>(&d.srec[max(t[q], 0)]);
+        }
+        int jb[kListBatch];
+#pragma unroll
+        for (int q = 0; q < kListBatch; ++q) jb[q] = t[q] >= 0 && inside(rec[q]) ? ldm<PERSIST>(&d.sorted[t[q]]) : -1;
+#pragma unroll
+        for (int q = 0; q < kListBatch; ++q)
+            if (jb[q] >= 0) take(jb[q]);
     }
+    if (!whole) {
+        // (a grid has at least three cells each way: the nine are different)
+        for (int c = 0; c < 9; ++c) {
+            const int cell = row[c / 3] + wrap_cell(cc.x + c % 3 - 1, A.gw);
+            for (int t = ldm<PERSIST>(&d.start[cell]), e = ldm<PERSIST>(&d.start[cell + 1]); t < e; ++t)
+                if (t != own && inside(ldm<PERSIST>(&d.srec[t]))) take(ldm<PERSIST>(&d.sorted[t]));
+        }
+    }
+    d.bref[(size_t)i * k.wpn] = w0;
+    for (int w = 1; w < k.wpn; ++w) d.bref[(size_t)i * k.wpn + w] = __ldcg(&d.bits[(size_t)i * k.wpn + w]);
     const size_t N = (size_t)k.N;
     for (int q = 0; q < n; ++q) d.nbr[q * N + i] = lst[q];
     d.nbr_cnt[i] = n;
     if (d.pq) {
         d.sref[i] = qi;
     } else {
-        const double2 u = ldm<PERSIST>(&cur_u<PERSIST>(d)[i]);
-        d.sref[i] = make_float4((float)u.x, (float)u.y, 0.f, 0.f);
+        d.sref[i] = make_float4((float)ui.x, (float)ui.y, 0.f, 0.f);
     }
     if (over) atomicAdd(&d.status[PD_STATUS_OVERFLOW], 1);
 }
@@ -1087,7 +1119,7 @@ __device__ __forceinline__ void finish_node32_total(const DevPtrs &d, const KPar
         d.v[vin ^ 1][i] = vn;
         if constexpr (PERSIST) {
             if (advance_node32(d, k, i, n.u, vn, ax, ay, n.xs, n.sref, d.ub[vin], d.pqb[vin]))
-                *(volatile int *)d.rebuild_next = 1;
+                *(volatile int *)s_raise = 1;
         }
     }
     d.af[i] = make_float2(ax, ay);
@@ -1518,7 +1550,7 @@ __device__ __forceinline__ void node_epilogue64(const DevPtrs &d, const KParams 
     const int2 cell = ldm<PERSIST>(&d.cell[i]);
     const int ag = __ldg(&d.g_agg[gi]);
     const double inv_m = __ldg(&d.g_invm[gi]);
-    const int4 wc = ldm<PERSIST>(&d.wall_cell[ag]);
+    const int4 wc = ldm<PERSIST>(&cur_wall<PERSIST>(d)[ag]);
     double Fwx = 0.0, Fwy = 0.0;
     const bool walls = !cells_far_from_walls(cell, wc);
     if (walls) {
@@ -1526,7 +1558,7 @@ __device__ __forceinline__ void node_epilogue64(const DevPtrs &d, const KParams 
         const AggParams &A = d.agg[ag];
         const double rho = k.mat ? __ldg(&d.g_rho[gi]) : k.rho;
         const double Kn = k.mat ? 18.0 * __ldg(&d.g_k[gi]) / A.pe5 : A.Kn;
-        wall_force64(k, A, Kn, rho, ldm<PERSIST>(d.t_now), pi.x, pi.y, vi.x, vi.y, __ldg(&d.V[i]), Fwx, Fwy,
+        wall_force64(k, A, Kn, rho, cur_time<PERSIST>(d), pi.x, pi.y, vi.x, vi.y, __ldg(&d.V[i]), Fwx, Fwy,
                      d.status);
     }
     if (k.store) {
@@ -1705,31 +1737,31 @@ __device__ __forceinline__ void tile_forward32(const KParams &k, uint32_t alive,
             }
         }
     }
-    if (excess > 0.f || alive != nd.st.x) {
-        // a bond breaks, lies in the guard band or is broken: markers and the sum again
+    // broken bonds (their other node has them broken too, unless the caller set
+    // the bits of one direction only)
+    for (uint32_t m = nd.st.x & ~alive & ~((1u << kPairHalf) - 1u); m; m &= m - 1u)
+        mine[(__ffs(m) - 1 - kPairHalf) * S].x = __uint_as_float(kPairNone);
+    if (excess > 0.f) {
+        // a bond breaks or lies in the guard band: markers and the sum again
         Fx = Fy = 0.f;
-        for (uint32_t m = nd.st.x & ~((1u << kPairHalf) - 1u); m; m &= m - 1u) {
+        for (uint32_t m = alive & ~((1u << kPairHalf) - 1u); m; m &= m - 1u) {
             const int o = __ffs(m) - 1, di = stn_di(o), dj = stn_dj(o), n = di * di + dj * dj;
             float2 *const at = &mine[(o - kPairHalf) * S];
-            unsigned mark = kPairNone;
-            if ((alive >> o) & 1u) {
-                BondGeom32 g;
-                const int r = bond_classify32(win[di + stn_row(nd.st, dj)], phi, pli, (float)n, stn_sqrt_n(n), nd.gq, s0_lo,
-                                              nd.gc.y * (1.0f + k.guard), g);
-                if (r == 0) {
-                    Fx = __fadd_rn(Fx, at->x);
-                    Fy = __fadd_rn(Fy, at->y);
-                    continue;
-                }
-                mark = r == 1 ? kPairBroken : kPairGuard;
-                if (r == 2) {
-                    note |= kNoteGuard;
-                } else if (OWN) {
-                    atomicOr(bw, stn_bit(nd.st.x, o));
-                    note |= kNoteBroke;
-                }
+            BondGeom32 g;
+            const int r = bond_classify32(win[di + stn_row(nd.st, dj)], phi, pli, (float)n, stn_sqrt_n(n), nd.gq, s0_lo,
+                                          nd.gc.y * (1.0f + k.guard), g);
+            if (r == 0) {
+                Fx = __fadd_rn(Fx, at->x);
+                Fy = __fadd_rn(Fy, at->y);
+                continue;
             }
-            at->x = __uint_as_float(mark);
+            at->x = __uint_as_float(r == 1 ? kPairBroken : kPairGuard);
+            if (r == 2) {
+                note |= kNoteGuard;
+            } else if (OWN) {
+                atomicOr(bw, stn_bit(nd.st.x, o));
+                note |= kNoteBroke;
+            }
         }
     }
 }
@@ -2207,7 +2239,7 @@ __device__ __forceinline__ void node_epilogue32(const DevPtrs &d, const KParams 
     const double2 vi = n.v;
     const int ag = __ldg(&d.g_agg[gi]);
     const float inv_m = __ldg(&d.g_invmf[gi]);
-    const int4 wc = ldm<PERSIST>(&d.wall_cell[ag]);
+    const int4 wc = ldm<PERSIST>(&cur_wall<PERSIST>(d)[ag]);
     Sums32 f = fin;
     if constexpr (!PERSIST) {
         // learned modal surrogate: between judge steps an active grain's bond force
@@ -2229,7 +2261,7 @@ __device__ __forceinline__ void node_epilogue32(const DevPtrs &d, const KParams 
         const double Kn = k.mat ? 18.0 * __ldg(&d.g_k[gi]) / A.pe5 : A.Kn;
         const double rho = k.mat ? __ldg(&d.g_rho[gi]) : k.rho;
         const float Knf = k.mat ? __ldg(&d.g_kf[gi]) : A.knf, rhof = __ldg(&d.gc[gi]).w;
-        wall_force32(k, A, Knf, rhof, Kn, rho, ldm<PERSIST>(d.t_now), pi.x, pi.y, vi.x, vi.y, __ldg(&d.V[i]), Fwx,
+        wall_force32(k, A, Knf, rhof, Kn, rho, cur_time<PERSIST>(d), pi.x, pi.y, vi.x, vi.y, __ldg(&d.V[i]), Fwx,
                      Fwy, d.status);
     }
     // the lane-sum pass may have summed the parts already (f.bx / f.by hold the total)
@@ -2338,14 +2370,14 @@ __device__ __forceinline__ void special_node64(const DevPtrs &d, const KParams &
         f.ny = add_in_order(f.ny, ny, m);
     }
     // walls: thread l takes wall l, thread 4 + c corner c
-    const bool walls = node && !cells_far_from_walls(cell, ldm<PERSIST>(&d.wall_cell[ag]));
+    const bool walls = node && !cells_far_from_walls(cell, ldm<PERSIST>(&cur_wall<PERSIST>(d)[ag]));
     double Fwx = 0.0, Fwy = 0.0;
     if (__any_sync(0xffffffffu, walls)) {
         double gx = 0.0, gy = 0.0;
         if (walls) {
             const double rho = k.mat ? __ldg(&d.g_rho[gi]) : k.rho;
             const double Kn = k.mat ? 18.0 * __ldg(&d.g_k[gi]) / A.pe5 : A.Kn;
-            const double t = ldm<PERSIST>(d.t_now), V = __ldg(&d.V[ii]);
+            const double t = cur_time<PERSIST>(d), V = __ldg(&d.V[ii]);
             bool past, past2;
             if (lane < 4) {
                 const double dl = wall_distance(A, lane, t, pi.x, pi.y, past);

@@ -389,7 +389,7 @@ size_t layout(pd_ctx *c, char *base) {
     carve(base, off, d.agg, (size_t)c->n_agg);
     carve(base, off, d.key, N);
     carve(base, off, d.cell, N);
-    carve(base, off, d.wall_cell, (size_t)c->n_agg);
+    carve(base, off, d.wall_cell, 2 * (size_t)c->n_agg);
     carve(base, off, d.count, c->T);
     carve(base, off, d.start, (size_t)c->T + 1);
     carve(base, off, d.rank, N);
@@ -401,6 +401,7 @@ size_t layout(pd_ctx *c, char *base) {
     carve(base, off, d.rebuild, 1);
     carve(base, off, d.pred_done, 1);
     carve(base, off, d.rebuild_next, 1);
+    carve(base, off, d.rebuild3, 3);
     carve(base, off, d.pred_ok, 1);
     carve(base, off, d.spec, N);
     carve(base, off, d.spec_n, 2);
@@ -410,7 +411,7 @@ size_t layout(pd_ctx *c, char *base) {
     carve(base, off, d.blocksums, std::max<size_t>(c->T / pd::kScanTile + 2, 16 * 1024));
     carve(base, off, d.step, 1);
     carve(base, off, d.t_now, 1);
-    carve(base, off, d.bar, 2);
+    carve(base, off, d.bar, 3);
     carve(base, off, d.status, PD_STATUS_COUNT);
     carve(base, off, d.diag_part, (size_t)c->kp.n_diag_blocks * PD_DIAG_COUNT);
     carve(base, off, d.diag_out, PD_DIAG_COUNT);
@@ -1075,7 +1076,7 @@ int pd_bind_arena(pd_ctx *c, void *arena, size_t bytes) {
     for (size_t g = 0; g < G; ++g) gkf[g] = (float)(18.0 * c->g_k[g] / c->aggp[c->g_agg[g]].pe5);
     PD_CUDA(cudaMemcpyAsync(d.g_kf, gkf.data(), 4 * G, cudaMemcpyHostToDevice, s));
     PD_CUDA(cudaMemcpyAsync(d.agg, c->aggp.data(), sizeof(pd::AggParams) * c->aggp.size(), cudaMemcpyHostToDevice, s));
-    PD_CUDA(cudaMemsetAsync(d.bar, 0, 2 * sizeof(unsigned), s));
+    PD_CUDA(cudaMemsetAsync(d.bar, 0, 3 * sizeof(unsigned), s));
     PD_CUDA(cudaMemsetAsync(d.t_now, 0, sizeof(double), s));
     // cell counts are zero between rebuilds; the first force evaluation rebuilds
     PD_CUDA(cudaMemsetAsync(d.count, 0, sizeof(int) * c->T, s));
@@ -1528,7 +1529,7 @@ int pd_clear_status(pd_ctx *c) {
     cudaStream_t s = c->stream;
     PD_CUDA(cudaMemsetAsync(d.status, 0, sizeof(int) * PD_STATUS_COUNT, s));
     if (d.mlp_err) PD_CUDA(cudaMemsetAsync(d.mlp_err, 0, sizeof(int), s));
-    PD_CUDA(cudaMemsetAsync(d.bar, 0, 2 * sizeof(unsigned), s));
+    PD_CUDA(cudaMemsetAsync(d.bar, 0, 3 * sizeof(unsigned), s));
     PD_CUDA(cudaMemsetAsync(d.pred_done, 0, sizeof(unsigned), s));
     PD_CUDA(cudaMemsetAsync(d.pred_ok, 0, sizeof(int), s));
     PD_CUDA(cudaMemsetAsync(d.rebuild_next, 0, sizeof(int), s));
@@ -1619,7 +1620,7 @@ int pd_autotune(pd_ctx *c, double *report) {
         PD_CUDA(cudaMemcpyAsync(d.bits, d.bbits, 4 * N * c->wpn, cudaMemcpyDeviceToDevice, s));
         PD_CUDA(cudaMemcpyAsync(d.step, &step0, 8, cudaMemcpyHostToDevice, s));
         PD_CUDA(cudaMemcpyAsync(d.status, st0, sizeof(st0), cudaMemcpyHostToDevice, s));
-        PD_CUDA(cudaMemsetAsync(d.bar, 0, 2 * sizeof(unsigned), s));
+        PD_CUDA(cudaMemsetAsync(d.bar, 0, 3 * sizeof(unsigned), s));
         PD_CUDA(cudaMemsetAsync(d.pred_ok, 0, sizeof(int), s));
         PD_CUDA(cudaStreamSynchronize(s));
         return PD_OK;

@@ -103,7 +103,8 @@ struct DevPtrs {
     float4 *sref;       // at the last rebuild: FP32 split pq, FP64 path (float u, 0, 0)
     int *rebuild;       // nonzero: rebuild the lists before the next force phase (cleared by the force phase)
     unsigned *pred_done;  // blocks of the displacement update that have finished (last-block election)
-    int *rebuild_next;  // FP32-split persistent kernel: the next step's rebuild flag, raised in the velocity update
+    int *rebuild_next;  // FP32-split persistent kernel: the next launch's rebuild flag, raised in the velocity update
+    int *rebuild3;      // the same between the steps of a launch: word st % 3 for step st
     int *pred_ok;       // nonzero: ub / pqb of the other parity hold the next step's u and pq (persistent kernel)
     uint4 *srec;        // position of sorted[t] in cell order: FP32 split pq, FP64 p (16 bytes)
     void *fsum;         // split force phase: per-node lane sums, six components of N floats (FP32) or doubles
@@ -114,7 +115,7 @@ struct DevPtrs {
     long long *step;
     double *t_now;      // time of the force evaluation that follows the predict phase
     int *status;        // PD_STATUS_COUNT counters
-    unsigned *bar;      // grid barrier: [0] arrivals, [1] generation
+    unsigned *bar;      // grid barriers: [0] arrivals, [1] generation of the first; [2] arrivals of the later ones
     double *diag_part;  // per-block diagnostic partial sums
     double *diag_out;   // PD_DIAG_COUNT
     double *obs_gdam;   // particle damage of every grain (G)
@@ -131,6 +132,7 @@ struct DevPtrs {
     double *g_invm;     // per grain: 1 / (rho V)
     float *g_invmf;     // the same as floats (FP32-split contexts)
     int4 *wall_cell;    // per aggregate: grid cells of its walls x_lo, x_hi, y_lo, y_hi at the current time
+                        // (two halves: the persistent kernel's steps alternate)
     // autotuner backup of the state
     double2 *bu, *bv, *ba;
     float2 *af;         // FP32-split contexts: the acceleration, a = F / m + g rounded to float (d.a unused)

@@ -133,7 +133,7 @@ __device__ __forceinline__ void run_plain_nodes(const DevPtrs &d, const KParams 
             if (active) {
                 const Update32 n{sm.v[at], sm.u[at], sm.xs[at], sm.sref[at], sm.a[at], sm.cell[at]};
                 const int gi = __ldg(&d.grain[i]);
-                special = contact || k.store || !cells_far_from_walls(n.cell, ldm<true>(&d.wall_cell[__ldg(&d.g_agg[gi])]));
+                special = contact || k.store || !cells_far_from_walls(n.cell, ldm<true>(&cur_wall<true>(d)[__ldg(&d.g_agg[gi])]));
                 if (special) reinterpret_cast<float2 *>(d.fsum)[i] = make_float2(f.bx, f.by);
                 else finish_node32_total<true>(d, k, i, vin, 1, n, f.bx, f.by, false, 0.0, 0.0, __ldg(&d.g_invmf[gi]));
             }
@@ -146,7 +146,7 @@ __device__ __forceinline__ void run_plain_nodes(const DevPtrs &d, const KParams 
                 const int gi = __ldg(&d.grain[i]);
                 const double2 v = ldm<true>(&d.v[vin][i]), a = ldm<true>(&d.a[i]);
                 special = contact || k.store ||
-                          !cells_far_from_walls(ldm<true>(&d.cell[i]), ldm<true>(&d.wall_cell[__ldg(&d.g_agg[gi])]));
+                          !cells_far_from_walls(ldm<true>(&d.cell[i]), ldm<true>(&cur_wall<true>(d)[__ldg(&d.g_agg[gi])]));
                 if (special) reinterpret_cast<double2 *>(d.fsum)[i] = make_double2(f.bx, f.by);
                 else finish_node64_total<true>(d, k, i, vin, 1, v, a, f.bx, f.by, false, 0.0, 0.0, __ldg(&d.g_invm[gi]));
             }
@@ -291,13 +291,16 @@ cudaError_t launch_force_impl(const DevPtrs &d, const KParams &k, int vin, int u
 // ---------------------------------------------------------------------------
 // persistent step kernel
 
-// Grid barrier with a bounded wait: the last block to arrive resets the
-// arrival count and advances the generation; the others sleep-poll the
-// generation for at most max_spins rounds (kBarrierSpins unless a test
-// shortens it), then set status[PD_STATUS_TIMEOUT] and report failure (the
-// kernel then returns, so the device never hangs).  Co-residency of all blocks
-// is guaranteed by the cooperative launch.
-__device__ __forceinline__ bool grid_barrier(const DevPtrs &d, long long max_spins) {
+// Grid barriers with a bounded wait.  Co-residency of all blocks is guaranteed
+// by the cooperative launch.  A wait polls at most max_spins times
+// (kBarrierSpins unless a test shortens it), then sets
+// status[PD_STATUS_TIMEOUT] and reports failure (the kernel then returns, so
+// the device never hangs); the others see the status at a later poll.
+//
+// The first barrier of a launch: the last block to arrive resets the arrival
+// count and advances the generation that the others poll, so nothing depends
+// on what an earlier launch (with another grid, or given up) left behind.
+__device__ __forceinline__ bool grid_barrier_first(const DevPtrs &d, long long max_spins) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -322,6 +325,36 @@ __device__ __forceinline__ bool grid_barrier(const DevPtrs &d, long long max_spi
             }
         }
         __threadfence();
+    }
+    __syncthreads();
+    return ok != 0;
+}
+
+// The later ones: a release-increment of a counter that block 0 cleared before
+// the launch's first barrier, and an acquire-poll until all arrivals of this
+// barrier (the epoch-th) are in: one trip to L2 and back after the last
+// arrival, where the reset and the generation above take two more.  (3.5 us a
+// barrier with the latter on 304 blocks.)
+__device__ __forceinline__ bool grid_barrier(const DevPtrs &d, long long max_spins, unsigned &epoch) {
+    __shared__ int ok;
+    ++epoch;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned *const count = d.bar + 2;
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+        const unsigned target = epoch * gridDim.x;
+        ok = 1;
+        for (long long n = 1;; ++n) {
+            unsigned c;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(count) : "memory");
+            if ((int)(c - target) >= 0) break;
+            if (n > max_spins || ((n & 63) == 0 && *(volatile int *)&d.status[PD_STATUS_TIMEOUT])) {
+                atomicExch(&d.status[PD_STATUS_TIMEOUT], 1);
+                ok = 0;
+                break;
+            }
+            __nanosleep(20);
+        }
     }
     __syncthreads();
     return ok != 0;
@@ -385,49 +418,69 @@ __device__ __forceinline__ int block_scan1(int &v, int *sm) {
 //     R3 exclusive scan of the counts -> cell starts (counts cleared)
 //     R4 counting-sort scatter of the node indices
 //     R5 candidate lists
-//   E  forces, acceleration and velocity update
-// s_cur_u / s_cur_pq hold this step's current displacement and positions
-// (parity vin ^ 1).  Cell counts are zero on entry and on exit.  False when a
-// grid barrier gave up (the kernel then returns).
+//   E  forces, acceleration and velocity update (one thread per node and the
+//      fused force phase: plain nodes, then special ones)
+// The barrier after A is left out where A was taken by the step before (FP32
+// split, after the first step): what it published is then known already.
+//   * The time of the step follows from the step counter at the launch.
+//   * The wall cells of step st lie in half st & 1 of wall_cell, written during
+//     the step before.
+//   * The rebuild flag of step st is word st % 3 of rebuild3, raised by the
+//     velocity updates of step st - 1 and cleared during step st - 2 (every
+//     block has read the word in step st - 3, and none raises it before
+//     st - 1).
+// s_cur_* hold this step's displacement, positions, time, wall cells and the
+// word its rebuild test raises.  Cell counts are zero on entry and on exit.
+// False when a grid barrier gave up (the kernel then returns).
 template <bool FP32, int LANES, int BLOCK>
 __device__ __forceinline__ bool persistent_step(const DevPtrs &d, const KParams &k, int vin, int st, int nsteps,
-                                                bool predicted, int *sm, long long &s_step) {
+                                                bool predicted, long long step0, unsigned &epoch, int *sm) {
     const int nthreads = gridDim.x * BLOCK;
     const int gtid = blockIdx.x * BLOCK + threadIdx.x;
     const unsigned T = k.T;
     const unsigned slice = (T / 4 + gridDim.x - 1) / gridDim.x * 4;
     const unsigned lo = min(T, blockIdx.x * slice), hi = min(T, lo + slice);
-    // A (the step counter's load is issued first, so that its latency
-    // overlaps the displacement update of block 0's nodes)
-    const long long s = (blockIdx.x == 0 && threadIdx.x == 0) ? __ldcg(d.step) + 1 : 0;
-    if (st == 0) prefetch_force_inputs(d, k, gtid, nthreads);
-    if (!predicted) {
-        bool need = false;
-        for (int i = gtid; i < k.N; i += nthreads) need |= predict_node<true>(d, k, i, vin, 1);
-        if (__any_sync(0xffffffffu, need) && (threadIdx.x & 31) == 0) *(volatile int *)d.rebuild = 1;
-    }
-    if (blockIdx.x == 0) {
-        if (threadIdx.x == 0) {
-            *d.step = s;
-            *d.t_now = (double)s * k.dt;
-            s_step = s;
-            if (st == 0) d.spec_n[0] = d.spec_n[1] = 0;
-            if constexpr (FP32) {
-                // the previous velocity update's rebuild test becomes this step's
-                // flag (no block reads the flag before the barrier below)
-                if (predicted && *(volatile int *)d.rebuild_next) *(volatile int *)d.rebuild = 1;
-                *(volatile int *)d.rebuild_next = 0;
-            }
+    const bool known = FP32 && st > 0;
+    if (!known) {
+        // A
+        if (st == 0) prefetch_force_inputs(d, k, gtid, nthreads);
+        if (!predicted) {
+            bool need = false;
+            for (int i = gtid; i < k.N; i += nthreads) need |= predict_node<true>(d, k, i, vin, 1);
+            if (__any_sync(0xffffffffu, need) && (threadIdx.x & 31) == 0) *(volatile int *)d.rebuild = 1;
         }
-        __syncthreads();
-        wall_cells(d, k, (double)s_step * k.dt);
+        if (blockIdx.x == 0) {
+            if (st == 0 && threadIdx.x == 0) {
+                d.bar[2] = 0u;
+                d.spec_n[0] = d.spec_n[1] = 0;
+                if constexpr (FP32) {
+                    // the last launch's rebuild test becomes this step's flag (no
+                    // block reads the flag before the barrier below)
+                    if (predicted && *(volatile int *)d.rebuild_next) *(volatile int *)d.rebuild = 1;
+                    *(volatile int *)d.rebuild_next = 0;
+                    d.rebuild3[0] = d.rebuild3[1] = d.rebuild3[2] = 0;
+                }
+            }
+            wall_cells(d, k, (double)(step0 + st + 1) * k.dt, d.wall_cell + (st & 1) * k.n_agg);
+        }
+        if (st == 0 ? !grid_barrier_first(d, k.bar_spins) : !grid_barrier(d, k.bar_spins, epoch)) return false;
     }
-    if (!grid_barrier(d, k.bar_spins)) return false;
-    if (__ldcg(d.rebuild)) {
+    const bool rebuild = __ldcg(known ? &d.rebuild3[st % 3] : d.rebuild) != 0;
+    if (gtid == 0) {
+        if (FP32) d.rebuild3[(st + 2) % 3] = 0;
+        if (st + 1 == nsteps) {
+            *d.step = step0 + nsteps;
+            *d.t_now = (double)(step0 + nsteps) * k.dt;
+        }
+    }
+    // the next step's wall cells, by the block with the shortest run of nodes
+    if (FP32 && st + 1 < nsteps && blockIdx.x == gridDim.x - 1)
+        wall_cells(d, k, (double)(step0 + st + 2) * k.dt, d.wall_cell + ((st + 1) & 1) * k.n_agg);
+    if (rebuild) {
         // R1
         for (int i = gtid; i < k.N; i += kBinBatch * nthreads) bin_nodes<true>(d, k, i, nthreads);
-        if (!grid_barrier(d, k.bar_spins)) return false;
-        // R2 (four cells a thread; T is a multiple of 4)
+        if (!grid_barrier(d, k.bar_spins, epoch)) return false;
+        // R2 (four cells a load; T is a multiple of 4)
         int part = 0;
         for (unsigned b = lo + 4 * threadIdx.x; b < hi; b += 4 * BLOCK) {
             const int4 c = __ldcg(reinterpret_cast<const int4 *>(&d.count[b]));
@@ -435,36 +488,45 @@ __device__ __forceinline__ bool persistent_step(const DevPtrs &d, const KParams 
         }
         part = block_sum<BLOCK>(part, sm);
         if (threadIdx.x == 0) d.blocksums[blockIdx.x] = part;
-        if (!grid_barrier(d, k.bar_spins)) return false;
-        // R3
+        if (!grid_barrier(d, k.bar_spins, epoch)) return false;
+        // R3 (kScan4 loads of four cells a thread and round)
+        constexpr unsigned kScan4 = 4;
         int off = 0;
         for (int b = threadIdx.x; b < (int)blockIdx.x; b += BLOCK) off += __ldcg(&d.blocksums[b]);
         off = block_sum<BLOCK>(off, sm);
-        for (unsigned b0 = lo; b0 < hi; b0 += 4 * BLOCK) {
-            const unsigned b = b0 + 4 * threadIdx.x;
-            int4 c = make_int4(0, 0, 0, 0);
-            if (b < hi) {
-                c = __ldcg(reinterpret_cast<const int4 *>(&d.count[b]));
-                *reinterpret_cast<int4 *>(&d.count[b]) = make_int4(0, 0, 0, 0);
-            }
-            int at = (c.x + c.y) + (c.z + c.w);
+        for (unsigned b0 = lo; b0 < hi; b0 += 4 * kScan4 * BLOCK) {
+            const unsigned b = b0 + 4 * kScan4 * threadIdx.x;
+            int4 c[kScan4];
+            int at = 0;
+#pragma unroll
+            for (unsigned q = 0; q < kScan4; ++q)
+                c[q] = b + 4 * q < hi ? __ldcg(reinterpret_cast<const int4 *>(&d.count[b + 4 * q])) : make_int4(0, 0, 0, 0);
+#pragma unroll
+            for (unsigned q = 0; q < kScan4; ++q) at += (c[q].x + c[q].y) + (c[q].z + c[q].w);
             const int tot = block_scan1<BLOCK>(at, sm);
             at += off;
-            if (b < hi) *reinterpret_cast<int4 *>(&d.start[b]) = make_int4(at, at + c.x, at + c.x + c.y, at + c.x + c.y + c.z);
+#pragma unroll
+            for (unsigned q = 0; q < kScan4; ++q) {
+                if (b + 4 * q >= hi) break;
+                *reinterpret_cast<int4 *>(&d.count[b + 4 * q]) = make_int4(0, 0, 0, 0);
+                *reinterpret_cast<int4 *>(&d.start[b + 4 * q]) =
+                    make_int4(at, at + c[q].x, at + c[q].x + c[q].y, at + c[q].x + c[q].y + c[q].z);
+                at += (c[q].x + c[q].y) + (c[q].z + c[q].w);
+            }
             off += tot;
         }
         if (gtid == 0) d.start[T] = k.N;
-        if (!grid_barrier(d, k.bar_spins)) return false;
+        if (!grid_barrier(d, k.bar_spins, epoch)) return false;
         // R4
         for (int i = gtid; i < k.N; i += kBinBatch * nthreads) scatter_nodes<true>(d, k, i, nthreads);
-        if (!grid_barrier(d, k.bar_spins)) return false;
+        if (!grid_barrier(d, k.bar_spins, epoch)) return false;
         // R5 (every block has read the flag: clear it for the next step)
         if (gtid == 0) {
             *d.rebuild = 0;
             atomicAdd(&d.status[PD_STATUS_REBUILDS], 1);
         }
         for (int i = gtid; i < k.N; i += nthreads) build_list_node<true>(d, k, i);
-        if (!grid_barrier(d, k.bar_spins)) return false;
+        if (!grid_barrier(d, k.bar_spins, epoch)) return false;
     }
     // E
     if constexpr (LANES == 1) {
@@ -473,26 +535,26 @@ __device__ __forceinline__ bool persistent_step(const DevPtrs &d, const KParams 
         if (k.split || !k.pair) {
             run_nodes<FP32, true, BLOCK>(d, k, lo0, hi0, vin, 1, !k.split);
             if (k.split) {
-                if (!grid_barrier(d, k.bar_spins)) return false;
+                if (!grid_barrier(d, k.bar_spins, epoch)) return false;
                 for (int i = gtid; i < k.N; i += nthreads) epilogue_node<FP32, true>(d, k, i, vin, 1);
             }
         } else {
             run_plain_nodes<FP32, BLOCK>(d, k, lo0, hi0, vin, st & 1);
-            if (!grid_barrier(d, k.bar_spins)) return false;
+            if (!grid_barrier(d, k.bar_spins, epoch)) return false;
             if (gtid == 0) d.spec_n[(st + 1) & 1] = 0;
             run_special_nodes<FP32, BLOCK>(d, k, vin, st & 1);
         }
     } else if (k.split) {
         const long long total = (((long long)LANES * k.N + 31) / 32) * 32;
         for (long long t = gtid; t < total; t += nthreads) sums_node<FP32, true, LANES>(d, k, (int)(t / LANES), (int)(t % LANES), vin);
-        if (!grid_barrier(d, k.bar_spins)) return false;
+        if (!grid_barrier(d, k.bar_spins, epoch)) return false;
         for (int i = gtid; i < k.N; i += nthreads) epilogue_node<FP32, true>(d, k, i, vin, 1);
     } else {
         for (int node0 = blockIdx.x * (BLOCK / LANES); node0 < k.N; node0 += gridDim.x * (BLOCK / LANES))
             force_block<FP32, true, LANES, BLOCK>(d, k, node0, vin, 1);
     }
     // the end of the launch orders the last step before whatever follows
-    return st + 1 >= nsteps || grid_barrier(d, k.bar_spins);
+    return st + 1 >= nsteps || grid_barrier(d, k.bar_spins, epoch);
 }
 
 // nsteps time steps in one cooperative launch, phases separated by bounded
@@ -504,19 +566,23 @@ template <bool FP32, int LANES, int BLOCK>
 __global__ void __launch_bounds__(BLOCK, run_blocks(BLOCK))
     k_persistent(DevPtrs d, KParams k, int vin, int nsteps) {
     __shared__ int sm[33];
-    __shared__ long long s_step;
     // wait test: the withheld block never arrives, so the others' barrier waits run out
     if ((int)blockIdx.x == k.withhold_block) return;
     // read by every thread before the first grid barrier; written only after it
     const bool pred0 = FP32 && *(volatile int *)d.pred_ok != 0;
+    const long long step0 = __ldcg(d.step);
+    unsigned epoch = 0;
     for (int st = 0; st < nsteps; ++st) {
         if (threadIdx.x == 0) {
             s_cur_u = d.ub[vin ^ 1];
             s_cur_pq = d.pqb[vin ^ 1];
+            s_cur_t = (double)(step0 + st + 1) * k.dt;
+            s_cur_wall = d.wall_cell + (st & 1) * k.n_agg;
+            s_raise = st + 1 < nsteps ? &d.rebuild3[(st + 1) % 3] : d.rebuild_next;
         }
         __syncthreads();
         const bool predicted = FP32 && (st > 0 || pred0);
-        if (!persistent_step<FP32, LANES, BLOCK>(d, k, vin, st, nsteps, predicted, sm, s_step)) return;
+        if (!persistent_step<FP32, LANES, BLOCK>(d, k, vin, st, nsteps, predicted, step0, epoch, sm)) return;
         vin ^= 1;
     }
     // the next launch may skip its first update phase (the end of this launch
