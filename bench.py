@@ -441,7 +441,8 @@ def _launches(mode: int, steps: int, rebuilds: int) -> int:
     """Kernels launched by `steps` timed steps: the displacement update and the
     force phase (one or two kernels) every step, plus the six rebuild kernels
     (bin, three scan kernels, scatter, lists) in the steps whose conditional
-    node ran them; the persistent kernel is one launch per step."""
+    node ran them (a lower bound up to 65536 nodes, where one rebuild kernel is
+    launched every step); the persistent kernel is one launch per step."""
     if mode & 1:
         return steps
     if mode & 4:      # rebuild kernels launched every step
@@ -946,8 +947,8 @@ def run_ours(args):
         "list_rebuilds": {"timed_steps": args.steps, key: rebuilds,
                           **({"fp64": rebuilds64} if sim64 is not None else {}),
                           "note": "contact candidate lists (radius R_c + 0.1 R_c) rebuilt only when a node has "
-                                  "moved 0.45 skin (inside the persistent kernel, or in a conditional graph node "
-                                  "on the kernel-graph path)"},
+                                  "moved 0.45 skin (inside the persistent kernel, or on the kernel-graph "
+                                  "path by one cluster's kernel or, beyond 65536 nodes, in a conditional node)"},
         "cpu_baseline": None,
         "e2e": e2e,
         "clocks": clk,

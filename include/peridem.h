@@ -202,8 +202,8 @@ int pd_bind_arena(pd_ctx *ctx, void *device_arena, size_t bytes);
  * the context stream; the step sequence runs as captured CUDA graphs.  The
  * contact neighbourhoods S^nbr (Algorithm 1, nodes within R_c) are taken from
  * per-node candidate lists of radius R_c + skin (skin = 0.1 R_c), rebuilt by
- * a grid counting sort in a conditional graph node only in steps where
- * some node has moved more than 0.45 skin since the last rebuild; every pair
+ * a grid counting sort only in steps where some node has moved more than
+ * 0.45 skin since the last rebuild; every pair
  * is still tested against R_c exactly, so the forces are those of a full
  * search.  status[PD_STATUS_REBUILDS] counts the rebuilds.
  * Errors: PD_ESTATE (not bound), PD_EINVAL (n_steps < 0), PD_ECUDA.
@@ -336,7 +336,8 @@ int pd_autotune(pd_ctx *ctx, double *report);
  * the force phase split in two passes (lane sums through device memory, then
  * walls and update one thread per node); modes 4-7 = modes 0-3 with the
  * candidate-list rebuild kernels launched every step (returning at once when no
- * rebuild is due) instead of behind a conditional graph node (same results;
+ * rebuild is due) instead of behind a conditional graph node or, up to 65536
+ * nodes, in one launch of one thread-block cluster (same results;
  * the persistent kernel ignores this bit; profilers that cannot trace kernels
  * of graphs with conditional nodes need it); lanes 1, 2, 4 or 8 threads per
  * node (1 = textbook summation order); block 128 or 256 threads (persistent

@@ -6,7 +6,7 @@
 #include <algorithm>
 #include <cstring>
 
-#include "pd_device.cuh"
+#include "pd_rebuild.cuh"
 
 namespace pd {
 
@@ -70,6 +70,26 @@ __global__ void __launch_bounds__(kBlock) k_build_list(DevPtrs d, KParams k) {
     // rebuild (the grid covers max(N, T / 4) threads: one int4 per thread)
     if ((unsigned)i < k.T / 4) reinterpret_cast<int4 *>(d.count)[i] = make_int4(0, 0, 0, 0);
     if (i < k.N) build_list_node<false>(d, k, i);
+}
+
+// The whole rebuild by one cluster of kClusterBlocks blocks, for few nodes: the
+// hardware brings a cluster's blocks onto the chip together and has a barrier
+// for them, so the kernel graph needs one launch, which returns at once when
+// the flag is clear: 3 us, where a conditional graph node around the six kernels
+// below costs every step about 15 us.  (Two disks of 3218 nodes, FP64: 46 to
+// 32 us a step; 4 materials, 5740 nodes, FP32 split: 44 to 24.)  A rebuild
+// itself takes 30 to 90 us, as much as the six kernels at up to kClusterNodes.
+constexpr int kClusterBlocks = 8, kClusterThreads = 1024;
+__global__ void __cluster_dims__(kClusterBlocks, 1, 1) __launch_bounds__(kClusterThreads, 1)
+    k_rebuild_cluster(DevPtrs d, KParams k) {
+    __shared__ int sm[33];
+    if (!__ldcg(d.rebuild)) return;
+    rebuild_lists<false, kClusterThreads>(d, k, blockIdx.x, kClusterBlocks, sm, [] {
+        __threadfence();
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        __threadfence();
+        return true;
+    });
 }
 
 // Block-wide exclusive scan of kScanItems values per thread.
@@ -363,6 +383,11 @@ cudaError_t launch_rebuild(const DevPtrs &d, const KParams &k, cudaStream_t s) {
     k_scan_apply<<<nb, kScanThreads, 0, s>>>(d.count, d.blocksums, d.start, k.T, k.N, d.rebuild);
     k_scatter<<<nn, kBlock, 0, s>>>(d, k);
     k_build_list<<<nblk(std::max<long long>(k.N, k.T / 4), kBlock), kBlock, 0, s>>>(d, k);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_rebuild_cluster(const DevPtrs &d, const KParams &k, cudaStream_t s) {
+    k_rebuild_cluster<<<kClusterBlocks, kClusterThreads, 0, s>>>(d, k);
     return cudaGetLastError();
 }
 

@@ -549,7 +549,9 @@ cudaError_t record_step(pd_ctx *c, int vin, cudaStream_t s, bool timed = false) 
     cudaGraph_t g = nullptr;
     if ((e = cudaStreamGetCaptureInfo(s, &cs, nullptr, &g)) != cudaSuccess) return e;
     if (cs != cudaStreamCaptureStatusActive || !g) return cudaErrorStreamCaptureUnmatched;
-    const int use_cond = (c->mode & 4) ? 0 : 1;
+    // few nodes: the rebuild is one launch, else the body of a conditional node
+    const bool cluster = c->N <= pd::kClusterNodes && !(c->mode & 4);
+    const int use_cond = (c->mode & 4) || cluster ? 0 : 1;
     cudaGraphConditionalHandle cond = 0;
     if (use_cond && (e = cudaGraphConditionalHandleCreate(&cond, g, 0, cudaGraphCondAssignDefault)) != cudaSuccess)
         return e;
@@ -571,6 +573,8 @@ cudaError_t record_step(pd_ctx *c, int vin, cudaStream_t s, bool timed = false) 
         // path modes 4-7: the rebuild kernels run every step and return at once
         // when the flag is clear (no conditional node)
         if ((e = pd::launch_rebuild(dv, c->kp, s)) != cudaSuccess) return e;
+    } else if (cluster) {
+        if ((e = pd::launch_rebuild_cluster(dv, c->kp, s)) != cudaSuccess) return e;
     } else {
         const cudaGraphNode_t *deps = nullptr;
         size_t nd = 0;
@@ -1632,6 +1636,7 @@ int pd_autotune(pd_ctx *c, double *report) {
     // 1, 2, 4 or 8 threads per node for every mode
     // modes 4 and 6: the kernel graph with the rebuild kernels launched every
     // step (returning at once without the flag) instead of the conditional node
+    // or the one-cluster rebuild
     for (int m : {0, 1, 2, 3, 4, 6}) {
         for (int lanes : {1, 2, 4, 8}) {
             if (c->prm.lanes && lanes != c->prm.lanes) continue;

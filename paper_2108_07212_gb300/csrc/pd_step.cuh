@@ -5,7 +5,7 @@
 
 #include <type_traits>
 
-#include "pd_device.cuh"
+#include "pd_rebuild.cuh"
 
 namespace pd {
 
@@ -291,133 +291,12 @@ cudaError_t launch_force_impl(const DevPtrs &d, const KParams &k, int vin, int u
 // ---------------------------------------------------------------------------
 // persistent step kernel
 
-// Grid barriers with a bounded wait.  Co-residency of all blocks is guaranteed
-// by the cooperative launch.  A wait polls at most max_spins times
-// (kBarrierSpins unless a test shortens it), then sets
-// status[PD_STATUS_TIMEOUT] and reports failure (the kernel then returns, so
-// the device never hangs); the others see the status at a later poll.
-//
-// The first barrier of a launch: the last block to arrive resets the arrival
-// count and advances the generation that the others poll, so nothing depends
-// on what an earlier launch (with another grid, or given up) left behind.
-__device__ __forceinline__ bool grid_barrier_first(const DevPtrs &d, long long max_spins) {
-    __shared__ int ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        volatile unsigned *gen = d.bar + 1;
-        const unsigned g = *gen;
-        __threadfence();
-        const unsigned arrived = atomicAdd(d.bar, 1u);
-        ok = 1;
-        if (arrived == gridDim.x - 1) {
-            atomicExch(d.bar, 0u);
-            __threadfence();
-            atomicAdd(d.bar + 1, 1u);
-        } else {
-            long long n = 0;
-            while (*gen == g) {
-                if (++n > max_spins || *(volatile int *)&d.status[PD_STATUS_TIMEOUT]) {
-                    atomicExch(&d.status[PD_STATUS_TIMEOUT], 1);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(64);
-            }
-        }
-        __threadfence();
-    }
-    __syncthreads();
-    return ok != 0;
-}
-
-// The later ones: a release-increment of a counter that block 0 cleared before
-// the launch's first barrier, and an acquire-poll until all arrivals of this
-// barrier (the epoch-th) are in: one trip to L2 and back after the last
-// arrival, where the reset and the generation above take two more.  (3.5 us a
-// barrier with the latter on 304 blocks.)
-__device__ __forceinline__ bool grid_barrier(const DevPtrs &d, long long max_spins, unsigned &epoch) {
-    __shared__ int ok;
-    ++epoch;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned *const count = d.bar + 2;
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
-        const unsigned target = epoch * gridDim.x;
-        ok = 1;
-        for (long long n = 1;; ++n) {
-            unsigned c;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(count) : "memory");
-            if ((int)(c - target) >= 0) break;
-            if (n > max_spins || ((n & 63) == 0 && *(volatile int *)&d.status[PD_STATUS_TIMEOUT])) {
-                atomicExch(&d.status[PD_STATUS_TIMEOUT], 1);
-                ok = 0;
-                break;
-            }
-            __nanosleep(20);
-        }
-    }
-    __syncthreads();
-    return ok != 0;
-}
-
-template <int BLOCK>
-__device__ __forceinline__ int block_sum(int v, int *sm) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) sm[warp] = v;
-    __syncthreads();
-    int t = 0;
-    if (threadIdx.x < 32) {
-        t = (lane < BLOCK / 32) ? sm[lane] : 0;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
-        if (lane == 0) sm[32] = t;
-    }
-    __syncthreads();
-    return sm[32];
-}
-
-// Exclusive scan of one value per thread over the block; returns the total.
-template <int BLOCK>
-__device__ __forceinline__ int block_scan1(int &v, int *sm) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = v;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += y;
-    }
-    __syncthreads();
-    if (lane == 31) sm[warp] = incl;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        int w = (lane < BLOCK / 32) ? sm[lane] : 0;
-        int wi = w;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, wi, off);
-            if (lane >= off) wi += y;
-        }
-        sm[lane] = wi - w;
-        if (lane == 31) sm[32] = wi;
-    }
-    __syncthreads();
-    v = sm[warp] + incl - v;
-    return sm[32];
-}
-
 // One time step of the persistent kernel, all phases:
 //   A  displacement update, positions, rebuild test       (Algorithm 1)
 //      (FP32 split: taken by the previous step's velocity update instead,
 //      except in the first step of a launch that finds no valid prediction)
-//   when some node moved kSkinTrigger * skin since the last rebuild:
-//     R1 cell counts
-//     R2 per-block sums of the cell counts
-//     R3 exclusive scan of the counts -> cell starts (counts cleared)
-//     R4 counting-sort scatter of the node indices
-//     R5 candidate lists
+//   R  the candidate lists, when some node moved kSkinTrigger * skin since the
+//      last rebuild (rebuild_lists)
 //   E  forces, acceleration and velocity update (one thread per node and the
 //      fused force phase: plain nodes, then special ones)
 // The barrier after A is left out where A was taken by the step before (FP32
@@ -430,16 +309,12 @@ __device__ __forceinline__ int block_scan1(int &v, int *sm) {
 //     block has read the word in step st - 3, and none raises it before
 //     st - 1).
 // s_cur_* hold this step's displacement, positions, time, wall cells and the
-// word its rebuild test raises.  Cell counts are zero on entry and on exit.
-// False when a grid barrier gave up (the kernel then returns).
+// word its rebuild test raises.  False when a grid barrier gave up (the kernel then returns).
 template <bool FP32, int LANES, int BLOCK>
 __device__ __forceinline__ bool persistent_step(const DevPtrs &d, const KParams &k, int vin, int st, int nsteps,
                                                 bool predicted, long long step0, unsigned &epoch, int *sm) {
     const int nthreads = gridDim.x * BLOCK;
     const int gtid = blockIdx.x * BLOCK + threadIdx.x;
-    const unsigned T = k.T;
-    const unsigned slice = (T / 4 + gridDim.x - 1) / gridDim.x * 4;
-    const unsigned lo = min(T, blockIdx.x * slice), hi = min(T, lo + slice);
     const bool known = FP32 && st > 0;
     if (!known) {
         // A
@@ -476,58 +351,9 @@ __device__ __forceinline__ bool persistent_step(const DevPtrs &d, const KParams 
     // the next step's wall cells, by the block with the shortest run of nodes
     if (FP32 && st + 1 < nsteps && blockIdx.x == gridDim.x - 1)
         wall_cells(d, k, (double)(step0 + st + 2) * k.dt, d.wall_cell + ((st + 1) & 1) * k.n_agg);
-    if (rebuild) {
-        // R1
-        for (int i = gtid; i < k.N; i += kBinBatch * nthreads) bin_nodes<true>(d, k, i, nthreads);
-        if (!grid_barrier(d, k.bar_spins, epoch)) return false;
-        // R2 (four cells a load; T is a multiple of 4)
-        int part = 0;
-        for (unsigned b = lo + 4 * threadIdx.x; b < hi; b += 4 * BLOCK) {
-            const int4 c = __ldcg(reinterpret_cast<const int4 *>(&d.count[b]));
-            part += (c.x + c.y) + (c.z + c.w);
-        }
-        part = block_sum<BLOCK>(part, sm);
-        if (threadIdx.x == 0) d.blocksums[blockIdx.x] = part;
-        if (!grid_barrier(d, k.bar_spins, epoch)) return false;
-        // R3 (kScan4 loads of four cells a thread and round)
-        constexpr unsigned kScan4 = 4;
-        int off = 0;
-        for (int b = threadIdx.x; b < (int)blockIdx.x; b += BLOCK) off += __ldcg(&d.blocksums[b]);
-        off = block_sum<BLOCK>(off, sm);
-        for (unsigned b0 = lo; b0 < hi; b0 += 4 * kScan4 * BLOCK) {
-            const unsigned b = b0 + 4 * kScan4 * threadIdx.x;
-            int4 c[kScan4];
-            int at = 0;
-#pragma unroll
-            for (unsigned q = 0; q < kScan4; ++q)
-                c[q] = b + 4 * q < hi ? __ldcg(reinterpret_cast<const int4 *>(&d.count[b + 4 * q])) : make_int4(0, 0, 0, 0);
-#pragma unroll
-            for (unsigned q = 0; q < kScan4; ++q) at += (c[q].x + c[q].y) + (c[q].z + c[q].w);
-            const int tot = block_scan1<BLOCK>(at, sm);
-            at += off;
-#pragma unroll
-            for (unsigned q = 0; q < kScan4; ++q) {
-                if (b + 4 * q >= hi) break;
-                *reinterpret_cast<int4 *>(&d.count[b + 4 * q]) = make_int4(0, 0, 0, 0);
-                *reinterpret_cast<int4 *>(&d.start[b + 4 * q]) =
-                    make_int4(at, at + c[q].x, at + c[q].x + c[q].y, at + c[q].x + c[q].y + c[q].z);
-                at += (c[q].x + c[q].y) + (c[q].z + c[q].w);
-            }
-            off += tot;
-        }
-        if (gtid == 0) d.start[T] = k.N;
-        if (!grid_barrier(d, k.bar_spins, epoch)) return false;
-        // R4
-        for (int i = gtid; i < k.N; i += kBinBatch * nthreads) scatter_nodes<true>(d, k, i, nthreads);
-        if (!grid_barrier(d, k.bar_spins, epoch)) return false;
-        // R5 (every block has read the flag: clear it for the next step)
-        if (gtid == 0) {
-            *d.rebuild = 0;
-            atomicAdd(&d.status[PD_STATUS_REBUILDS], 1);
-        }
-        for (int i = gtid; i < k.N; i += nthreads) build_list_node<true>(d, k, i);
-        if (!grid_barrier(d, k.bar_spins, epoch)) return false;
-    }
+    if (rebuild && !rebuild_lists<true, BLOCK>(d, k, blockIdx.x, gridDim.x, sm,
+                                               [&] { return grid_barrier(d, k.bar_spins, epoch); }))
+        return false;
     // E
     if constexpr (LANES == 1) {
         const int len = run_length(k.N, gridDim.x);
