@@ -445,24 +445,23 @@ __device__ __forceinline__ void wall_force32(const KParams &k, const AggParams &
 // Float-float (hi + lo) of a double from its bits: hi holds the top 24
 // significand bits, lo the next 24 (the last five are dropped: 2^-48 relative).
 // Integer operations and one conversion of a 24-bit integer, no FP64
-// instruction.  Magnitudes below 2^-79 lose lo, below 2^-126 become 0.
+// instruction.  Magnitudes below 2^-79 lose lo, below 2^-126 become 0; beyond
+// the float range, inf and NaN are carried as inf or NaN.  Without branches, so
+// that the chains of several bonds interleave (see bond_terms64).
 __device__ __forceinline__ void dbl_to_ff(double x, float &hi, float &lo) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
     const int e = (int)((b >> 52) & 0x7FF);
-    if (e < 897) {
-        hi = lo = 0.f;
-        return;
-    }
-    if (e > 1150) {                     // beyond the float range, inf or NaN: carried as inf or NaN
-        hi = lo = e == 2047 && (b & 0xFFFFFFFFFFFFFull) ? __int_as_float(0x7FC00000) : __uint_as_float(sign | 0x7F800000u);
-        return;
-    }
     const unsigned long long m = b & 0xFFFFFFFFFFFFFull;
-    hi = __uint_as_float(sign | ((unsigned)(e - 896) << 23) | (unsigned)(m >> 29));
     // fraction bits 28..5 carry the weight 2^(e - 1023 - 47)
     const float scale = e > 943 ? __uint_as_float((unsigned)(e - 943) << 23) : 0.f;
-    lo = __uint_as_float(sign | __float_as_uint(__uint2float_rn((unsigned)(m >> 5) & 0xFFFFFFu) * scale));
+    const float h = __uint_as_float(sign | ((unsigned)(e - 896) << 23) | (unsigned)(m >> 29));
+    const float l = __uint_as_float(sign | __float_as_uint(__uint2float_rn((unsigned)(m >> 5) & 0xFFFFFFu) * scale));
+    const float big = e == 2047 && m ? __int_as_float(0x7FC00000) : __uint_as_float(sign | 0x7F800000u);
+    const float off = e < 897 ? 0.f : big;
+    const bool in = (unsigned)(e - 897) <= 1150u - 897u;
+    hi = in ? h : off;
+    lo = in ? l : off;
 }
 
 // Correctly rounded (to nearest) square root of a positive normal double, in
@@ -482,7 +481,7 @@ __device__ __forceinline__ void dbl_to_ff(double x, float &hi, float &lo) {
 // random inputs by pd_check_sqrt).
 __device__ __forceinline__ double sqrt_rn_int(double x) {
     const unsigned long long D = (unsigned long long)__double_as_longlong(x);
-    if (D == 0ull || (D >> 52) >= 0x7FFull) return x;   // 0, inf, NaN (negative inputs do not occur)
+    const bool same = D == 0ull || (D >> 52) >= 0x7FFull;   // 0, inf, NaN (negative inputs do not occur)
     const int E = (int)(D >> 52) - 1023;
     const unsigned long long M = (D & 0xFFFFFFFFFFFFFull) | (1ull << 52);
     const int odd = E & 1;
@@ -512,12 +511,13 @@ __device__ __forceinline__ double sqrt_rn_int(double x) {
     const float rf = __int2float_rn((int)(long long)((r_hi << 32) | (r_lo >> 32))) * 4294967296.0f;
     long long Q = Y + __float2int_rn(rf * (r * 1.1102230246251565e-16f));   // R / (2 Y), 1 / (2 Y) = r 2^-53
     long long R = (long long)(n_lo - (unsigned long long)Q * (unsigned long long)Q);
-    if (R < 0) {
-        Q -= 1;
-        R += 2 * Q + 1;
-    }
+    const long long Q1 = Q - 1;
+    const bool below = R < 0;
+    Q = below ? Q1 : Q;
+    R += below ? 2 * Q1 + 1 : 0;
     Q += R > Q ? 1 : 0;
-    return __longlong_as_double(((long long)(eL + 1023) << 52) + (Q - (1ll << 52)));
+    const double root = __longlong_as_double(((long long)(eL + 1023) << 52) + (Q - (1ll << 52)));
+    return same ? x : root;
 }
 
 // float-float arithmetic (Dekker / Knuth error-free transformations with FMA)
@@ -1238,25 +1238,48 @@ struct Sums32 {
 // quotient by |xi|, the break decision away from the threshold and the bond
 // force c_w w s V_x V_y (d / L) are float-float (relative error ~1e-14; a bond
 // whose stretch lies within 1e-6 of s0 is decided by the FP64 quotient).
-// cwVV = c_w V^2 (one grain: V_y = V_x).
-__device__ __forceinline__ bool bond_force64(double2 pi, double2 pj, double xi, ff cwVV, ff inv_eps, float s0f,
-                                             double s0, int micro, ff &fx, ff &fy) {
-    const double dx = __dsub_rn(pj.x, pi.x), dy = __dsub_rn(pj.y, pi.y);
-    const double L = sqrt_rn_int(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
-    const double diff = __dsub_rn(L, xi);                       // |xi| s, exact as in FP64
-    const ff dff = to_ff(diff), xff = to_ff(xi);
-    // break test |diff| > s0 |xi| in float, the FP64 quotient near the threshold
-    const float lhs = fabsf(dff.hi), rhs = s0f * xff.hi;
-    bool brk = lhs > rhs;
-    if (fabsf(lhs - rhs) <= 1e-6f * rhs) brk = fabs(__ddiv_rn(diff, xi)) > s0;
-    if (brk) return false;
-    // c_w w V_x V_y (diff / |xi|) / L  (w = 1 - |xi| / eps for the conic micromodulus)
-    ff c = cwVV;
-    if (micro) c = ff_mul(c, ff_add({1.0f, 0.f}, ff_mul({-xff.hi, -xff.lo}, inv_eps)));
-    const ff t = ff_mul(ff_mul(c, dff), ff_rcp(ff_mul(xff, to_ff(L))));
+// c = c_w w V^2 (one grain: V_y = V_x; w = 1, or 1 - |xi| / eps for the conic
+// micromodulus).
+//
+// A bond is a chain of some 200 dependent 32-bit operations.  bond_terms64 has
+// no branch, so a thread's bonds of a batch run interleaved; the rare decisions
+// (near the threshold, broken) follow the batch.  (Bond tiles of 1.03M nodes
+// with a branch at each special case and at each bond, the 12 bonds unrolled:
+// 37% of the issue slots, a sixth of the stalls for instructions to arrive.)
+__device__ __forceinline__ ff bond_conic64(ff cwVV, double xi, ff inv_eps) {
+    const ff x = to_ff(xi);
+    return ff_mul(cwVV, ff_add({1.0f, 0.f}, ff_mul({-x.hi, -x.lo}, inv_eps)));
+}
+__device__ __forceinline__ double bond_diff64(double2 pi, double2 pj, double xi, double &dx, double &dy, double &L) {
+    dx = __dsub_rn(pj.x, pi.x);
+    dy = __dsub_rn(pj.y, pi.y);
+    L = sqrt_rn_int(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
+    return __dsub_rn(L, xi);                                    // |xi| s, exact as in FP64
+}
+// The bond's force, as if it held, and the float decision: broken, and whether
+// it is near the threshold and takes bond_breaks64's.
+__device__ __forceinline__ void bond_terms64(double2 pi, double2 pj, double xi, ff c, float s0f, ff &fx, ff &fy,
+                                             bool &broken, bool &near) {
+    double dx, dy, L;
+    const ff dff = to_ff(bond_diff64(pi, pj, xi, dx, dy, L)), xff = to_ff(xi);
+    const float lhs = fabsf(dff.hi), rhs = s0f * xff.hi;        // |diff| > s0 |xi|
+    broken = lhs > rhs;
+    near = fabsf(lhs - rhs) <= 1e-6f * rhs;
+    const ff t = ff_mul(ff_mul(c, dff), ff_rcp(ff_mul(xff, to_ff(L))));     // c (diff / |xi|) / L
     fx = ff_mul(t, to_ff(dx));
     fy = ff_mul(t, to_ff(dy));
-    return true;
+}
+__device__ __forceinline__ bool bond_breaks64(double2 pi, double2 pj, double xi, double s0) {
+    double dx, dy, L;
+    return fabs(__ddiv_rn(bond_diff64(pi, pj, xi, dx, dy, L), xi)) > s0;
+}
+// One bond: false when it breaks at this evaluation.
+__device__ __forceinline__ bool bond_force64(double2 pi, double2 pj, double xi, ff cwVV, ff inv_eps, float s0f,
+                                             double s0, int micro, ff &fx, ff &fy) {
+    bool broken, near;
+    bond_terms64(pi, pj, xi, micro ? bond_conic64(cwVV, xi, inv_eps) : cwVV, s0f, fx, fy, broken, near);
+    if (near) broken = bond_breaks64(pi, pj, xi, s0);
+    return !broken;
 }
 
 // The forward half of node ii's stencil bonds (alive: the intact ones), FP64
@@ -1270,34 +1293,48 @@ __device__ __forceinline__ uint32_t tile_forward64(const DevPtrs &d, const KPara
     const int at = kCarry + (int)threadIdx.x;
     uint32_t formed = 0u;
     constexpr int kBatch = 4;
-#pragma unroll
+#pragma unroll 1
     for (int m0 = 0; m0 < kPairHalf; m0 += kBatch) {
+        const uint32_t live = alive >> (kPairHalf + m0);
+        const auto to = [&](int m) { return ii + stn_di(kPairHalf + m0 + m) + stn_row(st, stn_dj(kPairHalf + m0 + m)); };
         double2 pb[kBatch];
         double xb[kBatch];
 #pragma unroll
         for (int m = 0; m < kBatch; ++m) {
-            const int o = kPairHalf + m0 + m;
-            const bool live = (alive >> o) & 1u;
-            pb[m] = ldm<PERSIST>(&d.p[live ? ii + stn_di(o) + stn_row(st, stn_dj(o)) : ii]);
-            xb[m] = live ? __ldg(&d.xif[(size_t)(m0 + m) * k.N + ii]) : 1.0;
+            pb[m] = ldm<PERSIST>(&d.p[(live >> m) & 1u ? to(m) : ii]);
+            xb[m] = (live >> m) & 1u ? __ldg(&d.xif[(size_t)(m0 + m) * k.N + ii]) : 1.0;
+        }
+        ff c[kBatch], fx[kBatch], fy[kBatch];
+        uint32_t broken = 0u, near = 0u;
+#pragma unroll
+        for (int m = 0; m < kBatch; ++m) c[m] = cwVV;
+        if (k.micro) {
+#pragma unroll
+            for (int m = 0; m < kBatch; ++m) c[m] = bond_conic64(cwVV, xb[m], inv_eps);
         }
 #pragma unroll
         for (int m = 0; m < kBatch; ++m) {
-            const int o = kPairHalf + m0 + m;
-            unsigned mark = kPairNone;
-            ff fx = {0.f, 0.f}, fy = fx;
-            if ((alive >> o) & 1u) {
-                if (bond_force64(pi, pb[m], xb[m], cwVV, inv_eps, s0f, s0, k.micro, fx, fy)) {
-                    mark = 0u;
-                    formed |= 1u << o;
-                } else {
-                    mark = kPairBroken;
-                    if (OWN) atomicOr(&d.bits[(size_t)ii * k.wpn], stn_bit(st.x, o));
-                    note |= kNoteBroke;
-                }
-            }
-            slot[(m0 + m) * S + at] = make_float4(mark ? __uint_as_float(mark) : fx.hi, fx.lo, fy.hi, fy.lo);
+            bool b, n;
+            bond_terms64(pi, pb[m], xb[m], c[m], s0f, fx[m], fy[m], b, n);
+            broken |= (b && ((live >> m) & 1u)) ? 1u << m : 0u;
+            near |= (n && ((live >> m) & 1u)) ? 1u << m : 0u;
         }
+        for (; near; near &= near - 1u) {
+            const int m = __ffs(near) - 1;
+            const bool b = bond_breaks64(pi, ldm<PERSIST>(&d.p[to(m)]), __ldg(&d.xif[(size_t)(m0 + m) * k.N + ii]), s0);
+            broken = b ? broken | (1u << m) : broken & ~(1u << m);
+        }
+        if (broken) {
+            note |= kNoteBroke;
+            for (uint32_t b = broken; OWN && b; b &= b - 1u)
+                atomicOr(&d.bits[(size_t)ii * k.wpn], stn_bit(st.x, kPairHalf + m0 + __ffs(b) - 1));
+        }
+#pragma unroll
+        for (int m = 0; m < kBatch; ++m) {
+            const unsigned mark = !((live >> m) & 1u) ? kPairNone : ((broken >> m) & 1u) ? kPairBroken : 0u;
+            slot[(m0 + m) * S + at] = make_float4(mark ? __uint_as_float(mark) : fx[m].hi, fx[m].lo, fy[m].hi, fy[m].lo);
+        }
+        formed |= (live & ((1u << kBatch) - 1u) & ~broken) << (kPairHalf + m0);
     }
     return formed;
 }
@@ -1492,33 +1529,62 @@ __device__ __forceinline__ void force_node64(const DevPtrs &d, const KParams &k,
         r0 = active ? __ldg(&d.row_ptr[ii]) : 0;
         r1 = active ? __ldg(&d.row_ptr[ii + 1]) : 0;
     }
-    constexpr int kBondBatch64 = 4;
-    for (int b0 = r0 + lane; b0 < r1 && csr; b0 += kBondBatch64 * LANES) {
-        int jb[kBondBatch64];
-        uint32_t wb[kBondBatch64];
-        double xb[kBondBatch64];
-        double2 pb[kBondBatch64];
+    // six bonds loaded, three evaluated at a time: a full row of 24 is 4, 2, 1
+    // rounds of loads and 8, 4, 2, 1 of evaluations with 1, 2, 4, 8 threads
+    constexpr int kLoad = 6, kEval = 3;
+    for (int b0 = r0 + lane; b0 < r1 && csr; b0 += kLoad * LANES) {
+        int jb[kLoad];
+        uint32_t wb[kLoad];
+        double xb[kLoad];
+        double2 pb[kLoad];
 #pragma unroll
-        for (int m = 0; m < kBondBatch64; ++m) {
+        for (int m = 0; m < kLoad; ++m) {
             const int b = b0 + m * LANES;
             jb[m] = b < r1 ? __ldg(&d.col[b]) : -1;
             xb[m] = b < r1 ? __ldg(&d.xi[b]) : 1.0;
             wb[m] = b - r0 < 32 ? w0 : (b < r1 ? __ldcg(&bw[(b - r0) >> 5]) : 0u);
         }
+        uint32_t live = 0u;
 #pragma unroll
-        for (int m = 0; m < kBondBatch64; ++m) pb[m] = ldm<PERSIST>(&d.p[jb[m] < 0 ? ii : jb[m]]);
+        for (int m = 0; m < kLoad; ++m) {
+            pb[m] = ldm<PERSIST>(&d.p[jb[m] < 0 ? ii : jb[m]]);
+            live |= (jb[m] >= 0 && !((wb[m] >> ((b0 + m * LANES - r0) & 31)) & 1u)) ? 1u << m : 0u;
+        }
 #pragma unroll
-        for (int m = 0; m < kBondBatch64; ++m) {
-            const int kk = b0 + m * LANES - r0;
-            if (jb[m] < 0 || ((wb[m] >> (kk & 31)) & 1u)) continue;
-            ff fx, fy;
-            if (!bond_force64(pi, pb[m], xb[m], cwVV, inv_eps, s0f, s0, k.micro, fx, fy)) {
+        for (int m0 = 0; m0 < kLoad; m0 += kEval) {
+            if (!(live >> m0)) break;
+            ff c[kEval], fx[kEval], fy[kEval];
+            uint32_t broken = 0u, near = 0u;
+#pragma unroll
+            for (int m = 0; m < kEval; ++m) c[m] = cwVV;
+            if (k.micro) {
+#pragma unroll
+                for (int m = 0; m < kEval; ++m) c[m] = bond_conic64(cwVV, xb[m0 + m], inv_eps);
+            }
+#pragma unroll
+            for (int m = 0; m < kEval; ++m) {
+                bool b, n;
+                bond_terms64(pi, pb[m0 + m], xb[m0 + m], c[m], s0f, fx[m], fy[m], b, n);
+                broken |= b ? 1u << (m0 + m) : 0u;
+                near |= n ? 1u << (m0 + m) : 0u;
+            }
+            broken &= live;
+            for (near &= live; near; near &= near - 1u) {
+                const int m = __ffs(near) - 1, b = b0 + m * LANES;
+                const bool brk = bond_breaks64(pi, ldm<PERSIST>(&d.p[__ldg(&d.col[b])]), __ldg(&d.xi[b]), s0);
+                broken = brk ? broken | (1u << m) : broken & ~(1u << m);
+            }
+            for (uint32_t m = broken; m; m &= m - 1u) {
+                const int kk = b0 + (__ffs(m) - 1) * LANES - r0;
                 atomicOr(&bw[kk >> 5], 1u << (kk & 31));
                 note |= kNoteBroke;
-                continue;
             }
-            Fbx = ff_add(Fbx, fx);
-            Fby = ff_add(Fby, fy);
+#pragma unroll
+            for (int m = 0; m < kEval; ++m) {
+                const bool ok = ((live & ~broken) >> (m0 + m)) & 1u;
+                Fbx = ff_add(Fbx, ok ? fx[m] : ff{0.f, 0.f});
+                Fby = ff_add(Fby, ok ? fy[m] : ff{0.f, 0.f});
+            }
         }
     }
     __syncwarp();

@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kBlock, FP32 ? 8 : 4) k_sums(DevPtrs d, KParam
 }
 
 template <bool FP32>
-__global__ void __launch_bounds__(256, 6) k_epilogue(DevPtrs d, KParams k, int vin, int update_v) {
+__global__ void __launch_bounds__(256, FP32 ? 6 : 2) k_epilogue(DevPtrs d, KParams k, int vin, int update_v) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < k.N) epilogue_node<FP32, false>(d, k, i, vin, update_v);
 }
