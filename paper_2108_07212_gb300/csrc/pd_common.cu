@@ -72,19 +72,20 @@ __global__ void __launch_bounds__(kBlock) k_build_list(DevPtrs d, KParams k) {
     if (i < k.N) build_list_node<false>(d, k, i);
 }
 
-// The whole rebuild by one cluster of kClusterBlocks blocks, for few nodes: the
-// hardware brings a cluster's blocks onto the chip together and has a barrier
-// for them, so the kernel graph needs one launch, which returns at once when
-// the flag is clear: 3 us, where a conditional graph node around the six kernels
-// below costs every step about 15 us.  (Two disks of 3218 nodes, FP64: 46 to
-// 32 us a step; 4 materials, 5740 nodes, FP32 split: 44 to 24.)  A rebuild
-// itself takes 30 to 90 us, as much as the six kernels at up to kClusterNodes.
-constexpr int kClusterBlocks = 8, kClusterThreads = 1024;
-__global__ void __cluster_dims__(kClusterBlocks, 1, 1) __launch_bounds__(kClusterThreads, 1)
-    k_rebuild_cluster(DevPtrs d, KParams k) {
+// The whole rebuild by one cluster of blocks, for few nodes: the hardware brings
+// a cluster's blocks onto the chip together and has a barrier for them, so the
+// kernel graph needs one launch, which returns at once when the flag is clear:
+// 3 us, where a conditional graph node around the six kernels below costs every
+// step about 15 us.  (Two disks of 386 nodes, FP64: 46 to 32 us a step; 4
+// materials, 49907 nodes, FP32 split: 33 to 26.)  A rebuild is bound by the
+// latency of a thread's nodes one after the other: 8 blocks up to
+// kClusterNodes8 nodes (one node a thread), else 16 where the chip takes such
+// a cluster (49907 nodes: 94 us by 8).
+constexpr int kClusterThreads = 1024, kClusterNodes8 = 8 * kClusterThreads;
+__global__ void __launch_bounds__(kClusterThreads, 1) k_rebuild_cluster(DevPtrs d, KParams k) {
     __shared__ int sm[33];
     if (!__ldcg(d.rebuild)) return;
-    rebuild_lists<false, kClusterThreads>(d, k, blockIdx.x, kClusterBlocks, sm, [] {
+    rebuild_lists<false, kClusterThreads>(d, k, blockIdx.x, gridDim.x, sm, [] {
         __threadfence();
         asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
         __threadfence();
@@ -397,8 +398,26 @@ cudaError_t launch_rebuild(const DevPtrs &d, const KParams &k, cudaStream_t s) {
 }
 
 cudaError_t launch_rebuild_cluster(const DevPtrs &d, const KParams &k, cudaStream_t s) {
-    k_rebuild_cluster<<<kClusterBlocks, kClusterThreads, 0, s>>>(d, k);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg{};
+    cfg.blockDim = dim3(kClusterThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int blocks = 8;
+    if (k.N > kClusterNodes8 &&
+        cudaFuncSetAttribute(k_rebuild_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+        cfg.gridDim = dim3(16);
+        at.val.clusterDim.x = 16;
+        int fit = 0;
+        if (cudaOccupancyMaxActiveClusters(&fit, k_rebuild_cluster, &cfg) == cudaSuccess && fit > 0) blocks = 16;
+    }
+    cudaGetLastError();                     // a cluster of 16 that the chip does not take is no error
+    cfg.gridDim = dim3(blocks);
+    at.val.clusterDim.x = blocks;
+    return cudaLaunchKernelEx(&cfg, k_rebuild_cluster, d, k);
 }
 
 cudaError_t launch_force(const DevPtrs &d, const KParams &k, int vin, int update_v, cudaStream_t s, int phase) {

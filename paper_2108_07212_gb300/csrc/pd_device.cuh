@@ -1462,14 +1462,64 @@ __device__ __forceinline__ int candidate(const DevPtrs &d, const KParams &k, int
     return q < nc ? ldm<PERSIST>(&d.nbr[(size_t)q * k.N + ii]) : fresh_partner(d, k, ii, r0, q - nc);
 }
 
-// Contact forces of node ii, FP64 path: every LANES-th of its nc + nb candidates.
-template <bool PERSIST, int LANES>
-__device__ __forceinline__ void contacts64(const DevPtrs &d, const KParams &k, int ii, int lane, int vin, int gi, int nc,
-                                           int nb, int r0, int r1, double2 pi, double &Fsx, double &Fsy, double &Fnx,
+// The candidates of the nodes of a warp (several threads per node: thread 0 of
+// each gives node ii and its number n of candidates, the others n = 0), one per
+// thread, 32 at a time: pair(node, q, sx, sy, nx, ny) for candidate q of a node.
+// Each node's forces are then added in the order of its candidates, into its
+// thread 0.  A contact is a chain of divisions and square roots (FP64: about
+// 4 us on the 2-lane pipe, which a warp occupies as long for one pair as for
+// 32), and few nodes of a warp have any: with every thread working through its
+// share of its own node's, the warp took as many chains as the longest share.
+// (19681 nodes of a settled box, FP64, 2 threads per node: 50 to 40 us a step;
+// FP32 split 21 to 18.)
+// Every thread of the warp calls it.
+template <class T, class Pair>
+__device__ __forceinline__ void warp_contacts(int ii, int n, T &Fsx, T &Fsy, T &Fnx, T &Fny, Pair pair) {
+    constexpr unsigned kAll = 0xffffffffu;
+    if (!__any_sync(kAll, n > 0)) return;
+    const int lane = threadIdx.x & 31;
+    int start = n;                          // exclusive prefix of n
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(kAll, start, off);
+        if (lane >= off) start += y;
+    }
+    const int total = __shfl_sync(kAll, start, 31);
+    start -= n;
+    for (int p0 = 0; p0 < total; p0 += 32) {
+        // pair p belongs to the last thread whose prefix is not beyond p
+        const int p = p0 + lane;
+        int own = 0;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1)
+            if (__shfl_sync(kAll, start, own + off) <= p) own += off;
+        const int node = __shfl_sync(kAll, ii, own), q = p - __shfl_sync(kAll, start, own);
+        T a = 0, b = 0, c = 0, e = 0;
+        if (p < total) pair(node, q, a, b, c, e);
+        __syncwarp();
+        const int lo = max(start, p0), m = min(start + n, p0 + 32) - lo;
+        for (int t = 0; __any_sync(kAll, t < m); ++t) {
+            const int src = (lo + t) & 31;
+            const T va = __shfl_sync(kAll, a, src), vb = __shfl_sync(kAll, b, src);
+            const T vc = __shfl_sync(kAll, c, src), ve = __shfl_sync(kAll, e, src);
+            if (t < m) {
+                Fsx += va;
+                Fsy += vb;
+                Fnx += vc;
+                Fny += ve;
+            }
+        }
+    }
+}
+
+// Contact forces of node ii, FP64 path, by one thread: its nc + nb candidates.
+template <bool PERSIST>
+__device__ __forceinline__ void contacts64(const DevPtrs &d, const KParams &k, int ii, int vin, int gi, int nc, int nb,
+                                           int r0, int r1, double2 pi, double &Fsx, double &Fsy, double &Fnx,
                                            double &Fny) {
     const AggParams &A = d.agg[__ldg(&d.g_agg[gi])];
     const double2 vi = ldm<PERSIST>(&d.v[vin][ii]);
-    for (int q = lane; q < nc + nb; q += LANES) {
+    for (int q = 0; q < nc + nb; ++q) {
         const int j = candidate<PERSIST>(d, k, ii, nc, r0, q);
         double a, b, c, e;
         contact_pair64<PERSIST>(d, k, A, ii, j, vin, gi, r0, r1, pi, ldm<PERSIST>(&d.p[j]), vi, a, b, c, e);
@@ -1593,7 +1643,18 @@ __device__ __forceinline__ void force_node64(const DevPtrs &d, const KParams &k,
     const int nb = fresh_bonds(d, k, ii, any_lane<LANES>(w0 != 0u || (note & kNoteBroke) || (active && k.wpn > 1)));
     double Fsx = 0.0, Fsy = 0.0, Fnx = 0.0, Fny = 0.0;
     contact = nc + nb > 0;
-    if (INLINE && contact) contacts64<PERSIST, LANES>(d, k, ii, lane, vin, gi, nc, nb, r0, r1, pi, Fsx, Fsy, Fnx, Fny);
+    if constexpr (LANES == 1) {
+        if (INLINE && contact) contacts64<PERSIST>(d, k, ii, vin, gi, nc, nb, r0, r1, pi, Fsx, Fsy, Fnx, Fny);
+    } else {
+        warp_contacts(ii, lane == 0 ? nc + nb : 0, Fsx, Fsy, Fnx, Fny,
+                      [&](int x, int q, double &sx, double &sy, double &nx, double &ny) {
+                          const int g = __ldg(&d.grain[x]), b0 = __ldg(&d.row_ptr[x]), b1 = __ldg(&d.row_ptr[x + 1]);
+                          const int j = candidate<PERSIST>(d, k, x, ldm<PERSIST>(&d.nbr_cnt[x]), b0, q);
+                          contact_pair64<PERSIST>(d, k, d.agg[__ldg(&d.g_agg[g])], x, j, vin, g, b0, b1,
+                                                  ldm<PERSIST>(&d.p[x]), ldm<PERSIST>(&d.p[j]),
+                                                  ldm<PERSIST>(&d.v[vin][x]), sx, sy, nx, ny);
+                      });
+    }
     __syncwarp();
     out.bx = lane_sum<LANES>(f2d_bits(Fbx.hi) + f2d_bits(Fbx.lo));
     out.by = lane_sum<LANES>(f2d_bits(Fby.hi) + f2d_bits(Fby.lo));
@@ -1976,14 +2037,14 @@ __device__ __forceinline__ void contact_pair32(const DevPtrs &d, const KParams &
     }
 }
 
-// Contact forces of node ii, FP32 split: every LANES-th of its nc + nb candidates.
-template <bool PERSIST, int LANES>
-__device__ __forceinline__ void contacts32(const DevPtrs &d, const KParams &k, int ii, int lane, int vin, int gi, int nc,
-                                           int nb, int r0, int r1, float2 phi, float2 pli, float4 gq, float4 gc, float &Fsx,
+// Contact forces of node ii, FP32 split, by one thread: its nc + nb candidates.
+template <bool PERSIST>
+__device__ __forceinline__ void contacts32(const DevPtrs &d, const KParams &k, int ii, int vin, int gi, int nc, int nb,
+                                           int r0, int r1, float2 phi, float2 pli, float4 gq, float4 gc, float &Fsx,
                                            float &Fsy, float &Fnx, float &Fny) {
     const AggParams &A = d.agg[__ldg(&d.g_agg[gi])];
     const double2 vi64 = ldm<PERSIST>(&d.v[vin][ii]);      // start-of-step velocity
-    for (int q = lane; q < nc + nb; q += LANES) {
+    for (int q = 0; q < nc + nb; ++q) {
         const int j = candidate<PERSIST>(d, k, ii, nc, r0, q);
         float a, b, c, e;
         contact_pair32<PERSIST>(d, k, A, ii, j, vin, gi, r0, r1, phi, pli, gq, gc, ldm<PERSIST>(&cur_pq<PERSIST>(d)[j]),
@@ -2126,9 +2187,16 @@ __device__ __forceinline__ void force_node32(const DevPtrs &d, const KParams &k,
     float Fsx = 0.f, Fsy = 0.f, Fnx = 0.f, Fny = 0.f;
     const int nc = active ? ldm<PERSIST>(&d.nbr_cnt[ii]) : 0;
     const int nb = fresh_bonds(d, k, ii, any_lane<LANES>(w0 != 0u || (note & kNoteBroke) || (active && k.wpn > 1)));
-    if (nc + nb > 0)
-        contacts32<PERSIST, LANES>(d, k, ii, lane, vin, gi, nc, nb, r0, r1, phi, pli, gq, gc, Fsx, Fsy, Fnx, Fny);
-    __syncwarp();
+    warp_contacts(ii, lane == 0 ? nc + nb : 0, Fsx, Fsy, Fnx, Fny,
+                  [&](int x, int q, float &sx, float &sy, float &nx, float &ny) {
+                      const int g = __ldg(&d.grain[x]), b0 = __ldg(&d.row_ptr[x]), b1 = __ldg(&d.row_ptr[x + 1]);
+                      const int j = candidate<PERSIST>(d, k, x, ldm<PERSIST>(&d.nbr_cnt[x]), b0, q);
+                      const float4 qx = ldm<PERSIST>(&cur_pq<PERSIST>(d)[x]);
+                      contact_pair32<PERSIST>(d, k, d.agg[__ldg(&d.g_agg[g])], x, j, vin, g, b0, b1,
+                                              make_float2(qx.x, qx.y), make_float2(qx.z, qx.w), __ldg(&d.gq[g]),
+                                              __ldg(&d.gc[g]), ldm<PERSIST>(&cur_pq<PERSIST>(d)[j]),
+                                              ldm<PERSIST>(&d.v[vin][x]), sx, sy, nx, ny);
+                  });
     out.bx = lane_sum<LANES>(Fbx);
     out.by = lane_sum<LANES>(Fby);
     out.sx = lane_sum<LANES>(Fsx);
@@ -2264,7 +2332,7 @@ __device__ __forceinline__ void tile_nodes32(const DevPtrs &d, const KParams &k,
                 const int nb = fresh_bonds(d, k, i, w0 != 0u || (note & kNoteBroke));
                 contact = nc + nb > 0;
                 if (INLINE && contact)
-                    contacts32<PERSIST, 1>(d, k, i, 0, vin, gi, nc, nb, r0, r1, phi, pli, nd.gq, nd.gc, f.sx, f.sy, f.nx,
+                    contacts32<PERSIST>(d, k, i, vin, gi, nc, nb, r0, r1, phi, pli, nd.gq, nd.gc, f.sx, f.sy, f.nx,
                                            f.ny);
                 if (sur && judge) d.sur_fb[i] = make_float2(f.bx, f.by);   // full bond force for the judge
             }

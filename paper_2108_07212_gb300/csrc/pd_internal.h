@@ -271,9 +271,8 @@ cudaError_t launch_predict(const DevPtrs &d, const KParams &k, int vin, int adva
 // Rebuild of the contact candidate lists (kernels return at once when the
 // rebuild flag is clear).
 cudaError_t launch_rebuild(const DevPtrs &d, const KParams &k, cudaStream_t s);
-// The same in one launch of one cluster, for up to kClusterNodes nodes (a
-// cluster has 8192 threads, a rebuild by it takes about a node's latency for
-// every 8192).
+// The same in one launch of one cluster, for up to kClusterNodes nodes: 8192 or
+// 16384 threads, so a rebuild takes about a node's latency for every 16384.
 constexpr int kClusterNodes = 1 << 16;
 cudaError_t launch_rebuild_cluster(const DevPtrs &d, const KParams &k, cudaStream_t s);
 // Force phase; with the split variant, phase 1 launches only the lane sums

@@ -247,8 +247,10 @@ __global__ void __launch_bounds__(kBlock, FP32 ? 8 : 4) k_sums(DevPtrs d, KParam
     sums_node<FP32, false, LANES>(d, k, tid / LANES, tid % LANES, vin);
 }
 
+// (Registers for the wall terms: at 40 a thread their chain went through 1.3 to
+// 1.5 KB of spills; a step near the walls, 49907 nodes FP32 split: 12 us.)
 template <bool FP32>
-__global__ void __launch_bounds__(256, FP32 ? 6 : 2) k_epilogue(DevPtrs d, KParams k, int vin, int update_v) {
+__global__ void __launch_bounds__(256, FP32 ? 3 : 2) k_epilogue(DevPtrs d, KParams k, int vin, int update_v) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < k.N) epilogue_node<FP32, false>(d, k, i, vin, update_v);
 }
