@@ -1155,8 +1155,7 @@ int pd_bind_arena(pd_ctx *c, void *arena, size_t bytes) {
     std::vector<float> gq, gcf;
     std::vector<double> invm;
     std::vector<uint32_t> colx;
-    std::vector<uint4> stn;
-    std::vector<double> xs, xif;
+    std::vector<double> xs;
     PD_CUDA(k.fp32 ? pd::init_tiles32() : pd::init_tiles64());
     if (p.precision == PD_FP32_SPLIT) {
         // per grain: h, h^2 as a float-float pair, V as float
@@ -1202,68 +1201,24 @@ int pd_bind_arena(pd_ctx *c, void *arena, size_t bytes) {
         }
         PD_CUDA(cudaMemcpyAsync(d.gc, gcf.data(), 16 * G, cudaMemcpyHostToDevice, s));
     }
-    // lattice stencil of the bonds (FP64 path: with the forward bonds' reference lengths)
+    // lattice stencil of the bonds (FP64 path: with the forward bonds' reference
+    // lengths; the lattice indices pass through the lane sums' scratch)
     c->kp.stencil = has_stencil(c) ? 1 : 0;
     k.pair = 0;
     if (c->kp.stencil) {
-        stn.assign(N, make_uint4(pd::kStnIrregular, 0u, 0u, 0u));
-        if (!k.fp32) xif.assign(12 * N, 1.0);
-        size_t irregular = 0;
-        int reach = 0;             // farthest bond along the node numbering
-        for (size_t x = 0; x < N; ++x) {
-            uint32_t mask = 0;
-            int D[5] = {0, 0, 0, 0, 0};
-            bool seen[5] = {false, false, false, false, false}, ok = true;
-            int last = -1;
-            for (int b = c->row_ptr[x]; b < c->row_ptr[x + 1] && ok; ++b) {
-                const int j = c->col[b];
-                const int di = c->lat[2 * (size_t)j] - c->lat[2 * x], dj = c->lat[2 * (size_t)j + 1] - c->lat[2 * x + 1];
-                if (di < -2 || di > 2 || dj < -2 || dj > 2) { ok = false; break; }
-                const int oo = (dj + 2) * 5 + (di + 2), o = oo < 12 ? oo : oo - 1;
-                const long long base = (long long)j - (long long)x - di;
-                if (o <= last) ok = false;                      // CSR order must be the offset order
-                last = o;
-                if (!seen[dj + 2]) { seen[dj + 2] = true; D[dj + 2] = (int)std::max<long long>(-40000, std::min<long long>(40000, base)); }
-                else if (D[dj + 2] != base) ok = false;
-                if (dj == 0 && base != 0) ok = false;
-                if (D[dj + 2] < -32768 || D[dj + 2] > 32767) ok = false;
-                mask |= 1u << o;
-                reach = std::max(reach, std::abs(j - (int)x));
-            }
-            if (!ok) {
-                stn[x] = make_uint4(pd::kStnIrregular, 0u, 0u, (unsigned)c->row_ptr[x]);
-                ++irregular;
-                continue;
-            }
-            auto u16 = [](int v) { return (uint32_t)(uint16_t)(int16_t)v; };
-            stn[x] = make_uint4(mask, u16(D[0]) | (u16(D[1]) << 16), u16(D[3]) | (u16(D[4]) << 16),
-                                (unsigned)c->row_ptr[x]);
-            if (!k.fp32) {
-                int b = c->row_ptr[x];
-                for (int o = 0; o < 24; ++o) {
-                    if (!((mask >> o) & 1u)) continue;
-                    if (o >= 12) xif[(size_t)(o - 12) * N + x] = c->xi[b];
-                    ++b;
-                }
-            }
+        const int2 *lat = d.lat;
+        if (!lat) {
+            PD_CUDA(cudaMemcpyAsync(d.fsum, c->lat.data(), 8 * N, cudaMemcpyHostToDevice, s));
+            lat = static_cast<const int2 *>(d.fsum);
         }
-        c->stn_irregular = irregular;
-        k.pair = reach <= pd::kCarry ? 1 : 0;
-        // a node that forms a bond relies on the other node's list having it too
-        for (size_t x = 0; x < N && k.pair; ++x) {
-            const uint4 &a = stn[x];
-            if (a.x & pd::kStnIrregular) continue;
-            for (int o = 0; o < 24; ++o) {
-                if (!((a.x >> o) & 1u)) continue;
-                const int oo = o < 12 ? o : o + 1, dj = oo / 5 - 2, di = oo % 5 - 2;
-                const uint32_t w = dj < 0 ? a.y : a.z;
-                const int row = dj == 0 ? 0 : (int)(int16_t)(uint16_t)((dj == -2 || dj == 1) ? w & 0xFFFFu : w >> 16);
-                const uint32_t other = stn[x + di + row].x;
-                if (!(other & pd::kStnIrregular) && !((other >> (23 - o)) & 1u)) k.pair = 0;
-            }
-        }
-        PD_CUDA(cudaMemcpyAsync(d.stn, stn.data(), 16 * N, cudaMemcpyHostToDevice, s));
-        if (!k.fp32) PD_CUDA(cudaMemcpyAsync(d.xif, xif.data(), 8 * xif.size(), cudaMemcpyHostToDevice, s));
+        int *const found = reinterpret_cast<int *>(d.diag_out);
+        int got[pd::kStencilFound];
+        PD_CUDA(cudaMemsetAsync(found, 0, sizeof(got), s));
+        PD_CUDA(pd::launch_stencil(d, c->kp, lat, found, s));
+        PD_CUDA(cudaMemcpyAsync(got, found, sizeof(got), cudaMemcpyDeviceToHost, s));
+        PD_CUDA(cudaStreamSynchronize(s));
+        c->stn_irregular = (size_t)got[0];
+        k.pair = got[1] <= pd::kCarry && !got[2] ? 1 : 0;
     }
     // per grain 1 / (rho V): the update multiplies by it (an FP64 division per
     // node and component costs about nine FP64 operations on GB300)

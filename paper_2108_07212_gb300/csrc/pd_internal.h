@@ -275,6 +275,12 @@ cudaError_t launch_rebuild(const DevPtrs &d, const KParams &k, cudaStream_t s);
 // 16384 threads, so a rebuild takes about a node's latency for every 16384.
 constexpr int kClusterNodes = 1 << 16;
 cudaError_t launch_rebuild_cluster(const DevPtrs &d, const KParams &k, cudaStream_t s);
+// The nodes' bond stencils (DevPtrs::stn; FP64 path: xif) from the uploaded CSR
+// rows and the lattice indices.  found (kStencilFound zeroed ints): nodes whose
+// bonds do not follow the stencil, the farthest bond along the node numbering,
+// whether a stencil bond is missing from the other node's list.
+constexpr int kStencilFound = 3;
+cudaError_t launch_stencil(const DevPtrs &d, const KParams &k, const int2 *lat, int *found, cudaStream_t s);
 // Force phase; with the split variant, phase 1 launches only the lane sums
 // and phase 2 only the epilogue (0: both; the fused variant takes only 0).
 cudaError_t launch_force(const DevPtrs &d, const KParams &k, int vin, int update_v, cudaStream_t s, int phase = 0);
