@@ -87,7 +87,8 @@ __global__ void __launch_bounds__(kClusterThreads, 1) k_rebuild_cluster(DevPtrs 
     if (!__ldcg(d.rebuild)) return;
     rebuild_lists<false, kClusterThreads>(d, k, blockIdx.x, gridDim.x, sm, [] {
         __threadfence();
-        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        // (not the aligned form: a warp's threads come here from loops of different lengths)
+        asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
         __threadfence();
         return true;
     });
