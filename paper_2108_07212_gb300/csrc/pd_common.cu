@@ -96,8 +96,8 @@ __global__ void __launch_bounds__(kClusterThreads, 1) k_rebuild_cluster(DevPtrs 
 
 // The bond stencil of each node: a mask of the offsets its bonds have, the node
 // distance of each lattice row, and its first bond; marked irregular when its
-// CSR row is not in the order of the offsets, a row of the lattice has a gap or
-// a bond is longer.  (On the host, with a copy of 12 lengths a node, this took
+// CSR row is not in the order of the offsets, a row of the lattice has a gap
+// (kStnGap) or a bond is longer.  (On the host, with a copy of 12 lengths a node, this took
 // 80 of the 660 ms in which 521k nodes of the FP64 path are set up.)
 __global__ void __launch_bounds__(kBlock) k_stencil(DevPtrs d, KParams k, const int2 *__restrict__ lat, int *found) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(kBlock) k_stencil(DevPtrs d, KParams k, const 
     const int2 lx = lat[x];
     uint32_t mask = 0u;
     int D[5] = {0, 0, 0, 0, 0}, seen = 0, last = -1, reach = 0;
-    bool ok = true;
+    bool ok = true, rows = true;
     for (int b = r0; b < r1 && ok; ++b) {
         const int j = d.col[b];
         const int2 lj = lat[j];
@@ -123,17 +123,17 @@ __global__ void __launch_bounds__(kBlock) k_stencil(DevPtrs d, KParams k, const 
         for (int r = 0; r < 5; ++r) {
             if (r != dj + 2) continue;
             if (!((seen >> r) & 1)) D[r] = base;
-            else if (D[r] != base) ok = false;
+            else if (D[r] != base) rows = false;
         }
         seen |= 1 << (dj + 2);
-        if (dj == 0 && base != 0) ok = false;
-        if (base < -32768 || base > 32767) ok = false;
+        if (dj == 0 && base != 0) rows = false;
+        if (base < -32768 || base > 32767) rows = false;
         mask |= 1u << o;
         reach = max(reach, abs(j - x));
     }
     atomicMax(&found[1], reach);
-    if (!ok) {
-        mask = kStnIrregular;
+    if (!ok || !rows) {
+        mask = ok ? mask | kStnIrregular | kStnGap : kStnIrregular;
         D[0] = D[1] = D[3] = D[4] = 0;
         atomicAdd(&found[0], 1);
     }
@@ -152,12 +152,14 @@ __global__ void __launch_bounds__(kBlock) k_stencil(DevPtrs d, KParams k, const 
 __global__ void __launch_bounds__(kBlock) k_stencil_check(DevPtrs d, KParams k, int *found) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= k.N) return;
-    const uint4 st = d.stn[x];
-    if (st.x & kStnIrregular) return;
+    uint4 st = d.stn[x];
+    const bool gap = st.x & kStnGap;
+    if ((st.x & kStnIrregular) && !gap) return;
+    st.x &= kStnBits;
     for (int o = 0; o < 24; ++o) {
         if (!((st.x >> o) & 1u)) continue;
-        const uint32_t other = d.stn[x + stn_di(o) + stn_row(st, stn_dj(o))].x;
-        if (!(other & kStnIrregular) && !((other >> (23 - o)) & 1u)) found[2] = 1;
+        const uint32_t other = d.stn[x + stn_to(d, st, gap, x, o)].x;
+        if ((!(other & kStnIrregular) || (other & kStnGap)) && !((other >> (23 - o)) & 1u)) found[2] = 1;
     }
 }
 

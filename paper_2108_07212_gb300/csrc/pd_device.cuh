@@ -869,6 +869,18 @@ __device__ __forceinline__ int stn_row(const uint4 &st, int dj) {
     return dj == -2 ? (int)(short)(st.y & 0xFFFFu) : (dj == -1 ? (int)(short)(st.y >> 16)
            : (dj == 0 ? 0 : (dj == 1 ? (int)(short)(st.z & 0xFFFFu) : (int)(short)(st.z >> 16))));
 }
+// Where the bond at offset o of node ii (it has one there) leads, as a difference
+// of node numbers; gap: the node's columns tell (see kStnGap).  (Left to the
+// general bond loop, these nodes and the markers that their neighbours found
+// held a tile's other warps up: a box of 233k nodes with seven in a thousand at
+// the edge of a hole took 68 us a step in the FP32 split and 193 in FP64, now 30
+// and 118; as many nodes without holes, 25 and 88.  The tile functions come
+// twice, for warps with and without such a node: a test at each bond cost 4 %.)
+__device__ __forceinline__ int stn_to(const DevPtrs &d, const uint4 &st, bool gap, int ii, int o) {
+    int off = stn_di(o) + stn_row(st, stn_dj(o));
+    if (gap) off = __ldg(&d.col[(int)st.w + __popc(st.x & ((1u << o) - 1u))]) - ii;
+    return off;
+}
 // Bits of the stencil's intact bonds: the broken-bond bits w follow the order
 // of the node's bonds (the rank of the offset among the stencil bits), so each
 // set bit clears the stencil bit of that rank (a node seldom has a broken
@@ -1284,11 +1296,11 @@ __device__ __forceinline__ bool bond_force64(double2 pi, double2 pj, double xi, 
 
 // The forward half of node ii's stencil bonds (alive: the intact ones), FP64
 // path, into the thread's slots; returns the offsets whose force is there.
-// OWN: the block owns the node and records its broken bonds.
-template <bool PERSIST, int BLOCK, bool OWN>
+// own: the block owns the node and records its broken bonds.
+template <bool PERSIST, int BLOCK, bool GAP>
 __device__ __forceinline__ uint32_t tile_forward64(const DevPtrs &d, const KParams &k, int ii, uint32_t alive,
-                                                   const uint4 &st, double2 pi, ff cwVV, ff inv_eps, float s0f,
-                                                   double s0, float4 *slot, unsigned &note) {
+                                                   const uint4 &st, bool gap, double2 pi, ff cwVV, ff inv_eps,
+                                                   float s0f, double s0, float4 *slot, unsigned &note, bool own) {
     constexpr int S = PairTile<float4, BLOCK>::kStride;
     const int at = kCarry + (int)threadIdx.x;
     uint32_t formed = 0u;
@@ -1296,7 +1308,7 @@ __device__ __forceinline__ uint32_t tile_forward64(const DevPtrs &d, const KPara
 #pragma unroll 1
     for (int m0 = 0; m0 < kPairHalf; m0 += kBatch) {
         const uint32_t live = alive >> (kPairHalf + m0);
-        const auto to = [&](int m) { return ii + stn_di(kPairHalf + m0 + m) + stn_row(st, stn_dj(kPairHalf + m0 + m)); };
+        const auto to = [&](int m) { return ii + stn_to(d, st, GAP && gap, ii, kPairHalf + m0 + m); };
         double2 pb[kBatch];
         double xb[kBatch];
 #pragma unroll
@@ -1326,7 +1338,7 @@ __device__ __forceinline__ uint32_t tile_forward64(const DevPtrs &d, const KPara
         }
         if (broken) {
             note |= kNoteBroke;
-            for (uint32_t b = broken; OWN && b; b &= b - 1u)
+            for (uint32_t b = broken; own && b; b &= b - 1u)
                 atomicOr(&d.bits[(size_t)ii * k.wpn], stn_bit(st.x, kPairHalf + m0 + __ffs(b) - 1));
         }
 #pragma unroll
@@ -1341,10 +1353,10 @@ __device__ __forceinline__ uint32_t tile_forward64(const DevPtrs &d, const KPara
 
 // The bond sum of node ii, FP64 path: the backward half from the slots of the
 // nodes that formed it, then the node's own forward slots.
-template <bool PERSIST, int BLOCK>
+template <bool PERSIST, int BLOCK, bool GAP>
 __device__ __forceinline__ void tile_sum64(const DevPtrs &d, const KParams &k, int ii, uint32_t alive, uint32_t formed,
-                                           const uint4 &st, double2 pi, ff cwVV, ff inv_eps, float s0f, double s0,
-                                           const float4 *slot, ff &Fx, ff &Fy, unsigned &note) {
+                                           const uint4 &st, bool gap, double2 pi, ff cwVV, ff inv_eps, float s0f,
+                                           double s0, const float4 *slot, ff &Fx, ff &Fy, unsigned &note) {
     constexpr int S = PairTile<float4, BLOCK>::kStride;
     const int at = kCarry + (int)threadIdx.x;
     const uint32_t back = alive & ((1u << kPairHalf) - 1u);
@@ -1352,7 +1364,7 @@ __device__ __forceinline__ void tile_sum64(const DevPtrs &d, const KParams &k, i
 #pragma unroll
     for (int o = 0; o < kPairHalf; ++o) {
         const bool in = (back >> o) & 1u;
-        const float4 v = slot[(kPairHalf - 1 - o) * S + (in ? at + stn_di(o) + stn_row(st, stn_dj(o)) : at)];
+        const float4 v = slot[(kPairHalf - 1 - o) * S + at + (in ? stn_to(d, st, GAP && gap, ii, o) : 0)];
         const bool ok = in && v.x == v.x;
         if (ok) got |= 1u << o;
         Fx = ff_add(Fx, ok ? ff{-v.x, -v.y} : ff{0.f, 0.f});
@@ -1363,7 +1375,7 @@ __device__ __forceinline__ void tile_sum64(const DevPtrs &d, const KParams &k, i
         Fx = Fy = {0.f, 0.f};
         for (uint32_t m = back; m; m &= m - 1u) {
             const int o = __ffs(m) - 1;
-            const int off = stn_di(o) + stn_row(st, stn_dj(o));
+            const int off = stn_to(d, st, GAP && gap, ii, o);
             const float4 v = slot[(kPairHalf - 1 - o) * S + at + off];
             unsigned mark = __float_as_uint(v.x);
             if (mark == kPairNone) {
@@ -1555,8 +1567,10 @@ __device__ __forceinline__ void force_node64(const DevPtrs &d, const KParams &k,
     unsigned note = 0u;
     int r0, r1;
     if constexpr (LANES == 1) {
-        const uint4 st = (k.stencil && active) ? __ldg(&d.stn[ii]) : make_uint4(kStnIrregular, 0u, 0u, 0u);
-        csr = (st.x & kStnIrregular) != 0u || !k.pair;
+        uint4 st = (k.stencil && active) ? __ldg(&d.stn[ii]) : make_uint4(kStnIrregular, 0u, 0u, 0u);
+        const bool gap = st.x & kStnGap;
+        csr = ((st.x & kStnIrregular) && !gap) || !k.pair;
+        st.x &= kStnBits;
         r0 = (int)st.w;
         r1 = r0 + __popc(st.x);
         if (csr) {
@@ -1565,15 +1579,18 @@ __device__ __forceinline__ void force_node64(const DevPtrs &d, const KParams &k,
         }
         if (k.pair) {
             const uint32_t alive = csr ? 0u : stn_alive(st.x, w0);
-            if (warm) {
-                tile_forward64<PERSIST, BLOCK, false>(d, k, ii, alive, st, pi, cwVV, inv_eps, s0f, s0, slot, note);
-                return;
-            }
+            const bool gaps = __any_sync(0xffffffffu, gap);
             const uint32_t formed =
-                tile_forward64<PERSIST, BLOCK, true>(d, k, ii, alive, st, pi, cwVV, inv_eps, s0f, s0, slot, note);
+                gaps ? tile_forward64<PERSIST, BLOCK, true>(d, k, ii, alive, st, gap, pi, cwVV, inv_eps, s0f, s0, slot,
+                                                            note, !warm)
+                     : tile_forward64<PERSIST, BLOCK, false>(d, k, ii, alive, st, gap, pi, cwVV, inv_eps, s0f, s0,
+                                                             slot, note, !warm);
+            if (warm) return;
             __syncthreads();
-            tile_sum64<PERSIST, BLOCK>(d, k, ii, alive, formed, st, pi, cwVV, inv_eps, s0f, s0, slot, Fbx, Fby,
-                                       note);
+            if (gaps) tile_sum64<PERSIST, BLOCK, true>(d, k, ii, alive, formed, st, gap, pi, cwVV, inv_eps, s0f, s0,
+                                                       slot, Fbx, Fby, note);
+            else tile_sum64<PERSIST, BLOCK, false>(d, k, ii, alive, formed, st, gap, pi, cwVV, inv_eps, s0f, s0, slot,
+                                                   Fbx, Fby, note);
         }
     } else {
         r0 = active ? __ldg(&d.row_ptr[ii]) : 0;
@@ -1820,7 +1837,8 @@ struct Tile32 {
 // What the bond loop takes from a node's grain and list.
 struct BondNode32 {
     float4 qi, gq, gc;      // position; (h, h^2 hi, h^2 lo, V); (c_w, s0, eps, rho)
-    uint4 st;               // stencil record
+    uint4 st;               // stencil record (its 24 bits)
+    bool gap;               // of a node with kStnGap
 };
 
 // The forward half of a node's stencil bonds: their forces into the thread's
@@ -1829,14 +1847,15 @@ struct BondNode32 {
 // offsets: a slot of an absent bond holds what the arithmetic makes of the
 // wrong position (nobody reads it: bonds are in both nodes' lists), and one
 // comparison over the largest excess of a stretch tells whether the general
-// pass after it is needed.  OWN: the block owns the node (broken-bond word bw)
+// pass after it is needed.  own: the block owns the node (broken-bond word bw)
 // and records its broken bonds.
-template <int BLOCK, bool OWN, bool MICRO>
-__device__ __forceinline__ void tile_forward32(const KParams &k, uint32_t alive, const BondNode32 &nd, const float4 *win,
-                                               float2 *mine, uint32_t *bw, float &Fx, float &Fy, unsigned &note) {
+template <int BLOCK, bool GAP>
+__device__ __forceinline__ void tile_forward32(const DevPtrs &d, const KParams &k, int ii, uint32_t alive,
+                                               const BondNode32 &nd, const float4 *win, float2 *mine, uint32_t *bw, float &Fx, float &Fy, unsigned &note, bool own,
+                                               bool micro) {
     constexpr int S = PairTile<float2, BLOCK>::kStride;
     const float2 phi = make_float2(nd.qi.x, nd.qi.y), pli = make_float2(nd.qi.z, nd.qi.w);
-    const float VV = nd.gq.w * nd.gq.w, inv_eps = MICRO ? 1.0f / nd.gc.z : 0.f;
+    const float VV = nd.gq.w * nd.gq.w, inv_eps = micro ? 1.0f / nd.gc.z : 0.f;
     const float s0_lo = nd.gc.y * (1.0f - k.guard);
     const float4 *const row[3] = {win, win + stn_row(nd.st, 1), win + stn_row(nd.st, 2)};
     float excess = 0.f;
@@ -1845,17 +1864,25 @@ __device__ __forceinline__ void tile_forward32(const KParams &k, uint32_t alive,
 #pragma unroll
     for (int m0 = 0; m0 < kPairHalf; m0 += kBatch) {
         float4 qb[kBatch];
+        if (!GAP || !nd.gap) {
 #pragma unroll
-        for (int m = 0; m < kBatch; ++m) {
-            const int o = kPairHalf + m0 + m;
-            qb[m] = row[stn_dj(o)][stn_di(o)];
+            for (int m = 0; m < kBatch; ++m) {
+                const int o = kPairHalf + m0 + m;
+                qb[m] = row[stn_dj(o)][stn_di(o)];
+            }
+        } else {
+#pragma unroll
+            for (int m = 0; m < kBatch; ++m) {
+                const int o = kPairHalf + m0 + m;
+                qb[m] = win[(nd.st.x >> o) & 1u ? stn_to(d, nd.st, true, ii, o) : 0];
+            }
         }
 #pragma unroll
         for (int m = 0; m < kBatch; ++m) {
             const int o = kPairHalf + m0 + m, di = stn_di(o), dj = stn_dj(o), n = di * di + dj * dj;
             BondGeom32 g;
             bond_geom32(qb[m], phi, pli, (float)n, stn_sqrt_n(n), nd.gq, g, (n & (n - 1)) == 0);
-            const float2 f = bond_force32(g, nd.gc.x, inv_eps, VV, MICRO);
+            const float2 f = bond_force32(g, nd.gc.x, inv_eps, VV, micro);
             mine[(m0 + m) * S] = f;
             if ((alive >> o) & 1u) {
                 excess = fmaxf(excess, bond_excess32(g, s0_lo));      // (a NaN stretch counts as intact)
@@ -1875,7 +1902,7 @@ __device__ __forceinline__ void tile_forward32(const KParams &k, uint32_t alive,
             const int o = __ffs(m) - 1, di = stn_di(o), dj = stn_dj(o), n = di * di + dj * dj;
             float2 *const at = &mine[(o - kPairHalf) * S];
             BondGeom32 g;
-            const int r = bond_classify32(win[di + stn_row(nd.st, dj)], phi, pli, (float)n, stn_sqrt_n(n), nd.gq, s0_lo,
+            const int r = bond_classify32(win[stn_to(d, nd.st, GAP && nd.gap, ii, o)], phi, pli, (float)n, stn_sqrt_n(n), nd.gq, s0_lo,
                                           nd.gc.y * (1.0f + k.guard), g);
             if (r == 0) {
                 Fx = __fadd_rn(Fx, at->x);
@@ -1885,7 +1912,7 @@ __device__ __forceinline__ void tile_forward32(const KParams &k, uint32_t alive,
             at->x = __uint_as_float(r == 1 ? kPairBroken : kPairGuard);
             if (r == 2) {
                 note |= kNoteGuard;
-            } else if (OWN) {
+            } else if (own) {
                 atomicOr(bw, stn_bit(nd.st.x, o));
                 note |= kNoteBroke;
             }
@@ -1895,18 +1922,31 @@ __device__ __forceinline__ void tile_forward32(const KParams &k, uint32_t alive,
 
 // The backward half of node ii's bonds, from the slots of the nodes that formed
 // them: its sum in (Fx, Fy).
-template <bool PERSIST, int BLOCK>
+template <bool PERSIST, int BLOCK, bool GAP>
 __device__ __forceinline__ void tile_backward32(const DevPtrs &d, const KParams &k, int ii, uint32_t alive,
                                                 const BondNode32 &nd, const float2 *mine, float &Fx, float &Fy,
                                                 unsigned &note) {
     constexpr int S = PairTile<float2, BLOCK>::kStride;
     const float2 *const row[3] = {mine + stn_row(nd.st, -2), mine + stn_row(nd.st, -1), mine};
     Fx = Fy = 0.f;
+    if (!GAP || !nd.gap) {
 #pragma unroll
-    for (int o = 0; o < kPairHalf; ++o) {
-        // (a row without bonds has offset 0: some slot of the tile)
-        const float2 v = row[stn_dj(o) + 2][(kPairHalf - 1 - o) * S + stn_di(o)];
-        if ((alive >> o) & 1u) {
+        for (int o = 0; o < kPairHalf; ++o) {
+            // (a row without bonds has offset 0: some slot of the tile)
+            const float2 v = row[stn_dj(o) + 2][(kPairHalf - 1 - o) * S + stn_di(o)];
+            if ((alive >> o) & 1u) {
+                Fx = __fsub_rn(Fx, v.x);
+                Fy = __fsub_rn(Fy, v.y);
+            }
+        }
+    } else {
+        int off[kPairHalf];
+#pragma unroll
+        for (int o = 0; o < kPairHalf; ++o) off[o] = (alive >> o) & 1u ? stn_to(d, nd.st, true, ii, o) : 0;
+#pragma unroll
+        for (int o = 0; o < kPairHalf; ++o) {
+            if (!((alive >> o) & 1u)) continue;
+            const float2 v = mine[(kPairHalf - 1 - o) * S + off[o]];
             Fx = __fsub_rn(Fx, v.x);
             Fy = __fsub_rn(Fy, v.y);
         }
@@ -1916,7 +1956,7 @@ __device__ __forceinline__ void tile_backward32(const DevPtrs &d, const KParams 
         const float2 phi = make_float2(nd.qi.x, nd.qi.y), pli = make_float2(nd.qi.z, nd.qi.w);
         Fx = Fy = 0.f;
         for (uint32_t m = alive & ((1u << kPairHalf) - 1u); m; m &= m - 1u) {
-            const int o = __ffs(m) - 1, di = stn_di(o), dj = stn_dj(o), off = di + stn_row(nd.st, dj);
+            const int o = __ffs(m) - 1, di = stn_di(o), dj = stn_dj(o), off = stn_to(d, nd.st, GAP && nd.gap, ii, o);
             const float2 v = mine[(kPairHalf - 1 - o) * S + off];
             unsigned mark = __float_as_uint(v.x);
             if (mark == kPairNone) {
@@ -2274,7 +2314,10 @@ __device__ __forceinline__ void tile_nodes32(const DevPtrs &d, const KParams &k,
         }
         nd.gq = __ldg(&d.gq[gi]);
         nd.gc = __ldg(&d.gc[gi]);
-        const bool stencil = !(nd.st.x & kStnIrregular);
+        nd.gap = nd.st.x & kStnGap;
+        const bool gaps = __any_sync(0xffffffffu, nd.gap);
+        const bool stencil = !(nd.st.x & kStnIrregular) || nd.gap;
+        nd.st.x &= kStnBits;
         // learned modal surrogate: between judge steps an active grain skips the
         // bond loop; the epilogue adds its surrogate bond force instead
         bool sur = false, judge = false;
@@ -2290,13 +2333,9 @@ __device__ __forceinline__ void tile_nodes32(const DevPtrs &d, const KParams &k,
         uint32_t *bw = &d.bits[(size_t)(active ? i : 0) * k.wpn];
         float fx = 0.f, fy = 0.f;
         if (bonds && stencil) {
-            if (k.micro) {
-                if (warm) tile_forward32<BLOCK, false, true>(k, alive, nd, win, mine, bw, fx, fy, note);
-                else tile_forward32<BLOCK, true, true>(k, alive, nd, win, mine, bw, fx, fy, note);
-            } else {
-                if (warm) tile_forward32<BLOCK, false, false>(k, alive, nd, win, mine, bw, fx, fy, note);
-                else tile_forward32<BLOCK, true, false>(k, alive, nd, win, mine, bw, fx, fy, note);
-            }
+            if (gaps) tile_forward32<BLOCK, true>(d, k, i, alive, nd, win, mine, bw, fx, fy, note, !warm, k.micro != 0);
+            else if (k.micro) tile_forward32<BLOCK, false>(d, k, i, alive, nd, win, mine, bw, fx, fy, note, !warm, true);
+            else tile_forward32<BLOCK, false>(d, k, i, alive, nd, win, mine, bw, fx, fy, note, !warm, false);
         } else {
 #pragma unroll
             for (int q = 0; q < kPairHalf; ++q)
@@ -2311,7 +2350,8 @@ __device__ __forceinline__ void tile_nodes32(const DevPtrs &d, const KParams &k,
             Sums32 f{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             bool contact = false;
             if (active) {
-                tile_backward32<PERSIST, BLOCK>(d, k, i, alive, nd, mine, f.bx, f.by, note);
+                if (gaps) tile_backward32<PERSIST, BLOCK, true>(d, k, i, alive, nd, mine, f.bx, f.by, note);
+                else tile_backward32<PERSIST, BLOCK, false>(d, k, i, alive, nd, mine, f.bx, f.by, note);
                 f.bx = __fadd_rn(f.bx, fx);
                 f.by = __fadd_rn(f.by, fy);
                 const float2 phi = make_float2(nd.qi.x, nd.qi.y), pli = make_float2(nd.qi.z, nd.qi.w);

@@ -32,10 +32,12 @@ constexpr uint32_t kColMask = (1u << kColBits) - 1u;
 // neighbour rows are contiguous runs near it the neighbour at offset o is node
 // x + di + D[dj], and the CSR order of its bonds is the order of o.  Per node:
 //   x: bit o = bond at offset o exists (reference list), bit 31 = irregular
-//      (a row with a gap near the node: its bonds are read from the CSR columns)
+//      (its bonds are read from the CSR columns); bit 30, with bit 31: only
+//      because a row near the node has a gap (a hole's edge), bits 0..23 and the
+//      order of the columns hold all the same
 //   y: D[-2] | D[-1] << 16, z: D[1] | D[2] << 16 (16-bit two's complement)
 //   w: first bond of the node's CSR row
-constexpr uint32_t kStnIrregular = 0x80000000u;
+constexpr uint32_t kStnIrregular = 0x80000000u, kStnGap = 0x40000000u, kStnBits = 0x00FFFFFFu;
 // Nodes before a run of nodes whose bond forces it can use (see PairTile): two
 // lattice rows of a grain of up to 32 lattice spacings a radius (the finest
 // workloads have 23).
