@@ -35,10 +35,14 @@ sys.path.insert(0, ROOT)
 METRIC = "node-steps/s and bond evals/s vs plain FP64 GPU path at stated error; % HBM peak"
 # algorithmic bytes of the plain FP64 force phase: per node the FP64 position p,
 # v and a read (48 B), v and a written (32 B), volume (8 B), grain, row pointer,
-# broken-bond word and contact-list length (16 B), hash-grid cell (8 B); per
-# directed bond the column and the FP64 reference length (12 B)
+# broken-bond word and contact-list length (16 B), grid cell (8 B); per
+# directed bond the column and the FP64 reference length (12 B).  With one
+# thread per node each bond is evaluated once: the stencil record for the row
+# pointer (12 B more) and the 12 forward reference lengths (96 B) per node,
+# and no per-bond stream
 BYTES_PER_NODE_FP64 = 112
 BYTES_PER_BOND_FP64 = 12
+BYTES_PER_NODE_FP64_TILE = 220
 # the FP64 displacement update: X, u, v and a read (64 B), u and p written (32 B)
 BYTES_UPDATE_FP64 = 96
 # GB300 FP64 pipe: 2 lanes per SM per cycle on 152 SMs; a warp instruction on
@@ -49,7 +53,7 @@ N_SM = 152
 # here: horizon 3 h): the lane sums read the float-float position pq (16 B), the stencil record
 # (16 B), grain, broken-bond word and contact-list length (12 B) and write the force total (8 B);
 # the epilogue reads the force total (8 B), the FP64 v (16 B), the FP32 a (8 B), grain (4 B) and
-# the hash-grid cell of the wall test (8 B) and writes v and a (24 B).  120 B per node and no
+# the grid cell of the wall test (8 B) and writes v and a (24 B).  120 B per node and no
 # per-bond stream (nodes whose lattice row has a gap read CSR columns instead, 4 B per bond, not
 # counted).  The fused force phase (one kernel, the force total stays on chip) reads the same
 # inputs once: 100 B per node.
@@ -71,6 +75,16 @@ def fp32_bytes_per_node(mode: int, whole: bool) -> int:
     if not whole:
         return force
     return force + (BYTES_UPDATE_FP32_FUSED if mode & 1 else BYTES_UPDATE_FP32)
+
+
+def fp64_bytes(path: dict, whole: bool):
+    """Algorithmic bytes per node and per directed bond of the FP64 force phase
+    of a step path, or of its whole step."""
+    per_node, per_bond = ((BYTES_PER_NODE_FP64_TILE, 0) if path.get("lanes") == 1 else
+                          (BYTES_PER_NODE_FP64, BYTES_PER_BOND_FP64))
+    return per_node + (BYTES_UPDATE_FP64 if whole else 0), per_bond
+
+
 B_STATUS_REBUILDS = 5    # status slot counting the contact candidate-list rebuilds
 
 
@@ -512,15 +526,15 @@ def _roof_fp64(sim, f_ms, path, workload, clk, hbm):
     table = FP64_INST.get(workload, {}) if kernel_digest() == FP64_INST_DIGEST else {}
     inst = sum(table[n] for n in names) if all(n in table for n in names) else None
     # the persistent kernel is the whole step: the displacement update's bytes too
-    per_node = BYTES_PER_NODE_FP64 + (BYTES_UPDATE_FP64 if m & 1 else 0)
-    nbytes = per_node * sim.N + BYTES_PER_BOND_FP64 * sim.n_bonds
+    per_node, per_bond = fp64_bytes(path, bool(m & 1))
+    nbytes = per_node * sim.N + per_bond * sim.n_bonds
     hbm_a = nbytes / (f_ms / 1e3) / 1e9
     achieved = None if inst is None else 32.0 * inst / (f_ms / 1e3) / 1e12
     return {"bound": "alu", "kernel": _force_kernels(m, False), "achieved": achieved, "peak": peak,
             "unit": "T FP64 lane-ops/s", "frac": None if achieved is None else achieved / peak,
             "traffic": force_phase_traffic(path, False, workload),
             "hbm": {"achieved": hbm_a, "peak": hbm, "unit": "GB/s", "frac": hbm_a / hbm,
-                    "note": f"{per_node} B/node + {BYTES_PER_BOND_FP64} B/bond (of measured)"},
+                    "note": f"{per_node} B/node + {per_bond} B/bond (of measured)"},
             "note": f"peak = {N_SM} SMs x {FP64_LANES_PER_SM_CYCLE} FP64 lanes/cycle x {mhz:.0f} MHz (derived); "
                     + ("achieved = 32 x %d FP64-pipe warp instructions (ncu) / mean event time %.1f us"
                        % (inst, f_ms * 1e3) if inst is not None else
@@ -916,7 +930,7 @@ def run_ours(args):
                         + ("; the workload is too small to load 152 SMs, so the phase is latency-bound"
                            if sim.N < 100000 else "")}
     if prec == B.PD_FP64:
-        step_per_node, step_per_bond = BYTES_UPDATE_FP64 + BYTES_PER_NODE_FP64, BYTES_PER_BOND_FP64
+        step_per_node, step_per_bond = fp64_bytes(tuned[key], True)
     else:
         step_per_node, step_per_bond = fp32_bytes_per_node(tuned[key]["mode"], True), BYTES_PER_BOND_FP32
     step_bytes = step_per_node * sim.N + step_per_bond * sim.n_bonds
