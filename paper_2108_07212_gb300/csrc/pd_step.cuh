@@ -249,8 +249,12 @@ __global__ void __launch_bounds__(kBlock, FP32 ? 8 : 4) k_sums(DevPtrs d, KParam
 
 // (Registers for the wall terms: at 40 a thread their chain went through 1.3 to
 // 1.5 KB of spills; a step near the walls, 49907 nodes FP32 split: 12 us.)
-template <bool FP32>
-__global__ void __launch_bounds__(256, FP32 ? 3 : 2) k_epilogue(DevPtrs d, KParams k, int vin, int update_v) {
+// (kManyNodes: with ten waves of blocks the pass is bound by memory, and the warps
+// that 40 registers allow are worth more: surrogate step of 2.03M nodes, 232 us
+// with 80, 207 with 40.)
+constexpr int kManyNodes = 1 << 20;
+template <bool FP32, int PERSM = FP32 ? 3 : 2>
+__global__ void __launch_bounds__(256, PERSM) k_epilogue(DevPtrs d, KParams k, int vin, int update_v) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < k.N) epilogue_node<FP32, false>(d, k, i, vin, update_v);
 }
@@ -283,7 +287,9 @@ cudaError_t launch_force_impl(const DevPtrs &d, const KParams &k, int vin, int u
                 if constexpr (FP32) k_sums<FP32, 1><<<grid, kBlock, 0, s>>>(d, k, vin);
             } else if (const cudaError_t e = launch_force_run<FP32>(d, k, vin, 0, s, 0)) return e;
         }
-        if (phase != 1) k_epilogue<FP32><<<(unsigned)((k.N + 255) / 256), 256, 0, s>>>(d, k, vin, update_v);
+        const unsigned nb = (unsigned)((k.N + 255) / 256);
+        if (phase != 1 && FP32 && k.sur && k.N > kManyNodes) k_epilogue<FP32, 6><<<nb, 256, 0, s>>>(d, k, vin, update_v);
+        else if (phase != 1) k_epilogue<FP32><<<nb, 256, 0, s>>>(d, k, vin, update_v);
         return cudaGetLastError();
     }
     if (phase != 0) return cudaErrorInvalidValue;
