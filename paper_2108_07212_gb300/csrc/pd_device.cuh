@@ -1597,8 +1597,15 @@ __device__ __forceinline__ void force_node64(const DevPtrs &d, const KParams &k,
         r1 = active ? __ldg(&d.row_ptr[ii + 1]) : 0;
     }
     // six bonds loaded, three evaluated at a time: a full row of 24 is 4, 2, 1
-    // rounds of loads and 8, 4, 2, 1 of evaluations with 1, 2, 4, 8 threads
+    // rounds of loads and 8, 4, 2, 1 of evaluations with 1, 2, 4, 8 threads.
+    // (One copy of the evaluation for both halves of a round, which moves the
+    // second half's operands down: a bond is some 200 instructions, and a step
+    // that starts with cold caches waits for its code more than for data.  Two
+    // copies, 4 threads per node: 49.7 us a step of a settled box of 19681 nodes
+    // with L2 flushed before it, one: 45.0; 48 bonds a node, 87340 nodes: 104.7
+    // and 98.2.)
     constexpr int kLoad = 6, kEval = 3;
+    static_assert(kLoad == 2 * kEval, "a round is two evaluations");
     for (int b0 = r0 + lane; b0 < r1 && csr; b0 += kLoad * LANES) {
         int jb[kLoad];
         uint32_t wb[kLoad];
@@ -1617,40 +1624,42 @@ __device__ __forceinline__ void force_node64(const DevPtrs &d, const KParams &k,
             pb[m] = ldm<PERSIST>(&d.p[jb[m] < 0 ? ii : jb[m]]);
             live |= (jb[m] >= 0 && !((wb[m] >> ((b0 + m * LANES - r0) & 31)) & 1u)) ? 1u << m : 0u;
         }
-#pragma unroll
-        for (int m0 = 0; m0 < kLoad; m0 += kEval) {
-            if (!(live >> m0)) break;
+#pragma unroll 1
+        for (int bm = b0; live; bm += kEval * LANES, live >>= kEval) {
             ff c[kEval], fx[kEval], fy[kEval];
             uint32_t broken = 0u, near = 0u;
 #pragma unroll
             for (int m = 0; m < kEval; ++m) c[m] = cwVV;
             if (k.micro) {
 #pragma unroll
-                for (int m = 0; m < kEval; ++m) c[m] = bond_conic64(cwVV, xb[m0 + m], inv_eps);
+                for (int m = 0; m < kEval; ++m) c[m] = bond_conic64(cwVV, xb[m], inv_eps);
             }
 #pragma unroll
             for (int m = 0; m < kEval; ++m) {
                 bool b, n;
-                bond_terms64(pi, pb[m0 + m], xb[m0 + m], c[m], s0f, fx[m], fy[m], b, n);
-                broken |= b ? 1u << (m0 + m) : 0u;
-                near |= n ? 1u << (m0 + m) : 0u;
+                bond_terms64(pi, pb[m], xb[m], c[m], s0f, fx[m], fy[m], b, n);
+                broken |= b ? 1u << m : 0u;
+                near |= n ? 1u << m : 0u;
             }
-            broken &= live;
-            for (near &= live; near; near &= near - 1u) {
-                const int m = __ffs(near) - 1, b = b0 + m * LANES;
+            const uint32_t now = live & ((1u << kEval) - 1u);
+            broken &= now;
+            for (near &= now; near; near &= near - 1u) {
+                const int m = __ffs(near) - 1, b = bm + m * LANES;
                 const bool brk = bond_breaks64(pi, ldm<PERSIST>(&d.p[__ldg(&d.col[b])]), __ldg(&d.xi[b]), s0);
                 broken = brk ? broken | (1u << m) : broken & ~(1u << m);
             }
             for (uint32_t m = broken; m; m &= m - 1u) {
-                const int kk = b0 + (__ffs(m) - 1) * LANES - r0;
+                const int kk = bm + (__ffs(m) - 1) * LANES - r0;
                 atomicOr(&bw[kk >> 5], 1u << (kk & 31));
                 note |= kNoteBroke;
             }
 #pragma unroll
             for (int m = 0; m < kEval; ++m) {
-                const bool ok = ((live & ~broken) >> (m0 + m)) & 1u;
+                const bool ok = ((now & ~broken) >> m) & 1u;
                 Fbx = ff_add(Fbx, ok ? fx[m] : ff{0.f, 0.f});
                 Fby = ff_add(Fby, ok ? fy[m] : ff{0.f, 0.f});
+                pb[m] = pb[kEval + m];
+                xb[m] = xb[kEval + m];
             }
         }
     }
