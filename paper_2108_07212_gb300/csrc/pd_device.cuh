@@ -1478,53 +1478,39 @@ __device__ __forceinline__ int candidate(const DevPtrs &d, const KParams &k, int
     return q < nc ? ldm<PERSIST>(&d.nbr[(size_t)q * k.N + ii]) : fresh_partner(d, k, ii, r0, q - nc);
 }
 
-// The candidates of the nodes of a warp (several threads per node: thread 0 of
-// each gives node ii and its number n of candidates, the others n = 0), one per
-// thread, 32 at a time: pair(node, q, sx, sy, nx, ny) for candidate q of a node.
-// Each node's forces are then added in the order of its candidates, into its
-// thread 0.  A contact is a chain of divisions and square roots (FP64: about
-// 4 us on the 2-lane pipe, which a warp occupies as long for one pair as for
-// 32), and few nodes of a warp have any: with every thread working through its
-// share of its own node's, the warp took as many chains as the longest share.
-// (19681 nodes of a settled box, FP64, 2 threads per node: 50 to 40 us a step;
-// FP32 split 21 to 18.)
-// Every thread of the warp calls it.
-template <class T, class Pair>
-__device__ __forceinline__ void warp_contacts(int ii, int n, T &Fsx, T &Fsy, T &Fnx, T &Fny, Pair pair) {
-    constexpr unsigned kAll = 0xffffffffu;
-    if (!__any_sync(kAll, n > 0)) return;
-    const int lane = threadIdx.x & 31;
-    int start = n;                          // exclusive prefix of n
+// Adds the v of a group of LANES threads, thread by thread (the first n of them),
+// to the running sum `acc` of all its threads.
+template <int LANES, class T>
+__device__ __forceinline__ T add_in_order(T acc, T v, int n) {
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const int y = __shfl_up_sync(kAll, start, off);
-        if (lane >= off) start += y;
+    for (int l = 0; l < LANES; ++l) {
+        const T w = __shfl_sync(0xffffffffu, v, l, LANES);
+        if (l < n) acc += w;
     }
-    const int total = __shfl_sync(kAll, start, 31);
-    start -= n;
-    for (int p0 = 0; p0 < total; p0 += 32) {
-        // pair p belongs to the last thread whose prefix is not beyond p
-        const int p = p0 + lane;
-        int own = 0;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1)
-            if (__shfl_sync(kAll, start, own + off) <= p) own += off;
-        const int node = __shfl_sync(kAll, ii, own), q = p - __shfl_sync(kAll, start, own);
+    return acc;
+}
+
+// The n candidates of a node by its LANES threads, a candidate each:
+// pair(q, sx, sy, nx, ny) for candidate q; the forces are then added in the
+// order of the candidates, so the sums are those of one thread working through
+// them, in every thread of the node.  A contact is a chain of divisions and
+// square roots (FP64: about 4 us on the 2-lane pipe).  (Dealt to all threads of
+// the warp instead, every candidate began with a chain of loads for what its
+// node's threads hold: 19681 nodes settled, FP64, 4 threads per node, 27.7
+// us a step against 26.7, 8 threads 32.5 against 30.7, but 2 threads 26.1
+// against 30.2; 80171 nodes thrown at each other 62.8 against 57.9 with 4
+// threads, 63.0 against 60.5 with 2, FP32 split 28.7 against 26.6.)
+// Every thread of the warp calls it.
+template <int LANES, class T, class Pair>
+__device__ __forceinline__ void group_contacts(int lane, int n, T &Fsx, T &Fsy, T &Fnx, T &Fny, Pair pair) {
+    for (int q0 = 0; __any_sync(0xffffffffu, q0 < n); q0 += LANES) {
         T a = 0, b = 0, c = 0, e = 0;
-        if (p < total) pair(node, q, a, b, c, e);
+        if (q0 + lane < n) pair(q0 + lane, a, b, c, e);
         __syncwarp();
-        const int lo = max(start, p0), m = min(start + n, p0 + 32) - lo;
-        for (int t = 0; __any_sync(kAll, t < m); ++t) {
-            const int src = (lo + t) & 31;
-            const T va = __shfl_sync(kAll, a, src), vb = __shfl_sync(kAll, b, src);
-            const T vc = __shfl_sync(kAll, c, src), ve = __shfl_sync(kAll, e, src);
-            if (t < m) {
-                Fsx += va;
-                Fsy += vb;
-                Fnx += vc;
-                Fny += ve;
-            }
-        }
+        Fsx = add_in_order<LANES>(Fsx, a, n - q0);
+        Fsy = add_in_order<LANES>(Fsy, b, n - q0);
+        Fnx = add_in_order<LANES>(Fnx, c, n - q0);
+        Fny = add_in_order<LANES>(Fny, e, n - q0);
     }
 }
 
@@ -1676,22 +1662,21 @@ __device__ __forceinline__ void force_node64(const DevPtrs &d, const KParams &k,
     if constexpr (LANES == 1) {
         if (INLINE && contact) contacts64<PERSIST>(d, k, ii, vin, gi, nc, nb, r0, r1, pi, Fsx, Fsy, Fnx, Fny);
     } else {
-        warp_contacts(ii, lane == 0 ? nc + nb : 0, Fsx, Fsy, Fnx, Fny,
-                      [&](int x, int q, double &sx, double &sy, double &nx, double &ny) {
-                          const int g = __ldg(&d.grain[x]), b0 = __ldg(&d.row_ptr[x]), b1 = __ldg(&d.row_ptr[x + 1]);
-                          const int j = candidate<PERSIST>(d, k, x, ldm<PERSIST>(&d.nbr_cnt[x]), b0, q);
-                          contact_pair64<PERSIST>(d, k, d.agg[__ldg(&d.g_agg[g])], x, j, vin, g, b0, b1,
-                                                  ldm<PERSIST>(&d.p[x]), ldm<PERSIST>(&d.p[j]),
-                                                  ldm<PERSIST>(&d.v[vin][x]), sx, sy, nx, ny);
-                      });
+        group_contacts<LANES>(lane, nc + nb, Fsx, Fsy, Fnx, Fny,
+                              [&](int q, double &sx, double &sy, double &nx, double &ny) {
+                                  const int j = candidate<PERSIST>(d, k, ii, nc, r0, q);
+                                  contact_pair64<PERSIST>(d, k, d.agg[__ldg(&d.g_agg[gi])], ii, j, vin, gi, r0, r1, pi,
+                                                          ldm<PERSIST>(&d.p[j]), ldm<PERSIST>(&d.v[vin][ii]), sx, sy,
+                                                          nx, ny);
+                              });
     }
     __syncwarp();
     out.bx = lane_sum<LANES>(f2d_bits(Fbx.hi) + f2d_bits(Fbx.lo));
     out.by = lane_sum<LANES>(f2d_bits(Fby.hi) + f2d_bits(Fby.lo));
-    out.sx = lane_sum<LANES>(Fsx);
-    out.sy = lane_sum<LANES>(Fsy);
-    out.nx = lane_sum<LANES>(Fnx);
-    out.ny = lane_sum<LANES>(Fny);
+    out.sx = Fsx;
+    out.sy = Fsy;
+    out.nx = Fnx;
+    out.ny = Fny;
 }
 
 // Wall forces and the update of node i from its lane sums, one thread per node
@@ -2240,22 +2225,19 @@ __device__ __forceinline__ void force_node32(const DevPtrs &d, const KParams &k,
     float Fsx = 0.f, Fsy = 0.f, Fnx = 0.f, Fny = 0.f;
     const int nc = active ? ldm<PERSIST>(&d.nbr_cnt[ii]) : 0;
     const int nb = fresh_bonds(d, k, ii, any_lane<LANES>(w0 != 0u || (note & kNoteBroke) || (active && k.wpn > 1)));
-    warp_contacts(ii, lane == 0 ? nc + nb : 0, Fsx, Fsy, Fnx, Fny,
-                  [&](int x, int q, float &sx, float &sy, float &nx, float &ny) {
-                      const int g = __ldg(&d.grain[x]), b0 = __ldg(&d.row_ptr[x]), b1 = __ldg(&d.row_ptr[x + 1]);
-                      const int j = candidate<PERSIST>(d, k, x, ldm<PERSIST>(&d.nbr_cnt[x]), b0, q);
-                      const float4 qx = ldm<PERSIST>(&cur_pq<PERSIST>(d)[x]);
-                      contact_pair32<PERSIST>(d, k, d.agg[__ldg(&d.g_agg[g])], x, j, vin, g, b0, b1,
-                                              make_float2(qx.x, qx.y), make_float2(qx.z, qx.w), __ldg(&d.gq[g]),
-                                              __ldg(&d.gc[g]), ldm<PERSIST>(&cur_pq<PERSIST>(d)[j]),
-                                              ldm<PERSIST>(&d.v[vin][x]), sx, sy, nx, ny);
-                  });
+    group_contacts<LANES>(lane, nc + nb, Fsx, Fsy, Fnx, Fny,
+                          [&](int q, float &sx, float &sy, float &nx, float &ny) {
+                              const int j = candidate<PERSIST>(d, k, ii, nc, r0, q);
+                              contact_pair32<PERSIST>(d, k, d.agg[ag], ii, j, vin, gi, r0, r1, phi, pli, gq, gc,
+                                                      ldm<PERSIST>(&cur_pq<PERSIST>(d)[j]), ldm<PERSIST>(&d.v[vin][ii]),
+                                                      sx, sy, nx, ny);
+                          });
     out.bx = lane_sum<LANES>(Fbx);
     out.by = lane_sum<LANES>(Fby);
-    out.sx = lane_sum<LANES>(Fsx);
-    out.sy = lane_sum<LANES>(Fsy);
-    out.nx = lane_sum<LANES>(Fnx);
-    out.ny = lane_sum<LANES>(Fny);
+    out.sx = Fsx;
+    out.sy = Fsy;
+    out.nx = Fnx;
+    out.ny = Fny;
     if (sur && judge && lane == 0) d.sur_fb[i] = make_float2(out.bx, out.by);   // full bond force for the judge
 }
 
@@ -2490,17 +2472,6 @@ __device__ __forceinline__ void list_special(const DevPtrs &d, int which, int i,
 // FP64 pipe about 4 us -- and a node has up to a dozen.
 constexpr int kSpecialLanes = 8;
 
-// Adds the group's v, lane by lane, to the running sum `acc` of all its threads.
-template <class T>
-__device__ __forceinline__ T add_in_order(T acc, T v, int n) {
-#pragma unroll
-    for (int l = 0; l < kSpecialLanes; ++l) {
-        const T w = __shfl_sync(0xffffffffu, v, l, kSpecialLanes);
-        if (l < n) acc += w;
-    }
-    return acc;
-}
-
 // (node: the group has one; every thread of the warp calls it)
 template <bool PERSIST>
 __device__ __forceinline__ void special_node32(const DevPtrs &d, const KParams &k, int i, bool node, int vin) {
@@ -2523,10 +2494,10 @@ __device__ __forceinline__ void special_node32(const DevPtrs &d, const KParams &
                                     gc, ldm<PERSIST>(&cur_pq<PERSIST>(d)[j]), n.v, sx, sy, nx, ny);
         }
         const int m = nc + nb - q0;
-        f.sx = add_in_order(f.sx, sx, m);
-        f.sy = add_in_order(f.sy, sy, m);
-        f.nx = add_in_order(f.nx, nx, m);
-        f.ny = add_in_order(f.ny, ny, m);
+        f.sx = add_in_order<kSpecialLanes>(f.sx, sx, m);
+        f.sy = add_in_order<kSpecialLanes>(f.sy, sy, m);
+        f.nx = add_in_order<kSpecialLanes>(f.nx, nx, m);
+        f.ny = add_in_order<kSpecialLanes>(f.ny, ny, m);
     }
     if (node && lane == 0) node_epilogue32<PERSIST>(d, k, ii, gi, vin, 1, f, n);
 }
@@ -2551,10 +2522,10 @@ __device__ __forceinline__ void special_node64(const DevPtrs &d, const KParams &
             contact_pair64<PERSIST>(d, k, A, ii, j, vin, gi, r0, r1, pi, ldm<PERSIST>(&d.p[j]), vi, sx, sy, nx, ny);
         }
         const int m = nc + nb - q0;
-        f.sx = add_in_order(f.sx, sx, m);
-        f.sy = add_in_order(f.sy, sy, m);
-        f.nx = add_in_order(f.nx, nx, m);
-        f.ny = add_in_order(f.ny, ny, m);
+        f.sx = add_in_order<kSpecialLanes>(f.sx, sx, m);
+        f.sy = add_in_order<kSpecialLanes>(f.sy, sy, m);
+        f.nx = add_in_order<kSpecialLanes>(f.nx, nx, m);
+        f.ny = add_in_order<kSpecialLanes>(f.ny, ny, m);
     }
     // walls: thread l takes wall l, thread 4 + c corner c
     const bool walls = node && !cells_far_from_walls(cell, ldm<PERSIST>(&cur_wall<PERSIST>(d)[ag]));
@@ -2578,8 +2549,8 @@ __device__ __forceinline__ void special_node64(const DevPtrs &d, const KParams &
                 gy = -gy;
             }
         }
-        Fwx = add_in_order(0.0, gx, kSpecialLanes);
-        Fwy = add_in_order(0.0, gy, kSpecialLanes);
+        Fwx = add_in_order<kSpecialLanes>(0.0, gx, kSpecialLanes);
+        Fwy = add_in_order<kSpecialLanes>(0.0, gy, kSpecialLanes);
     }
     if (!node || lane != 0) return;
     const double inv_m = __ldg(&d.g_invm[gi]);
