@@ -1193,7 +1193,8 @@ constexpr unsigned kPairNone = 0x7FC0D000u, kPairBroken = 0x7FC0D001u, kPairGuar
 constexpr int kPairHalf = 12;     // forward offsets of the stencil
 // What a node's bond pass leaves to do: bonds in the guard band to decide, and
 // that one of its bonds broke at this evaluation.
-constexpr unsigned kNoteGuard = 1u, kNoteBroke = 2u;
+// (kNoteSeen: one of its broken-bond words has a bit; see fresh_bonds)
+constexpr unsigned kNoteGuard = 1u, kNoteBroke = 2u, kNoteSeen = 4u;
 template <class Slot, int BLOCK>
 struct PairTile {
     static constexpr int kStride = kCarry + BLOCK;      // carried slots, then the tile's
@@ -1613,6 +1614,7 @@ __device__ __forceinline__ void force_node64(const DevPtrs &d, const KParams &k,
         for (int m = 0; m < kLoad; ++m) {
             pb[m] = ldm<PERSIST>(&d.p[jb[m] < 0 ? ii : jb[m]]);
             live |= (jb[m] >= 0 && !((wb[m] >> ((b0 + m * LANES - r0) & 31)) & 1u)) ? 1u << m : 0u;
+            note |= wb[m] ? kNoteSeen : 0u;
         }
 #pragma unroll 1
         for (int bm = b0; live; bm += kEval * LANES, live >>= kEval) {
@@ -1656,7 +1658,7 @@ __device__ __forceinline__ void force_node64(const DevPtrs &d, const KParams &k,
     __syncwarp();
 
     const int nc = active ? ldm<PERSIST>(&d.nbr_cnt[ii]) : 0;
-    const int nb = fresh_bonds(d, k, ii, any_lane<LANES>(w0 != 0u || (note & kNoteBroke) || (active && k.wpn > 1)));
+    const int nb = fresh_bonds(d, k, ii, any_lane<LANES>(w0 != 0u || note != 0u));
     double Fsx = 0.0, Fsy = 0.0, Fnx = 0.0, Fny = 0.0;
     contact = nc + nb > 0;
     if constexpr (LANES == 1) {
@@ -2122,6 +2124,7 @@ __device__ __forceinline__ void csr_bonds32(const DevPtrs &d, const KParams &k, 
         for (int m = 0; m < kBondBatch; ++m) {
             const int b = b0 + m * LANES;
             const int kk = b - r0;
+            note |= wb[m] ? kNoteSeen : 0u;
             if (cb[m] == 0xFFFFFFFFu || ((wb[m] >> (kk & 31)) & 1u)) continue;
             const float nn = (float)(cb[m] >> kColBits);         // lattice offset di^2 + dj^2
             BondGeom32 bg;
@@ -2224,7 +2227,8 @@ __device__ __forceinline__ void force_node32(const DevPtrs &d, const KParams &k,
     __syncwarp();
     float Fsx = 0.f, Fsy = 0.f, Fnx = 0.f, Fny = 0.f;
     const int nc = active ? ldm<PERSIST>(&d.nbr_cnt[ii]) : 0;
-    const int nb = fresh_bonds(d, k, ii, any_lane<LANES>(w0 != 0u || (note & kNoteBroke) || (active && k.wpn > 1)));
+    const int nb = fresh_bonds(d, k, ii, any_lane<LANES>(w0 != 0u || (note & ~kNoteGuard) ||
+                                                         (active && !bonds && k.wpn > 1)));
     group_contacts<LANES>(lane, nc + nb, Fsx, Fsy, Fnx, Fny,
                           [&](int q, float &sx, float &sy, float &nx, float &ny) {
                               const int j = candidate<PERSIST>(d, k, ii, nc, r0, q);
