@@ -2221,7 +2221,9 @@ __device__ __forceinline__ void force_node32(const DevPtrs &d, const KParams &k,
     }
     if (!stencil && bonds)
         csr_bonds32<PERSIST, LANES>(d, k, ii, lane, r0, r1, phi, pli, gq, gc, s0_lo, s0_hi, w0, Fbx, Fby, note);
-    if (note & kNoteGuard)
+    // (all threads of the node: they share its offsets out in the loop above, its
+    // bonds in this pass, and a node without some offset has other ranks)
+    if (any_lane<LANES>(note & kNoteGuard))
         guard_bonds32<PERSIST>(d, k, ii, r0, r1, lane, LANES, stencil, phi, pli, gq, gc, gi, s0_lo, s0_hi, bw, Fbx, Fby,
                                 note);
     __syncwarp();
