@@ -1471,12 +1471,25 @@ __device__ __forceinline__ void contact_pair64(const DevPtrs &d, const KParams &
     }
 }
 
-// Candidate q of node ii: the nc of its list (ascending node index), then the
-// partners of the bonds broken since the rebuild; together every pair closer
-// than R_c without an intact bond.
+// Candidate q of node ii, in ascending node index: the nc of its list and the nb
+// partners of the bonds broken since the rebuild, merged; together every pair
+// closer than R_c without an intact bond.  (The order of a node's contact forces
+// then does not depend on when the lists were last rebuilt: a run continued from
+// a stored state, or batched with other aggregates, adds them as any other.)
 template <bool PERSIST>
-__device__ __forceinline__ int candidate(const DevPtrs &d, const KParams &k, int ii, int nc, int r0, int q) {
-    return q < nc ? ldm<PERSIST>(&d.nbr[(size_t)q * k.N + ii]) : fresh_partner(d, k, ii, r0, q - nc);
+__device__ __forceinline__ int candidate(const DevPtrs &d, const KParams &k, int ii, int nc, int nb, int r0, int q) {
+    const auto listed = [&](int at) { return ldm<PERSIST>(&d.nbr[(size_t)at * k.N + ii]); };
+    int at = 0;                             // list entries taken
+    for (int m = 0; m < nb; ++m) {
+        // (few nodes have one; both sequences ascend)
+        const int p = fresh_partner(d, k, ii, r0, m);
+        while (at < nc && listed(at) < p) {
+            if (at + m == q) return listed(at);
+            ++at;
+        }
+        if (at + m == q) return p;
+    }
+    return listed(q - nb);
 }
 
 // Adds the v of a group of LANES threads, thread by thread (the first n of them),
@@ -1523,7 +1536,7 @@ __device__ __forceinline__ void contacts64(const DevPtrs &d, const KParams &k, i
     const AggParams &A = d.agg[__ldg(&d.g_agg[gi])];
     const double2 vi = ldm<PERSIST>(&d.v[vin][ii]);
     for (int q = 0; q < nc + nb; ++q) {
-        const int j = candidate<PERSIST>(d, k, ii, nc, r0, q);
+        const int j = candidate<PERSIST>(d, k, ii, nc, nb, r0, q);
         double a, b, c, e;
         contact_pair64<PERSIST>(d, k, A, ii, j, vin, gi, r0, r1, pi, ldm<PERSIST>(&d.p[j]), vi, a, b, c, e);
         Fsx += a;
@@ -1666,7 +1679,7 @@ __device__ __forceinline__ void force_node64(const DevPtrs &d, const KParams &k,
     } else {
         group_contacts<LANES>(lane, nc + nb, Fsx, Fsy, Fnx, Fny,
                               [&](int q, double &sx, double &sy, double &nx, double &ny) {
-                                  const int j = candidate<PERSIST>(d, k, ii, nc, r0, q);
+                                  const int j = candidate<PERSIST>(d, k, ii, nc, nb, r0, q);
                                   contact_pair64<PERSIST>(d, k, d.agg[__ldg(&d.g_agg[gi])], ii, j, vin, gi, r0, r1, pi,
                                                           ldm<PERSIST>(&d.p[j]), ldm<PERSIST>(&d.v[vin][ii]), sx, sy,
                                                           nx, ny);
@@ -2085,7 +2098,7 @@ __device__ __forceinline__ void contacts32(const DevPtrs &d, const KParams &k, i
     const AggParams &A = d.agg[__ldg(&d.g_agg[gi])];
     const double2 vi64 = ldm<PERSIST>(&d.v[vin][ii]);      // start-of-step velocity
     for (int q = 0; q < nc + nb; ++q) {
-        const int j = candidate<PERSIST>(d, k, ii, nc, r0, q);
+        const int j = candidate<PERSIST>(d, k, ii, nc, nb, r0, q);
         float a, b, c, e;
         contact_pair32<PERSIST>(d, k, A, ii, j, vin, gi, r0, r1, phi, pli, gq, gc, ldm<PERSIST>(&cur_pq<PERSIST>(d)[j]),
                                 vi64, a, b, c, e);
@@ -2233,7 +2246,7 @@ __device__ __forceinline__ void force_node32(const DevPtrs &d, const KParams &k,
                                                          (active && !bonds && k.wpn > 1)));
     group_contacts<LANES>(lane, nc + nb, Fsx, Fsy, Fnx, Fny,
                           [&](int q, float &sx, float &sy, float &nx, float &ny) {
-                              const int j = candidate<PERSIST>(d, k, ii, nc, r0, q);
+                              const int j = candidate<PERSIST>(d, k, ii, nc, nb, r0, q);
                               contact_pair32<PERSIST>(d, k, d.agg[ag], ii, j, vin, gi, r0, r1, phi, pli, gq, gc,
                                                       ldm<PERSIST>(&cur_pq<PERSIST>(d)[j]), ldm<PERSIST>(&d.v[vin][ii]),
                                                       sx, sy, nx, ny);
@@ -2495,7 +2508,7 @@ __device__ __forceinline__ void special_node32(const DevPtrs &d, const KParams &
     for (int q0 = 0; __any_sync(0xffffffffu, q0 < nc + nb); q0 += kSpecialLanes) {
         float sx = 0.f, sy = 0.f, nx = 0.f, ny = 0.f;
         if (q0 + lane < nc + nb) {
-            const int j = candidate<PERSIST>(d, k, ii, nc, r0, q0 + lane);
+            const int j = candidate<PERSIST>(d, k, ii, nc, nb, r0, q0 + lane);
             contact_pair32<PERSIST>(d, k, A, ii, j, vin, gi, r0, r1, make_float2(qi.x, qi.y), make_float2(qi.z, qi.w), gq,
                                     gc, ldm<PERSIST>(&cur_pq<PERSIST>(d)[j]), n.v, sx, sy, nx, ny);
         }
@@ -2524,7 +2537,7 @@ __device__ __forceinline__ void special_node64(const DevPtrs &d, const KParams &
     for (int q0 = 0; __any_sync(0xffffffffu, q0 < nc + nb); q0 += kSpecialLanes) {
         double sx = 0.0, sy = 0.0, nx = 0.0, ny = 0.0;
         if (q0 + lane < nc + nb) {
-            const int j = candidate<PERSIST>(d, k, ii, nc, r0, q0 + lane);
+            const int j = candidate<PERSIST>(d, k, ii, nc, nb, r0, q0 + lane);
             contact_pair64<PERSIST>(d, k, A, ii, j, vin, gi, r0, r1, pi, ldm<PERSIST>(&d.p[j]), vi, sx, sy, nx, ny);
         }
         const int m = nc + nb - q0;

@@ -6,7 +6,8 @@ together below the contact radius makes such pairs exert self-contact forces at
 once: against the oracle, for bonds broken between the steps and in the step,
 on every form of the force phase.  In the step some stretches lie so close to
 the critical one that the FP32 split decides them in FP64, also at the edge of a
-grain, where a node lacks neighbours."""
+grain, where a node lacks neighbours.  And the order of a node's contacts does
+not depend on when its list was built."""
 import numpy as np
 import pytest
 
@@ -88,3 +89,32 @@ def test_contacts_of_fresh_breaks_match_the_oracle(prec, ratio, when):
         assert np.array_equal(S.get("BROKEN"), broken), path
         err = np.abs(S.get("ACC") - P.a).max() / np.abs(P.a).max()
         assert err <= TOL[prec], (path, err)
+
+
+@pytest.mark.parametrize("prec", [B.PD_FP64, B.PD_FP32_SPLIT])
+@pytest.mark.parametrize("path", PATHS)
+def test_order_of_contacts_does_not_depend_on_the_last_rebuild(prec, path):
+    """Half of the broken bonds are in the lists, half came after them; with the
+    lists rebuilt all are in: the same bits."""
+    w, P, u, v = _pressed(0.08)
+    br = _some_bonds(P, 3, 0.4)
+    listed = br * _some_bonds(P, 4, 0.5)
+    assert 0 < listed.sum() < br.sum()
+    runs = []
+    for rebuild in (False, True):
+        S = B.Simulation(w, precision=prec, device="cuda:0")
+        S.set_path(*path)
+        S.set("DISP", u)
+        S.set("BROKEN", listed)
+        S.eval_forces()
+        S.set("VEL", v)
+        S.set("ACC", np.zeros_like(v))
+        S.set("BROKEN", br)
+        if rebuild:
+            S.clear_status()
+        n = _rebuilds(S)
+        S.step(1)
+        assert _rebuilds(S) == n + rebuild
+        runs.append((S.get("ACC"), S.get("VEL"), S.get("BROKEN")))
+    for a, b in zip(*runs):
+        assert np.array_equal(a, b)
