@@ -21,8 +21,9 @@ LIB = os.path.join(OUT, "libperidem.so")
 INC = os.path.join(ROOT, "include")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-# (source, extra flags[, object name]): pd_persist.cu builds once per precision
-# and thread count per node, so that the persistent kernels compile in parallel
+# (source, extra flags[, object name]): pd_persist.cu builds once per precision,
+# thread count per node and with or without bond tiles, so that the persistent
+# kernels compile in parallel
 _FP64_FLAGS = ["-fmad=false"]
 # FP32-split force kernels: divisions and square roots to within 2 ulp (far
 # inside the path's 1e-5 force tolerance) instead of the IEEE sequences
@@ -34,8 +35,10 @@ CU_SOURCES = [
     ("pd_noalloc.cu", []),
     ("pd_mlp.cu", []),
     ("pd_surrogate.cu", []),
-] + [("pd_persist.cu", (_FP32_FLAGS if fp32 else _FP64_FLAGS) + [f"-DPD_PERSIST_FP32={fp32}", f"-DPD_PERSIST_LANES={lanes}"],
-      f"pd_persist{32 if fp32 else 64}_l{lanes}.o") for fp32 in (1, 0) for lanes in (1, 2, 4, 8)]
+] + [("pd_persist.cu", (_FP32_FLAGS if fp32 else _FP64_FLAGS) + [f"-DPD_PERSIST_FP32={fp32}", f"-DPD_PERSIST_LANES={lanes}",
+                                                                 f"-DPD_PERSIST_TILES={tiles}"],
+      f"pd_persist{32 if fp32 else 64}_l{lanes}{'t' if tiles else ''}.o")
+     for fp32 in (1, 0) for lanes, tiles in ((1, 1), (1, 0), (2, 0), (4, 0), (8, 0))]
 CPP_SOURCES = ["pd_host.cpp", "pd_basis.cpp"]
 
 

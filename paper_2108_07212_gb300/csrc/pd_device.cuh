@@ -1548,9 +1548,8 @@ __device__ __forceinline__ void contacts64(const DevPtrs &d, const KParams &k, i
 
 // (slot: the bond tile of a block of BLOCK threads with one thread per node,
 // and warm the pass before a run, which forms slots only and leaves `out`;
-// with more threads per node BLOCK is 0 and there is no tile.  contact: the node
-// has contact candidates; without INLINE its contact forces are left to a later
-// pass.)
+// without a tile BLOCK is 0.  contact: the node has contact candidates; without
+// INLINE (one thread per node) its contact forces are left to a later pass.)
 template <bool PERSIST, int LANES, int BLOCK, bool INLINE = true>
 __device__ __forceinline__ void force_node64(const DevPtrs &d, const KParams &k, int i, int lane, bool active,
                                              int vin, Sums64 &out, float4 *slot, bool warm, bool &contact) {
@@ -1570,10 +1569,10 @@ __device__ __forceinline__ void force_node64(const DevPtrs &d, const KParams &k,
     bool csr = true;           // bonds from the CSR columns
     unsigned note = 0u;
     int r0, r1;
-    if constexpr (LANES == 1) {
-        uint4 st = (k.stencil && active) ? __ldg(&d.stn[ii]) : make_uint4(kStnIrregular, 0u, 0u, 0u);
+    if constexpr (BLOCK > 0) {
+        uint4 st = active ? __ldg(&d.stn[ii]) : make_uint4(kStnIrregular, 0u, 0u, 0u);
         const bool gap = st.x & kStnGap;
-        csr = ((st.x & kStnIrregular) && !gap) || !k.pair;
+        csr = (st.x & kStnIrregular) && !gap;
         st.x &= kStnBits;
         r0 = (int)st.w;
         r1 = r0 + __popc(st.x);
@@ -1581,21 +1580,19 @@ __device__ __forceinline__ void force_node64(const DevPtrs &d, const KParams &k,
             r0 = active ? __ldg(&d.row_ptr[ii]) : 0;
             r1 = active ? __ldg(&d.row_ptr[ii + 1]) : 0;
         }
-        if (k.pair) {
-            const uint32_t alive = csr ? 0u : stn_alive(st.x, w0);
-            const bool gaps = __any_sync(0xffffffffu, gap);
-            const uint32_t formed =
-                gaps ? tile_forward64<PERSIST, BLOCK, true>(d, k, ii, alive, st, gap, pi, cwVV, inv_eps, s0f, s0, slot,
-                                                            note, !warm)
-                     : tile_forward64<PERSIST, BLOCK, false>(d, k, ii, alive, st, gap, pi, cwVV, inv_eps, s0f, s0,
-                                                             slot, note, !warm);
-            if (warm) return;
-            __syncthreads();
-            if (gaps) tile_sum64<PERSIST, BLOCK, true>(d, k, ii, alive, formed, st, gap, pi, cwVV, inv_eps, s0f, s0,
-                                                       slot, Fbx, Fby, note);
-            else tile_sum64<PERSIST, BLOCK, false>(d, k, ii, alive, formed, st, gap, pi, cwVV, inv_eps, s0f, s0, slot,
+        const uint32_t alive = csr ? 0u : stn_alive(st.x, w0);
+        const bool gaps = __any_sync(0xffffffffu, gap);
+        const uint32_t formed =
+            gaps ? tile_forward64<PERSIST, BLOCK, true>(d, k, ii, alive, st, gap, pi, cwVV, inv_eps, s0f, s0, slot,
+                                                        note, !warm)
+                 : tile_forward64<PERSIST, BLOCK, false>(d, k, ii, alive, st, gap, pi, cwVV, inv_eps, s0f, s0, slot,
+                                                         note, !warm);
+        if (warm) return;
+        __syncthreads();
+        if (gaps) tile_sum64<PERSIST, BLOCK, true>(d, k, ii, alive, formed, st, gap, pi, cwVV, inv_eps, s0f, s0, slot,
                                                    Fbx, Fby, note);
-        }
+        else tile_sum64<PERSIST, BLOCK, false>(d, k, ii, alive, formed, st, gap, pi, cwVV, inv_eps, s0f, s0, slot, Fbx,
+                                               Fby, note);
     } else {
         r0 = active ? __ldg(&d.row_ptr[ii]) : 0;
         r1 = active ? __ldg(&d.row_ptr[ii + 1]) : 0;

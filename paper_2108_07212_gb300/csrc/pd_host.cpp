@@ -1218,7 +1218,12 @@ int pd_bind_arena(pd_ctx *c, void *arena, size_t bytes) {
         PD_CUDA(cudaMemcpyAsync(got, found, sizeof(got), cudaMemcpyDeviceToHost, s));
         PD_CUDA(cudaStreamSynchronize(s));
         c->stn_irregular = (size_t)got[0];
-        k.pair = got[1] <= pd::kCarry && !got[2] ? 1 : 0;
+        int dev = 0, sms = 0;
+        PD_CUDA(cudaGetDevice(&dev));
+        PD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        const int run = pd::run_length((int)N, pd::kRunBlocksPerSm * sms);
+        k.pair = got[1] <= pd::kCarry && !got[2] && (k.fp32 || run > pd::kRunBlock) ? 1 : 0;
+        k.run = std::min(std::max(run, pd::kRunBlock), pd::kRunNodes);
     }
     // per grain 1 / (rho V): the update multiplies by it (an FP64 division per
     // node and component costs about nine FP64 operations on GB300)

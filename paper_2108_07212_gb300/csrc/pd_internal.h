@@ -42,6 +42,22 @@ constexpr uint32_t kStnIrregular = 0x80000000u, kStnGap = 0x40000000u, kStnBits 
 // lattice rows of a grain of up to 32 lattice spacings a radius (the finest
 // workloads have 23).
 constexpr int kCarry = 128;
+// Bond tiles on the multi-kernel path: blocks of kRunBlock threads, two an SM,
+// each with up to four tiles of nodes (long enough that the pass before a run
+// costs little, short enough that blocks with many contacts do not set the
+// kernel's time), fewer where that would leave some of the chip's blocks without
+// nodes.  (1024 each whatever the number: FP64, 157138 nodes 101 us a step, now
+// 93; FP32 split 35 and 32, 19681 nodes 26 and 13.5.)  FP64 needs more than one
+// tile a block for tiles to pay, since the pass before the run evaluates as many
+// bonds as they share; below that one thread takes all bonds of its node, and
+// the blocks are twice as many (sequence of launches, FP64, 19681 nodes 69 and
+// 27 us, 49438 nodes 70 and 34.5; persistent kernel 32.5 and 26.4, 44 and 34).
+// (In the FP32 split the two add a node's bonds in different orders.)
+constexpr int kRunBlock = 256, kRunNodes = 4 * kRunBlock, kRunBlocksPerSm = 2;
+// Nodes per block when N nodes are dealt to n of them: a multiple of the warp.
+__host__ __device__ inline int run_length(int N, int n) {
+    return (int)((((long long)N + n - 1) / n + 31) / 32 * 32);
+}
 // Threads per block of the node-parallel multi-kernel path.
 constexpr int kBlock = 128;
 // Scan tile: threads x items per thread.
@@ -188,7 +204,8 @@ struct KParams {
     int fp32;           // precision of the force phase
     int pf_bonds;       // > 0: prefetch the force phase's read-only arrays (this many bonds) into L2
     int stencil;        // bonds from the lattice stencil (DevPtrs::stn) instead of the columns
-    int pair;           // one thread per node: each stencil bond evaluated once (no row reaches past kCarry nodes)
+    int pair;           // one thread per node: each stencil bond evaluated once, in bond tiles (see kRunNodes)
+    int run;            // multi-kernel path with bond tiles: nodes per block
     // surrogate
     int sur;            // surrogate on
     int n_modes;        // modes of the basis (32)

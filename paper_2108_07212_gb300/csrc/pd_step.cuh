@@ -15,7 +15,6 @@ namespace pd {
 // integrates (FP64, converged warps).  Every thread of the block must call it.
 template <bool FP32, bool PERSIST, int LANES, int BLOCK>
 __device__ __forceinline__ void force_block(const DevPtrs &d, const KParams &k, int node0, int vin, int update_v) {
-    static_assert(LANES > 1, "one thread per node: tile_nodes");
     constexpr int NB = BLOCK / LANES;
     using Sums = typename std::conditional<FP32, Sums32, Sums64>::type;
     __shared__ Sums sm[NB];
@@ -63,37 +62,34 @@ __device__ __forceinline__ void store_sums(const DevPtrs &d, const KParams &k, i
 extern __shared__ __align__(16) unsigned char tile_smem[];
 
 // One thread per node, FP64 path: the nodes [lo, hi) in bond tiles of BLOCK
-// nodes (see PairTile).  All threads call out(i, sums, active, contact) as
-// tile_nodes32 does.  Every thread of the block calls it with the same range.
-template <bool PERSIST, int BLOCK, bool INLINE, class Out>
-__device__ __forceinline__ void tile_nodes64(const DevPtrs &d, const KParams &k, int lo, int hi, int vin, Out out) {
-    float4 *slot = reinterpret_cast<float4 *>(tile_smem);
+// nodes (see PairTile), or without TILES as many by themselves.  All threads
+// call out(i, sums, active, contact) as tile_nodes32 does.  Every thread of the
+// block calls it with the same range.
+template <bool PERSIST, int BLOCK, bool TILES, bool INLINE, class Out>
+__device__ __forceinline__ void run_nodes64(const DevPtrs &d, const KParams &k, int lo, int hi, int vin, Out out) {
+    [[maybe_unused]] float4 *slot = reinterpret_cast<float4 *>(tile_smem);
     // the pass before the run takes the nodes [lo - BLOCK, lo), of which the last kCarry have slots
-    for (int node0 = lo > 0 && lo < hi && k.pair ? lo - BLOCK : lo; node0 < hi; node0 += BLOCK) {
+    for (int node0 = TILES && lo > 0 && lo < hi ? lo - BLOCK : lo; node0 < hi; node0 += BLOCK) {
         const int i = node0 + (int)threadIdx.x;
         const bool warm = node0 < lo;
         const bool active = warm ? i >= max(0, lo - kCarry) : i < hi;
         Sums64 f;
         bool contact;
-        force_node64<PERSIST, 1, BLOCK, INLINE>(d, k, i, 0, active, vin, f, slot, warm, contact);
+        force_node64<PERSIST, 1, TILES ? BLOCK : 0, INLINE>(d, k, i, 0, active, vin, f, slot, warm, contact);
         if (!warm) out(i, f, active, contact);
-        __syncthreads();                   // the tile's slots have been read (or formed)
-        if (k.pair) PairTile<float4, BLOCK>::carry(slot);
-        __syncthreads();
+        if constexpr (TILES) {
+            __syncthreads();               // the tile's slots have been read (or formed)
+            PairTile<float4, BLOCK>::carry(slot);
+            __syncthreads();
+        }
     }
 }
 
-// Nodes per block when N nodes are dealt to n of them: a multiple of the warp.
-__host__ __device__ __forceinline__ int run_length(int N, int n) {
-    return (int)((((long long)N + n - 1) / n + 31) / 32 * 32);
-}
-
-// The forces of the nodes [lo, hi), one thread per node, by the calling block:
-// sums stored (split force phase), or each node's walls and update behind them.
-// Grains with rows too long for the carried slots (k.pair clear) take the
-// general bond loop.
+// The forces of the nodes [lo, hi) in bond tiles, one thread per node, by the
+// calling block: sums stored (split force phase), or each node's walls and
+// update behind them.
 template <bool FP32, bool PERSIST, int BLOCK>
-__device__ __forceinline__ void run_nodes(const DevPtrs &d, const KParams &k, int lo, int hi, int vin, int update_v,
+__device__ __forceinline__ void run_tiles(const DevPtrs &d, const KParams &k, int lo, int hi, int vin, int update_v,
                                           bool fused) {
     if constexpr (FP32) {
         auto out = [&](int i, const Sums32 &f, int, bool active, bool) {
@@ -102,18 +98,9 @@ __device__ __forceinline__ void run_nodes(const DevPtrs &d, const KParams &k, in
                                                 load_update32<PERSIST>(d, i, vin, update_v));
             else store_sums<true>(d, k, i, f);
         };
-        if (k.pair) {
-            tile_nodes32<PERSIST, BLOCK, true>(d, k, lo, hi, vin, false, *reinterpret_cast<Tile32<BLOCK> *>(tile_smem), out);
-            return;
-        }
-        for (int g = lo; g < hi; g += BLOCK) {
-            const int i = g + (int)threadIdx.x;
-            Sums32 f;
-            force_node32<PERSIST, 1>(d, k, i, 0, i < hi, vin, f);
-            out(i, f, 0, i < hi, false);
-        }
+        tile_nodes32<PERSIST, BLOCK, true>(d, k, lo, hi, vin, false, *reinterpret_cast<Tile32<BLOCK> *>(tile_smem), out);
     } else {
-        tile_nodes64<PERSIST, BLOCK, true>(d, k, lo, hi, vin, [&](int i, const Sums64 &f, bool active, bool) {
+        run_nodes64<PERSIST, BLOCK, true, true>(d, k, lo, hi, vin, [&](int i, const Sums64 &f, bool active, bool) {
             if (!active) return;
             if (fused) node_epilogue64<PERSIST>(d, k, i, vin, update_v, f);
             else store_sums<false>(d, k, i, f);
@@ -123,8 +110,9 @@ __device__ __forceinline__ void run_nodes(const DevPtrs &d, const KParams &k, in
 
 // The same for the persistent kernel's fused force phase: plain nodes are
 // updated at once, special ones (see list_special) put on list `which`.
-template <bool FP32, int BLOCK>
+template <bool FP32, int BLOCK, bool TILES>
 __device__ __forceinline__ void run_plain_nodes(const DevPtrs &d, const KParams &k, int lo, int hi, int vin, int which) {
+    static_assert(TILES || !FP32, "FP32 split without tiles: no list of special nodes");
     if constexpr (FP32) {
         Tile32<BLOCK> &sm = *reinterpret_cast<Tile32<BLOCK> *>(tile_smem);
         tile_nodes32<true, BLOCK, false>(d, k, lo, hi, vin, true, sm,
@@ -140,7 +128,7 @@ __device__ __forceinline__ void run_plain_nodes(const DevPtrs &d, const KParams 
             list_special(d, which, i, special);
         });
     } else {
-        tile_nodes64<true, BLOCK, false>(d, k, lo, hi, vin, [&](int i, const Sums64 &f, bool active, bool contact) {
+        run_nodes64<true, BLOCK, TILES, false>(d, k, lo, hi, vin, [&](int i, const Sums64 &f, bool active, bool contact) {
             bool special = false;
             if (active) {
                 const int gi = __ldg(&d.grain[i]);
@@ -180,21 +168,18 @@ constexpr int run_smem() {
 // the tile loop, 211 us against 183 us on 2.28M nodes.)
 constexpr int run_blocks(int block) { return 512 / block; }
 
-// Multi-kernel path, one thread per node: four tiles of nodes a block (long
-// enough that the pass before a run costs little, short enough that blocks with
-// many contacts do not set the kernel's time).
-constexpr int kRunBlock = 256, kRunNodes = 4 * kRunBlock;
+// Multi-kernel path, bond tiles: k.run nodes a block (see kRunNodes).
 template <bool FP32>
 __global__ void __launch_bounds__(kRunBlock, run_blocks(kRunBlock))
     k_force_run(DevPtrs d, KParams k, int vin, int update_v, int fused) {
     clear_rebuild(d);
-    const int lo = blockIdx.x * kRunNodes;
-    run_nodes<FP32, false, kRunBlock>(d, k, lo, min(lo + kRunNodes, k.N), vin, update_v, fused != 0);
+    const int lo = blockIdx.x * k.run;
+    run_tiles<FP32, false, kRunBlock>(d, k, lo, min(lo + k.run, k.N), vin, update_v, fused != 0);
 }
 
-// Multi-kernel path, several threads per node: one block per BLOCK / LANES nodes.
+// Multi-kernel path without tiles: one block per BLOCK / LANES nodes.
 template <bool FP32, int LANES>
-__global__ void __launch_bounds__(kBlock, FP32 ? 5 : 4) k_force(DevPtrs d, KParams k, int vin, int update_v) {
+__global__ void __launch_bounds__(kBlock, FP32 ? (LANES == 1 ? 8 : 5) : 4) k_force(DevPtrs d, KParams k, int vin, int update_v) {
     clear_rebuild(d);
     force_block<FP32, false, LANES, kBlock>(d, k, blockIdx.x * (kBlock / LANES), vin, update_v);
 }
@@ -261,7 +246,7 @@ __global__ void __launch_bounds__(256, PERSM) k_epilogue(DevPtrs d, KParams k, i
 
 template <bool FP32>
 cudaError_t launch_force_run(const DevPtrs &d, const KParams &k, int vin, int update_v, cudaStream_t s, int fused) {
-    k_force_run<FP32><<<(k.N + kRunNodes - 1) / kRunNodes, kRunBlock, run_smem<FP32, kRunBlock>(), s>>>(d, k, vin,
+    k_force_run<FP32><<<(k.N + k.run - 1) / k.run, kRunBlock, run_smem<FP32, kRunBlock>(), s>>>(d, k, vin,
                                                                                                      update_v, fused);
     return cudaGetLastError();
 }
@@ -281,21 +266,28 @@ cudaError_t launch_force_impl(const DevPtrs &d, const KParams &k, int vin, int u
             if (k.lanes == 8) k_sums<FP32, 8><<<grid, kBlock, 0, s>>>(d, k, vin);
             else if (k.lanes == 4) k_sums<FP32, 4><<<grid, kBlock, 0, s>>>(d, k, vin);
             else if (k.lanes == 2) k_sums<FP32, 2><<<grid, kBlock, 0, s>>>(d, k, vin);
-            else if (FP32 && k.sur) {
-                // grains on the surrogate have no bonds to share: more warps instead of
-                // tiles (2000 grains, 2.03M nodes: 232 us a step, in tiles 250)
-                if constexpr (FP32) k_sums<FP32, 1><<<grid, kBlock, 0, s>>>(d, k, vin);
-            } else if (const cudaError_t e = launch_force_run<FP32>(d, k, vin, 0, s, 0)) return e;
+            else if (!k.pair || (FP32 && k.sur))
+                // (grains on the surrogate have no bonds to share: more warps instead of
+                // tiles; 2000 grains, 2.03M nodes: 232 us a step, in tiles 250)
+                k_sums<FP32, 1><<<grid, kBlock, 0, s>>>(d, k, vin);
+            else if (const cudaError_t e = launch_force_run<FP32>(d, k, vin, 0, s, 0)) return e;
         }
         const unsigned nb = (unsigned)((k.N + 255) / 256);
-        if (phase != 1 && FP32 && k.sur && k.N > kManyNodes) k_epilogue<FP32, 6><<<nb, 256, 0, s>>>(d, k, vin, update_v);
-        else if (phase != 1) k_epilogue<FP32><<<nb, 256, 0, s>>>(d, k, vin, update_v);
+        if (phase == 1) return cudaGetLastError();
+        if constexpr (FP32) {
+            if (k.sur && k.N > kManyNodes) {
+                k_epilogue<FP32, 6><<<nb, 256, 0, s>>>(d, k, vin, update_v);
+                return cudaGetLastError();
+            }
+        }
+        k_epilogue<FP32><<<nb, 256, 0, s>>>(d, k, vin, update_v);
         return cudaGetLastError();
     }
     if (phase != 0) return cudaErrorInvalidValue;
     if (k.lanes == 8) k_force<FP32, 8><<<grid, kBlock, 0, s>>>(d, k, vin, update_v);
     else if (k.lanes == 4) k_force<FP32, 4><<<grid, kBlock, 0, s>>>(d, k, vin, update_v);
     else if (k.lanes == 2) k_force<FP32, 2><<<grid, kBlock, 0, s>>>(d, k, vin, update_v);
+    else if (!k.pair) k_force<FP32, 1><<<grid, kBlock, 0, s>>>(d, k, vin, update_v);
     else return launch_force_run<FP32>(d, k, vin, update_v, s, 1);
     return cudaGetLastError();
 }
@@ -309,8 +301,8 @@ cudaError_t launch_force_impl(const DevPtrs &d, const KParams &k, int vin, int u
 //      except in the first step of a launch that finds no valid prediction)
 //   R  the candidate lists, when some node moved kSkinTrigger * skin since the
 //      last rebuild (rebuild_lists)
-//   E  forces, acceleration and velocity update (one thread per node and the
-//      fused force phase: plain nodes, then special ones)
+//   E  forces, acceleration and velocity update (bond tiles, and in FP64 one
+//      thread per node, with the fused force phase: plain nodes, then special ones)
 // The barrier after A is left out where A was taken by the step before (FP32
 // split, after the first step): what it published is then known already.
 //   * The time of the step follows from the step counter at the launch.
@@ -322,7 +314,7 @@ cudaError_t launch_force_impl(const DevPtrs &d, const KParams &k, int vin, int u
 //     st - 1).
 // s_cur_* hold this step's displacement, positions, time, wall cells and the
 // word its rebuild test raises.  False when a grid barrier gave up (the kernel then returns).
-template <bool FP32, int LANES, int BLOCK>
+template <bool FP32, int LANES, int BLOCK, bool TILES>
 __device__ __forceinline__ bool persistent_step(const DevPtrs &d, const KParams &k, int vin, int st, int nsteps,
                                                 bool predicted, long long step0, unsigned &epoch, int *sm) {
     const int nthreads = gridDim.x * BLOCK;
@@ -367,26 +359,23 @@ __device__ __forceinline__ bool persistent_step(const DevPtrs &d, const KParams 
                                                [&] { return grid_barrier(d, k.bar_spins, epoch); }))
         return false;
     // E
-    if constexpr (LANES == 1) {
-        const int len = run_length(k.N, gridDim.x);
-        const int lo0 = (int)min((long long)k.N, (long long)blockIdx.x * len), hi0 = min(lo0 + len, k.N);
-        if (k.split || !k.pair) {
-            run_nodes<FP32, true, BLOCK>(d, k, lo0, hi0, vin, 1, !k.split);
-            if (k.split) {
-                if (!grid_barrier(d, k.bar_spins, epoch)) return false;
-                for (int i = gtid; i < k.N; i += nthreads) epilogue_node<FP32, true>(d, k, i, vin, 1);
-            }
+    const int len = run_length(k.N, gridDim.x);
+    const int lo0 = (int)min((long long)k.N, (long long)blockIdx.x * len), hi0 = min(lo0 + len, k.N);
+    if (k.split) {
+        if constexpr (TILES) {
+            run_tiles<FP32, true, BLOCK>(d, k, lo0, hi0, vin, 1, false);
         } else {
-            run_plain_nodes<FP32, BLOCK>(d, k, lo0, hi0, vin, st & 1);
-            if (!grid_barrier(d, k.bar_spins, epoch)) return false;
-            if (gtid == 0) d.spec_n[(st + 1) & 1] = 0;
-            run_special_nodes<FP32, BLOCK>(d, k, vin, st & 1);
+            const long long total = (((long long)LANES * k.N + 31) / 32) * 32;
+            for (long long t = gtid; t < total; t += nthreads)
+                sums_node<FP32, true, LANES>(d, k, (int)(t / LANES), (int)(t % LANES), vin);
         }
-    } else if (k.split) {
-        const long long total = (((long long)LANES * k.N + 31) / 32) * 32;
-        for (long long t = gtid; t < total; t += nthreads) sums_node<FP32, true, LANES>(d, k, (int)(t / LANES), (int)(t % LANES), vin);
         if (!grid_barrier(d, k.bar_spins, epoch)) return false;
         for (int i = gtid; i < k.N; i += nthreads) epilogue_node<FP32, true>(d, k, i, vin, 1);
+    } else if constexpr (TILES || (LANES == 1 && !FP32)) {
+        run_plain_nodes<FP32, BLOCK, TILES>(d, k, lo0, hi0, vin, st & 1);
+        if (!grid_barrier(d, k.bar_spins, epoch)) return false;
+        if (gtid == 0) d.spec_n[(st + 1) & 1] = 0;
+        run_special_nodes<FP32, BLOCK>(d, k, vin, st & 1);
     } else {
         for (int node0 = blockIdx.x * (BLOCK / LANES); node0 < k.N; node0 += gridDim.x * (BLOCK / LANES))
             force_block<FP32, true, LANES, BLOCK>(d, k, node0, vin, 1);
@@ -399,8 +388,13 @@ __device__ __forceinline__ bool persistent_step(const DevPtrs &d, const KParams 
 // grid barriers.  Every step reads its current displacement and positions
 // through s_cur_u / s_cur_pq, the buffers of its parity (the FP32 split keeps
 // two of each; the FP64 path one).
-// (Capped at 128 registers, four blocks of 128 threads per SM.)
-template <bool FP32, int LANES, int BLOCK>
+// (Capped at 128 registers, four blocks of 128 threads per SM.  What one thread
+// per node without tiles needs beside them is the L1 that tiles would take from
+// its gathers: horizon 4 h, 306907 nodes, blocks of 256, with the tiles' shared
+// memory FP32 split 75.7 us a step and FP64 284, without 62.5 and 240.  Twice
+// the threads at 64 registers: FP32 split 60.4, but 157138 nodes of it 38 us
+// for 43, 49438 nodes 17.9 for 16.4, 10010 nodes 8.8 for 8.1.)
+template <bool FP32, int LANES, int BLOCK, bool TILES>
 __global__ void __launch_bounds__(BLOCK, run_blocks(BLOCK))
     k_persistent(DevPtrs d, KParams k, int vin, int nsteps) {
     __shared__ int sm[33];
@@ -420,7 +414,7 @@ __global__ void __launch_bounds__(BLOCK, run_blocks(BLOCK))
         }
         __syncthreads();
         const bool predicted = FP32 && (st > 0 || pred0);
-        if (!persistent_step<FP32, LANES, BLOCK>(d, k, vin, st, nsteps, predicted, step0, epoch, sm)) return;
+        if (!persistent_step<FP32, LANES, BLOCK, TILES>(d, k, vin, st, nsteps, predicted, step0, epoch, sm)) return;
         vin ^= 1;
     }
     // the next launch may skip its first update phase (the end of this launch
@@ -428,14 +422,14 @@ __global__ void __launch_bounds__(BLOCK, run_blocks(BLOCK))
     if (FP32 && blockIdx.x == 0 && threadIdx.x == 0) *(volatile int *)d.pred_ok = 1;
 }
 
-template <bool FP32, int LANES, int BLOCK>
+template <bool FP32, int LANES, int BLOCK, bool TILES>
 cudaError_t launch_persistent_cfg(const DevPtrs &d, const KParams &k, int vin, int nsteps, cudaStream_t s) {
-    auto kern = k_persistent<FP32, LANES, BLOCK>;
+    auto kern = k_persistent<FP32, LANES, BLOCK, TILES>;
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const size_t smem = LANES == 1 ? run_smem<FP32, BLOCK>() : 0;
+    const size_t smem = TILES ? run_smem<FP32, BLOCK>() : 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BLOCK, smem)) != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     const long long need = ((long long)LANES * k.N + BLOCK - 1) / BLOCK;
@@ -453,10 +447,11 @@ cudaError_t launch_persistent_cfg(const DevPtrs &d, const KParams &k, int vin, i
     return cudaLaunchKernelEx(&cfg, kern, d, k, vin, nsteps);
 }
 
-// The persistent kernels of one precision and one thread count per node (both
-// block sizes), each instantiated in a translation unit of its own
-// (pd_persist.cu, compiled once per pair) so that they build in parallel.
-template <bool FP32, int LANES>
+// The persistent kernels of one precision and one thread count per node, with
+// or without tiles (both block sizes), each instantiated in a translation unit
+// of its own (pd_persist.cu, compiled once per combination) so that they build
+// in parallel.
+template <bool FP32, int LANES, bool TILES>
 cudaError_t launch_persistent_lanes(const DevPtrs &d, const KParams &k, int vin, int nsteps, int block,
                                     cudaStream_t s);
 
@@ -466,10 +461,11 @@ cudaError_t init_persistent_tiles();
 
 template <bool FP32>
 cudaError_t launch_persistent_impl(const DevPtrs &d, const KParams &k, int vin, int nsteps, int block, cudaStream_t s) {
-    if (k.lanes == 8) return launch_persistent_lanes<FP32, 8>(d, k, vin, nsteps, block, s);
-    if (k.lanes == 4) return launch_persistent_lanes<FP32, 4>(d, k, vin, nsteps, block, s);
-    if (k.lanes == 2) return launch_persistent_lanes<FP32, 2>(d, k, vin, nsteps, block, s);
-    return launch_persistent_lanes<FP32, 1>(d, k, vin, nsteps, block, s);
+    if (k.lanes == 8) return launch_persistent_lanes<FP32, 8, false>(d, k, vin, nsteps, block, s);
+    if (k.lanes == 4) return launch_persistent_lanes<FP32, 4, false>(d, k, vin, nsteps, block, s);
+    if (k.lanes == 2) return launch_persistent_lanes<FP32, 2, false>(d, k, vin, nsteps, block, s);
+    if (!k.pair) return launch_persistent_lanes<FP32, 1, false>(d, k, vin, nsteps, block, s);
+    return launch_persistent_lanes<FP32, 1, true>(d, k, vin, nsteps, block, s);
 }
 
 }  // namespace pd
