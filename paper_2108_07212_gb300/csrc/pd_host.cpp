@@ -283,24 +283,58 @@ void compute_aggregates(pd_ctx *c) {
 }
 
 // Contact grid of every aggregate: cells over its wall box at t = 0 and one
-// around it, at least 3 each way and, by shrinking both ways alike, at most
-// four per node (two beyond 2^28 nodes, for 32-bit cell indices), 64 at least.
+// around it, at least 3 each way and at most four per node (two beyond 2^28
+// nodes, for 32-bit cell indices), 64 at least.  A box with more cells keeps
+// those of the nodes' extent at the start, the longer way first brought to the
+// shorter where even these are too many, and the rest is shared out to both ways
+// alike: cells that wrap around pile nodes up, so the populated ones must not.
+// (Shrinking the whole box alike left one of 23 mm by 33 km three cells across:
+// an evaluation with rebuilt lists, 19681 nodes FP64, took 217 us in it against 81
+// in the close-fitting box of 23 by 33 mm; now 76 in both.)
 void compute_grid(pd_ctx *c) {
-    std::vector<int64_t> nodes(c->n_agg, 0);
-    for (int g = 0; g < c->G; ++g) nodes[c->g_agg[g]] += c->g_start[g + 1] - c->g_start[g];
+    std::vector<double> most(c->n_agg, 0.0);
+    for (int g = 0; g < c->G; ++g)
+        most[c->g_agg[g]] += (c->N > (int64_t(1) << 28) ? 2.0 : 4.0) * (double)(c->g_start[g + 1] - c->g_start[g]);
+    std::vector<double> gw(c->n_agg), gh(c->n_agg);
+    bool fits = true;
+    for (int a = 0; a < c->n_agg; ++a) {
+        const double *w = &c->agg_walls[8 * (size_t)a], cell = c->aggp[a].cell;
+        most[a] = std::max(64.0, most[a]);
+        gw[a] = std::max(3.0, std::ceil((w[1] - w[0]) / cell) + 2);
+        gh[a] = std::max(3.0, std::ceil((w[3] - w[2]) / cell) + 2);
+        fits &= gw[a] * gh[a] <= most[a];
+    }
+    std::vector<double> ext;                                // of the nodes: x_lo, x_hi, y_lo, y_hi
+    for (int a = 0; a < c->n_agg && !fits; ++a) ext.insert(ext.end(), {1e300, -1e300, 1e300, -1e300});
+    for (int g = 0; g < c->G && !fits; ++g) {
+        double *e = &ext[4 * (size_t)c->g_agg[g]];
+        for (int64_t i = c->g_start[g]; i < c->g_start[g + 1]; ++i)
+            for (int q = 0; q < 2; ++q) {
+                e[2 * q] = std::min(e[2 * q], c->X[2 * i + q]);
+                e[2 * q + 1] = std::max(e[2 * q + 1], c->X[2 * i + q]);
+            }
+    }
     int64_t total = 0;
     for (int a = 0; a < c->n_agg; ++a) {
         pd::AggParams &A = c->aggp[a];
-        const double *w = &c->agg_walls[8 * (size_t)a];
-        double gw = std::ceil((w[1] - w[0]) / A.cell) + 2, gh = std::ceil((w[3] - w[2]) / A.cell) + 2;
-        const double most = std::max(64.0, (c->N > (int64_t(1) << 28) ? 2.0 : 4.0) * (double)nodes[a]);
-        if (gw * gh > most) {
-            const double f = std::sqrt(most / (gw * gh));
-            gw = std::max(3.0, std::min(std::floor(gw * f), std::floor(most / 3)));
-            gh = std::max(3.0, std::floor(most / gw));
+        if (gw[a] * gh[a] > most[a]) {
+            const double *e = &ext[4 * (size_t)a];
+            double ew = std::min(gw[a], std::max(3.0, std::ceil((e[1] - e[0]) / A.cell) + 2));
+            double eh = std::min(gh[a], std::max(3.0, std::ceil((e[3] - e[2]) / A.cell) + 2));
+            if (ew * eh > most[a]) {
+                double &lo = ew < eh ? ew : eh, &hi = ew < eh ? eh : ew;
+                lo = std::min(lo, std::floor(std::sqrt(most[a])));
+                hi = std::floor(most[a] / lo);
+            } else {
+                ew = std::min(gw[a], std::floor(ew * std::sqrt(most[a] / (ew * eh))));
+                eh = std::min(gh[a], std::floor(most[a] / ew));
+                ew = std::min(gw[a], std::floor(most[a] / eh));
+            }
+            gw[a] = ew;
+            gh[a] = eh;
         }
-        A.gw = (int)std::max(gw, 3.0);
-        A.gh = (int)std::max(gh, 3.0);
+        A.gw = (int)gw[a];
+        A.gh = (int)gh[a];
         A.gbase = (int)total;
         total += (int64_t)A.gw * A.gh;
     }
