@@ -234,9 +234,10 @@ __global__ void __launch_bounds__(kBlock, FP32 ? 8 : 4) k_sums(DevPtrs d, KParam
 
 // (Registers for the wall terms: at 40 a thread their chain went through 1.3 to
 // 1.5 KB of spills; a step near the walls, 49907 nodes FP32 split: 12 us.)
-// (kManyNodes: with ten waves of blocks the pass is bound by memory, and the warps
-// that 40 registers allow are worth more: surrogate step of 2.03M nodes, 232 us
-// with 80, 207 with 40.)
+// (kManyNodes, FP32 split: with ten waves of blocks the pass is bound by memory,
+// and the warps that 40 registers allow are worth more.  Step with 80 and with 40:
+// 2.04M nodes, two threads each, 251 and 239 us, on the surrogate 232 and 207;
+// 1.24M 159 and 155, 801k 109 and 107, 521k 74 and 75.)
 constexpr int kManyNodes = 1 << 20;
 template <bool FP32, int PERSM = FP32 ? 3 : 2>
 __global__ void __launch_bounds__(256, PERSM) k_epilogue(DevPtrs d, KParams k, int vin, int update_v) {
@@ -275,7 +276,7 @@ cudaError_t launch_force_impl(const DevPtrs &d, const KParams &k, int vin, int u
         const unsigned nb = (unsigned)((k.N + 255) / 256);
         if (phase == 1) return cudaGetLastError();
         if constexpr (FP32) {
-            if (k.sur && k.N > kManyNodes) {
+            if (k.N > kManyNodes) {
                 k_epilogue<FP32, 6><<<nb, 256, 0, s>>>(d, k, vin, update_v);
                 return cudaGetLastError();
             }
