@@ -1610,7 +1610,9 @@ __device__ __forceinline__ void force_node64(const DevPtrs &d, const KParams &k,
     // that starts with cold caches waits for its code more than for data.  Two
     // copies, 4 threads per node: 49.7 us a step of a settled box of 19681 nodes
     // with L2 flushed before it, one: 45.0; 48 bonds a node, 87340 nodes: 104.7
-    // and 98.2.)
+    // and 98.2.  Two bonds a time, of four: 306907 nodes, 4 threads per node 182 us
+    // for 172, 8 threads 260 for 227, but horizon 2 h, whose rows of eight leave
+    // the third place empty, 2 threads 71 for 88.)
     constexpr int kLoad = 6, kEval = 3;
     static_assert(kLoad == 2 * kEval, "a round is two evaluations");
     for (int b0 = r0 + lane; b0 < r1 && csr; b0 += kLoad * LANES) {

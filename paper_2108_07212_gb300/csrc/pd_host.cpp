@@ -237,7 +237,7 @@ constexpr double kPiAgg = 3.14159265358979323846;
 // Per-aggregate contact constants (Sec. 4.1): R_c = rc_ratio h_min and
 // K_n = 18 k / (pi eps_c^5) with eps_c = horizon_ratio h_min, h_min the
 // smallest lattice spacing of the aggregate's grains; contact grid anchored at
-// the aggregate's lower-left wall corner with cells of side R_c.
+// the aggregate's lower-left wall corner, its cells a hair wider than R_c + skin.
 void compute_aggregates(pd_ctx *c) {
     const pd_params &p = c->prm;
     c->aggp.assign(c->n_agg, pd::AggParams{});

@@ -291,7 +291,13 @@ cudaError_t launch_predict(const DevPtrs &d, const KParams &k, int vin, int adva
 // rebuild flag is clear).
 cudaError_t launch_rebuild(const DevPtrs &d, const KParams &k, cudaStream_t s);
 // The same in one launch of one cluster, for up to kClusterNodes nodes: 8192 or
-// 16384 threads, so a rebuild takes about a node's latency for every 16384.
+// 16384 threads, so a rebuild takes about a node's latency for every 16384.  A
+// step of a calm state, behind a conditional node and with the cluster's launch:
+// 19681 nodes FP32 split 23.6 and 14.3 us, FP64 31.5 and 22.6; 64904 nodes 28.4
+// and 18.8, 52.9 and 43.2.  Of grains thrown at 20 m/s, with a rebuild every few
+// steps: 19681 nodes 29.0 and 21.2, 37.6 and 33.8; 49438 nodes 34.1 and 27.3, 53.0
+// and 51.8; 64904 nodes 37.2 and 34.5, 62.5 and 68.4: the line lies where the
+// six kernels win in such a state and lose in a calm one.
 constexpr int kClusterNodes = 1 << 16;
 cudaError_t launch_rebuild_cluster(const DevPtrs &d, const KParams &k, cudaStream_t s);
 // The nodes' bond stencils (DevPtrs::stn; FP64 path: xif) from the uploaded CSR

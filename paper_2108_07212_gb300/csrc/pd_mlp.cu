@@ -43,7 +43,7 @@ __device__ __forceinline__ float gelu_grad(float z) {
 }
 
 // ---------------------------------------------------------------------------
-// pieces of a tile of R = 32, 64, 96 or 128 samples on 512 threads: warp w reads
+// pieces of a tile of R = 32, 64 or 128 samples on 512 threads: warp w reads
 // TMEM lanes 32 (w % 4) .. 32 (w % 4) + 31 (its quarter of the samples) and
 // warpgroup w / 4 takes a quarter of a layer's columns.  The products always
 // have 128 sample rows (rows from R on hold whatever shared memory does and are
