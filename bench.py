@@ -77,11 +77,12 @@ def fp32_bytes_per_node(mode: int, whole: bool) -> int:
     return force + (BYTES_UPDATE_FP32_FUSED if mode & 1 else BYTES_UPDATE_FP32)
 
 
-def fp64_bytes(path: dict, whole: bool):
+def fp64_bytes(path: dict, whole: bool, nodes: int):
     """Algorithmic bytes per node and per directed bond of the FP64 force phase
-    of a step path, or of its whole step."""
-    per_node, per_bond = ((BYTES_PER_NODE_FP64_TILE, 0) if path.get("lanes") == 1 else
-                          (BYTES_PER_NODE_FP64, BYTES_PER_BOND_FP64))
+    of a step path, or of its whole step (one thread per node: bond tiles where
+    more than one falls to each of two blocks an SM)."""
+    tiles = path.get("lanes") == 1 and nodes > 2 * 256 * N_SM
+    per_node, per_bond = (BYTES_PER_NODE_FP64_TILE, 0) if tiles else (BYTES_PER_NODE_FP64, BYTES_PER_BOND_FP64)
     return per_node + (BYTES_UPDATE_FP64 if whole else 0), per_bond
 
 
@@ -393,28 +394,27 @@ def _timed_steps(sim, stream, flush, steps, warmup, torch):
 BYTES_PER_NODE_STEP_FP32_MAX = BYTES_UPDATE_FP32 + BYTES_PER_NODE_FP32
 
 
-# DRAM bytes (read + write) per launch of the force-phase kernels, per workload,
-# from one ncu capture (one pass) of the timed steps (the bench marks them with
-# cudaProfilerStart/Stop; path mode 6 = mode 2 without the conditional graph
-# node, which ncu cannot trace; the same kernels), e.g.
+# DRAM bytes (read + write) per launch of the force-phase kernels on the 500-grain
+# compaction, from one ncu capture (one pass) of the timed steps (the bench marks
+# them with cudaProfilerStart/Stop; path mode 6 = mode 2 without the conditional
+# graph node, which ncu cannot trace; the same kernels), e.g.
 #   ncu --metrics gpu__time_duration.sum,dram__bytes_read.sum,dram__bytes_write.sum --clock-control none
-#       --profile-from-start off -k regex:"k_sums|k_epilogue" --csv
-#       python bench.py --steps 3 --warmup 3 --legs= --no-cpu --path 6,1
+#       --profile-from-start off -k regex:"k_force_run|k_epilogue" --csv
+#       python bench.py --workload compaction500 --steps 3 --warmup 3 --legs= --no-cpu --path 6,1
 # (medians over the three captured launches; summaries under profiles/).  They
-# hold while the kernel sources hash to TRAFFIC_DIGEST; otherwise, or for a
-# kernel not captured, traffic is null.
+# hold while the kernel sources hash to CAPTURED[workload]; otherwise, or for a
+# kernel or workload not captured (the ensemble: counters are taken on small
+# contexts only), traffic is null.
 TRAFFIC = {
-    "ensemble64": {"k_persistent<1, 1, 256>": 1196907520, "k_persistent<0, 1, 256>": 3344664064,
-                   "k_sums<1, 1>": 356045568, "k_epilogue<1>": 421486080,
-                   "k_sums<0, 1>": 2233693952, "k_epilogue<0>": 584599552},
-    "compaction500": {"k_persistent<1, 1, 256>": 69165824, "k_persistent<0, 1, 256>": 244184320,
-                      "k_persistent<1, 1, 128>": 69178880, "k_persistent<0, 1, 128>": 243823872,
-                      "k_sums<1, 1>": 23607040, "k_epilogue<1>": 23026944,
-                      "k_sums<0, 1>": 170565120, "k_epilogue<0>": 31460864},
+    "compaction500": {"k_persistent<1, 1, 256, 1>": 66604288, "k_persistent<0, 1, 256, 1>": 141907200,
+                      "k_persistent<1, 1, 128, 1>": 66999296, "k_persistent<0, 1, 128, 1>": 145461248,
+                      "k_force_run<1>": 23030272, "k_epilogue<1, 3>": 23021568,
+                      "k_force_run<0>": 77035776, "k_epilogue<0, 2>": 31365120},
 }
-TRAFFIC_DIGEST = "1235532d82438481bf9c97cad09580c8b576d3ac"
-TRAFFIC_SOURCES = ("pd_device.cuh", "pd_step.cuh", "pd_step32.cu", "pd_step64.cu", "pd_persist.cu", "pd_common.cu",
-                   "pd_internal.h")
+CAPTURED = {"compaction500": "fed131ce2bd63361db6b265b635ef1beea5db3b2"}
+TRAFFIC_DIGEST = None     # sources at which every workload's figures were taken: the ensemble has none
+TRAFFIC_SOURCES = ("pd_device.cuh", "pd_rebuild.cuh", "pd_step.cuh", "pd_step32.cu", "pd_step64.cu", "pd_persist.cu",
+                   "pd_common.cu", "pd_internal.h")
 
 
 def kernel_digest() -> str:
@@ -428,16 +428,25 @@ def kernel_digest() -> str:
     return hsh.hexdigest()
 
 
-def force_phase_traffic(path: dict, fp32: bool, workload: str):
-    """Measured DRAM bytes of one force phase of the chosen path, or None."""
-    table = TRAFFIC.get(workload, {})
-    if not table or kernel_digest() != TRAFFIC_DIGEST:
-        return None
+def captured(table: dict, workload: str) -> dict:
+    """The workload's ncu figures, empty when its kernels have changed since."""
+    return table.get(workload, {}) if kernel_digest() == CAPTURED.get(workload) else {}
+
+
+def force_kernel_names(path: dict, fp32: bool) -> list:
+    """The kernels of one force phase of a large context as ncu prints them (one
+    thread per node: in bond tiles)."""
     p, m, l = ("1" if fp32 else "0"), path["mode"], path["lanes"]
     if m & 1:
-        names = [f"k_persistent<{p}, {l}, {path.get('block', 128)}>"]     # the whole step
-    else:
-        names = [f"k_sums<{p}, {l}>", f"k_epilogue<{p}>"] if (m >> 1) & 1 else [f"k_force<{p}, {l}>"]
+        return [f"k_persistent<{p}, {l}, {path.get('block', 128)}, {1 if l == 1 else 0}>"]     # the whole step
+    if (m >> 1) & 1:
+        return [f"k_force_run<{p}>" if l == 1 else f"k_sums<{p}, {l}>", f"k_epilogue<{p}, {3 if fp32 else 2}>"]
+    return [f"k_force_run<{p}>" if l == 1 else f"k_force<{p}, {l}>"]
+
+
+def force_phase_traffic(path: dict, fp32: bool, workload: str):
+    """Measured DRAM bytes of one force phase of the chosen path, or None."""
+    table, names = captured(TRAFFIC, workload), force_kernel_names(path, fp32)
     if not all(n in table for n in names):
         return None
     return float(sum(table[n] for n in names))
@@ -499,16 +508,12 @@ def _roof_fp32(sim, f_ms, hbm, label, path=None, workload=None):
 
 
 # Warp instructions on the FP64 pipe per launch of the FP64 force-phase kernels
-# (ncu smsp__inst_executed_pipe_fp64.sum, one launch each, --clock-control none;
-# profiles/force64_*.md), per workload; they hold while the kernel sources hash
-# to FP64_INST_DIGEST, otherwise the ALU roofline is left unmeasured.
+# (ncu smsp__inst_executed_pipe_fp64.sum in the captures above), per workload;
+# without them the ALU roofline is left unmeasured.
 FP64_INST = {
-    "ensemble64": {"k_persistent<0, 1, 256>": 36245494, "k_sums<0, 1>": 32548173,
-                   "k_epilogue<0>": 1674592},
-    "compaction500": {"k_persistent<0, 1, 256>": 2784267, "k_persistent<0, 1, 128>": 2784259,
-                      "k_sums<0, 1>": 2492904, "k_epilogue<0>": 130368},
+    "compaction500": {"k_persistent<0, 1, 256, 1>": 1787088, "k_persistent<0, 1, 128, 1>": 1787680,
+                      "k_force_run<0>": 1625376, "k_epilogue<0, 2>": 130368},
 }
-FP64_INST_DIGEST = "1235532d82438481bf9c97cad09580c8b576d3ac"
 
 
 def _roof_fp64(sim, f_ms, path, workload, clk, hbm):
@@ -520,13 +525,10 @@ def _roof_fp64(sim, f_ms, path, workload, clk, hbm):
     phase (algorithmic bytes / duration) is reported beside it."""
     mhz = (clk or {}).get("sm_mhz") or 2070.0
     peak = N_SM * FP64_LANES_PER_SM_CYCLE * mhz * 1e6 / 1e12          # tera lane-ops/s
-    m, l = path["mode"], path["lanes"]
-    names = [f"k_persistent<0, {l}, {path.get('block', 128)}>"] if m & 1 else (
-        [f"k_sums<0, {l}>", f"k_epilogue<0>"] if (m >> 1) & 1 else [f"k_force<0, {l}>"])
-    table = FP64_INST.get(workload, {}) if kernel_digest() == FP64_INST_DIGEST else {}
+    m, names, table = path["mode"], force_kernel_names(path, False), captured(FP64_INST, workload)
     inst = sum(table[n] for n in names) if all(n in table for n in names) else None
     # the persistent kernel is the whole step: the displacement update's bytes too
-    per_node, per_bond = fp64_bytes(path, bool(m & 1))
+    per_node, per_bond = fp64_bytes(path, bool(m & 1), sim.N)
     nbytes = per_node * sim.N + per_bond * sim.n_bonds
     hbm_a = nbytes / (f_ms / 1e3) / 1e9
     achieved = None if inst is None else 32.0 * inst / (f_ms / 1e3) / 1e12
@@ -930,7 +932,7 @@ def run_ours(args):
                         + ("; the workload is too small to load 152 SMs, so the phase is latency-bound"
                            if sim.N < 100000 else "")}
     if prec == B.PD_FP64:
-        step_per_node, step_per_bond = fp64_bytes(tuned[key], True)
+        step_per_node, step_per_bond = fp64_bytes(tuned[key], True, sim.N)
     else:
         step_per_node, step_per_bond = fp32_bytes_per_node(tuned[key]["mode"], True), BYTES_PER_BOND_FP32
     step_bytes = step_per_node * sim.N + step_per_bond * sim.n_bonds
