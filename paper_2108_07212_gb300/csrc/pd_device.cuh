@@ -1510,27 +1510,110 @@ __device__ __forceinline__ T add_in_order(T acc, T v, int n) {
     return acc;
 }
 
+// Not a zero of either sign (no FP64 instruction).
+__device__ __forceinline__ bool nonzero(double v) { return (unsigned long long)__double_as_longlong(v) << 1; }
+__device__ __forceinline__ bool nonzero(float v) { return __float_as_uint(v) << 1; }
+
 // The n candidates of a node by its LANES threads, a candidate each:
 // pair(q, sx, sy, nx, ny) for candidate q; the forces are then added in the
 // order of the candidates, so the sums are those of one thread working through
 // them, in every thread of the node.  A contact is a chain of divisions and
-// square roots (FP64: about 4 us on the 2-lane pipe).  (Dealt to all threads of
-// the warp instead, every candidate began with a chain of loads for what its
-// node's threads hold: 19681 nodes settled, FP64, 4 threads per node, 27.7
-// us a step against 26.7, 8 threads 32.5 against 30.7, but 2 threads 26.1
-// against 30.2; 80171 nodes thrown at each other 62.8 against 57.9 with 4
-// threads, 63.0 against 60.5 with 2, FP32 split 28.7 against 26.6.)
+// square roots (FP64: about 4 us on the 2-lane pipe).  Four or eight threads
+// work through their own node's: see warp_contacts.  (FP64: additions of zeros
+// only, as most candidates lie beyond R_c, are left out; 28.0 to 27.6 us a step.)
 // Every thread of the warp calls it.
 template <int LANES, class T, class Pair>
 __device__ __forceinline__ void group_contacts(int lane, int n, T &Fsx, T &Fsy, T &Fnx, T &Fny, Pair pair) {
     for (int q0 = 0; __any_sync(0xffffffffu, q0 < n); q0 += LANES) {
         T a = 0, b = 0, c = 0, e = 0;
         if (q0 + lane < n) pair(q0 + lane, a, b, c, e);
-        __syncwarp();
-        Fsx = add_in_order<LANES>(Fsx, a, n - q0);
-        Fsy = add_in_order<LANES>(Fsy, b, n - q0);
-        Fnx = add_in_order<LANES>(Fnx, c, n - q0);
-        Fny = add_in_order<LANES>(Fny, e, n - q0);
+        if (sizeof(T) == 4 || __any_sync(0xffffffffu, nonzero(a) || nonzero(b))) {
+            Fsx = add_in_order<LANES>(Fsx, a, n - q0);
+            Fsy = add_in_order<LANES>(Fsy, b, n - q0);
+        }
+        if (sizeof(T) == 4 || __any_sync(0xffffffffu, nonzero(c) || nonzero(e))) {
+            Fnx = add_in_order<LANES>(Fnx, c, n - q0);
+            Fny = add_in_order<LANES>(Fny, e, n - q0);
+        }
+    }
+}
+
+// What a contact takes from its own node, handed from the node's thread to the
+// one that works on the contact.
+struct ContactNode64 {
+    double px, py, vx, vy;
+    int ii, gi, ag, r0, r1, nc, nb, pad;
+};
+struct ContactNode32 {
+    float4 q;
+    double vx, vy;
+    int ii, gi, ag, r0, r1, nc, nb, pad;
+};
+template <class Node>
+__device__ __forceinline__ Node shfl_node(const Node &v, int src) {
+    constexpr int kWords = sizeof(Node) / 4 - 1;          // (not the padding)
+    Node r;
+#pragma unroll
+    for (int w = 0; w < kWords; ++w)
+        reinterpret_cast<int *>(&r)[w] = __shfl_sync(0xffffffffu, reinterpret_cast<const int *>(&v)[w], src);
+    return r;
+}
+
+// The candidates of the nodes of a warp (several threads per node: thread 0 of
+// each gives its node and the number n of its candidates, the others n = 0), one
+// per thread, 32 at a time: pair(node, q, sx, sy, nx, ny) for candidate q of a
+// node.  Each node's forces are then added in the order of its candidates, into
+// its thread 0.  A contact is a chain of divisions and square roots (FP64: about
+// 4 us on the 2-lane pipe, which a warp occupies as long for one pair as for
+// 32), and few nodes of a warp have any.
+// Two threads per node share their contacts so: a node's own two take half as
+// many chains as it has candidates, one after the other.  A step of a settled
+// box of 19681 nodes, by the node's own threads and dealt to the warp, hot and
+// with L2 flushed: FP64, 2 threads 31.7 and 28.1, 46.2 and 43.6 us; 4 threads 27.9
+// and 28.7, 40.1 and 42.1; FP32 split, 2 threads 13.4 and 12.7, 4 threads 12.8 and
+// 13.3.  (Without the node's data handed over, each contact began with a chain of
+// loads for it: FP64, 2 threads 31.0, flushed 48.3.)
+// Every thread of the warp calls it.
+template <class T, class Node, class Pair>
+__device__ __forceinline__ void warp_contacts(const Node &mine, int n, T &Fsx, T &Fsy, T &Fnx, T &Fny, Pair pair) {
+    constexpr unsigned kAll = 0xffffffffu;
+    if (!__any_sync(kAll, n > 0)) return;
+    const int lane = threadIdx.x & 31;
+    int start = n;                          // exclusive prefix of n
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(kAll, start, off);
+        if (lane >= off) start += y;
+    }
+    const int total = __shfl_sync(kAll, start, 31);
+    start -= n;
+    for (int p0 = 0; p0 < total; p0 += 32) {
+        // pair p belongs to the last thread whose prefix is not beyond p
+        const int p = p0 + lane;
+        int own = 0;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1)
+            if (__shfl_sync(kAll, start, own + off) <= p) own += off;
+        const int q = p - __shfl_sync(kAll, start, own);
+        const Node node = shfl_node(mine, own);
+        T a = 0, b = 0, c = 0, e = 0;
+        if (p < total) pair(node, q, a, b, c, e);
+        // (most candidates lie beyond R_c; adding their zeros changes no sum)
+        const unsigned some = __ballot_sync(kAll, nonzero(a) || nonzero(b) || nonzero(c) || nonzero(e));
+        const int lo = max(start - p0, 0), hi = min(start + n - p0, 32);
+        unsigned left = hi > lo ? some & (kAll >> (32 - hi)) & (kAll << lo) : 0u;
+        while (__any_sync(kAll, left != 0u)) {
+            const int src = left ? __ffs(left) - 1 : lane;
+            const T va = __shfl_sync(kAll, a, src), vb = __shfl_sync(kAll, b, src);
+            const T vc = __shfl_sync(kAll, c, src), ve = __shfl_sync(kAll, e, src);
+            if (left) {
+                Fsx += va;
+                Fsy += vb;
+                Fnx += vc;
+                Fny += ve;
+            }
+            left &= left - 1u;
+        }
     }
 }
 
@@ -1681,6 +1764,19 @@ __device__ __forceinline__ void force_node64(const DevPtrs &d, const KParams &k,
     contact = nc + nb > 0;
     if constexpr (LANES == 1) {
         if (INLINE && contact) contacts64<PERSIST>(d, k, ii, vin, gi, nc, nb, r0, r1, pi, Fsx, Fsy, Fnx, Fny);
+    } else if constexpr (LANES == 2) {
+        ContactNode64 mine = {};
+        if (contact) {
+            const double2 vi = ldm<PERSIST>(&d.v[vin][ii]);
+            mine = {pi.x, pi.y, vi.x, vi.y, ii, gi, __ldg(&d.g_agg[gi]), r0, r1, nc, nb, 0};
+        }
+        warp_contacts(mine, lane == 0 ? nc + nb : 0, Fsx, Fsy, Fnx, Fny,
+                      [&](const ContactNode64 &x, int q, double &sx, double &sy, double &nx, double &ny) {
+                          const int j = candidate<PERSIST>(d, k, x.ii, x.nc, x.nb, x.r0, q);
+                          contact_pair64<PERSIST>(d, k, d.agg[x.ag], x.ii, j, vin, x.gi, x.r0, x.r1,
+                                                  make_double2(x.px, x.py), ldm<PERSIST>(&d.p[j]),
+                                                  make_double2(x.vx, x.vy), sx, sy, nx, ny);
+                      });
     } else {
         group_contacts<LANES>(lane, nc + nb, Fsx, Fsy, Fnx, Fny,
                               [&](int q, double &sx, double &sy, double &nx, double &ny) {
@@ -2249,13 +2345,33 @@ __device__ __forceinline__ void force_node32(const DevPtrs &d, const KParams &k,
     const int nc = active ? ldm<PERSIST>(&d.nbr_cnt[ii]) : 0;
     const int nb = fresh_bonds(d, k, ii, any_lane<LANES>(w0 != 0u || (note & ~kNoteGuard) ||
                                                          (active && !bonds && k.wpn > 1)));
-    group_contacts<LANES>(lane, nc + nb, Fsx, Fsy, Fnx, Fny,
-                          [&](int q, float &sx, float &sy, float &nx, float &ny) {
-                              const int j = candidate<PERSIST>(d, k, ii, nc, nb, r0, q);
-                              contact_pair32<PERSIST>(d, k, d.agg[ag], ii, j, vin, gi, r0, r1, phi, pli, gq, gc,
-                                                      ldm<PERSIST>(&cur_pq<PERSIST>(d)[j]), ldm<PERSIST>(&d.v[vin][ii]),
-                                                      sx, sy, nx, ny);
-                          });
+    if constexpr (LANES == 1) {
+        if (nc + nb > 0)
+            contacts32<PERSIST>(d, k, ii, vin, gi, nc, nb, r0, r1, phi, pli, gq, gc, Fsx, Fsy, Fnx, Fny);
+    } else if constexpr (LANES == 2) {
+        ContactNode32 mine = {};
+        if (nc + nb > 0) {
+            const double2 vi = ldm<PERSIST>(&d.v[vin][ii]);
+            mine = {qi, vi.x, vi.y, ii, gi, ag, r0, r1, nc, nb, 0};
+        }
+        warp_contacts(mine, lane == 0 ? nc + nb : 0, Fsx, Fsy, Fnx, Fny,
+                      [&](const ContactNode32 &x, int q, float &sx, float &sy, float &nx, float &ny) {
+                          const int j = candidate<PERSIST>(d, k, x.ii, x.nc, x.nb, x.r0, q);
+                          contact_pair32<PERSIST>(d, k, d.agg[x.ag], x.ii, j, vin, x.gi, x.r0, x.r1,
+                                                  make_float2(x.q.x, x.q.y), make_float2(x.q.z, x.q.w),
+                                                  __ldg(&d.gq[x.gi]), __ldg(&d.gc[x.gi]),
+                                                  ldm<PERSIST>(&cur_pq<PERSIST>(d)[j]), make_double2(x.vx, x.vy), sx, sy,
+                                                  nx, ny);
+                      });
+    } else {
+        group_contacts<LANES>(lane, nc + nb, Fsx, Fsy, Fnx, Fny,
+                              [&](int q, float &sx, float &sy, float &nx, float &ny) {
+                                  const int j = candidate<PERSIST>(d, k, ii, nc, nb, r0, q);
+                                  contact_pair32<PERSIST>(d, k, d.agg[ag], ii, j, vin, gi, r0, r1, phi, pli, gq, gc,
+                                                          ldm<PERSIST>(&cur_pq<PERSIST>(d)[j]), ldm<PERSIST>(&d.v[vin][ii]),
+                                                          sx, sy, nx, ny);
+                              });
+    }
     out.bx = lane_sum<LANES>(Fbx);
     out.by = lane_sum<LANES>(Fby);
     out.sx = Fsx;
