@@ -285,12 +285,15 @@ void compute_aggregates(pd_ctx *c) {
 // Contact grid of every aggregate: cells over its wall box at t = 0 and one
 // around it, at least 3 each way and at most four per node (two beyond 2^28
 // nodes, for 32-bit cell indices), 64 at least.  A box with more cells keeps
-// those of the nodes' extent at the start, the longer way first brought to the
-// shorter where even these are too many, and the rest is shared out to both ways
-// alike: cells that wrap around pile nodes up, so the populated ones must not.
+// those of the nodes' extent at the start, and the rest is shared out to both
+// ways alike: cells that wrap around pile nodes up, so the populated ones must
+// not.  Where even the extent has too many, the longer way is first brought to
+// four times the shorter, then both shrink alike.
 // (Shrinking the whole box alike left one of 23 mm by 33 km three cells across:
 // an evaluation with rebuilt lists, 19681 nodes FP64, took 217 us in it against 81
-// in the close-fitting box of 23 by 33 mm; now 76 in both.)
+// in the close-fitting box of 23 by 33 mm; now 81 in both.  Bringing the longer
+// way to the shorter instead of to four times it made rebuilds by one cluster up
+// to 6 us slower in boxes of about that shape.)
 void compute_grid(pd_ctx *c) {
     std::vector<double> most(c->n_agg, 0.0);
     for (int g = 0; g < c->G; ++g)
@@ -323,8 +326,11 @@ void compute_grid(pd_ctx *c) {
             double eh = std::min(gh[a], std::max(3.0, std::ceil((e[3] - e[2]) / A.cell) + 2));
             if (ew * eh > most[a]) {
                 double &lo = ew < eh ? ew : eh, &hi = ew < eh ? eh : ew;
-                lo = std::min(lo, std::floor(std::sqrt(most[a])));
-                hi = std::floor(most[a] / lo);
+                hi = std::min(hi, std::max(4 * lo, std::floor(most[a] / lo)));
+                if (lo * hi > most[a]) {
+                    lo = std::floor(lo * std::sqrt(most[a] / (lo * hi)));
+                    hi = std::floor(most[a] / lo);
+                }
             } else {
                 ew = std::min(gw[a], std::floor(ew * std::sqrt(most[a] / (ew * eh))));
                 eh = std::min(gh[a], std::floor(most[a] / ew));
