@@ -1640,10 +1640,11 @@ int pd_autotune(pd_ctx *c, double *report) {
     for (int m : {0, 1, 2, 3, 4, 6}) {
         for (int lanes : {1, 2, 4, 8}) {
             if (c->prm.lanes && lanes != c->prm.lanes) continue;
-            // with bond tiles the persistent kernel's fused force phase shares the
-            // contacts of few nodes among all warps; the split one leaves each to
-            // a thread, which a trial on a state with few contacts does not show
-            if (m == 3 && lanes == 1 && c->kp.pair) continue;
+            // the persistent kernel's fused force phase with bond tiles, or in FP64
+            // one thread per node, shares the contacts of few nodes among all warps;
+            // the split one leaves each to a thread, which a trial on a state with
+            // few contacts does not show
+            if (m == 3 && lanes == 1 && (c->kp.pair || !c->kp.fp32)) continue;
             cands.push_back({m, lanes, 128});
             if (m & 1) cands.push_back({m, lanes, 256});
         }
