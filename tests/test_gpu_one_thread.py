@@ -18,10 +18,10 @@ TOL = {B.PD_FP64: 1e-12, B.PD_FP32_SPLIT: 1e-5}
 PATHS = [(0, 1, 128), (2, 1, 128), (1, 1, 128), (1, 1, 256), (3, 1, 128), (3, 1, 256)]
 
 
-def _grains(n, ratio=3.0):
-    """Grains of every shape, about 412 nodes each."""
+def _grains(n, ratio=3.0, h_ratio=15):
+    """Grains of every shape, about 412 nodes each (h_ratio 32: 1900)."""
     s = (n / 50) ** 0.5
-    w = I.settling(n_grains=n, h_ratio=15, box=(20e-3 * s + 3e-3, 30e-3 * s + 3e-3), seed=3)
+    w = I.settling(n_grains=n, h_ratio=h_ratio, box=(20e-3 * s + 3e-3, 30e-3 * s + 3e-3), seed=3)
     w.params["horizon_ratio"] = ratio
     return w
 
@@ -38,6 +38,7 @@ CASES = {
     "few": lambda: I.two_disks(h_ratio=4, k_bulk=5e5),                     # fewer nodes than a block
     "below": lambda: _grains(int(0.9 * _edge())),                          # the last FP64 sizes without tiles
     "above": lambda: _grains(int(1.15 * _edge())),                         # the first with
+    "wide": lambda: _grains(int(1.15 * _edge() * 412 / 1900), 3.0, 32),    # with, two rows of 63 nodes
 }
 
 
